@@ -11,6 +11,7 @@
 #include "kernels.cuh"
 #include "kernels_tc.cuh"
 #include "plan.hpp"
+#include "split_args.hpp"
 #include "stationary_args.hpp"
 #include "tc_stationary.cuh"
 
@@ -45,7 +46,7 @@ int ensure_device(ftp_plan* p)
         cudaFuncSetAttribute(bwd_group_tc_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemBudget) != cudaSuccess ||
         cudaFuncSetAttribute(filter_grad_tc_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcFgSmemBudget) != cudaSuccess ||
         cudaFuncSetAttribute(conv_tc_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcConvSmemBudget) != cudaSuccess ||
-        !st_prepare_device())
+        !st_prepare_device() || !split_prepare_device())
         return FTP_ERR_CUDA;
     if (!p->grad_stream) {
         cudaStream_t gs;
@@ -112,13 +113,32 @@ void fill_common(const ftp_plan* p, const GroupPlan& g, bool backward, const flo
     a.params = params;
 }
 
-int pack_filters(ftp_plan* p, const float* params, void* ws, cudaStream_t st)
+inline int* err_ptr(void* ws, const ftp_plan* p) { return reinterpret_cast<int*>(static_cast<unsigned char*>(ws) + p->ws.err_off); }
+
+// clear_error: the first launch of a pass that starts afresh also clears the error word of the split kernels' bounded waits
+int pack_filters(ftp_plan* p, const float* params, void* ws, bool clear_error, cudaStream_t st)
 {
     PackArgs pa{};
+    SplitPackArgs sa{};
+    sa.error = clear_error ? err_ptr(ws, p) : nullptr;
+    auto flush_split = [&]() {
+        if (!sa.n) return;
+        Timed t(p, st, 0, -1);
+        split_launch_pack(sa, params, st);
+        sa.n = sa.tiles = 0;
+    };
     for (const GroupPlan& g : p->groups)
         for (int i = 0; i < g.n_ops; ++i) {
             const OpDesc& op = g.fwd_ops[i];
             if (op.kind == kOpPool) continue;
+            if (g.sp.on) {
+                if (sa.n == kSplitPackLayers) flush_split();
+                uint4* base = reinterpret_cast<uint4*>(ws_ptr(ws, p->ws.sw_off));
+                sa.l[sa.n++] = SplitPackLayer{op.p_off, base + g.sp.wf_off, base + g.sp.wd_off, op.cin, op.cout, op.k, op.cin16, op.cout16,
+                                              g.sp.f.Ns, g.sp.f.kpc, g.sp.d.Ns, g.sp.d.kpc, sa.tiles};
+                sa.tiles += ((op.cin16 + 31) / 32) * ((op.cout16 + 31) / 32);
+                continue;
+            }
             if (pa.n == kMaxOps * 2) {   // flush a full batch
                 { Timed t(p, st, 0, -1);
                   pack_filters_kernel<<<dim3(64, pa.n), 256, 0, st>>>(pa, params, ws_ptr(ws, p->ws.wf_off), ws_ptr(ws, p->ws.wb_off)); }
@@ -130,11 +150,11 @@ int pack_filters(ftp_plan* p, const float* params, void* ws, cudaStream_t st)
         Timed t(p, st, 0, -1);
         pack_filters_kernel<<<dim3(64, pa.n), 256, 0, st>>>(pa, params, ws_ptr(ws, p->ws.wf_off), ws_ptr(ws, p->ws.wb_off));
     }
+    flush_split();
     return launched_ok() ? FTP_OK : FTP_ERR_CUDA;
 }
 
 inline bool is_tc(const ftp_plan* p) { return p->precision == FTP_BF16_FP32ACC; }
-inline int* err_ptr(void* ws, const ftp_plan* p) { return reinterpret_cast<int*>(static_cast<unsigned char*>(ws) + p->ws.err_off); }
 // Shared memory requested per block, so that exactly `ctas` blocks share an SM and the tensor memory
 // they allocate (512 / ctas columns each) is always available: more than half of the SM's 228 KB for
 // one block, more than a third for two.
@@ -190,6 +210,27 @@ bool encode_rows_map(unsigned char out[128], const void* base, int N, int planes
     CUtensorMap m;
     if (enc(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return false;
+    std::memcpy(out, &m, 128);
+    return true;
+}
+
+// Tensor map of a split map (three parts of bf16 planes, this GPU's memory) as flat planes {entries, planes, parts}, or as rows
+// {columns, rows, planes, parts}; an entry is two 8-byte elements, entries outside read as zeros.
+bool encode_split_map(unsigned char out[128], const uint4* base, const SplitGeom& g, bool rows, int box_x, int box_rows, int box_planes, int box_parts)
+{
+    tensor_map_encode_fn enc = tensor_map_encoder();
+    if (!enc || box_x > 128 || box_rows > 256) return false;
+    cuuint64_t dims[4]; cuuint64_t strides[3]; cuuint32_t box[4]; const cuuint32_t estr[4] = {1, 1, 1, 1};
+    int d = 0;
+    dims[d] = 2 * (cuuint64_t)(rows ? g.wp : g.tp); box[d++] = 2 * (cuuint32_t)box_x;
+    if (rows) { strides[d - 1] = (cuuint64_t)g.wp * 16; dims[d] = (cuuint64_t)g.rows; box[d++] = (cuuint32_t)box_rows; }
+    strides[d - 1] = (cuuint64_t)g.tp * 16; dims[d] = (cuuint64_t)g.planes; box[d++] = (cuuint32_t)box_planes;
+    strides[d - 1] = (cuuint64_t)g.planes * g.tp * 16; dims[d] = 3; box[d++] = (cuuint32_t)box_parts;
+    CUtensorMap m;
+    if (enc(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, d, const_cast<uint4*>(rows ? base + kSplitLead : base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return false;
     std::memcpy(out, &m, 128);
     return true;
@@ -418,13 +459,105 @@ bool stationary_backward(ftp_plan* p, const GroupPlan& g, int gi, const float* x
     return true;
 }
 
+// ---- split groups (split.cuh): one-conv groups of the fp32 path on the tensor cores ----
+inline uint4* split_ptr(void* ws, size_t off) { return reinterpret_cast<uint4*>(static_cast<unsigned char*>(ws) + off); }
+inline SplitGeom in_geom(const ftp_plan* p, const OpDesc& op) { return split_geom(p->N, op.cin, op.in_H, op.in_W); }      // input map
+inline SplitGeom dz_geom(const ftp_plan* p, const OpDesc& op) { return split_geom(p->N, op.cout, op.in_H, op.in_W); }     // conv output
+inline SplitGeom out_geom(const ftp_plan* p, const OpDesc& op) { return split_geom(p->N, op.cout, op.out_H, op.out_W); }  // after the pool
+inline bool split_at(const ftp_plan* p, int gi) { return gi >= 0 && gi < (int)p->groups.size() && p->groups[gi].sp.on; }
+
+bool split_conv_args(SplitConvArgs& a, const SplitConvPlan& c, const uint4* in, const SplitGeom& g, int K, int cout, int cout16)
+{
+    a.in = in;
+    a.g = g; a.K = K; a.nchunks = c.nchunks; a.kpc = c.kpc; a.cout = cout; a.cout16 = cout16;
+    a.Ns = c.Ns; a.slices = c.slices; a.nblk = c.nblk; a.mode = c.mode; a.R = c.R; a.Cw = c.Cw; a.tiles_x = c.tiles_x; a.tiles_y = c.tiles_y;
+    a.pitch = c.pitch; a.run_len = c.run_len; a.items = c.items;
+    a.a_plane = c.a_plane; a.a_bytes = c.a_bytes; a.a_block = K == 1 && c.mode == kSplitFlat ? 3 * c.kpc * 128 : 128; a.a_stages = c.a_stages; a.b_stage = c.b_stage; a.b_stages = c.b_stages; a.pool_bytes = c.pool_bytes;
+    if (c.mode != kSplitFlat) return encode_split_map(a.tmap, in, g, true, c.pitch, c.nruns, c.kpc, 3);
+    return K == 3 || encode_split_map(a.tmap, in, g, false, 128, 0, c.kpc, 3);
+}
+
+bool split_forward(ftp_plan* p, const GroupPlan& g, int gi, const float* x, const float* params, void* ws, cudaStream_t st)
+{
+    const OpDesc& op = g.fwd_ops[0];
+    uint4* in = split_ptr(ws, g.sp.in_off);
+    if (!split_at(p, gi - 1)) {                     // the group below wrote an fp32 map
+        Timed t(p, st, 9, gi);
+        split_launch_planes(map_ptr(p, x, ws, g.first), in, in_geom(p, op), op.cin, st);
+    }
+    SplitConvArgs a{};
+    if (!split_conv_args(a, g.sp.f, in, in_geom(p, op), op.k, op.cout, op.cout16)) return false;
+    a.w = split_ptr(ws, p->ws.sw_off) + g.sp.wf_off;
+    a.bias = params + op.p_off + (size_t)op.cout * op.cin * op.k * op.k;
+    a.error = err_ptr(ws, p); a.slope = op.slope; a.act = 1;
+    a.og = out_geom(p, op);
+    if (op.kind == kOpConvPool) a.arg = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(ws) + p->ws.arg_off[op.out_map - 1]);
+    if (split_at(p, gi + 1)) a.out_s = split_ptr(ws, p->groups[gi + 1].sp.in_off);
+    else a.out_f = const_cast<float*>(map_ptr(p, x, ws, op.out_map));
+    { Timed t(p, st, 1, gi);
+      split_launch_conv(a, g.sp.f.nb, g.sp.f.blocks, g.sp.f.smem, st); }
+    return launched_ok();
+}
+
+// dz (made here from the fp32 delta `dout`, unless the split group above has written it), filter gradient, and the input
+// delta: straight into the dz map of a split group below, else fp32 NCHW to `din` (null: not wanted).
+bool split_backward(ftp_plan* p, const GroupPlan& g, int gi, const float* x, const float* dout, float* din, void* ws, cudaStream_t st)
+{
+    const OpDesc& op = g.bwd_ops[0];
+    uint4* dz = split_ptr(ws, p->ws.sdz_off[gi & 1]);
+    if (!split_at(p, gi + 1)) {
+        SplitDeltaArgs d{};
+        d.d = dout; d.y = map_ptr(p, x, ws, op.out_map); d.dz = dz; d.g = dz_geom(p, op); d.low = out_geom(p, op);
+        d.C = op.cout; d.slope = op.slope; d.pool = op.kind == kOpConvPool ? 1 : 0;
+        if (d.pool) d.arg = reinterpret_cast<const unsigned long long*>(static_cast<unsigned char*>(ws) + p->ws.arg_off[op.out_map - 1]);
+        { Timed t(p, st, 6, gi);
+          split_launch_delta(d, st); }
+    }
+    {
+        const SplitFgPlan& t = g.sp.g;
+        SplitFgArgs f{};
+        f.dz = dz; f.x = split_ptr(ws, g.sp.in_off); f.g = dz_geom(p, op); f.x_planes = op.cin16 / 8;
+        f.partial = ws_ptr(ws, g.partial_off); f.set_floats = (long long)g.split_set_floats; f.tgp_off = op.tgp_off;
+        f.error = err_ptr(ws, p);
+        f.K = op.k; f.cout16 = op.cout16; f.cin16 = op.cin16;
+        f.Ms = t.Ms; f.slices = t.slices; f.ncols = t.ncols; f.units = t.units; f.nci = t.nci; f.rows3 = t.rows3;
+        f.E = t.E; f.e_lo = kSplitLead + f.g.wp; f.stages_total = t.stages_total; f.shares = t.shares;
+        f.nstages = t.nstages; f.stage_bytes = t.stage_bytes; f.x_entries = t.x_entries; f.dz_box = t.dz_box; f.x_box = t.x_box;
+        if (!encode_split_map(f.tmap_dz, dz, f.g, false, t.E, 0, t.dz_box, 3) ||
+            !encode_split_map(f.tmap_x, f.x, in_geom(p, op), false, t.x_entries, 0, t.x_box, 3)) return false;
+        Timed tm(p, st, 7, gi);
+        split_launch_fgrad(f, t.blocks, t.smem, st);
+    }
+    if (!launched_ok()) return false;
+    const bool below = split_at(p, gi - 1);
+    if (!below && !din) return true;
+    SplitConvArgs a{};
+    if (!split_conv_args(a, g.sp.d, dz, dz_geom(p, op), op.k, op.cin, op.cin16)) return false;
+    a.w = split_ptr(ws, p->ws.sw_off) + g.sp.wd_off; a.error = err_ptr(ws, p);
+    if (below) {
+        const OpDesc& lo = p->groups[gi - 1].fwd_ops[0];
+        a.out_s = split_ptr(ws, p->ws.sdz_off[(gi - 1) & 1]); a.og = dz_geom(p, lo);
+        a.prev_y = split_ptr(ws, g.sp.in_off); a.prev_slope = lo.slope;
+        if (lo.kind == kOpConvPool) a.prev_arg = reinterpret_cast<const unsigned long long*>(static_cast<unsigned char*>(ws) + p->ws.arg_off[lo.out_map - 1]);
+    } else {
+        a.out_f = din; a.og = a.g;
+    }
+    { Timed t(p, st, 8, gi);
+      split_launch_conv(a, g.sp.d.nb, g.sp.d.blocks, g.sp.d.smem, st); }
+    return launched_ok();
+}
+
 int forward_impl(ftp_plan* p, const float* x, const float* params, float* y, void* ws, cudaStream_t st)
 {
     if (is_tc(p)) return forward_tc(p, x, params, y, ws, st);
-    int rc = pack_filters(p, params, ws, st);
+    int rc = pack_filters(p, params, ws, true, st);
     if (rc != FTP_OK) return rc;
     for (size_t gi = 0; gi < p->groups.size(); ++gi) {
         const GroupPlan& g = p->groups[gi];
+        if (g.sp.on) {
+            if (!split_forward(p, g, (int)gi, x, params, ws, st)) return FTP_ERR_CUDA;
+            continue;
+        }
         if (g.st.on) {
             if (!stationary_forward(p, g, (int)gi, x, params, ws, st)) return FTP_ERR_CUDA;
             continue;
@@ -452,7 +585,7 @@ TcReduceLayer reduce_layer(const GroupPlan& g, const OpDesc& op, void* ws)
     if (g.col_cin16)
         return TcReduceLayer{op.p_off, ws_ptr(ws, g.partial_off), (long long)g.param_floats, op.tgp_off, g.sets(), g.col_cin, op.cout, 1,
                              g.col_cin16, op.cout16};
-    return TcReduceLayer{op.p_off, ws_ptr(ws, g.partial_off), (long long)g.param_floats, op.tgp_off, g.sets(), op.cin, op.cout, op.k,
+    return TcReduceLayer{op.p_off, ws_ptr(ws, g.partial_off), (long long)g.set_floats(), op.tgp_off, g.sets(), op.cin, op.cout, op.k,
                          op.cin16, op.cout16};
 }
 
@@ -615,6 +748,16 @@ int reduce_group_and_notify(ftp_plan* p, int gi, float* grad_out, void* ws, cuda
 {
     const GroupPlan& g = p->groups[gi];
     if (g.param_floats == 0) return FTP_OK;
+    if (g.sp.on) {
+        TcReduceArgs rg{};
+        rg.n = 1;
+        rg.l[0] = reduce_layer(g, g.bwd_ops[0], ws);
+        { Timed t(p, st, 5, gi);
+          reduce_sgd_tc_kernel<<<dim3(1184, 1), 128, 0, st>>>(rg, nullptr, 0.f, grad_out); }
+        if (!launched_ok()) return FTP_ERR_CUDA;
+        p->group_ready(p->group_ready_user, gi, g.param_begin, (long long)g.param_floats);
+        return FTP_OK;
+    }
     ReduceArgs ra{};
     ra.n = 1;
     ra.g[0] = ReduceGroup{g.param_begin, (long long)g.param_floats, ws_ptr(ws, g.partial_off), g.bwd.blocks};
@@ -636,6 +779,13 @@ int backward_impl(ftp_plan* p, const float* x, const float* dy, const float* par
     const int G = (int)p->groups.size();
     for (int gi = G - 1; gi >= 0; --gi) {
         const GroupPlan& g = p->groups[gi];
+        if (g.sp.on) {
+            const float* dout = gi == G - 1 ? dy : ws_ptr(ws, p->ws.dmap_off[gi + 1]);
+            float* din = gi == 0 ? dx : ws_ptr(ws, p->ws.dmap_off[gi]);
+            if (!split_backward(p, g, gi, x, dout, din, ws, st)) return FTP_ERR_CUDA;
+            if (p->group_ready) { const int rc = reduce_group_and_notify(p, gi, grad_out, ws, st); if (rc != FTP_OK) return rc; }
+            continue;
+        }
         if (g.st.on) {
             const float* dout = gi == G - 1 ? dy : ws_ptr(ws, p->ws.dmap_off[gi + 1]);
             float* din = gi == 0 ? dx : ws_ptr(ws, p->ws.dmap_off[gi]);
@@ -678,18 +828,36 @@ int backward_impl(ftp_plan* p, const float* x, const float* dy, const float* par
             p->fg_pending[turn] = false;
         }
     if (p->group_ready) return FTP_OK;       // every group's sets were summed right after its backward pass
-    ReduceArgs ra{};
+    TcReduceArgs rt{};
+    auto flush_split = [&]() {
+        if (!rt.n) return;
+        Timed t(p, st, 5, -1);
+        reduce_sgd_tc_kernel<<<dim3(1184, rt.n), 128, 0, st>>>(rt, sgd_params, lr, grad_out);
+        rt.n = 0;
+    };
     for (const GroupPlan& g : p->groups) {
-        if (g.param_floats == 0) continue;
+        if (!g.sp.on) continue;
+        if (rt.n == kMaxOps * 2) flush_split();
+        rt.l[rt.n++] = reduce_layer(g, g.bwd_ops[0], ws);
+    }
+    flush_split();
+    // the other groups, whose sets are arranged like the parameters: a launch per contiguous run of them
+    ReduceArgs ra{};
+    auto flush_run = [&]() {
+        if (!ra.n) return;
+        const long long first = ra.g[0].begin, total = ra.g[ra.n - 1].begin + ra.g[ra.n - 1].floats;
+        const int blocks = (int)std::min<long long>((total - first + 255) / 256, (long long)kSmCount * 16);
+        Timed t(p, st, 5, -1);
+        reduce_sgd_kernel<<<blocks, 256, 0, st>>>(ra, first, total, sgd_params, lr, grad_out);
+        ra.n = 0;
+    };
+    for (const GroupPlan& g : p->groups) {
+        if (g.sp.on) flush_run();
+        if (g.sp.on || g.param_floats == 0) continue;
         ra.g[ra.n++] = ReduceGroup{g.param_begin, (long long)g.param_floats, ws_ptr(ws, g.partial_off), g.bwd.blocks};
     }
-    if (ra.n) {
-        const long long total = (long long)p->param_floats;
-        const int blocks = (int)std::min<long long>((total + 255) / 256, (long long)kSmCount * 16);
-        { Timed t(p, st, 5, -1);
-          reduce_sgd_kernel<<<blocks, 256, 0, st>>>(ra, 0, total, sgd_params, lr, grad_out); }
-        if (!launched_ok()) return FTP_ERR_CUDA;
-    }
+    flush_run();
+    if (!launched_ok()) return FTP_ERR_CUDA;
     return FTP_OK;
 }
 
@@ -858,7 +1026,7 @@ int ftp_backward(ftp_plan* plan, const float* x, const float* dy, const float* p
     int rc = ensure_device(plan);
     if (rc != FTP_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    rc = is_tc(plan) ? pack_filters_tc(plan, params, workspace, st) : pack_filters(plan, params, workspace, st);
+    rc = is_tc(plan) ? pack_filters_tc(plan, params, workspace, st) : pack_filters(plan, params, workspace, false, st);
     if (rc != FTP_OK) return rc;
     return backward_impl(plan, x, dy, params, dx, dparams, nullptr, 0.f, workspace, st);
 }
@@ -1061,7 +1229,7 @@ int ftp_plan_check(ftp_plan* plan, void* workspace, void* stream)
 {
     if (!plan || !workspace) return FTP_ERR_ARG;
     if (cudaStreamSynchronize(static_cast<cudaStream_t>(stream)) != cudaSuccess) return FTP_ERR_CUDA;
-    if (!is_tc(plan)) return FTP_OK;
+    if (!is_tc(plan) && !plan->split) return FTP_OK;
     int word = 0;
     if (cudaMemcpy(&word, err_ptr(workspace, plan), 4, cudaMemcpyDeviceToHost) != cudaSuccess) return FTP_ERR_CUDA;
     return word ? FTP_ERR_TIMEOUT : FTP_OK;

@@ -3,6 +3,7 @@
 // generalised with explicit padding, sub-tiling for shared memory, workspace layout.
 // Pure C++; no CUDA calls.
 #include "plan.hpp"
+#include "split_args.hpp"
 
 #include <algorithm>
 #include <cmath>
@@ -638,6 +639,165 @@ void plan_stationary(const ftp_plan& p, GroupPlan& g, const PlanOpts& o)
     }
 }
 
+// ---- split kernels (split.cuh) ----
+inline double split_mma_cycles(int n) { return std::max(32.0 + n / 4.0, n / 2.0); }   // both operands in shared memory
+
+// Launch shape of conv_split_kernel.  Items are 128-entry blocks of the flat batch where the halo of a flat run fits, else
+// (wide maps, and always with a pool) tiles of R rows x Cw columns; the candidate with the least rounds of items over the
+// SMs x time of a chunk (tensor pipe, or loads at 22 bytes a cycle) wins.
+SplitConvPlan plan_split_conv(const SplitGeom& g, int K, int cout16, bool pool)
+{
+    SplitConvPlan best;
+    double best_cost = -1;
+    const int kpc = K == 3 ? 2 : std::min(4, g.planes), nchunks = (g.planes + kpc - 1) / kpc;
+    const int room = kSplitSmemBudget - kSplitHeader;
+    int slices = 0, Ns = 0, nb = 0;
+    auto consider = [&](int mode, int nblk, int R, int Cw) {
+        SplitConvPlan c;
+        c.Ns = Ns; c.slices = slices; c.nb = nb; c.nblk = nblk; c.kpc = kpc; c.nchunks = nchunks; c.mode = mode;
+        long long tiles;
+        if (mode == kSplitFlat) {
+            c.nruns = 1; c.run_len = nblk * 128 + (K == 3 ? 2 * g.wp + 2 : 0); c.pitch = g.wp;
+            c.a_plane = K == 1 ? 2048 : (int)align_up((size_t)c.run_len * 16, 128);
+            c.a_bytes = 3 * kpc * c.a_plane * (K == 1 ? nblk : 1);
+            tiles = (g.tp + nblk * 128 - 1) / (nblk * 128);
+        } else {
+            c.R = R; c.Cw = Cw; c.pitch = c.run_len = Cw + K - 1; c.nruns = R + K - 1;
+            if (c.pitch > 128 || c.nruns > 256) return;              // one box of a tensor map
+            c.a_plane = c.nruns * c.pitch * 16;                      // (blocks may read on into the planes behind: rows of no pixel)
+            c.a_bytes = (int)align_up((size_t)3 * kpc * c.a_plane, 128);
+            const int W = mode == kSplitPool ? g.W : g.wp, Hh = mode == kSplitPool ? g.H : g.rows;
+            c.tiles_x = (W + Cw - 1) / Cw; c.tiles_y = (Hh + R - 1) / R;
+            tiles = (long long)c.tiles_x * c.tiles_y * (mode == kSplitPool ? g.N : 1);
+        }
+        c.pool_bytes = pool ? nblk * 128 * 16 * 4 : 0;
+        c.b_stage = K * K * kpc * Ns * 16;
+        const int a_bytes = c.a_bytes;
+        c.a_stages = std::min(3, std::max(2, (K == 1 ? 3 : 2)));
+        for (; c.a_stages >= 2; --c.a_stages) {
+            c.b_stages = std::min(K == 1 ? 8 : 5, (room - c.pool_bytes - c.a_stages * a_bytes) / c.b_stage);
+            if (c.b_stages >= 3) break;
+        }
+        if (c.a_stages < 2 || a_bytes >= (1 << 20)) return;
+        const long long items = tiles * slices;
+        if (items > 0x7fffffffLL) return;
+        c.items = (int)items; c.blocks = (int)std::min<long long>(items, kSmCount);
+        c.smem = kSplitHeader + c.a_stages * a_bytes + c.b_stages * c.b_stage + c.pool_bytes;
+        const double mma = nblk * (K * K * 6.0 * (kpc / 2)) * split_mma_cycles(Ns);
+        const double load = (3.0 * kpc * c.nruns * c.run_len * 16 + 3.0 * c.b_stage) / 22.0;
+        const double cost = (double)((items + kSmCount - 1) / kSmCount) * (nchunks * std::max(mma, load) + 300.0) + nchunks * 200.0;
+        if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = c; best.on = 1; }
+    };
+    for (int most = 128; most >= 32; most /= 2) {        // narrower slices where they fill the SMs
+        slices = (cout16 + most - 1) / most; Ns = round_up((cout16 + slices - 1) / slices, 16);
+        if (most < 128 && Ns > most) continue;
+        nb = Ns <= 32 ? 4 : Ns <= 64 ? 2 : 1;
+        for (int nblk = 2 * nb; nblk >= 1; nblk /= 2) {
+            if (!pool) consider(kSplitFlat, nblk, 0, 0);
+            const int W = pool ? g.W : g.wp, Hh = pool ? g.H : g.rows, step = pool ? 2 : 1;
+            if (!pool && K == 1) continue;
+            for (int ncx = 1; ncx <= 24; ++ncx) {
+                const int Cw = round_up((W + ncx - 1) / ncx, step);
+                const int pitch = Cw + K - 1;
+                int R = std::min(nblk * 128 / pitch, Hh) / step * step;
+                if (R < step) continue;
+                const int bands = (Hh + R - 1) / R;
+                R = round_up((Hh + bands - 1) / bands, step);
+                if (R * pitch > nblk * 128) continue;
+                consider(pool ? kSplitPool : kSplitTile, nblk, R, Cw);
+            }
+        }
+    }
+    return best;
+}
+
+// Launch shape of fgrad_split_kernel: (slices of 64 or 128 output channels) x (slices of the input channels) x (window
+// rows) roles, each with `shares` equal runs of the stages: the number of shares with the fewest rounds of blocks per
+// share of the work, a partial set counted as a few microseconds of the reduction.
+SplitFgPlan plan_split_fg(const SplitGeom& g, int K, int cin16, int cout16)
+{
+    SplitFgPlan t;
+    t.Ms = cout16 <= 64 ? 64 : 128;
+    t.slices = (cout16 + t.Ms - 1) / t.Ms;
+    if (K == 3 && cin16 <= 32) { t.rows3 = 1; t.units = 3; t.ncols = cin16; t.nci = 1; }
+    else if (K == 3) { t.units = 3; t.nci = (cin16 + 127) / 128; t.ncols = round_up((cin16 + t.nci - 1) / t.nci, 16); }
+    else {
+        t.units = cin16 <= 128 ? 1 : 2;
+        const int per = 128 * t.units;
+        t.nci = (cin16 + per - 1) / per;
+        t.ncols = round_up(((cin16 + t.nci - 1) / t.nci + t.units - 1) / t.units, 16);
+    }
+    const int xpl = t.ncols / 8 * (K == 1 ? t.units : 1), tiles = t.rows3 ? 3 : 1;
+    for (t.E = 64; t.E >= 32; t.E /= 2) {
+        t.x_entries = t.E + (K == 3 ? (t.rows3 ? 8 : 2) : 0);           // (rows3: the three tiles start at multiples of 128 bytes)
+        t.stage_bytes = (int)align_up((size_t)3 * (t.Ms / 8 * t.E + tiles * xpl * t.x_entries) * 16, 128);
+        t.dz_box = std::min(t.Ms, cout16) / 8; t.x_box = xpl;
+        t.nstages = std::min(4, (kSplitSmemBudget - kSplitHeader) / t.stage_bytes);
+        if (t.nstages >= 2) break;
+    }
+    if (t.nstages < 2) return SplitFgPlan{};
+    t.smem = kSplitHeader + t.nstages * t.stage_bytes;
+    t.stages_total = ((g.rows - 2) * g.wp + t.E - 1) / t.E;
+    const int roles = t.slices * t.nci * (t.rows3 ? 1 : K);
+    double best = -1;
+    const double set_cost = (double)K * K * cin16 * cout16 * 8.0 / 5e6 * 1900.0;        // cycles to write and read one set of the layer
+    const double stage_cost = (K == 1 ? t.units : t.rows3 ? 9 : 3) * (t.E / 16) * 6 * (t.rows3 ? 26.0 : split_mma_cycles(t.ncols));
+    for (int shares = 1; shares <= std::min(t.stages_total, std::max(1, 2 * kSmCount / roles)); ++shares) {
+        const double rounds = (double)((roles * shares + kSmCount - 1) / kSmCount);
+        const double cost = rounds * (((t.stages_total + shares - 1) / shares) * stage_cost + 6000.0) + shares * set_cost;
+        if (best < 0 || cost < best) { best = cost; t.shares = shares; }
+    }
+    t.blocks = roles * t.shares;
+    return t;
+}
+
+// Whether the fp32 plan runs its one-conv groups on the split kernels: with the default options, and only where the layers
+// they take (1x1 or 3x3 window, at least 32 input channels) amount to kSplitMinMacs multiply-accumulates an image in a
+// forward pass.  Below that (the 8-layer stack on images of less than about 80 x 80 pixels) a step is mostly launches and
+// latencies, and the CUDA-core kernels, whose sums have the order of the fused stacks, keep the result bit-identical under
+// every grouping profile.  The rule does not look at the batch, so that the parts of a batch that is dealt out to several
+// replicas run as the whole does.
+bool split_wanted(const ftp_plan& p, const PlanOpts& o)
+{
+    if (p.precision != FTP_FP32 || o.stationary != 0) return false;
+    double macs = 0;
+    for (size_t i = 0; i < p.layers.size(); ++i) {
+        const ftp_layer& l = p.layers[i];
+        if (l.kind == FTP_CONV && (l.k == 1 || l.k == 3) && l.cin >= kStatMinCin)
+            macs += (double)p.maps[i].H * p.maps[i].W * l.cin * l.cout * l.k * l.k;
+    }
+    return macs >= kSplitMinMacs;
+}
+
+void plan_split(const ftp_plan& p, GroupPlan& g)
+{
+    g.sp = SplitPlan{};
+    if (!p.split || !g.st.on || g.st.thin) return;
+    const OpDesc& op = g.fwd_ops[0];
+    if (op.cin < kStatMinCin || op.in_W > 1008) return;
+    const SplitGeom in = split_geom(p.N, op.cin, op.in_H, op.in_W), out = split_geom(p.N, op.cout, op.in_H, op.in_W);
+    if ((long long)in.N * (in.H + 1) * in.wp > 0x3fffffffLL) return;
+    g.sp.f = plan_split_conv(in, op.k, op.cout16, op.kind == kOpConvPool);
+    g.sp.d = plan_split_conv(out, op.k, op.cin16, false);
+    g.sp.g = plan_split_fg(in, op.k, op.cin16, op.cout16);
+    g.sp.on = g.sp.f.on && g.sp.d.on && g.sp.g.shares > 0;
+}
+// 16-byte entries of one packed arrangement
+inline long long split_w_entries(const SplitConvPlan& c, int k) { return (long long)c.slices * c.nchunks * 3 * k * k * c.kpc * c.Ns; }
+
+// Time of one pass of a group on the split kernels: six products at the measured rate of the kernels, maps at 4 TB/s.
+double split_estimate_us(const ftp_plan& p, const GroupPlan& g, bool backward, bool need_dx)
+{
+    const OpDesc& op = g.fwd_ops[0];
+    const double px = (double)p.N * op.in_H * op.in_W, flops = 2.0 * px * op.cin16 * op.cout16 * op.k * op.k;
+    auto rate = [](int n) { return 150e6 * std::min(1.0, n / 2.0 / split_mma_cycles(n)); };
+    const double in_us = px * op.cin16 * 6.0 / 4e6, out_us = px * op.cout16 * 6.0 / 4e6;
+    if (!backward) return flops / rate(g.sp.f.Ns) + in_us + out_us + 10.0;
+    double t = flops / rate(g.sp.g.rows3 ? 40 : g.sp.g.ncols) * (128.0 / g.sp.g.Ms) + in_us + out_us + 12.0;
+    if (need_dx) t += flops / rate(g.sp.d.Ns) + in_us + out_us + 10.0;
+    return t;
+}
+
 // bf16 path: whether a conv layer runs as a group of its own with the weight-stationary filter gradient: window 1
 // or 3, rows of at most 256 tile entries, a saved bf16 map as input, i.e. not the first layer.  (Measured on B200
 // this beats the fused sub-tile stacks for every such layer of the YOLO stacks, by 2x to 6x for the backward pass of
@@ -924,6 +1084,8 @@ int make_group(const ftp_plan& p, const LayerOffsets& lo, int first, int last, c
                            g.bwd.y.scratch_off[g.bwd.y.count] *
                            g.bwd.x.scratch_off[g.bwd.x.count];
     plan_stationary(p, g, o);
+    plan_split(p, g);
+    g.split_set_floats = (size_t)tgp;
     plan_tc_filter_grad(p, g, o);
     // bf16 path: the fused kernels keep all output channels of an op in the 512 tensor-memory columns; wider layers
     // run on the banded kernels (a group of their own) or not at all
@@ -986,6 +1148,7 @@ int build_plan(ftp_plan& p, const ftp_layer* layers, int n_layers, int N, int C,
             return FTP_ERR_LAYERS;
         }
     }
+    p.split = split_wanted(p, popts);
     p.param_floats = (size_t)params;
     p.wf_floats = (size_t)(tcp ? twf : wf);
     p.wb_floats = (size_t)(tcp ? twf : wb);
@@ -1011,6 +1174,7 @@ int build_plan(ftp_plan& p, const ftp_layer* layers, int n_layers, int N, int C,
     // puts it at least 3 % ahead; the margin keeps the model's error (about 10 % per group) from
     // trading a measured-good default for a predicted tie.
     auto estimate = [&](const GroupPlan& g) {
+        if (g.sp.on) return split_estimate_us(p, g, false, false) + split_estimate_us(p, g, true, g.first > 1);
         if (g.st.on) return stationary_estimate_us(p, g, false, false) + stationary_estimate_us(p, g, true, g.first > 1);
         if (g.tfg.on) return tc_stationary_estimate_us(p, g, false, false) + tc_stationary_estimate_us(p, g, true, g.first > 1);
         double f[kCostTerms];
@@ -1131,8 +1295,12 @@ int build_plan(ftp_plan& p, const ftp_layer* layers, int n_layers, int N, int C,
                 if (op.kind == kOpConvPool) ws.arg_off[op.out_map - 1] = take((size_t)N * c16 * s.H * s.W);
                 continue;
             }
-            ws.map_off[op.out_map - 1] = take((size_t)N * s.C * s.H * s.W * 4);
-            if (op.kind == kOpConvPool) ws.arg_off[op.out_map - 1] = take((size_t)N * s.C * s.H * s.W);
+            if (!(g.sp.on && &g != &p.groups.back() && (&g)[1].sp.on))       // (between split groups the map exists in split form only)
+                ws.map_off[op.out_map - 1] = take((size_t)N * s.C * s.H * s.W * 4);
+            if (op.kind == kOpConvPool) {
+                const SplitGeom sg = split_geom(N, s.C, s.H, s.W);
+                ws.arg_off[op.out_map - 1] = take(g.sp.on ? (size_t)sg.planes * sg.tp * 8 : (size_t)N * s.C * s.H * s.W);
+            }
         }
     // Deltas at the inputs of the executed groups 1..: the backward pass of group gi reads the one at its output
     // (index gi + 1) and writes the one at its input (index gi), so two areas, taken in turn, hold them all.
@@ -1141,6 +1309,7 @@ int build_plan(ftp_plan& p, const ftp_layer* layers, int n_layers, int N, int C,
         size_t need[2] = {0, 0};
         for (int gi = 1; gi < n_exec; ++gi) {
             if (p.groups[gi].tfg.on && p.groups[gi - 1].tfg.on) continue;   // bf16 one-conv groups hand over dz planes instead
+            if (p.groups[gi].sp.on && p.groups[gi - 1].sp.on) continue;     // ... and so do split groups
             const MapShape& s = p.maps[p.groups[gi].first - 1];
             const size_t bytes = tcp ? (size_t)N * round_up(s.C, 16) * s.H * s.W * 2     // bf16 planes
                                      : (size_t)N * s.C * s.H * s.W * 4;
@@ -1169,7 +1338,7 @@ int build_plan(ftp_plan& p, const ftp_layer* layers, int n_layers, int N, int C,
     for (int gi = 0; gi < n_exec; ++gi) {
         const GroupPlan& g = p.groups[gi];
         scratch = std::max(scratch, g.bwd.scratch_floats);
-        if (g.st.on && !g.st.thin)
+        if (g.st.on && !g.st.thin && !g.sp.on)
             dz[0] = dz[1] = std::max(dz[0], (size_t)N * g.fwd_ops[0].cout * g.fwd_ops[0].in_H * g.fwd_ops[0].in_W * 4);
         if (g.tfg.on) dz[gi & 1] = std::max(dz[gi & 1], (size_t)N * g.fwd_ops[0].cout16 * g.fwd_ops[0].in_H * g.fwd_ops[0].in_W * 2);
         if (gi == 0 && g.col_cin16) dz[1] = std::max(dz[1], (size_t)N * g.col_cin16 * H * W * 2);   // delta of the unrolled input
@@ -1181,8 +1350,31 @@ int build_plan(ftp_plan& p, const ftp_layer* layers, int n_layers, int N, int C,
     ws.wf_off = take(p.wf_floats * (tcp ? 2 : 4));
     ws.wb_off = take(p.wb_floats * (tcp ? 2 : 4));
     ws.err_off = take(256);
+    // split groups: the input of each as a split map, two dz maps (taken by the groups with an even / odd index: a group's
+    // input-delta kernel writes the dz of the group below while it reads its own), the packed filters
+    {
+        size_t sdz[2] = {0, 0};
+        long long sw = 0;
+        bool any = false;
+        for (int gi = 0; gi < n_exec; ++gi) {
+            GroupPlan& g = p.groups[gi];
+            if (!g.sp.on) continue;
+            any = true;
+            const OpDesc& op = g.fwd_ops[0];
+            off += kSplitSlack;
+            g.sp.in_off = take(split_bytes(split_geom(N, op.cin, op.in_H, op.in_W)));
+            sdz[gi & 1] = std::max(sdz[gi & 1], split_bytes(split_geom(N, op.cout, op.in_H, op.in_W)));
+            g.sp.wf_off = sw; sw += split_w_entries(g.sp.f, op.k);
+            g.sp.wd_off = sw; sw += split_w_entries(g.sp.d, op.k);
+        }
+        if (any) {
+            for (int i = 0; i < 2; ++i) { off += kSplitSlack; ws.sdz_off[i] = take(sdz[i]); }
+            off += kSplitSlack;
+            ws.sw_off = take((size_t)sw * 16);
+        }
+    }
     ws.partial_off = off;
-    for (GroupPlan& g : p.groups) g.partial_off = take((size_t)g.sets() * g.param_floats * 4);
+    for (GroupPlan& g : p.groups) g.partial_off = take((size_t)g.sets() * g.set_floats() * 4);
     ws.grad_off = take(p.param_floats * 4);
     ws.total = off;
     return FTP_OK;
@@ -1192,7 +1384,8 @@ int cost_terms(const ftp_plan& p, int pass, int group, int need_dx, double terms
 {
     if (group < 0 || group >= (int)p.groups.size() || pass < 0 || pass > 1 || !terms) return FTP_ERR_ARG;
     pass_cost_terms(p, p.groups[group], pass == 1, need_dx != 0, terms);
-    if (est_us) *est_us = p.groups[group].st.on  ? stationary_estimate_us(p, p.groups[group], pass == 1, need_dx != 0)
+    if (est_us) *est_us = p.groups[group].sp.on  ? split_estimate_us(p, p.groups[group], pass == 1, need_dx != 0)
+                        : p.groups[group].st.on  ? stationary_estimate_us(p, p.groups[group], pass == 1, need_dx != 0)
                         : p.groups[group].tfg.on ? tc_stationary_estimate_us(p, p.groups[group], pass == 1, need_dx != 0)
                                                  : pass_estimate_us(p.precision, pass == 1, terms);
     return FTP_OK;

@@ -162,9 +162,37 @@ constexpr int kTcMaxColChunks = 8;            // a band spans at most 126 column
 constexpr int kTcFgHeader = 1024;             // barriers, tensor-memory slot, a core matrix of ones
 constexpr int kTcFgSmemBudget = 200 * 1024;   // header + two stages
 
+// Split execution of a one-conv group of the fp32 path (split.cuh): the contractions on the tensor cores, every fp32
+// operand as the sum of three bf16 values.
+enum { kSplitFlat = 0, kSplitTile = 1, kSplitPool = 2 };
+struct SplitConvPlan {
+    int on = 0;
+    int Ns = 0, slices = 0, nb = 0, nblk = 0;   // output channels per item and slices; accumulator blocks per epilogue warp / per item
+    int kpc = 0, nchunks = 0;                   // 8-channel planes per chunk, chunks
+    int mode = 0, R = 0, Cw = 0, tiles_x = 0, tiles_y = 0, pitch = 0, nruns = 0, run_len = 0;
+    int a_plane = 0, a_bytes = 0, a_stages = 0, b_stage = 0, b_stages = 0, pool_bytes = 0, smem = 0;
+    int items = 0, blocks = 0;
+};
+struct SplitFgPlan {
+    int Ms = 0, slices = 0, ncols = 0, units = 0, nci = 0, rows3 = 0;
+    int E = 0, stages_total = 0, shares = 0, blocks = 0;
+    int nstages = 0, stage_bytes = 0, x_entries = 0, dz_box = 0, x_box = 0, smem = 0;
+};
+struct SplitPlan {
+    int on = 0;
+    SplitConvPlan f, d;                         // forward, input delta
+    SplitFgPlan g;
+    size_t in_off = 0;                          // workspace: the group's input as a split map
+    long long wf_off = 0, wd_off = 0;           // 16-byte entries into the packed filters
+};
+constexpr int kSplitSmemBudget = 226 * 1024;
+constexpr int kSplitHeader = 2048;
+constexpr double kSplitMinMacs = 1.0e8;   // see split_wanted in plan.cpp
+
 struct GroupPlan {
     int first = 0, last = 0;        // 1-based layers
     StatPlan st;
+    SplitPlan sp;                   // fp32 path: on = this one-conv group runs on the split kernels (st describes its CUDA-core form)
     TcFgPlan tfg;
     TcConvPlan cf, cd;              // tfg.on: the forward convolution and the input-delta convolution (dz planes in, delta planes
                                     //   out: the conv with the channel counts exchanged and the filters rotated) as banded kernels
@@ -172,13 +200,15 @@ struct GroupPlan {
     // on a window-unrolled copy of the network input (channel ci * 9 + ky * 3 + kx of a pixel = the input of channel ci
     // at window position (ky, kx)); the parameters keep their places, since W[co][ci][ky][kx] IS W'[co][ci * 9 + ky * 3 + kx].
     int col_cin = 0, col_cin16 = 0;     // 9 cin and its padding to 16 (0: not this route)
-    int sets() const { return tfg.on ? tfg.shares : bwd.blocks; }   // partial gradient sets the reduction sums
+    int sets() const { return tfg.on ? tfg.shares : sp.on ? sp.g.shares : bwd.blocks; }   // partial gradient sets the reduction sums
     int n_ops = 0;
     OpDesc fwd_ops[kMaxOps];
     OpDesc bwd_ops[kMaxOps];
     PassPlan fwd, bwd;
     std::vector<Span> tile_y, tile_x;   // user-tile partition of the group's output map
     size_t param_floats = 0;            // floats of this group's partial gradient set (tensor-core path: padded layout)
+    size_t split_set_floats = 0;        // ... of a group on the split kernels (padded layout as on the tensor-core path)
+    size_t set_floats() const { return sp.on ? split_set_floats : param_floats; }
     long long param_begin = 0;          // offset of the group's first parameter in params
     size_t partial_off = 0;             // float offset of the group's partial sets in the workspace
     double macs_done = 0, macs_untiled = 0;
@@ -196,6 +226,8 @@ struct Workspace {                 // byte offsets, all 256-aligned
     size_t dz_off = 0, dz_bytes = 0;   // one-conv groups: two areas (taken in turn, the second dz_bytes behind the first) for the
                                        // delta in front of the activation at the conv's resolution
     size_t wf_off = 0, wb_off = 0; // packed filters
+    size_t sw_off = 0;             // packed filters of the split groups
+    size_t sdz_off[2] = {0, 0};    // split groups: dz maps of the groups with an even / odd index
     size_t partial_off = 0;
     size_t grad_off = 0;           // summed gradient (ftp_step keeps it internal)
     size_t loss_off = 0;           // per-block partial sums of the MSE
@@ -215,6 +247,7 @@ struct ftp_plan {
     std::vector<ftp_group> user_groups;     // the requested grouping profile
     std::vector<ftp::GroupPlan> groups;     // the executed groups (a requested group may be cut, see build_plan)
     int N = 0, grid_y = 0, grid_x = 0, precision = 0;
+    bool split = false;                     // fp32 path: one-conv groups with enough input channels run on the split kernels
     int tc_tma = 1;                         // bf16 path: tiles of saved bf16 maps are copied by TMA (0: by the threads)
     size_t param_floats = 0;
     size_t wf_floats = 0, wb_floats = 0;    // packed filters (tensor-core path: counted in bf16 elements)
