@@ -115,12 +115,23 @@ void fill_common(const ftp_plan* p, const GroupPlan& g, bool backward, const flo
 
 inline int* err_ptr(void* ws, const ftp_plan* p) { return reinterpret_cast<int*>(static_cast<unsigned char*>(ws) + p->ws.err_off); }
 
-// clear_error: the first launch of a pass that starts afresh also clears the error word of the split kernels' bounded waits
-int pack_filters(ftp_plan* p, const float* params, void* ws, bool clear_error, cudaStream_t st)
+// Which packed arrangements a call needs: a forward pass the one, a backward pass the other.  The packing of a pass that starts
+// afresh (kPackForward) also clears the error word of the bounded waits.
+enum { kPackForward = 1, kPackDelta = 2 };
+
+void add_pack_tiles(PackTilesArgs& a, PackTilesLayer l)
+{
+    l.tile_begin = a.tiles;
+    a.l[a.n++] = l;
+    a.tiles += ((l.cin16 + 31) / 32) * ((l.cout16 + 31) / 32);
+}
+
+int pack_filters(ftp_plan* p, const float* params, void* ws, int dirs, cudaStream_t st)
 {
     PackArgs pa{};
-    SplitPackArgs sa{};
-    sa.error = clear_error ? err_ptr(ws, p) : nullptr;
+    PackTilesArgs sa{};
+    pa.dirs = sa.dirs = dirs;
+    sa.error = (dirs & kPackForward) ? err_ptr(ws, p) : nullptr;
     auto flush_split = [&]() {
         if (!sa.n) return;
         Timed t(p, st, 0, -1);
@@ -132,11 +143,10 @@ int pack_filters(ftp_plan* p, const float* params, void* ws, bool clear_error, c
             const OpDesc& op = g.fwd_ops[i];
             if (op.kind == kOpPool) continue;
             if (g.sp.on) {
-                if (sa.n == kSplitPackLayers) flush_split();
+                if (sa.n == kPackTilesLayers) flush_split();
                 uint4* base = reinterpret_cast<uint4*>(ws_ptr(ws, p->ws.sw_off));
-                sa.l[sa.n++] = SplitPackLayer{op.p_off, base + g.sp.wf_off, base + g.sp.wd_off, op.cin, op.cout, op.k, op.cin16, op.cout16,
-                                              g.sp.f.Ns, g.sp.f.kpc, g.sp.d.Ns, g.sp.d.kpc, sa.tiles};
-                sa.tiles += ((op.cin16 + 31) / 32) * ((op.cout16 + 31) / 32);
+                add_pack_tiles(sa, PackTilesLayer{op.p_off, base + g.sp.wf_off, base + g.sp.wd_off, op.cin, op.cout, op.k, op.cin16, op.cout16,
+                                                  g.sp.f.Ns, g.sp.f.kpc, g.sp.d.Ns, g.sp.d.kpc, 0});
                 continue;
             }
             if (pa.n == kMaxOps * 2) {   // flush a full batch
@@ -299,36 +309,53 @@ void fill_common_tc(const ftp_plan* p, const GroupPlan& g, bool backward, const 
     }
 }
 
-int pack_filters_tc(ftp_plan* p, const float* params, void* ws, cudaStream_t st)
+int pack_filters_tc(ftp_plan* p, const float* params, void* ws, int dirs, cudaStream_t st)
 {
     __nv_bfloat16* wf = reinterpret_cast<__nv_bfloat16*>(ws_ptr(ws, p->ws.wf_off));
     __nv_bfloat16* wb = reinterpret_cast<__nv_bfloat16*>(ws_ptr(ws, p->ws.wb_off));
     TcPackArgs pa{};
+    PackTilesArgs ba{};
+    pa.dirs = ba.dirs = dirs;
+    int* clear = (dirs & kPackForward) ? err_ptr(ws, p) : nullptr;       // by the first launch
     auto flush = [&]() {
         if (!pa.n) return;
+        pa.error = clear; clear = nullptr;
         Timed t(p, st, 0, -1);
         pack_filters_tc_kernel<<<dim3(64, pa.n), 256, 0, st>>>(pa, params, wf, wb);
         pa.n = 0;
+    };
+    auto flush_banded = [&]() {
+        if (!ba.n) return;
+        ba.error = clear; clear = nullptr;
+        Timed t(p, st, 0, -1);
+        pack_banded_kernel<<<ba.tiles, 256, 0, st>>>(ba, params);
+        ba.n = ba.tiles = 0;
     };
     for (const GroupPlan& g : p->groups)
         for (int i = 0; i < g.n_ops; ++i) {
             const OpDesc& op = g.fwd_ops[i];
             if (op.kind == kOpPool) continue;
-            if (pa.n == kMaxOps * 2) flush();
+            if (!g.tfg.on) {
+                if (pa.n == kMaxOps * 2) flush();
+                pa.l[pa.n++] = TcPackLayer{op.p_off, op.twf_off, op.cin, op.cout, op.k, op.cin16, op.cout16};
+                continue;
+            }
+            if (ba.n == kPackTilesLayers) flush_banded();
             // (first layer on the window-unrolled input: a 1x1 conv with 9 cin input channels, same parameters)
-            if (g.col_cin16) pa.l[pa.n++] = TcPackLayer{op.p_off, op.twf_off, g.col_cin, op.cout, 1, g.col_cin16, op.cout16,
-                                                        1, g.cf.Ns, g.cf.kpc, g.cd.Ns, g.cd.kpc};
-            else pa.l[pa.n++] = TcPackLayer{op.p_off, op.twf_off, op.cin, op.cout, op.k, op.cin16, op.cout16,
-                                            g.tfg.on ? 1 : 0, g.cf.Ns, g.cf.kpc, g.cd.Ns, g.cd.kpc};
+            const bool col = g.col_cin16 != 0;
+            add_pack_tiles(ba, PackTilesLayer{op.p_off, reinterpret_cast<uint4*>(wf + op.twf_off), reinterpret_cast<uint4*>(wb + op.twb_off),
+                                              col ? g.col_cin : op.cin, op.cout, col ? 1 : op.k, col ? g.col_cin16 : op.cin16, op.cout16,
+                                              g.cf.Ns, g.cf.kpc, g.cd.Ns, g.cd.kpc, 0});
         }
     flush();
+    flush_banded();
+    if (clear && cudaMemsetAsync(clear, 0, 4, st) != cudaSuccess) return FTP_ERR_CUDA;       // a plan without convolutions
     return launched_ok() ? FTP_OK : FTP_ERR_CUDA;
 }
 
-int forward_tc(ftp_plan* p, const float* x, const float* params, float* y, void* ws, cudaStream_t st)
+int forward_tc(ftp_plan* p, const float* x, const float* params, float* y, void* ws, int pack, cudaStream_t st)
 {
-    if (cudaMemsetAsync(err_ptr(ws, p), 0, 4, st) != cudaSuccess) return FTP_ERR_CUDA;
-    int rc = pack_filters_tc(p, params, ws, st);
+    int rc = pack_filters_tc(p, params, ws, pack, st);
     if (rc != FTP_OK) return rc;
     for (size_t gi = 0; gi < p->groups.size(); ++gi) {
         const GroupPlan& g = p->groups[gi];
@@ -547,10 +574,11 @@ bool split_backward(ftp_plan* p, const GroupPlan& g, int gi, const float* x, con
     return launched_ok();
 }
 
-int forward_impl(ftp_plan* p, const float* x, const float* params, float* y, void* ws, cudaStream_t st)
+// pack: the packed arrangements to make (kPackForward, with kPackDelta when the backward pass follows in the same call)
+int forward_impl(ftp_plan* p, const float* x, const float* params, float* y, void* ws, int pack, cudaStream_t st)
 {
-    if (is_tc(p)) return forward_tc(p, x, params, y, ws, st);
-    int rc = pack_filters(p, params, ws, true, st);
+    if (is_tc(p)) return forward_tc(p, x, params, y, ws, pack, st);
+    int rc = pack_filters(p, params, ws, pack, st);
     if (rc != FTP_OK) return rc;
     for (size_t gi = 0; gi < p->groups.size(); ++gi) {
         const GroupPlan& g = p->groups[gi];
@@ -584,9 +612,53 @@ TcReduceLayer reduce_layer(const GroupPlan& g, const OpDesc& op, void* ws)
 {
     if (g.col_cin16)
         return TcReduceLayer{op.p_off, ws_ptr(ws, g.partial_off), (long long)g.param_floats, op.tgp_off, g.sets(), g.col_cin, op.cout, 1,
-                             g.col_cin16, op.cout16};
+                             g.col_cin16, op.cout16, 1};
     return TcReduceLayer{op.p_off, ws_ptr(ws, g.partial_off), (long long)g.set_floats(), op.tgp_off, g.sets(), op.cin, op.cout, op.k,
-                         op.cin16, op.cout16};
+                         op.cin16, op.cout16, 1};
+}
+
+// Sums the partial sets of executed groups [first, last]: whole gradients (grad_out) and / or the update.
+int reduce_groups(ftp_plan* p, int first, int last, float* sgd_params, float lr, float* grad_out, void* ws, int timed_group, cudaStream_t st)
+{
+    TcReduceArgs ra{};
+    auto flush = [&]() {
+        if (!ra.n) return;
+        Timed t(p, st, 5, timed_group);
+        reduce_sgd_tc_kernel<<<dim3(1184, ra.n), 128, 0, st>>>(ra, sgd_params, lr, grad_out);
+        ra.n = 0;
+    };
+    for (int gi = first; gi <= last; ++gi) {
+        const GroupPlan& g = p->groups[gi];
+        if (g.param_floats == 0) continue;
+        if (!is_tc(p) && !g.sp.on) {                     // sets arranged like the parameters
+            if (ra.n == kMaxOps * 2) flush();
+            ra.l[ra.n++] = TcReduceLayer{g.param_begin, ws_ptr(ws, g.partial_off), (long long)g.param_floats, 0, g.sets(),
+                                               (int)g.param_floats, 1, 1, (int)g.param_floats, 1, 0};
+            continue;
+        }
+        for (int i = 0; i < g.n_ops; ++i) {
+            if (g.bwd_ops[i].kind == kOpPool) continue;
+            if (ra.n == kMaxOps * 2) flush();
+            ra.l[ra.n++] = reduce_layer(g, g.bwd_ops[i], ws);
+        }
+    }
+    flush();
+    return launched_ok() ? FTP_OK : FTP_ERR_CUDA;
+}
+
+// ftp_step_grad_groups: the sum of ONE executed group's partial sets, launched as soon as its backward pass is
+// queued, and the caller's notification.  Same per-parameter sums as the reduction over all groups.
+int reduce_group_and_notify(ftp_plan* p, int gi, float* grad_out, void* ws, cudaStream_t st)
+{
+    const GroupPlan& g = p->groups[gi];
+    if (g.param_floats == 0) return FTP_OK;
+    const int rc = reduce_groups(p, gi, gi, nullptr, 0.f, grad_out, ws, gi, st);
+    if (rc != FTP_OK) return rc;
+    long long floats = 0;
+    for (int i = 0; i < g.n_ops; ++i)
+        if (g.bwd_ops[i].kind != kOpPool) floats += (long long)g.bwd_ops[i].cout * g.bwd_ops[i].cin * g.bwd_ops[i].k * g.bwd_ops[i].k + g.bwd_ops[i].cout;
+    p->group_ready(p->group_ready_user, gi, g.param_begin, floats);
+    return FTP_OK;
 }
 
 // Backward pass of a one-conv bf16 group: dz planes at the conv's resolution, the filter gradient by the
@@ -689,20 +761,9 @@ int backward_tc(ftp_plan* p, const float* x, const float* dy, const float* param
           if (g.bwd.ctas == 2) bwd_group_tc_kernel<256><<<g.bwd.blocks, 256, smem, st>>>(a, tile_bytes, kTcTmemCols / 2, g.bwd.stages);
           else bwd_group_tc_kernel<512><<<g.bwd.blocks, 512, smem, st>>>(a, tile_bytes, kTcTmemCols, g.bwd.stages); }
         if (!launched_ok()) return FTP_ERR_CUDA;
-        if (p->group_ready && g.param_floats) {       // ftp_step_grad_groups: this group's sets are summed right away
-            TcReduceArgs rg{};
-            for (int i = 0; i < g.n_ops; ++i) {
-                const OpDesc& op = g.bwd_ops[i];
-                if (op.kind == kOpPool) continue;
-                rg.l[rg.n++] = reduce_layer(g, op, ws);
-            }
-            { Timed t(p, st, 5, gi);
-              reduce_sgd_tc_kernel<<<dim3(1184, rg.n), 128, 0, st>>>(rg, nullptr, 0.f, grad_out); }
-            if (!launched_ok()) return FTP_ERR_CUDA;
-            long long floats = 0;
-            for (int i = 0; i < g.n_ops; ++i)
-                if (g.bwd_ops[i].kind != kOpPool) floats += (long long)g.bwd_ops[i].cout * g.bwd_ops[i].cin * g.bwd_ops[i].k * g.bwd_ops[i].k + g.bwd_ops[i].cout;
-            p->group_ready(p->group_ready_user, gi, g.param_begin, floats);
+        if (p->group_ready) {                         // ftp_step_grad_groups: this group's sets are summed right away
+            const int rc = reduce_group_and_notify(p, gi, grad_out, ws, st);
+            if (rc != FTP_OK) return rc;
         }
         if (a.need_dx && !g.tfg.on) {
             const MapShape& s = p->maps[g.first - 1];
@@ -724,50 +785,7 @@ int backward_tc(ftp_plan* p, const float* x, const float* dy, const float* param
         }
     }
     if (p->group_ready) return launched_ok() ? FTP_OK : FTP_ERR_CUDA;      // summed group by group above
-    TcReduceArgs ra{};
-    auto flush = [&]() {
-        if (!ra.n) return;
-        Timed t(p, st, 5, -1);
-        reduce_sgd_tc_kernel<<<dim3(1184, ra.n), 128, 0, st>>>(ra, sgd_params, lr, grad_out);
-        ra.n = 0;
-    };
-    for (const GroupPlan& g : p->groups)
-        for (int i = 0; i < g.n_ops; ++i) {
-            const OpDesc& op = g.bwd_ops[i];
-            if (op.kind == kOpPool) continue;
-            if (ra.n == kMaxOps * 2) flush();
-            ra.l[ra.n++] = reduce_layer(g, op, ws);
-        }
-    flush();
-    return launched_ok() ? FTP_OK : FTP_ERR_CUDA;
-}
-
-// ftp_step_grad_groups: the sum of ONE executed group's partial sets, launched as soon as its backward pass is
-// queued, and the caller's notification.  Same per-parameter sums as the reduction over all groups.
-int reduce_group_and_notify(ftp_plan* p, int gi, float* grad_out, void* ws, cudaStream_t st)
-{
-    const GroupPlan& g = p->groups[gi];
-    if (g.param_floats == 0) return FTP_OK;
-    if (g.sp.on) {
-        TcReduceArgs rg{};
-        rg.n = 1;
-        rg.l[0] = reduce_layer(g, g.bwd_ops[0], ws);
-        { Timed t(p, st, 5, gi);
-          reduce_sgd_tc_kernel<<<dim3(1184, 1), 128, 0, st>>>(rg, nullptr, 0.f, grad_out); }
-        if (!launched_ok()) return FTP_ERR_CUDA;
-        p->group_ready(p->group_ready_user, gi, g.param_begin, (long long)g.param_floats);
-        return FTP_OK;
-    }
-    ReduceArgs ra{};
-    ra.n = 1;
-    ra.g[0] = ReduceGroup{g.param_begin, (long long)g.param_floats, ws_ptr(ws, g.partial_off), g.bwd.blocks};
-    const long long first = g.param_begin, total = g.param_begin + (long long)g.param_floats;
-    const int blocks = (int)std::min<long long>(((long long)g.param_floats + 255) / 256, (long long)kSmCount * 16);
-    { Timed t(p, st, 5, gi);
-      reduce_sgd_kernel<<<blocks, 256, 0, st>>>(ra, first, total, nullptr, 0.f, grad_out); }
-    if (!launched_ok()) return FTP_ERR_CUDA;
-    p->group_ready(p->group_ready_user, gi, first, (long long)g.param_floats);
-    return FTP_OK;
+    return reduce_groups(p, 0, G - 1, sgd_params, lr, grad_out, ws, -1, st);
 }
 
 // Backward of all groups in reverse order, halo sums at the group inputs, then the cross-tile
@@ -828,37 +846,7 @@ int backward_impl(ftp_plan* p, const float* x, const float* dy, const float* par
             p->fg_pending[turn] = false;
         }
     if (p->group_ready) return FTP_OK;       // every group's sets were summed right after its backward pass
-    TcReduceArgs rt{};
-    auto flush_split = [&]() {
-        if (!rt.n) return;
-        Timed t(p, st, 5, -1);
-        reduce_sgd_tc_kernel<<<dim3(1184, rt.n), 128, 0, st>>>(rt, sgd_params, lr, grad_out);
-        rt.n = 0;
-    };
-    for (const GroupPlan& g : p->groups) {
-        if (!g.sp.on) continue;
-        if (rt.n == kMaxOps * 2) flush_split();
-        rt.l[rt.n++] = reduce_layer(g, g.bwd_ops[0], ws);
-    }
-    flush_split();
-    // the other groups, whose sets are arranged like the parameters: a launch per contiguous run of them
-    ReduceArgs ra{};
-    auto flush_run = [&]() {
-        if (!ra.n) return;
-        const long long first = ra.g[0].begin, total = ra.g[ra.n - 1].begin + ra.g[ra.n - 1].floats;
-        const int blocks = (int)std::min<long long>((total - first + 255) / 256, (long long)kSmCount * 16);
-        Timed t(p, st, 5, -1);
-        reduce_sgd_kernel<<<blocks, 256, 0, st>>>(ra, first, total, sgd_params, lr, grad_out);
-        ra.n = 0;
-    };
-    for (const GroupPlan& g : p->groups) {
-        if (g.sp.on) flush_run();
-        if (g.sp.on || g.param_floats == 0) continue;
-        ra.g[ra.n++] = ReduceGroup{g.param_begin, (long long)g.param_floats, ws_ptr(ws, g.partial_off), g.bwd.blocks};
-    }
-    flush_run();
-    if (!launched_ok()) return FTP_ERR_CUDA;
-    return FTP_OK;
+    return reduce_groups(p, 0, G - 1, sgd_params, lr, grad_out, ws, -1, st);
 }
 
 bool aligned256(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 255u) == 0; }
@@ -1016,7 +1004,7 @@ int ftp_forward(ftp_plan* plan, const float* x, const float* params, float* y, v
     if (!plan || !x || !params || !workspace || !aligned256(workspace)) return FTP_ERR_ARG;
     int rc = ensure_device(plan);
     if (rc != FTP_OK) return rc;
-    return forward_impl(plan, x, params, y, workspace, static_cast<cudaStream_t>(stream));
+    return forward_impl(plan, x, params, y, workspace, kPackForward, static_cast<cudaStream_t>(stream));
 }
 
 int ftp_backward(ftp_plan* plan, const float* x, const float* dy, const float* params, float* dx, float* dparams,
@@ -1026,7 +1014,7 @@ int ftp_backward(ftp_plan* plan, const float* x, const float* dy, const float* p
     int rc = ensure_device(plan);
     if (rc != FTP_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    rc = is_tc(plan) ? pack_filters_tc(plan, params, workspace, st) : pack_filters(plan, params, workspace, false, st);
+    rc = is_tc(plan) ? pack_filters_tc(plan, params, workspace, kPackDelta, st) : pack_filters(plan, params, workspace, kPackDelta, st);
     if (rc != FTP_OK) return rc;
     return backward_impl(plan, x, dy, params, dx, dparams, nullptr, 0.f, workspace, st);
 }
@@ -1041,7 +1029,7 @@ static int step_impl(ftp_plan* plan, const float* x, const float* dy, const floa
     if (rc != FTP_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     float* y32 = (is_tc(plan) && target) ? ws_ptr(workspace, plan->ws.y32_off) : nullptr;
-    rc = forward_impl(plan, x, params, y32, workspace, st);
+    rc = forward_impl(plan, x, params, y32, workspace, kPackForward | kPackDelta, st);
     if (rc != FTP_OK) return rc;
     const float* delta = dy;
     if (target_ready && cudaStreamWaitEvent(st, target_ready, 0) != cudaSuccess) return FTP_ERR_CUDA;

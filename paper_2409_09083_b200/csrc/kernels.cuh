@@ -37,10 +37,7 @@ struct HaloSumArgs {
 };
 
 struct PackLayer { long long p_off, wf_off, wb_off; int cin, cout, k, cout_pad, cin_pad; };
-struct PackArgs { int n; PackLayer l[kMaxOps * 2]; };
-
-struct ReduceGroup { long long begin, floats; const float* partial; int sets; };
-struct ReduceArgs { int n; ReduceGroup g[64]; };
+struct PackArgs { int n, dirs; PackLayer l[kMaxOps * 2]; };
 
 __device__ __forceinline__ float leaky(float z, float slope) { return z > 0.f ? z : slope * z; }
 // derivative of the leaky ReLU, decided from the activation's output (same sign as its input)
@@ -989,7 +986,8 @@ __global__ void pack_filters_kernel(const __grid_constant__ PackArgs A, const fl
     const PackLayer L = A.l[blockIdx.y];
     const int KK = L.k * L.k;
     const long long nf = (long long)L.cin * KK * L.cout_pad, nb = (long long)L.cout * KK * L.cin_pad;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nf + nb; e += (long long)gridDim.x * blockDim.x) {
+    const long long lo = (A.dirs & 1) ? 0 : nf, hi = (A.dirs & 2) ? nf + nb : nf;             // forward arrangement, rotated one
+    for (long long e = lo + blockIdx.x * (long long)blockDim.x + threadIdx.x; e < hi; e += (long long)gridDim.x * blockDim.x) {
         if (e < nf) {
             const int co = (int)(e % L.cout_pad); long long t = e / L.cout_pad;
             const int tap = (int)(t % KK); const int ci = (int)(t / KK);
@@ -1000,24 +998,6 @@ __global__ void pack_filters_kernel(const __grid_constant__ PackArgs A, const fl
             const int tapr = (int)(t % KK); const int co = (int)(t / KK);
             wb[L.wb_off + f] = ci < L.cin ? params[L.p_off + ((long long)co * L.cin + ci) * KK + (KK - 1 - tapr)] : 0.f;
         }
-    }
-}
-
-// Cross-tile reduction of the partial gradient sets in a fixed order, fused with the update
-// (Section 4.1: the sets are summed once per batch and the result updates F_l).
-__global__ void reduce_sgd_kernel(const __grid_constant__ ReduceArgs A, long long first, long long total, float* __restrict__ params,
-                                  float lr, float* __restrict__ grad_out)
-{
-    // parameters first .. total - 1 (the groups of A cover them)
-    for (long long e = first + blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
-        int g = 0;
-        while (g + 1 < A.n && e >= A.g[g + 1].begin) ++g;
-        const long long local = e - A.g[g].begin;
-        const float* p = A.g[g].partial + local;
-        float s = 0.f;
-        for (int k = 0; k < A.g[g].sets; ++k) s += p[(size_t)k * A.g[g].floats];
-        if (grad_out) grad_out[e] = s;
-        if (params) params[e] = params[e] - lr * s;
     }
 }
 

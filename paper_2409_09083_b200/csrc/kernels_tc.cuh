@@ -10,10 +10,13 @@
 // memory use the same plane arrangement, [n][C16/8][H][W][8] bf16.
 #pragma once
 
+#include <algorithm>
+
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include "plan.hpp"
+#include "pack.cuh"
 #include "tc.cuh"
 
 namespace ftp {
@@ -881,11 +884,16 @@ __global__ void halo_sum_planes_kernel(const __grid_constant__ HaloSumArgs A)
     }
 }
 
-// Cross-tile reduction of the partial gradient sets of the tensor-core path in a fixed order, fused
-// with the update.  A set holds each layer as [window position][cout16][cin16] + [cout16] bias.
-struct TcReduceLayer { long long p_off; const float* partial; long long set_floats, tgp_off; int sets, cin, cout, k, cin16, cout16; };
+// Cross-tile reduction of the partial gradient sets in a fixed order, fused with the update (Section 4.1: the sets are
+// summed once per batch and the result updates F_l).
+// One layer's slice of the partial sets ([tap][cout16][cin16] filters, then the bias), or a whole group whose sets are arranged
+// like the parameters (cout = k = 1, cin = floats of a set, no bias).
+struct TcReduceLayer { long long p_off; const float* partial; long long set_floats, tgp_off; int sets, cin, cout, k, cin16, cout16, bias; };
 struct TcReduceArgs { int n; TcReduceLayer l[kMaxOps * 2]; };
 
+// 16 loads in flight a thread: with 4 (296 sets of the 896 parameters of an fp32 first layer) the sums were a chain of latencies,
+// 52 us of an 8-layer step, now 27 us.  Measured and dropped: 3x3 tiles that leave through shared memory as contiguous runs of the
+// parameters, with the sets dealt out to warps or with several tiles a block (73-140 us on a 16-layer stack, this 75 us).
 __global__ void reduce_sgd_tc_kernel(const __grid_constant__ TcReduceArgs A, float* __restrict__ params, float lr,
                                      float* __restrict__ grad_out)
 {
@@ -893,7 +901,7 @@ __global__ void reduce_sgd_tc_kernel(const __grid_constant__ TcReduceArgs A, flo
     // bulk of the traffic); the one write per parameter goes to its place in the caller's arrangement.
     const TcReduceLayer L = A.l[blockIdx.y];
     const int KK = L.k * L.k;
-    const long long nf = (long long)KK * L.cout16 * L.cin16, total = nf + L.cout16;
+    const long long nf = (long long)KK * L.cout16 * L.cin16, total = nf + (L.bias ? L.cout16 : 0);
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
         long long dst;
         if (e < nf) {
@@ -928,51 +936,21 @@ __global__ void planes_to_nchw_kernel(const __nv_bfloat16* __restrict__ src, flo
     }
 }
 
-// Filters -> the two packed bf16 arrangements of the tensor-core kernels:
+// Filters -> the two packed bf16 arrangements of the fused stack kernels:
 //   wf[tap][cin16/8][cout16][8]   B operand of the forward pass   (rows = cout, K = cin)
 //   wb[tap'][cout16/8][cin16][8]  B operand of the delta pass, tap' = K*K-1-tap (rotated 180 degrees; rows = cin, K = cout)
-// Layers run by the banded kernels (sliced != 0) get instead, per pass, the arrangement in which the filters one block
-// needs for one chunk of input channels are contiguous (one bulk copy):
-//   wf[slice][chunk][tap][kpc_f][ns_f][8]    rows = output channels slice*ns_f .., K = input channels (chunk*kpc_f + j)*8 ..
-//   wb[slice][chunk][tap'][kpc_d][ns_d][8]   rows = input channels slice*ns_d ..,  K = output channels (chunk*kpc_d + j)*8 ..
-// with zeros beyond the layer's channel counts.
-struct TcPackLayer { long long p_off, w_off; int cin, cout, k, cin16, cout16; int sliced, ns_f, kpc_f, ns_d, kpc_d; };
-struct TcPackArgs { int n; TcPackLayer l[kMaxOps * 2]; };
+struct TcPackLayer { long long p_off, w_off; int cin, cout, k, cin16, cout16; };
+struct TcPackArgs { int n, dirs; int* error; TcPackLayer l[kMaxOps * 2]; };       // dirs: 1 wf, 2 wb, 3 both; error: word to clear, or null
 
 __global__ void pack_filters_tc_kernel(const __grid_constant__ TcPackArgs A, const float* __restrict__ params,
                                        __nv_bfloat16* __restrict__ wf, __nv_bfloat16* __restrict__ wb)
 {
+    if (A.error && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *A.error = 0;
     const TcPackLayer L = A.l[blockIdx.y];
     const int KK = L.k * L.k;
-    if (L.sliced) {
-        const int nch_f = (L.cin16 / 8 + L.kpc_f - 1) / L.kpc_f, nch_d = (L.cout16 / 8 + L.kpc_d - 1) / L.kpc_d;
-        const long long per_f = (long long)((L.cout16 + L.ns_f - 1) / L.ns_f) * nch_f * KK * L.kpc_f * L.ns_f * 8;
-        const long long per_d = (long long)((L.cin16 + L.ns_d - 1) / L.ns_d) * nch_d * KK * L.kpc_d * L.ns_d * 8;
-        // one thread per 16-byte entry (8 contraction channels of one row): the position is worked out once per entry
-        const long long ent_f = per_f / 8, ent_d = per_d / 8;
-        for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < ent_f + ent_d; e += (long long)gridDim.x * blockDim.x) {
-            const bool fwd = e < ent_f;
-            const int ns = fwd ? L.ns_f : L.ns_d, kpc = fwd ? L.kpc_f : L.kpc_d, nch = fwd ? nch_f : nch_d;
-            long long t = fwd ? e : e - ent_f;
-            const int r = (int)(t % ns); t /= ns;
-            const int j = (int)(t % kpc); t /= kpc;
-            const int tap = (int)(t % KK); t /= KK;
-            const int c = (int)(t % nch); const int sl = (int)(t / nch);
-            const int row = sl * ns + r, k0 = (c * kpc + j) * 8;                  // output row of the GEMM, first contraction channel
-            const int ptap = fwd ? tap : KK - 1 - tap;
-            float v[8];
-#pragma unroll
-            for (int c8 = 0; c8 < 8; ++c8) {
-                const int co = fwd ? row : k0 + c8, ci = fwd ? k0 + c8 : row;
-                v[c8] = (co < L.cout && ci < L.cin) ? __ldg(params + L.p_off + ((long long)co * L.cin + ci) * KK + ptap) : 0.f;
-            }
-            uint4* dst = reinterpret_cast<uint4*>(fwd ? wf + L.w_off : wb + L.w_off) + (fwd ? e : e - ent_f);
-            *dst = tcd::pack8(v);
-        }
-        return;
-    }
     const long long per = (long long)KK * L.cin16 * L.cout16;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < 2 * per; e += (long long)gridDim.x * blockDim.x) {
+    const long long lo = (A.dirs & 1) ? 0 : per, hi = (A.dirs & 2) ? 2 * per : per;
+    for (long long e = lo + blockIdx.x * (long long)blockDim.x + threadIdx.x; e < hi; e += (long long)gridDim.x * blockDim.x) {
         if (e < per) {
             const int c8 = (int)(e % 8); long long t = e / 8;
             const int co = (int)(t % L.cout16); t /= L.cout16;
@@ -990,6 +968,13 @@ __global__ void pack_filters_tc_kernel(const __grid_constant__ TcPackArgs A, con
             wb[L.w_off + f] = __float2bfloat16(v);
         }
     }
+}
+
+// ... and of the banded kernels (pack.cuh)
+__global__ void __launch_bounds__(256) pack_banded_kernel(const __grid_constant__ PackTilesArgs A, const float* __restrict__ params)
+{
+    __shared__ float s[kPackSmemFloats];
+    pack_tiles<1>(A, params, s, [](const float* v, uint4* p) { p[0] = tcd::pack8(v); });
 }
 
 }  // namespace ftp

@@ -1265,6 +1265,7 @@ int build_plan(ftp_plan& p, const ftp_layer* layers, int n_layers, int N, int C,
         for (const GroupPlan& g : cut) p.groups.push_back(g);
     }
     if (p.groups.size() > 64) return FTP_ERR_GROUPS;
+    if (p.split) p.split = std::any_of(p.groups.begin(), p.groups.end(), [](const GroupPlan& g) { return g.sp.on != 0; });
     const int n_exec = (int)p.groups.size();
 
     // device tables

@@ -48,7 +48,7 @@ void split_launch_delta(const SplitDeltaArgs& a, void* stream)
     sp::split_delta_kernel<<<helper_blocks((long long)a.low.planes * a.low.tp), 256, 0, static_cast<cudaStream_t>(stream)>>>(a);
 }
 
-void split_launch_pack(const SplitPackArgs& a, const float* params, void* stream)
+void split_launch_pack(const PackTilesArgs& a, const float* params, void* stream)
 {
     sp::pack_split_kernel<<<a.tiles, 256, 0, static_cast<cudaStream_t>(stream)>>>(a, params);
 }

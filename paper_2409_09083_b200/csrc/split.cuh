@@ -26,6 +26,7 @@
 //   fgrad_split_kernel   filter and bias gradient
 #pragma once
 
+#include "pack.cuh"
 #include "split_args.hpp"
 #include "tc.cuh"
 
@@ -853,44 +854,10 @@ __global__ void split_delta_kernel(const __grid_constant__ SplitDeltaArgs A)
     }
 }
 
-// Filters -> the packed split arrangements, per slice and chunk the parts b0, b1, b2 one after another:
-//   wf[slice][chunk][part][tap][kpc][Ns][8]   rows = output channels, contraction = input channels     (forward)
-//   wd[slice][chunk][part][tap'][kpc][Ns][8]  rows = input channels, contraction = output channels, rotated (input delta)
-// A block takes a tile of 32 x 32 channels through shared memory: the filters of 32 input channels are one contiguous
-// run of an output channel's row, and both outputs leave as runs of 16-byte entries of neighbouring rows.
-__global__ void __launch_bounds__(256) pack_split_kernel(const __grid_constant__ SplitPackArgs A, const float* __restrict__ params)
+__global__ void __launch_bounds__(256) pack_split_kernel(const __grid_constant__ PackTilesArgs A, const float* __restrict__ params)
 {
-    __shared__ float s[32 * (32 * 9 + 1)];
-    if (A.error && blockIdx.x == 0 && threadIdx.x == 0) *A.error = 0;
-    int l = 0;
-    while (l + 1 < A.n && (int)blockIdx.x >= A.l[l + 1].tile_begin) ++l;
-    const SplitPackLayer& L = A.l[l];
-    const int KK = L.k * L.k, t = (int)blockIdx.x - L.tile_begin;
-    const int tci = (L.cin16 + 31) / 32, co0 = t / tci * 32, ci0 = t % tci * 32;
-    const int pitch = 32 * KK + 1;                            // odd: rows (output channels) of a column fall into different banks
-    const int nci = min(32, L.cin - ci0), run = nci * KK;
-    for (int r = threadIdx.x >> 5; r < 32; r += 8)
-        for (int j = threadIdx.x & 31; j < 32 * KK; j += 32)
-            s[r * pitch + j] = (co0 + r < L.cout && j < run) ? __ldg(params + L.p_off + ((long long)(co0 + r) * L.cin + ci0) * KK + j) : 0.f;
-    __syncthreads();
-    const int total = 32 * 4 * KK;
-    for (int i = threadIdx.x; i < 2 * total; i += 256) {
-        const bool fwd = i < total;
-        const int j = fwd ? i : i - total, r = j & 31, o = (j >> 5) & 3, tap = j >> 7;   // row of the operand, octet of contraction channels
-        const int row = (fwd ? co0 : ci0) + r, k0 = (fwd ? ci0 : co0) + o * 8;
-        if (row >= (fwd ? L.cout16 : L.cin16) || k0 >= (fwd ? L.cin16 : L.cout16)) continue;
-        const int ns = fwd ? L.ns_f : L.ns_d, kpc = fwd ? L.kpc_f : L.kpc_d;
-        const int nch = ((fwd ? L.cin16 : L.cout16) / 8 + kpc - 1) / kpc;
-        float v[8];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) v[c] = fwd ? s[r * pitch + (o * 8 + c) * KK + tap] : s[(o * 8 + c) * pitch + r * KK + KK - 1 - tap];
-        uint4 p0, p1, p2;
-        split8(v, p0, p1, p2);
-        const int sl = row / ns, rr = row - sl * ns, kp = k0 / 8, ch = kp / kpc, kj = kp - ch * kpc;
-        const size_t stage = (size_t)KK * kpc * ns;
-        uint4* dst = (fwd ? L.wf : L.wd) + ((size_t)sl * nch + ch) * 3 * stage + ((size_t)tap * kpc + kj) * ns + rr;
-        dst[0] = p0; dst[stage] = p1; dst[2 * stage] = p2;
-    }
+    __shared__ float s[kPackSmemFloats];
+    pack_tiles<3>(A, params, s, [](const float* v, uint4* p) { split8(v, p[0], p[1], p[2]); });
 }
 
 }  // namespace sp

@@ -80,10 +80,15 @@ void split_launch_fgrad(const SplitFgArgs& a, int blocks, int smem, void* stream
 void split_launch_planes(const float* src, uint4* dst, const SplitGeom& g, int C, void* stream);
 void split_launch_delta(const SplitDeltaArgs& a, void* stream);
 
-// One layer of the packing launch: 32 x 32 channel tiles [tile_begin, next layer's tile_begin).
-struct SplitPackLayer { long long p_off; uint4* wf; uint4* wd; int cin, cout, k, cin16, cout16, ns_f, kpc_f, ns_d, kpc_d, tile_begin; };
-constexpr int kSplitPackLayers = 32;
-struct SplitPackArgs { int n, tiles; int* error; SplitPackLayer l[kSplitPackLayers]; };
-void split_launch_pack(const SplitPackArgs& a, const float* params, void* stream);
+// Packing launches (pack.cuh): 32 x 32 channel tiles [tile_begin, next layer's tile_begin) of a layer.
+struct PackTilesLayer { long long p_off; uint4* wf; uint4* wd; int cin, cout, k, cin16, cout16, ns_f, kpc_f, ns_d, kpc_d, tile_begin; };
+constexpr int kPackTilesLayers = 32;
+struct PackTilesArgs {
+    int n, tiles;
+    int dirs;                       // 1: forward arrangement, 2: input delta, 3: both
+    int* error;                     // error word to clear, or null
+    PackTilesLayer l[kPackTilesLayers];
+};
+void split_launch_pack(const PackTilesArgs& a, const float* params, void* stream);   // three parts
 
 }  // namespace ftp
