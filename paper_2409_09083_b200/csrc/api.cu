@@ -82,6 +82,7 @@ struct Timed {
             cudaEventRecord(static_cast<cudaEvent_t>(p->ev_begin[slot]), st);
         }
     }
+    LaunchStream ls() const { return LaunchStream{st, !p->timing}; }       // (events between two launches keep them apart anyway)
     ~Timed() { if (slot >= 0) cudaEventRecord(static_cast<cudaEvent_t>(p->ev_end[slot]), st); }
 };
 
@@ -135,7 +136,7 @@ int pack_filters(ftp_plan* p, const float* params, void* ws, int dirs, cudaStrea
     auto flush_split = [&]() {
         if (!sa.n) return;
         Timed t(p, st, 0, -1);
-        split_launch_pack(sa, params, st);
+        split_launch_pack(sa, params, t.ls());
         sa.n = sa.tiles = 0;
     };
     for (const GroupPlan& g : p->groups)
@@ -151,14 +152,14 @@ int pack_filters(ftp_plan* p, const float* params, void* ws, int dirs, cudaStrea
             }
             if (pa.n == kMaxOps * 2) {   // flush a full batch
                 { Timed t(p, st, 0, -1);
-                  pack_filters_kernel<<<dim3(64, pa.n), 256, 0, st>>>(pa, params, ws_ptr(ws, p->ws.wf_off), ws_ptr(ws, p->ws.wb_off)); }
+                  launch(pack_filters_kernel, dim3(64, pa.n), 256, 0, t.ls(), pa, params, ws_ptr(ws, p->ws.wf_off), ws_ptr(ws, p->ws.wb_off)); }
                 pa.n = 0;
             }
             pa.l[pa.n++] = PackLayer{op.p_off, op.wf_off, op.wb_off, op.cin, op.cout, op.k, op.cout_pad, op.cin_pad};
         }
     if (pa.n) {
         Timed t(p, st, 0, -1);
-        pack_filters_kernel<<<dim3(64, pa.n), 256, 0, st>>>(pa, params, ws_ptr(ws, p->ws.wf_off), ws_ptr(ws, p->ws.wb_off));
+        launch(pack_filters_kernel, dim3(64, pa.n), 256, 0, t.ls(), pa, params, ws_ptr(ws, p->ws.wf_off), ws_ptr(ws, p->ws.wb_off));
     }
     flush_split();
     return launched_ok() ? FTP_OK : FTP_ERR_CUDA;
@@ -246,6 +247,9 @@ bool encode_split_map(unsigned char out[128], const uint4* base, const SplitGeom
     return true;
 }
 
+// Tensor-core cycles of one MMA with N accumulator columns and both operands in shared memory (M = 128, K = 16)
+inline double tc_mma_cycles(int n) { return std::max(32.0 + n / 4.0, n / 2.0); }
+
 // One launch of the banded convolution kernel: `in` planes (cin16 channels) -> `out` planes (cout16 channels).
 struct PrevLayer { const uint4* y; const unsigned long long* arg; float slope; };   // see TcConvRowsArgs::prev_y
 
@@ -264,8 +268,9 @@ bool launch_tc_conv(ftp_plan* p, const TcConvPlan& c, int kind, int gi, const vo
     a.Ns = c.Ns; a.slices = c.slices; a.R = c.R; a.Wp = c.Wp; a.bands_img = c.bands_img; a.nblk = c.nblk; a.kpc = c.kpc;
     a.ncc = c.ncc; a.Cw = c.Cw; a.items = c.items; a.pool_planes = c.pool_planes; a.nbuf = c.nbuf;
     a.x_plane = c.x_plane; a.stage_bytes = c.stage_bytes; a.stages = c.stages;
+    a.hurry = (double)((c.items + c.blocks - 1) / c.blocks) * c.nblk * K * K * (cin16 / 16) * tc_mma_cycles(c.Ns) < kHurryCycles;
     { Timed tm(p, st, kind, gi);
-      conv_tc_rows_kernel<<<c.blocks, kTcConvThreads, c.smem_bytes, st>>>(a); }
+      launch(conv_tc_rows_kernel, c.blocks, kTcConvThreads, one_block_smem(c.smem_bytes), tm.ls(), a); }
     return launched_ok();
 }
 
@@ -321,14 +326,14 @@ int pack_filters_tc(ftp_plan* p, const float* params, void* ws, int dirs, cudaSt
         if (!pa.n) return;
         pa.error = clear; clear = nullptr;
         Timed t(p, st, 0, -1);
-        pack_filters_tc_kernel<<<dim3(64, pa.n), 256, 0, st>>>(pa, params, wf, wb);
+        launch(pack_filters_tc_kernel, dim3(64, pa.n), 256, 0, t.ls(), pa, params, wf, wb);
         pa.n = 0;
     };
     auto flush_banded = [&]() {
         if (!ba.n) return;
         ba.error = clear; clear = nullptr;
         Timed t(p, st, 0, -1);
-        pack_banded_kernel<<<ba.tiles, 256, 0, st>>>(ba, params);
+        launch(pack_banded_kernel, ba.tiles, 256, 0, t.ls(), ba, params);
         ba.n = ba.tiles = 0;
     };
     for (const GroupPlan& g : p->groups)
@@ -368,7 +373,7 @@ int forward_tc(ftp_plan* p, const float* x, const float* params, float* y, void*
             if (g.col_cin16) {                  // first layer: a 1x1 conv on the window-unrolled network input
                 uint4* col = reinterpret_cast<uint4*>(ws_ptr(ws, p->ws.col_off));
                 { Timed t(p, st, 9, (int)gi);
-                  launch_unroll_windows(x, col, p->N, op.cin, op.in_H, op.in_W, st); }
+                  launch_unroll_windows(x, col, p->N, op.cin, op.in_H, op.in_W, t.ls()); }
                 if (!launched_ok()) return FTP_ERR_CUDA;
                 in = col;
             }
@@ -383,8 +388,8 @@ int forward_tc(ftp_plan* p, const float* x, const float* params, float* y, void*
           const size_t smem = tc_smem(g.fwd.smem_bytes, g.fwd.ctas);
           const int blocks = std::min(items, kSmCount * g.fwd.ctas), tile_bytes = (int)(smem - tc_fixed_bytes(g.fwd.stages));
           // two blocks of 256 threads per SM, or one of 512: the phases around the MMAs want all the warps they can get
-          if (g.fwd.ctas == 2) fwd_group_tc_kernel<256><<<blocks, 256, smem, st>>>(a, tile_bytes, kTcTmemCols / 2, g.fwd.stages);
-          else fwd_group_tc_kernel<512><<<blocks, 512, smem, st>>>(a, tile_bytes, kTcTmemCols, g.fwd.stages); }
+          if (g.fwd.ctas == 2) launch(fwd_group_tc_kernel<256>, blocks, 256, smem, t.ls(), a, tile_bytes, kTcTmemCols / 2, g.fwd.stages);
+          else launch(fwd_group_tc_kernel<512>, blocks, 512, smem, t.ls(), a, tile_bytes, kTcTmemCols, g.fwd.stages); }
         if (!launched_ok()) return FTP_ERR_CUDA;
     }
     if (y) {
@@ -392,7 +397,7 @@ int forward_tc(ftp_plan* p, const float* x, const float* params, float* y, void*
         const size_t total = (size_t)p->N * s.C * s.H * s.W;
         const int blocks = (int)std::min<size_t>((total + 255) / 256, (size_t)kSmCount * 16);
         ++p->launches;
-        planes_to_nchw_kernel<<<blocks, 256, 0, st>>>(
+        launch(planes_to_nchw_kernel, blocks, 256, 0, LaunchStream{st, !p->timing}, 
             reinterpret_cast<const __nv_bfloat16*>(map_ptr(p, x, ws, (int)p->layers.size() + 1)), y, p->N, s.C,
             (s.C + 15) / 16 * 16, s.H, s.W);
         if (!launched_ok()) return FTP_ERR_CUDA;
@@ -414,7 +419,7 @@ bool stationary_forward(ftp_plan* p, const GroupPlan& g, int gi, const float* x,
     a.N = p->N; a.Cin = op.cin; a.Cout = op.cout; a.CoutPad = op.cout_pad; a.H = op.in_H; a.W = op.in_W;
     a.slope = op.slope; a.act = 1; a.pool = g.st.pool;
     { Timed t(p, st, 1, gi);
-      st_launch_conv_rows(a, op.k, g.st.fwd_co_tile, g.st.fwd_threads, g.st.fwd_blocks, st); }
+      st_launch_conv_rows(a, op.k, g.st.fwd_co_tile, g.st.fwd_threads, g.st.fwd_blocks, t.ls()); }
     return launched_ok();
 }
 
@@ -436,7 +441,7 @@ bool stationary_backward(ftp_plan* p, const GroupPlan& g, int gi, const float* x
         t.N = p->N; t.Cin = op.cin; t.Cout = op.cout; t.OH = op.out_H; t.OW = op.out_W;
         t.tiles_y = g.st.thin_tiles_y; t.tiles_x = g.st.thin_tiles_x; t.slope = op.slope;
         { Timed tm(p, st, 3, gi);
-          st_launch_thin_bwd(t, g.st.thin_blocks, st); }
+          st_launch_thin_bwd(t, g.st.thin_blocks, tm.ls()); }
         return launched_ok();
     }
     // The filter gradient and the input delta both read dZ and nothing else of each other, so the filter gradient
@@ -455,7 +460,7 @@ bool stationary_backward(ftp_plan* p, const GroupPlan& g, int gi, const float* x
         p->fg_pending[turn] = false;
     }
     { Timed t(p, st, 6, gi);
-      st_launch_delta_act(dout, y, arg, dz, count, op.out_W, op.slope, g.st.pool, st); }
+      st_launch_delta_act(dout, y, arg, dz, count, op.out_W, op.slope, g.st.pool, t.ls()); }
     if (!launched_ok()) return false;
     if (side && (cudaEventRecord(static_cast<cudaEvent_t>(p->ev_dz[turn]), st) != cudaSuccess ||
                  cudaStreamWaitEvent(gs, static_cast<cudaEvent_t>(p->ev_dz[turn]), 0) != cudaSuccess)) return false;
@@ -466,7 +471,7 @@ bool stationary_backward(ftp_plan* p, const GroupPlan& g, int gi, const float* x
     f.N = p->N; f.Cin = op.cin; f.Cout = op.cout; f.H = H; f.W = W;
     f.stages = g.st.fg_stages; f.splits = g.st.fg_splits;
     { Timed t(p, gs, 7, gi);
-      st_launch_filter_grad_rows(f, op.k, g.st.fg_blocks, gs); }
+      st_launch_filter_grad_rows(f, op.k, g.st.fg_blocks, t.ls()); }
     if (!launched_ok()) return false;
     if (side) {
         if (cudaEventRecord(static_cast<cudaEvent_t>(p->ev_fg[turn]), gs) != cudaSuccess) return false;
@@ -480,7 +485,7 @@ bool stationary_backward(ftp_plan* p, const GroupPlan& g, int gi, const float* x
         a.N = p->N; a.Cin = op.cout; a.Cout = op.cin; a.CoutPad = op.cin_pad; a.H = H; a.W = W;
         a.slope = 0.f; a.act = 0; a.pool = 0;
         { Timed t(p, st, 8, gi);
-          st_launch_conv_rows(a, op.k, g.st.dx_co_tile, g.st.dx_threads, g.st.dx_blocks, st); }
+          st_launch_conv_rows(a, op.k, g.st.dx_co_tile, g.st.dx_threads, g.st.dx_blocks, t.ls()); }
         if (!launched_ok()) return false;
     }
     return true;
@@ -510,7 +515,7 @@ bool split_forward(ftp_plan* p, const GroupPlan& g, int gi, const float* x, cons
     uint4* in = split_ptr(ws, g.sp.in_off);
     if (!split_at(p, gi - 1)) {                     // the group below wrote an fp32 map
         Timed t(p, st, 9, gi);
-        split_launch_planes(map_ptr(p, x, ws, g.first), in, in_geom(p, op), op.cin, st);
+        split_launch_planes(map_ptr(p, x, ws, g.first), in, in_geom(p, op), op.cin, t.ls());
     }
     SplitConvArgs a{};
     if (!split_conv_args(a, g.sp.f, in, in_geom(p, op), op.k, op.cout, op.cout16)) return false;
@@ -522,7 +527,7 @@ bool split_forward(ftp_plan* p, const GroupPlan& g, int gi, const float* x, cons
     if (split_at(p, gi + 1)) a.out_s = split_ptr(ws, p->groups[gi + 1].sp.in_off);
     else a.out_f = const_cast<float*>(map_ptr(p, x, ws, op.out_map));
     { Timed t(p, st, 1, gi);
-      split_launch_conv(a, g.sp.f.nb, g.sp.f.blocks, g.sp.f.smem, st); }
+      split_launch_conv(a, g.sp.f.nb, g.sp.f.blocks, g.sp.f.smem, t.ls()); }
     return launched_ok();
 }
 
@@ -538,7 +543,7 @@ bool split_backward(ftp_plan* p, const GroupPlan& g, int gi, const float* x, con
         d.C = op.cout; d.slope = op.slope; d.pool = op.kind == kOpConvPool ? 1 : 0;
         if (d.pool) d.arg = reinterpret_cast<const unsigned long long*>(static_cast<unsigned char*>(ws) + p->ws.arg_off[op.out_map - 1]);
         { Timed t(p, st, 6, gi);
-          split_launch_delta(d, st); }
+          split_launch_delta(d, t.ls()); }
     }
     {
         const SplitFgPlan& t = g.sp.g;
@@ -553,7 +558,7 @@ bool split_backward(ftp_plan* p, const GroupPlan& g, int gi, const float* x, con
         if (!encode_split_map(f.tmap_dz, dz, f.g, false, t.E, 0, t.dz_box, 3) ||
             !encode_split_map(f.tmap_x, f.x, in_geom(p, op), false, t.x_entries, 0, t.x_box, 3)) return false;
         Timed tm(p, st, 7, gi);
-        split_launch_fgrad(f, t.blocks, t.smem, st);
+        split_launch_fgrad(f, t.blocks, t.smem, tm.ls());
     }
     if (!launched_ok()) return false;
     const bool below = split_at(p, gi - 1);
@@ -570,7 +575,7 @@ bool split_backward(ftp_plan* p, const GroupPlan& g, int gi, const float* x, con
         a.out_f = din; a.og = a.g;
     }
     { Timed t(p, st, 8, gi);
-      split_launch_conv(a, g.sp.d.nb, g.sp.d.blocks, g.sp.d.smem, st); }
+      split_launch_conv(a, g.sp.d.nb, g.sp.d.blocks, g.sp.d.smem, t.ls()); }
     return launched_ok();
 }
 
@@ -593,8 +598,8 @@ int forward_impl(ftp_plan* p, const float* x, const float* params, float* y, voi
         GroupArgs a;
         fill_common(p, g, false, x, params, ws, a);
         { Timed t(p, st, 1, (int)gi);
-          if (max_window(g) <= 3) fwd_group_kernel<3><<<dim3(a.R * a.Q, p->N), kThreads, g.fwd.smem_bytes, st>>>(a);
-          else fwd_group_kernel<7><<<dim3(a.R * a.Q, p->N), kThreads, g.fwd.smem_bytes, st>>>(a); }
+          if (max_window(g) <= 3) launch(fwd_group_kernel<3>, dim3(a.R * a.Q, p->N), kThreads, g.fwd.smem_bytes, t.ls(), a);
+          else launch(fwd_group_kernel<7>, dim3(a.R * a.Q, p->N), kThreads, g.fwd.smem_bytes, t.ls(), a); }
         if (!launched_ok()) return FTP_ERR_CUDA;
     }
     if (y) {
@@ -624,7 +629,7 @@ int reduce_groups(ftp_plan* p, int first, int last, float* sgd_params, float lr,
     auto flush = [&]() {
         if (!ra.n) return;
         Timed t(p, st, 5, timed_group);
-        reduce_sgd_tc_kernel<<<dim3(1184, ra.n), 128, 0, st>>>(ra, sgd_params, lr, grad_out);
+        launch(reduce_sgd_tc_kernel, dim3(1184, ra.n), 128, 0, t.ls(), ra, sgd_params, lr, grad_out);
         ra.n = 0;
     };
     for (int gi = first; gi <= last; ++gi) {
@@ -689,7 +694,7 @@ bool tc_filter_grad(ftp_plan* p, const GroupPlan& g, int gi, const TcGroupArgs& 
     const size_t total = (size_t)p->N * (op.cout16 / 8) * op.out_H * op.out_W;
     if (!dz_ready) {
         { Timed tm(p, st, 6, gi);
-          delta_act_planes_kernel<<<(int)std::min<size_t>((total + 255) / 256, (size_t)kSmCount * 16), 256, 0, st>>>(d); }
+          launch(delta_act_planes_kernel, (int)std::min<size_t>((total + 255) / 256, (size_t)kSmCount * 16), 256, 0, tm.ls(), d); }
         if (!launched_ok()) return false;
     }
 
@@ -706,8 +711,9 @@ bool tc_filter_grad(ftp_plan* p, const GroupPlan& g, int gi, const TcGroupArgs& 
     f.Ms = t.Ms; f.slices = t.slices; f.ncols = t.ncols; f.nci = t.nci;
     f.R = t.R; f.Wp = t.Wp; f.bands_img = t.bands_img; f.bands = t.bands; f.shares = t.shares;
     f.dz_plane = t.dz_plane; f.x_plane = t.x_plane; f.stage_bytes = t.stage_bytes;
+    f.hurry = (double)((t.bands + t.shares - 1) / t.shares) * (t.k * t.k + 1) * ((t.R * t.Wp + 15) / 16) * tc_mma_cycles(t.ncols) < kHurryCycles;
     { Timed tm(p, st, 7, gi);
-      filter_grad_tc_rows_kernel<<<t.blocks, kTcFgThreads, t.smem_bytes, st>>>(f); }
+      launch(filter_grad_tc_rows_kernel, t.blocks, kTcFgThreads, one_block_smem(t.smem_bytes), tm.ls(), f); }
     if (!launched_ok()) return false;
 
     // input delta: the convolution of dz with the rotated filters (dz planes in, delta planes out)
@@ -731,7 +737,7 @@ bool tc_filter_grad(ftp_plan* p, const GroupPlan& g, int gi, const TcGroupArgs& 
                         a.error, st))
         return false;
     { Timed tm(p, st, 10, gi);
-      launch_fold_windows(reinterpret_cast<const __nv_bfloat16*>(dz_below), dx, p->N, op.cin, op.in_H, op.in_W, st); }
+      launch_fold_windows(reinterpret_cast<const __nv_bfloat16*>(dz_below), dx, p->N, op.cin, op.in_H, op.in_W, tm.ls()); }
     return launched_ok();
 }
 
@@ -758,8 +764,8 @@ int backward_tc(ftp_plan* p, const float* x, const float* dy, const float* param
         { Timed t(p, st, 3, gi);
           const size_t smem = tc_smem(g.bwd.smem_bytes, g.bwd.ctas);
           const int tile_bytes = (int)(smem - tc_fixed_bytes(g.bwd.stages));
-          if (g.bwd.ctas == 2) bwd_group_tc_kernel<256><<<g.bwd.blocks, 256, smem, st>>>(a, tile_bytes, kTcTmemCols / 2, g.bwd.stages);
-          else bwd_group_tc_kernel<512><<<g.bwd.blocks, 512, smem, st>>>(a, tile_bytes, kTcTmemCols, g.bwd.stages); }
+          if (g.bwd.ctas == 2) launch(bwd_group_tc_kernel<256>, g.bwd.blocks, 256, smem, t.ls(), a, tile_bytes, kTcTmemCols / 2, g.bwd.stages);
+          else launch(bwd_group_tc_kernel<512>, g.bwd.blocks, 512, smem, t.ls(), a, tile_bytes, kTcTmemCols, g.bwd.stages); }
         if (!launched_ok()) return FTP_ERR_CUDA;
         if (p->group_ready) {                         // ftp_step_grad_groups: this group's sets are summed right away
             const int rc = reduce_group_and_notify(p, gi, grad_out, ws, st);
@@ -779,8 +785,8 @@ int backward_tc(ftp_plan* p, const float* x, const float* dy, const float* param
             const int blocks = (int)std::min<size_t>((rows + 7) / 8, (size_t)kSmCount * 16);
             const size_t tab = (size_t)(2 * h.W + 2 * h.H + 3 * h.Q + 3 * h.R + 2) * sizeof(int);
             { Timed t(p, st, 4, gi);
-              if (planes) halo_sum_planes_kernel<<<blocks, 256, tab, st>>>(h);
-              else halo_sum_kernel<<<blocks, 256, tab, st>>>(h); }
+              if (planes) launch(halo_sum_planes_kernel, blocks, 256, tab, t.ls(), h);
+              else launch(halo_sum_kernel, blocks, 256, tab, t.ls(), h); }
             if (!launched_ok()) return FTP_ERR_CUDA;
         }
     }
@@ -820,8 +826,8 @@ int backward_impl(ftp_plan* p, const float* x, const float* dy, const float* par
         
         a.need_dx = (gi > 0 || dx != nullptr) ? 1 : 0;
         { Timed t(p, st, 3, gi);
-          if (max_window(g) <= 3) bwd_group_kernel<3><<<g.bwd.blocks, kThreads, g.bwd.smem_bytes, st>>>(a);
-          else bwd_group_kernel<7><<<g.bwd.blocks, kThreads, g.bwd.smem_bytes, st>>>(a); }
+          if (max_window(g) <= 3) launch(bwd_group_kernel<3>, g.bwd.blocks, kThreads, g.bwd.smem_bytes, t.ls(), a);
+          else launch(bwd_group_kernel<7>, g.bwd.blocks, kThreads, g.bwd.smem_bytes, t.ls(), a); }
         if (!launched_ok()) return FTP_ERR_CUDA;
         if (p->group_ready) { const int rc = reduce_group_and_notify(p, gi, grad_out, ws, st); if (rc != FTP_OK) return rc; }
         if (a.need_dx) {
@@ -836,7 +842,7 @@ int backward_impl(ftp_plan* p, const float* x, const float* dy, const float* par
             const size_t rows = (size_t)p->N * s.C * s.H;
             const int blocks = (int)std::min<size_t>((rows + 7) / 8, (size_t)kSmCount * 16);
             { Timed t(p, st, 4, gi);
-              halo_sum_kernel<<<blocks, 256, (size_t)(2 * h.W + 2 * h.H + 3 * h.Q + 3 * h.R + 2) * sizeof(int), st>>>(h); }
+              launch(halo_sum_kernel, blocks, 256, (size_t)(2 * h.W + 2 * h.H + 3 * h.Q + 3 * h.R + 2) * sizeof(int), t.ls(), h); }
             if (!launched_ok()) return FTP_ERR_CUDA;
         }
     }
@@ -1039,11 +1045,11 @@ static int step_impl(ftp_plan* plan, const float* x, const float* dy, const floa
         float* d = ws_ptr(workspace, plan->ws.dy_off);
         float* sums = ws_ptr(workspace, plan->ws.loss_off);
         { Timed t(plan, st, 2, -1);
-          mse_delta_kernel<<<plan->loss_blocks, 256, 0, st>>>(y32 ? y32 : map_ptr(plan, x, workspace, (int)plan->layers.size() + 1),
+          launch(mse_delta_kernel, plan->loss_blocks, 256, 0, t.ls(), y32 ? y32 : map_ptr(plan, x, workspace, (int)plan->layers.size() + 1),
                                                              target, d, M, sums); }
         if (loss_out) {
             Timed t(plan, st, 2, -1);
-            mse_finish_kernel<<<1, 256, 0, st>>>(sums, plan->loss_blocks, M, loss_out);
+            launch(mse_finish_kernel, 1, 256, 0, t.ls(), sums, plan->loss_blocks, M, loss_out);
         }
         if (!launched_ok()) return FTP_ERR_CUDA;
         delta = d;
@@ -1061,10 +1067,10 @@ int ftp_loss_mse(ftp_plan* plan, const float* y, const float* target, float* dy,
     float* d = dy ? dy : ws_ptr(workspace, plan->ws.dy_off);
     float* sums = ws_ptr(workspace, plan->ws.loss_off);
     { Timed t(plan, st, 2, -1);
-      mse_delta_kernel<<<plan->loss_blocks, 256, 0, st>>>(y, target, d, M, sums); }
+      launch(mse_delta_kernel, plan->loss_blocks, 256, 0, t.ls(), y, target, d, M, sums); }
     if (loss_out) {
         Timed t(plan, st, 2, -1);
-        mse_finish_kernel<<<1, 256, 0, st>>>(sums, plan->loss_blocks, M, loss_out);
+        launch(mse_finish_kernel, 1, 256, 0, t.ls(), sums, plan->loss_blocks, M, loss_out);
     }
     return launched_ok() ? FTP_OK : FTP_ERR_CUDA;
 }

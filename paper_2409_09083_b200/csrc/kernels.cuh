@@ -8,6 +8,7 @@
 
 #include <cuda_runtime.h>
 
+#include "launch.cuh"
 #include "plan.hpp"
 
 namespace ftp {
@@ -698,6 +699,8 @@ __device__ __forceinline__ void bias_grad_tile(const float* __restrict__ d, int 
 template <int KMAX>
 __global__ void __launch_bounds__(kThreads, 1) fwd_group_kernel(const __grid_constant__ GroupArgs A)
 {
+    next_launch();
+    previous_launches();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int* hdr = reinterpret_cast<int*>(smem_raw);
     float* sm = reinterpret_cast<float*>(smem_raw + kSmemHeader);
@@ -779,6 +782,8 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_group_kernel(const __grid_con
 template <int KMAX>
 __global__ void __launch_bounds__(kThreads, 1) bwd_group_kernel(const __grid_constant__ GroupArgs A)
 {
+    next_launch();
+    previous_launches();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int* hdr = reinterpret_cast<int*>(smem_raw);
     unsigned char* smb = smem_raw + kSmemHeader;
@@ -918,6 +923,8 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_group_kernel(const __grid_con
 // (row, column) order: the backward boundary exchange at a group input.
 __global__ void halo_sum_kernel(const __grid_constant__ HaloSumArgs A)
 {
+    next_launch();
+    previous_launches();
     // The cover / span / offset tables go to shared memory first: every output value walks through
     // three of them in a row, which from global memory is three dependent round trips.
     extern __shared__ int halo_tab[];
@@ -983,6 +990,8 @@ __global__ void halo_sum_kernel(const __grid_constant__ HaloSumArgs A)
 __global__ void pack_filters_kernel(const __grid_constant__ PackArgs A, const float* __restrict__ params,
                                     float* __restrict__ wf, float* __restrict__ wb)
 {
+    next_launch();
+    previous_launches();
     const PackLayer L = A.l[blockIdx.y];
     const int KK = L.k * L.k;
     const long long nf = (long long)L.cin * KK * L.cout_pad, nb = (long long)L.cout * KK * L.cin_pad;
@@ -1011,6 +1020,8 @@ __global__ void sgd_kernel(float* __restrict__ params, const float* __restrict__
 __global__ void mse_delta_kernel(const float* __restrict__ y, const float* __restrict__ t, float* __restrict__ d,
                                  size_t M, float* __restrict__ block_sums)
 {
+    next_launch();
+    previous_launches();
     __shared__ float red[256];
     const float scale = 2.0f / (float)M;
     float s = 0.f;
@@ -1031,6 +1042,8 @@ __global__ void mse_delta_kernel(const float* __restrict__ y, const float* __res
 // Sums the per-block partial sums in a fixed order (strided per thread, then a tree) and writes the mean.
 __global__ void mse_finish_kernel(const float* __restrict__ block_sums, int n, size_t M, float* __restrict__ loss)
 {
+    next_launch();
+    previous_launches();
     __shared__ float red[256];
     float s = 0.f;
     for (int i = threadIdx.x; i < n; i += 256) s += block_sums[i];

@@ -497,6 +497,8 @@ __device__ __forceinline__ void filter_grad_mma(Pipe& p, uint32_t dz_run /*addre
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 2 : 1) fwd_group_tc_kernel(const __grid_constant__ TcGroupArgs A, int tile_bytes, int tmem_cols, int stages)
 {
+    next_launch();
+    previous_launches();
     using namespace tcd;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Header* H = reinterpret_cast<Header*>(smem_raw);
@@ -626,6 +628,8 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 2 : 1) fwd_group_tc_
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 2 : 1) bwd_group_tc_kernel(const __grid_constant__ TcGroupArgs A, int tile_bytes, int tmem_cols, int stages)
 {
+    next_launch();
+    previous_launches();
     using namespace tcd;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Header* H = reinterpret_cast<Header*>(smem_raw);
@@ -814,6 +818,8 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 2 : 1) bwd_group_tc_
 // as the bf16 planes the previous group's backward reads.  One warp per row (n, plane, y).
 __global__ void halo_sum_planes_kernel(const __grid_constant__ HaloSumArgs A)
 {
+    next_launch();
+    previous_launches();
     extern __shared__ int halo_tab[];
     int* xcover = halo_tab;              int* xspan = xcover + 2 * A.W;   int* xoff = xspan + 2 * A.Q;
     int* ycover = xoff + A.Q + 1;        int* yspan = ycover + 2 * A.H;   int* yoff = yspan + 2 * A.R;
@@ -897,6 +903,7 @@ struct TcReduceArgs { int n; TcReduceLayer l[kMaxOps * 2]; };
 __global__ void reduce_sgd_tc_kernel(const __grid_constant__ TcReduceArgs A, float* __restrict__ params, float lr,
                                      float* __restrict__ grad_out)
 {
+    previous_launches();
     // Threads walk the set's own arrangement, so the reads of every set are coalesced (the sets are the
     // bulk of the traffic); the one write per parameter goes to its place in the caller's arrangement.
     const TcReduceLayer L = A.l[blockIdx.y];
@@ -927,6 +934,7 @@ __global__ void reduce_sgd_tc_kernel(const __grid_constant__ TcReduceArgs A, flo
 __global__ void planes_to_nchw_kernel(const __nv_bfloat16* __restrict__ src, float* __restrict__ dst, int N, int C, int C16,
                                       int H, int W)
 {
+    previous_launches();
     const size_t total = (size_t)N * C * H * W;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
         const int x = (int)(e % W); size_t t = e / W;
@@ -945,6 +953,8 @@ struct TcPackArgs { int n, dirs; int* error; TcPackLayer l[kMaxOps * 2]; };     
 __global__ void pack_filters_tc_kernel(const __grid_constant__ TcPackArgs A, const float* __restrict__ params,
                                        __nv_bfloat16* __restrict__ wf, __nv_bfloat16* __restrict__ wb)
 {
+    next_launch();
+    previous_launches();
     if (A.error && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *A.error = 0;
     const TcPackLayer L = A.l[blockIdx.y];
     const int KK = L.k * L.k;
@@ -973,6 +983,7 @@ __global__ void pack_filters_tc_kernel(const __grid_constant__ TcPackArgs A, con
 // ... and of the banded kernels (pack.cuh)
 __global__ void __launch_bounds__(256) pack_banded_kernel(const __grid_constant__ PackTilesArgs A, const float* __restrict__ params)
 {
+    previous_launches();
     __shared__ float s[kPackSmemFloats];
     pack_tiles<1>(A, params, s, [](const float* v, uint4* p) { p[0] = tcd::pack8(v); });
 }

@@ -28,29 +28,29 @@ bool split_prepare_device()
     return cudaFuncSetAttribute(sp::fgrad_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmemBudget) == cudaSuccess;
 }
 
-void split_launch_conv(const SplitConvArgs& a, int nb, int blocks, int smem, void* stream)
+void split_launch_conv(const SplitConvArgs& a, int nb, int blocks, int smem, LaunchStream ls)
 {
-    conv_kernel(a.K, nb)<<<blocks, sp::kConvThreads, smem, static_cast<cudaStream_t>(stream)>>>(a);
+    launch(conv_kernel(a.K, nb), blocks, sp::kConvThreads, one_block_smem(smem), ls, a);
 }
 
-void split_launch_fgrad(const SplitFgArgs& a, int blocks, int smem, void* stream)
+void split_launch_fgrad(const SplitFgArgs& a, int blocks, int smem, LaunchStream ls)
 {
-    sp::fgrad_split_kernel<<<blocks, sp::kFgThreads, smem, static_cast<cudaStream_t>(stream)>>>(a);
+    launch(sp::fgrad_split_kernel, blocks, sp::kFgThreads, one_block_smem(smem), ls, a);
 }
 
-void split_launch_planes(const float* src, uint4* dst, const SplitGeom& g, int C, void* stream)
+void split_launch_planes(const float* src, uint4* dst, const SplitGeom& g, int C, LaunchStream ls)
 {
-    sp::split_planes_kernel<<<helper_blocks((long long)g.planes * g.tp), 256, 0, static_cast<cudaStream_t>(stream)>>>(src, dst, g, C);
+    launch(sp::split_planes_kernel, helper_blocks((long long)g.planes * g.tp), 256, 0, ls, src, dst, g, C);
 }
 
-void split_launch_delta(const SplitDeltaArgs& a, void* stream)
+void split_launch_delta(const SplitDeltaArgs& a, LaunchStream ls)
 {
-    sp::split_delta_kernel<<<helper_blocks((long long)a.low.planes * a.low.tp), 256, 0, static_cast<cudaStream_t>(stream)>>>(a);
+    launch(sp::split_delta_kernel, helper_blocks((long long)a.low.planes * a.low.tp), 256, 0, ls, a);
 }
 
-void split_launch_pack(const PackTilesArgs& a, const float* params, void* stream)
+void split_launch_pack(const PackTilesArgs& a, const float* params, LaunchStream ls)
 {
-    sp::pack_split_kernel<<<a.tiles, 256, 0, static_cast<cudaStream_t>(stream)>>>(a, params);
+    launch(sp::pack_split_kernel, a.tiles, 256, 0, ls, a, params);
 }
 
 }  // namespace ftp

@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_split_kernel(const __gri
         fence_mbar_init();
     }
     if (warp == 0) { __syncwarp(); tmem_alloc(smem_u32(&H->tmem_base), (uint32_t)kTcTmemCols); }
+    previous_launches();
     // entries of the output map that no item covers
     if (A.out_s) {
         if (A.mode == kSplitPool) zero_margins(A.out_s, A.og, kSplitLead + A.og.wp, kSplitLead + A.og.rows * A.og.wp);
@@ -612,6 +613,7 @@ __global__ void __launch_bounds__(kFgThreads, 1) fgrad_split_kernel(const __grid
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
+    previous_launches();
     const uint32_t tmem = H->tmem_base;
 
     auto wait = [&](unsigned long long* bar, uint32_t parity, unsigned sleep_ns = 0) {
@@ -802,6 +804,7 @@ __global__ void __launch_bounds__(kFgThreads, 1) fgrad_split_kernel(const __grid
 // fp32 NCHW map -> split map, zero entries included.  One thread per entry and 8-channel plane.
 __global__ void split_planes_kernel(const float* __restrict__ src, uint4* __restrict__ dst, const __grid_constant__ SplitGeom g, int C)
 {
+    previous_launches();
     const long long total = (long long)g.planes * g.tp;
     const size_t HW = (size_t)g.H * g.W, part = (size_t)g.planes * g.tp;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
@@ -820,6 +823,7 @@ __global__ void split_planes_kernel(const float* __restrict__ src, uint4* __rest
 // writes the four members of the window.
 __global__ void split_delta_kernel(const __grid_constant__ SplitDeltaArgs A)
 {
+    previous_launches();
     const SplitGeom& g = A.low;
     const long long total = (long long)g.planes * g.tp;
     const size_t HW = (size_t)g.H * g.W, part = (size_t)A.g.planes * A.g.tp;
@@ -856,6 +860,7 @@ __global__ void split_delta_kernel(const __grid_constant__ SplitDeltaArgs A)
 
 __global__ void __launch_bounds__(256) pack_split_kernel(const __grid_constant__ PackTilesArgs A, const float* __restrict__ params)
 {
+    previous_launches();
     __shared__ float s[kPackSmemFloats];
     pack_tiles<3>(A, params, s, [](const float* v, uint4* p) { split8(v, p[0], p[1], p[2]); });
 }

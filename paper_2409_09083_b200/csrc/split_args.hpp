@@ -6,6 +6,7 @@
 
 #include <vector_types.h>
 
+#include "launch_stream.hpp"
 #include "plan.hpp"
 
 namespace ftp {
@@ -75,10 +76,10 @@ struct SplitDeltaArgs {             // fp32 NCHW delta -> dz split map
 };
 
 bool split_prepare_device();
-void split_launch_conv(const SplitConvArgs& a, int nb, int blocks, int smem, void* stream);
-void split_launch_fgrad(const SplitFgArgs& a, int blocks, int smem, void* stream);
-void split_launch_planes(const float* src, uint4* dst, const SplitGeom& g, int C, void* stream);
-void split_launch_delta(const SplitDeltaArgs& a, void* stream);
+void split_launch_conv(const SplitConvArgs& a, int nb, int blocks, int smem, LaunchStream ls);
+void split_launch_fgrad(const SplitFgArgs& a, int blocks, int smem, LaunchStream ls);
+void split_launch_planes(const float* src, uint4* dst, const SplitGeom& g, int C, LaunchStream ls);
+void split_launch_delta(const SplitDeltaArgs& a, LaunchStream ls);
 
 // Packing launches (pack.cuh): 32 x 32 channel tiles [tile_begin, next layer's tile_begin) of a layer.
 struct PackTilesLayer { long long p_off; uint4* wf; uint4* wd; int cin, cout, k, cin16, cout16, ns_f, kpc_f, ns_d, kpc_d, tile_begin; };
@@ -89,6 +90,6 @@ struct PackTilesArgs {
     int* error;                     // error word to clear, or null
     PackTilesLayer l[kPackTilesLayers];
 };
-void split_launch_pack(const PackTilesArgs& a, const float* params, void* stream);   // three parts
+void split_launch_pack(const PackTilesArgs& a, const float* params, LaunchStream ls);   // three parts
 
 }  // namespace ftp

@@ -11,13 +11,13 @@ namespace ftp {
 namespace {
 
 template <int K, int CO, int VEC, int T>
-void launch_conv(const ConvRowsArgs& a, int blocks, cudaStream_t st)
+void launch_conv(const ConvRowsArgs& a, int blocks, LaunchStream st)
 {
-    conv_rows_kernel<K, CO, VEC, T><<<blocks, T, StGeom<K, CO, T>::smem_bytes, st>>>(a);
+    launch(conv_rows_kernel<K, CO, VEC, T>, blocks, T, StGeom<K, CO, T>::smem_bytes, st, a);
 }
 
 template <int K, int CO, int T>
-void launch_conv_vec(const ConvRowsArgs& a, int blocks, cudaStream_t st)
+void launch_conv_vec(const ConvRowsArgs& a, int blocks, LaunchStream st)
 {
     if ((a.W & 3) == 0) launch_conv<K, CO, 4, T>(a, blocks, st);
     else if ((a.W & 1) == 0) launch_conv<K, CO, 2, T>(a, blocks, st);
@@ -58,7 +58,7 @@ size_t st_conv_smem_bytes(int k, int co_tile, int threads)
 size_t st_filter_grad_smem_bytes(int k) { return k == 3 ? FgGeom<3>::smem_bytes : kF1SmemBytes; }
 
 template <int T>
-void launch_conv_t(const ConvRowsArgs& a, int k, int co_tile, int blocks, cudaStream_t st)
+void launch_conv_t(const ConvRowsArgs& a, int k, int co_tile, int blocks, LaunchStream st)
 {
     if (k == 3 && co_tile == 64) launch_conv_vec<3, 64, T>(a, blocks, st);
     else if (k == 3) launch_conv_vec<3, 32, T>(a, blocks, st);
@@ -66,40 +66,37 @@ void launch_conv_t(const ConvRowsArgs& a, int k, int co_tile, int blocks, cudaSt
     else launch_conv_vec<1, 32, T>(a, blocks, st);
 }
 
-void st_launch_conv_rows(ConvRowsArgs& a, int k, int co_tile, int threads, int blocks, void* stream)
+void st_launch_conv_rows(ConvRowsArgs& a, int k, int co_tile, int threads, int blocks, LaunchStream st)
 {
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
     a.rp_img = (a.H + 1) / 2; a.x_tiles = (a.W + kStCols - 1) / kStCols; a.co_tiles = (a.Cout + co_tile - 1) / co_tile;
     if (threads == 128) launch_conv_t<128>(a, k, co_tile, blocks, st);
     else launch_conv_t<256>(a, k, co_tile, blocks, st);
 }
 
-void st_launch_filter_grad_rows(FilterGradRowsArgs& a, int k, int blocks, void* stream)
+void st_launch_filter_grad_rows(FilterGradRowsArgs& a, int k, int blocks, LaunchStream st)
 {
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
     a.rp_img = (a.H + 1) / 2; a.x_tiles = (a.W + kStCols - 1) / kStCols;
     a.co_tiles = (a.Cout + kFgCo - 1) / kFgCo; a.ci_tiles = (a.Cin + kFgCi - 1) / kFgCi;
-    if (k == 3) { filter_grad_rows_kernel<3><<<blocks, kStThreads, FgGeom<3>::smem_bytes, st>>>(a); return; }
+    if (k == 3) { launch(filter_grad_rows_kernel<3>, blocks, kStThreads, FgGeom<3>::smem_bytes, st, a); return; }
     // 1 x 1: a contraction over the flat pixels of an image, 64 x 128 channel slices
     a.co_tiles = (a.Cout + kF1Co - 1) / kF1Co; a.ci_tiles = (a.Cin + kF1Ci - 1) / kF1Ci;
-    filter_grad_1x1_kernel<<<blocks, kStThreads, kF1SmemBytes, st>>>(a);
+    launch(filter_grad_1x1_kernel, blocks, kStThreads, kF1SmemBytes, st, a);
 }
 
 void st_launch_delta_act(const float* dy, const float* y, const unsigned char* arg, float* dz, size_t count, int pooled_width,
-                         float slope, int pool, void* stream)
+                         float slope, int pool, LaunchStream st)
 {
     const int blocks = (int)std::min<size_t>((count + 255) / 256, (size_t)kSmCount * 16);
-    delta_act_kernel<<<blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(dy, y, arg, dz, count, pooled_width, slope, pool);
+    launch(delta_act_kernel, blocks, 256, 0, st, dy, y, arg, dz, count, pooled_width, slope, pool);
 }
 
-void st_launch_thin_bwd(const ThinBwdArgs& a, int blocks, void* stream)
+void st_launch_thin_bwd(const ThinBwdArgs& a, int blocks, LaunchStream st)
 {
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
     switch (a.Cin) {
-    case 1: thin_bwd_kernel<1><<<blocks, kStThreads, kThinSmemBytes, st>>>(a); break;
-    case 2: thin_bwd_kernel<2><<<blocks, kStThreads, kThinSmemBytes, st>>>(a); break;
-    case 3: thin_bwd_kernel<3><<<blocks, kStThreads, kThinSmemBytes, st>>>(a); break;
-    default: thin_bwd_kernel<4><<<blocks, kStThreads, kThinSmemBytes, st>>>(a); break;
+    case 1: launch(thin_bwd_kernel<1>, blocks, kStThreads, kThinSmemBytes, st, a); break;
+    case 2: launch(thin_bwd_kernel<2>, blocks, kStThreads, kThinSmemBytes, st, a); break;
+    case 3: launch(thin_bwd_kernel<3>, blocks, kStThreads, kThinSmemBytes, st, a); break;
+    default: launch(thin_bwd_kernel<4>, blocks, kStThreads, kThinSmemBytes, st, a); break;
     }
 }
 

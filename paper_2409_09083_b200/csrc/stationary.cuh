@@ -24,6 +24,7 @@
 
 #include <cuda_runtime.h>
 
+#include "launch.cuh"
 #include "plan.hpp"
 #include "stationary_args.hpp"
 
@@ -77,6 +78,7 @@ template <int N> __device__ __forceinline__ void st_wait() { asm volatile("cp.as
 template <int K, int CO, int VEC, int T = kStThreads>
 __global__ void __launch_bounds__(T, 512 / T) conv_rows_kernel(const __grid_constant__ ConvRowsArgs A)
 {
+    previous_launches();
     using G = StGeom<K, CO, T>;
     extern __shared__ __align__(16) float st_smem[];
     constexpr int KK = K * K, P = G::P, RR = G::RR;
@@ -271,6 +273,7 @@ template <int K> struct FgGeom {
 template <int K>
 __global__ void __launch_bounds__(kStThreads, 2) filter_grad_rows_kernel(const __grid_constant__ FilterGradRowsArgs A)
 {
+    previous_launches();
     using G = FgGeom<K>;
     extern __shared__ __align__(16) float st_smem[];
     constexpr int KK = K * K, P = G::P, RR = G::RR;
@@ -398,6 +401,7 @@ constexpr int kF1SmemBytes = 2 * kF1Stage * 4;
 
 __global__ void __launch_bounds__(kStThreads, 3) filter_grad_1x1_kernel(const __grid_constant__ FilterGradRowsArgs A)
 {
+    previous_launches();
     extern __shared__ __align__(16) float st_smem[];
     const int tid = threadIdx.x, lane = tid & 31;
     const int cig = tid & 15, cog = tid >> 4;              // a warp: 16 input-channel groups x 2 output-channel groups
@@ -486,6 +490,7 @@ __global__ void __launch_bounds__(kStThreads, 3) filter_grad_1x1_kernel(const __
 __global__ void delta_act_kernel(const float* __restrict__ dy, const float* __restrict__ y, const unsigned char* __restrict__ arg,
                                  float* __restrict__ dz, size_t count /*elements of dy*/, int OW /*pooled width*/, float slope, int pool)
 {
+    previous_launches();
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x) {
         const float v = dy[e] * (y[e] > 0.f ? 1.f : slope);
         if (!pool) { dz[e] = v; continue; }
@@ -530,6 +535,7 @@ constexpr int kThinSmemBytes = (kThinSmemV + kThinSmemX + kThinSmemW) * 4 + kThi
 template <int CIN>
 __global__ void __launch_bounds__(kStThreads, 2) thin_bwd_kernel(const __grid_constant__ ThinBwdArgs A)
 {
+    previous_launches();
     extern __shared__ __align__(16) float st_smem[];
     float* sv = st_smem;                                   // [pooled pixel][33]: v per output channel
     float* sx = sv + kThinSmemV;                           // [ci][row][col]: input patch, global row 2 py0 - 1 at row 0

@@ -38,6 +38,7 @@ struct TcFilterGradArgs {
     float* partial;                           // partial sets of the group
     long long set_floats, tgp_off;            // floats per set, offset of this layer inside a set
     int* error;
+    int hurry;                                // a short launch: see kHurryCycles in launch.cuh
     int N, K, cout16, cin16;
     int Ms, slices;                           // output channels per block (64 or 128) and number of such slices
     int ncols, nci;                           // input channels per block (multiple of 16) and number of such slices
@@ -58,6 +59,7 @@ struct DeltaActPlanesArgs {
 // window): the same arithmetic and roundings as the fused backward kernel applies when it fills its dz tile.
 __global__ void delta_act_planes_kernel(const __grid_constant__ DeltaActPlanesArgs A)
 {
+    previous_launches();
     const int planes = A.cout16 / 8;
     const size_t total = (size_t)A.N * planes * A.out_H * A.out_W;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
@@ -99,6 +101,7 @@ __global__ void delta_act_planes_kernel(const __grid_constant__ DeltaActPlanesAr
 template <int C>
 __global__ void unroll_windows_kernel(const float* __restrict__ x, uint4* __restrict__ col, int N, int H, int W)
 {
+    previous_launches();
     constexpr int planes = (9 * C + 15) / 16 * 2;
     const size_t HW = (size_t)H * W, total = (size_t)N * HW;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
@@ -132,6 +135,7 @@ __global__ void unroll_windows_kernel(const float* __restrict__ x, uint4* __rest
 template <int C>
 __global__ void fold_windows_kernel(const __nv_bfloat16* __restrict__ dcol, float* __restrict__ dx, int N, int H, int W)
 {
+    previous_launches();
     constexpr int planes = (9 * C + 15) / 16 * 2;
     const size_t HW = (size_t)H * W, total = (size_t)N * HW;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
@@ -158,30 +162,30 @@ __global__ void fold_windows_kernel(const __nv_bfloat16* __restrict__ dcol, floa
 }
 
 // the two kernels for the channel counts the route takes (9 C <= 64)
-inline void launch_unroll_windows(const float* x, uint4* col, int N, int C, int H, int W, cudaStream_t st)
+inline void launch_unroll_windows(const float* x, uint4* col, int N, int C, int H, int W, LaunchStream st)
 {
     const int blocks = (int)std::min<size_t>(((size_t)N * H * W + 255) / 256, (size_t)kSmCount * 16);
     switch (C) {
-        case 1: unroll_windows_kernel<1><<<blocks, 256, 0, st>>>(x, col, N, H, W); break;
-        case 2: unroll_windows_kernel<2><<<blocks, 256, 0, st>>>(x, col, N, H, W); break;
-        case 3: unroll_windows_kernel<3><<<blocks, 256, 0, st>>>(x, col, N, H, W); break;
-        case 4: unroll_windows_kernel<4><<<blocks, 256, 0, st>>>(x, col, N, H, W); break;
-        case 5: unroll_windows_kernel<5><<<blocks, 256, 0, st>>>(x, col, N, H, W); break;
-        case 6: unroll_windows_kernel<6><<<blocks, 256, 0, st>>>(x, col, N, H, W); break;
-        default: unroll_windows_kernel<7><<<blocks, 256, 0, st>>>(x, col, N, H, W); break;
+        case 1: launch(unroll_windows_kernel<1>, blocks, 256, 0, st, x, col, N, H, W); break;
+        case 2: launch(unroll_windows_kernel<2>, blocks, 256, 0, st, x, col, N, H, W); break;
+        case 3: launch(unroll_windows_kernel<3>, blocks, 256, 0, st, x, col, N, H, W); break;
+        case 4: launch(unroll_windows_kernel<4>, blocks, 256, 0, st, x, col, N, H, W); break;
+        case 5: launch(unroll_windows_kernel<5>, blocks, 256, 0, st, x, col, N, H, W); break;
+        case 6: launch(unroll_windows_kernel<6>, blocks, 256, 0, st, x, col, N, H, W); break;
+        default: launch(unroll_windows_kernel<7>, blocks, 256, 0, st, x, col, N, H, W); break;
     }
 }
-inline void launch_fold_windows(const __nv_bfloat16* dcol, float* dx, int N, int C, int H, int W, cudaStream_t st)
+inline void launch_fold_windows(const __nv_bfloat16* dcol, float* dx, int N, int C, int H, int W, LaunchStream st)
 {
     const int blocks = (int)std::min<size_t>(((size_t)N * H * W + 255) / 256, (size_t)kSmCount * 16);
     switch (C) {
-        case 1: fold_windows_kernel<1><<<blocks, 256, 0, st>>>(dcol, dx, N, H, W); break;
-        case 2: fold_windows_kernel<2><<<blocks, 256, 0, st>>>(dcol, dx, N, H, W); break;
-        case 3: fold_windows_kernel<3><<<blocks, 256, 0, st>>>(dcol, dx, N, H, W); break;
-        case 4: fold_windows_kernel<4><<<blocks, 256, 0, st>>>(dcol, dx, N, H, W); break;
-        case 5: fold_windows_kernel<5><<<blocks, 256, 0, st>>>(dcol, dx, N, H, W); break;
-        case 6: fold_windows_kernel<6><<<blocks, 256, 0, st>>>(dcol, dx, N, H, W); break;
-        default: fold_windows_kernel<7><<<blocks, 256, 0, st>>>(dcol, dx, N, H, W); break;
+        case 1: launch(fold_windows_kernel<1>, blocks, 256, 0, st, dcol, dx, N, H, W); break;
+        case 2: launch(fold_windows_kernel<2>, blocks, 256, 0, st, dcol, dx, N, H, W); break;
+        case 3: launch(fold_windows_kernel<3>, blocks, 256, 0, st, dcol, dx, N, H, W); break;
+        case 4: launch(fold_windows_kernel<4>, blocks, 256, 0, st, dcol, dx, N, H, W); break;
+        case 5: launch(fold_windows_kernel<5>, blocks, 256, 0, st, dcol, dx, N, H, W); break;
+        case 6: launch(fold_windows_kernel<6>, blocks, 256, 0, st, dcol, dx, N, H, W); break;
+        default: launch(fold_windows_kernel<7>, blocks, 256, 0, st, dcol, dx, N, H, W); break;
     }
 }
 
@@ -228,6 +232,7 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
+    previous_launches();
     const uint32_t tmem = H->tmem_base;
 
     auto wait = [&](unsigned long long* bar, uint32_t parity, unsigned sleep_ns = 0) {
@@ -300,6 +305,8 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
     if (!have && nb > 0) mbar_wait(smem_u32(&H->done), 0, 200000000ll);   // gave up: the MMAs under way still end first
     fence_after_sync();
 
+    if (A.hurry) next_launch();
+
     // tensor memory -> this share's partial set; lane quarter q holds rows 32q.. (Ms = 128) or rows 16q.. in its
     // first 16 lanes (Ms = 64).  The slices of the blocks are disjoint: plain stores.
     const int q = warp & 3, half = warp >> 2;
@@ -359,6 +366,7 @@ struct TcConvRowsArgs {
     uint4* out;                               // output planes [N][cout16/8][OH][OW] (OH = H / 2 with the pool)
     unsigned long long* arg;                  // pool: arg-max bytes in the same arrangement
     int* error;
+    int hurry;                                // a short launch: see kHurryCycles in launch.cuh
     int N, K, cin16, cout16, cout, H, W, pool;
     float slope;
     int Ns, slices;                           // output channels per item, number of slices
@@ -415,6 +423,7 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
+    previous_launches();
     const uint32_t tmem = H->tmem_base;
 
     auto wait = [&](unsigned long long* bar, uint32_t parity, unsigned sleep_ns = 0) {
@@ -674,6 +683,7 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
             if (lane == 0) mbar_arrive(smem_u32(&H->tfree[buf]));
         }
     }
+    if (A.hurry) next_launch();
     __syncthreads();
     // every MMA of the block has completed before the tensor memory goes back (also when a wait gave up)
     if (warp == 0) {
