@@ -148,7 +148,7 @@ int pack_filters(ftp_plan* p, const float* params, void* ws, int dirs, cudaStrea
                 uint4* base = reinterpret_cast<uint4*>(ws_ptr(ws, p->ws.sw_off));
                 add_pack_tiles(sa, PackTilesLayer{op.p_off, base + g.sp.wf_off, base + g.sp.wd_off, op.cin, op.cout, op.k, op.cin16, op.cout16,
                                                   g.sp.f.Ns, g.sp.f.kpc, g.sp.d.Ns, g.sp.d.kpc, 0});
-                continue;
+                if (!g.sp.rows_fwd) continue;
             }
             if (pa.n == kMaxOps * 2) {   // flush a full batch
                 { Timed t(p, st, 0, -1);
@@ -405,8 +405,18 @@ int forward_tc(ftp_plan* p, const float* x, const float* params, float* y, void*
     return FTP_OK;
 }
 
-// One-conv group run weight-stationary (stationary.cuh): the convolution with bias, activation and, where a
-// pool follows, the 2x2 maximum and its arg-max, written to the group's output map.
+// ---- split groups (split.cuh): one-conv groups of the fp32 path on the tensor cores ----
+inline uint4* split_ptr(void* ws, size_t off) { return reinterpret_cast<uint4*>(static_cast<unsigned char*>(ws) + off); }
+inline SplitGeom in_geom(const ftp_plan* p, const OpDesc& op) { return split_geom(p->N, op.cin, op.in_H, op.in_W); }      // input map
+inline SplitGeom dz_geom(const ftp_plan* p, const OpDesc& op) { return split_geom(p->N, op.cout, op.in_H, op.in_W); }     // conv output
+inline SplitGeom out_geom(const ftp_plan* p, const OpDesc& op) { return split_geom(p->N, op.cout, op.out_H, op.out_W); }  // after the pool
+inline bool split_at(const ftp_plan* p, int gi) { return gi >= 0 && gi < (int)p->groups.size() && p->groups[gi].sp.on; }
+// Whether the map between groups gi and gi + 1 exists as fp32 NCHW: always but between two groups of these kernels whose upper
+// one also runs its forward pass on them
+inline bool nchw_above(const ftp_plan* p, int gi) { return !split_at(p, gi) || !split_at(p, gi + 1) || p->groups[gi + 1].sp.rows_fwd; }
+
+// One-conv group whose forward pass runs weight-stationary (stationary.cuh): the convolution with bias, activation and, where a
+// pool follows, the 2x2 maximum and its arg-max, written to the group's output map, in split form too (or only) for a split group above.
 bool stationary_forward(ftp_plan* p, const GroupPlan& g, int gi, const float* x, const float* params, void* ws, cudaStream_t st)
 {
     const OpDesc& op = g.fwd_ops[0];
@@ -414,8 +424,11 @@ bool stationary_forward(ftp_plan* p, const GroupPlan& g, int gi, const float* x,
     a.in = map_ptr(p, x, ws, g.first);
     a.w = ws_ptr(ws, p->ws.wf_off) + op.wf_off;
     a.bias = params + op.p_off + (size_t)op.cout * op.cin * op.k * op.k;
-    a.out = const_cast<float*>(map_ptr(p, x, ws, op.out_map));
-    a.arg = g.st.pool ? static_cast<unsigned char*>(ws) + p->ws.arg_off[op.out_map - 1] : nullptr;
+    a.out = nchw_above(p, gi) ? const_cast<float*>(map_ptr(p, x, ws, op.out_map)) : nullptr;
+    a.og = out_geom(p, op);
+    if (split_at(p, gi + 1)) a.out_s = split_ptr(ws, p->groups[gi + 1].sp.in_off);
+    unsigned char* arg = g.st.pool ? static_cast<unsigned char*>(ws) + p->ws.arg_off[op.out_map - 1] : nullptr;
+    if (g.sp.on) a.arg_s = reinterpret_cast<unsigned long long*>(arg); else a.arg = arg;
     a.N = p->N; a.Cin = op.cin; a.Cout = op.cout; a.CoutPad = op.cout_pad; a.H = op.in_H; a.W = op.in_W;
     a.slope = op.slope; a.act = 1; a.pool = g.st.pool;
     { Timed t(p, st, 1, gi);
@@ -491,13 +504,6 @@ bool stationary_backward(ftp_plan* p, const GroupPlan& g, int gi, const float* x
     return true;
 }
 
-// ---- split groups (split.cuh): one-conv groups of the fp32 path on the tensor cores ----
-inline uint4* split_ptr(void* ws, size_t off) { return reinterpret_cast<uint4*>(static_cast<unsigned char*>(ws) + off); }
-inline SplitGeom in_geom(const ftp_plan* p, const OpDesc& op) { return split_geom(p->N, op.cin, op.in_H, op.in_W); }      // input map
-inline SplitGeom dz_geom(const ftp_plan* p, const OpDesc& op) { return split_geom(p->N, op.cout, op.in_H, op.in_W); }     // conv output
-inline SplitGeom out_geom(const ftp_plan* p, const OpDesc& op) { return split_geom(p->N, op.cout, op.out_H, op.out_W); }  // after the pool
-inline bool split_at(const ftp_plan* p, int gi) { return gi >= 0 && gi < (int)p->groups.size() && p->groups[gi].sp.on; }
-
 bool split_conv_args(SplitConvArgs& a, const SplitConvPlan& c, const uint4* in, const SplitGeom& g, int K, int cout, int cout16)
 {
     a.in = in;
@@ -513,10 +519,11 @@ bool split_forward(ftp_plan* p, const GroupPlan& g, int gi, const float* x, cons
 {
     const OpDesc& op = g.fwd_ops[0];
     uint4* in = split_ptr(ws, g.sp.in_off);
-    if (!split_at(p, gi - 1)) {                     // the group below wrote an fp32 map
+    if (gi == 0 || !p->groups[gi - 1].st.on) {      // a fused stack below wrote an fp32 map only
         Timed t(p, st, 9, gi);
         split_launch_planes(map_ptr(p, x, ws, g.first), in, in_geom(p, op), op.cin, t.ls());
     }
+    if (g.sp.rows_fwd) return stationary_forward(p, g, gi, x, params, ws, st);
     SplitConvArgs a{};
     if (!split_conv_args(a, g.sp.f, in, in_geom(p, op), op.k, op.cout, op.cout16)) return false;
     a.w = split_ptr(ws, p->ws.sw_off) + g.sp.wf_off;
@@ -525,7 +532,7 @@ bool split_forward(ftp_plan* p, const GroupPlan& g, int gi, const float* x, cons
     a.og = out_geom(p, op);
     if (op.kind == kOpConvPool) a.arg = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(ws) + p->ws.arg_off[op.out_map - 1]);
     if (split_at(p, gi + 1)) a.out_s = split_ptr(ws, p->groups[gi + 1].sp.in_off);
-    else a.out_f = const_cast<float*>(map_ptr(p, x, ws, op.out_map));
+    if (nchw_above(p, gi)) a.out_f = const_cast<float*>(map_ptr(p, x, ws, op.out_map));
     { Timed t(p, st, 1, gi);
       split_launch_conv(a, g.sp.f.nb, g.sp.f.blocks, g.sp.f.smem, t.ls()); }
     return launched_ok();

@@ -781,6 +781,12 @@ void plan_split(const ftp_plan& p, GroupPlan& g)
     g.sp.d = plan_split_conv(out, op.k, op.cin16, false);
     g.sp.g = plan_split_fg(in, op.k, op.cin16, op.cout16);
     g.sp.on = g.sp.f.on && g.sp.d.on && g.sp.g.shares > 0;
+    // Forward pass of the layers with at most 32 input channels: by the multiply-add kernel, whose sums they have always had.  Such a
+    // layer stands at the highest resolution, where the sign and pool decisions that fall on near-ties are most numerous and
+    // each moves a whole delta at the network input by up to its root mean square; bit for bit the same maps keep them
+    // where they were.  Its contraction is the shortest (288 terms), so it gains least: 16 x 304 x 304, 32 -> 64: 1.1 ms, on the
+    // split kernel 0.44 ms.
+    g.sp.rows_fwd = g.sp.on && op.cin <= 32;
 }
 // 16-byte entries of one packed arrangement
 inline long long split_w_entries(const SplitConvPlan& c, int k) { return (long long)c.slices * c.nchunks * 3 * k * k * c.kpc * c.Ns; }
@@ -792,7 +798,7 @@ double split_estimate_us(const ftp_plan& p, const GroupPlan& g, bool backward, b
     const double px = (double)p.N * op.in_H * op.in_W, flops = 2.0 * px * op.cin16 * op.cout16 * op.k * op.k;
     auto rate = [](int n) { return 150e6 * std::min(1.0, n / 2.0 / split_mma_cycles(n)); };
     const double in_us = px * op.cin16 * 6.0 / 4e6, out_us = px * op.cout16 * 6.0 / 4e6;
-    if (!backward) return flops / rate(g.sp.f.Ns) + in_us + out_us + 10.0;
+    if (!backward) return flops / (g.sp.rows_fwd ? kStatTflops * 1e6 : rate(g.sp.f.Ns)) + in_us + out_us + 10.0;
     double t = flops / rate(g.sp.g.rows3 ? 40 : g.sp.g.ncols) * (128.0 / g.sp.g.Ms) + in_us + out_us + 12.0;
     if (need_dx) t += flops / rate(g.sp.d.Ns) + in_us + out_us + 10.0;
     return t;
@@ -1296,7 +1302,8 @@ int build_plan(ftp_plan& p, const ftp_layer* layers, int n_layers, int N, int C,
                 if (op.kind == kOpConvPool) ws.arg_off[op.out_map - 1] = take((size_t)N * c16 * s.H * s.W);
                 continue;
             }
-            if (!(g.sp.on && &g != &p.groups.back() && (&g)[1].sp.on))       // (between split groups the map exists in split form only)
+            // (between split groups the map exists in split form only)
+            if (!(g.sp.on && &g != &p.groups.back() && (&g)[1].sp.on && !(&g)[1].sp.rows_fwd))
                 ws.map_off[op.out_map - 1] = take((size_t)N * s.C * s.H * s.W * 4);
             if (op.kind == kOpConvPool) {
                 const SplitGeom sg = split_geom(N, s.C, s.H, s.W);

@@ -180,6 +180,7 @@ struct SplitFgPlan {
 };
 struct SplitPlan {
     int on = 0;
+    int rows_fwd = 0;                           // forward pass by conv_rows_kernel (see plan_split)
     SplitConvPlan f, d;                         // forward, input delta
     SplitFgPlan g;
     size_t in_off = 0;                          // workspace: the group's input as a split map
@@ -192,7 +193,7 @@ constexpr double kSplitMinMacs = 1.0e8;   // see split_wanted in plan.cpp
 struct GroupPlan {
     int first = 0, last = 0;        // 1-based layers
     StatPlan st;
-    SplitPlan sp;                   // fp32 path: on = this one-conv group runs on the split kernels (st describes its CUDA-core form)
+    SplitPlan sp;                   // fp32 path: on = this one-conv group runs on the split kernels (st: its forward with rows_fwd)
     TcFgPlan tfg;
     TcConvPlan cf, cd;              // tfg.on: the forward convolution and the input-delta convolution (dz planes in, delta planes
                                     //   out: the conv with the channel counts exchanged and the filters rotated) as banded kernels

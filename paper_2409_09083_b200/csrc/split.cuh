@@ -28,36 +28,13 @@
 
 #include "pack.cuh"
 #include "split_args.hpp"
+#include "split_parts.cuh"
 #include "tc.cuh"
 
 namespace ftp {
 namespace sp {
 
 using namespace tc;
-
-// three bf16 parts of eight values; the first one rounded to 6 significant bits (nearest, ties away from zero)
-__device__ __forceinline__ void split8(const float* v, uint4& p0, uint4& p1, uint4& p2)
-{
-    uint32_t* a = &p0.x; uint32_t* b = &p1.x; uint32_t* c = &p2.x;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float x = v[2 * i], y = v[2 * i + 1];
-        const uint32_t bx = (__float_as_uint(x) + 0x20000u) & 0xfffc0000u, by = (__float_as_uint(y) + 0x20000u) & 0xfffc0000u;
-        a[i] = __byte_perm(bx, by, 0x7632);
-        const float rx = x - __uint_as_float(bx), ry = y - __uint_as_float(by);
-        const __nv_bfloat162 h1 = __floats2bfloat162_rn(rx, ry);
-        const float2 f1 = __bfloat1622float2(h1);
-        const __nv_bfloat162 h2 = __floats2bfloat162_rn(rx - f1.x, ry - f1.y);
-        b[i] = *reinterpret_cast<const uint32_t*>(&h1);
-        c[i] = *reinterpret_cast<const uint32_t*>(&h2);
-    }
-}
-__device__ __forceinline__ void store_split(uint4* base, size_t part_stride, size_t at, const float* v)
-{
-    uint4 p0, p1, p2;
-    split8(v, p0, p1, p2);
-    base[at] = p0; base[at + part_stride] = p1; base[at + 2 * part_stride] = p2;
-}
 
 // 32 lanes x 32 consecutive fp32 columns of tensor memory
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
@@ -74,27 +51,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// pixel of an entry (n, y, x); false: a zero entry of the map (edge column, row between images, lead or tail)
-__device__ __forceinline__ bool pixel_of(const SplitGeom& g, int e, int& n, int& y, int& x)
-{
-    const int r = e - kSplitLead, row = r / g.wp;
-    x = r - row * g.wp;
-    const int t = row - 1;
-    n = t / (g.H + 1); y = t - n * (g.H + 1);
-    return r >= 0 && t >= 0 && row < g.rows && x < g.W && y < g.H;
-}
-
-// zeros to the entries of every plane of a split map in front of `lo` and from `hi` on (all threads of the grid)
-__device__ __forceinline__ void zero_margins(uint4* out, const SplitGeom& g, int lo, int hi)
-{
-    const int per = lo + (g.tp - hi);
-    const long long total = 3ll * g.planes * per;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const int pl = (int)(i / per), j = (int)(i - (long long)pl * per);
-        out[(size_t)pl * g.tp + (j < lo ? j : hi + j - lo)] = make_uint4(0, 0, 0, 0);
-    }
 }
 
 constexpr int kMaxA = 3, kMaxB = 8;

@@ -26,6 +26,7 @@
 
 #include "launch.cuh"
 #include "plan.hpp"
+#include "split_parts.cuh"
 #include "stationary_args.hpp"
 
 namespace ftp {
@@ -79,6 +80,7 @@ template <int K, int CO, int VEC, int T = kStThreads>
 __global__ void __launch_bounds__(T, 512 / T) conv_rows_kernel(const __grid_constant__ ConvRowsArgs A)
 {
     previous_launches();
+    if (A.out_s) sp::zero_frame(A.out_s, A.og);
     using G = StGeom<K, CO, T>;
     extern __shared__ __align__(16) float st_smem[];
     constexpr int KK = K * K, P = G::P, RR = G::RR;
@@ -205,43 +207,73 @@ __global__ void __launch_bounds__(T, 512 / T) conv_rows_kernel(const __grid_cons
     const int rp = rp0 + rp_l;
     const int n = rp / A.rp_img, y = (rp - n * A.rp_img) * 2, x = x0 + cq_l * 4;
     if (n >= A.N || x >= A.W) return;
+    const int plane8 = (co0 >> 3) + cg;                      // 8-channel plane of this thread's output channels
+    const size_t opart = (size_t)A.og.planes * A.og.tp;
     if (!A.pool) {
+        if (A.out) {
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const int co = co0 + cg * 8 + c;
-            if (co >= A.Cout) break;
+            for (int c = 0; c < 8; ++c) {
+                const int co = co0 + cg * 8 + c;
+                if (co >= A.Cout) break;
 #pragma unroll
-            for (int p = 0; p < 2; ++p) {
-                if (y + p >= A.H) break;
-                float o[4];
+                for (int p = 0; p < 2; ++p) {
+                    if (y + p >= A.H) break;
+                    float o[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) { const float z = val(p, j, c); o[j] = A.act ? (z > 0.f ? z : A.slope * z) : z; }
-                float* dst = A.out + (((size_t)n * A.Cout + co) * A.H + y + p) * A.W + x;
-                if (x + 3 < A.W && (A.W & 3) == 0) *reinterpret_cast<float4*>(dst) = make_float4(o[0], o[1], o[2], o[3]);
-                else
+                    for (int j = 0; j < 4; ++j) { const float z = val(p, j, c); o[j] = A.act ? (z > 0.f ? z : A.slope * z) : z; }
+                    float* dst = A.out + (((size_t)n * A.Cout + co) * A.H + y + p) * A.W + x;
+                    if (x + 3 < A.W && (A.W & 3) == 0) *reinterpret_cast<float4*>(dst) = make_float4(o[0], o[1], o[2], o[3]);
+                    else
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) if (x + j < A.W) dst[j] = o[j];
+                        for (int j = 0; j < 4; ++j) if (x + j < A.W) dst[j] = o[j];
+                }
             }
+        }
+        if (A.out_s && plane8 < A.og.planes) {
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (y + p >= A.H || x + j >= A.W) continue;
+                    float o[8];
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) { const float z = val(p, j, c); o[c] = A.act ? (z > 0.f ? z : A.slope * z) : z; }
+                    sp::store_split(A.out_s, opart, (size_t)plane8 * A.og.tp + kSplitLead + (size_t)(1 + n * (A.H + 1) + y + p) * A.og.wp + x + j, o);
+                }
         }
     } else {
         const int OH = A.H >> 1, OW = A.W >> 1;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const int co = co0 + cg * 8 + c;
-            if (co >= A.Cout) break;
+        for (int h = 0; h < 2; ++h) {
+            if (x + 2 * h >= A.W) break;
+            float best[8];
+            unsigned long long am = 0ull;
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                if (x + 2 * h >= A.W) break;
+            for (int c = 0; c < 8; ++c) {
                 float v00 = val(0, 2 * h, c), v01 = val(0, 2 * h + 1, c), v10 = val(1, 2 * h, c), v11 = val(1, 2 * h + 1, c);
                 v00 = v00 > 0.f ? v00 : A.slope * v00; v01 = v01 > 0.f ? v01 : A.slope * v01;
                 v10 = v10 > 0.f ? v10 : A.slope * v10; v11 = v11 > 0.f ? v11 : A.slope * v11;
-                float best = v00; int am = 0;
-                if (v01 > best) { best = v01; am = 1; }
-                if (v10 > best) { best = v10; am = 2; }
-                if (v11 > best) { best = v11; am = 3; }
-                const size_t gi = (((size_t)n * A.Cout + co) * OH + (y >> 1)) * OW + (x >> 1) + h;
-                A.out[gi] = best;
-                if (A.arg) A.arg[gi] = (unsigned char)am;
+                best[c] = v00; unsigned m = 0;
+                if (v01 > best[c]) { best[c] = v01; m = 1; }
+                if (v10 > best[c]) { best[c] = v10; m = 2; }
+                if (v11 > best[c]) { best[c] = v11; m = 3; }
+                am |= (unsigned long long)m << (8 * c);
+            }
+            const int py = y >> 1, px = (x >> 1) + h;
+            if (A.out || A.arg) {
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const int co = co0 + cg * 8 + c;
+                    if (co >= A.Cout) break;
+                    const size_t gi = (((size_t)n * A.Cout + co) * OH + py) * OW + px;
+                    if (A.out) A.out[gi] = best[c];
+                    if (A.arg) A.arg[gi] = (unsigned char)(am >> (8 * c));
+                }
+            }
+            if (plane8 < A.og.planes && (A.out_s || A.arg_s)) {
+                const size_t e = (size_t)plane8 * A.og.tp + kSplitLead + (size_t)(1 + n * (OH + 1) + py) * A.og.wp + px;
+                if (A.out_s) sp::store_split(A.out_s, opart, e, best);
+                if (A.arg_s) A.arg_s[e] = am;
             }
         }
     }

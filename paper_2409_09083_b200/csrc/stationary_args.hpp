@@ -5,6 +5,7 @@
 
 #include "launch_stream.hpp"
 #include "plan.hpp"
+#include "split_args.hpp"
 
 namespace ftp {
 
@@ -13,6 +14,10 @@ struct ConvRowsArgs {
     const float* w;         // [Cin][K*K][CoutPad]: per input channel and tap, the 8-padded output channels
     const float* bias;      // [Cout] or null
     float* out;             // [N][Cout][H][W], or the pooled map [N][Cout][H/2][W/2] when pool != 0
+    // Where a group on the split kernels (split.cuh) reads the output: the same map in split form, its arg-max bytes as words of a
+    // plane; `out` and `arg` may then be null.  (out_s null: not wanted)
+    uint4* out_s; unsigned long long* arg_s;
+    SplitGeom og;
     unsigned char* arg;     // pool: arg-max (dy * 2 + dx, first maximum in row-major order) per pooled value
     int N, Cin, Cout, CoutPad, H, W;
     float slope;            // leaky-ReLU slope (act != 0)
