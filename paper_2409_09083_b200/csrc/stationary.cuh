@@ -594,42 +594,58 @@ __global__ void __launch_bounds__(kStThreads, 2) thin_bwd_kernel(const __grid_co
         const int n = tile / tiles_img, ty = (tile % tiles_img) / A.tiles_x, tx = tile % A.tiles_x;
         const int py0 = ty * kThinTH, px0 = tx * kThinTW;
         __syncthreads();                                   // the previous tile has been consumed
-        // stage v and arg-max: one warp per output channel at a time, lanes along the 10 x 34 pooled pixels of the tile
-        for (int co = warp; co < A.Cout; co += kStThreads / 32) {
-            const size_t base = ((size_t)n * A.Cout + co) * pplane;
-            // (all loads of a channel are issued before the first value is used: the loop is unrolled whole)
-            constexpr int kIt = (kThinPH * kThinPW + 31) / 32;
-            float dv[kIt], yv[kIt]; unsigned char av[kIt];
+        // Stage v and arg-max, lanes along the 10 x 34 pooled pixels of the tile, a warp takes four output channels.  Addresses are
+        // clamped into the map and the loads unconditional, so that 36 of them are in flight per thread: as conditional
+        // loads they were issued one by one and took two fifths of the kernel's warp cycles (16 images of 608 x 608, 3 -> 32
+        // channels: 1073 -> 660 us; what bounds the rest is instruction issue and shared-memory reads.  Packed multiply-adds
+        // with the filters staged in pairs, or the channels of a pixel in one 16-byte read, were slower: 690 and 700 us).
+        constexpr int kWarps = kStThreads / 32, kCos = kThinMaxCout / kWarps, kPix = kThinPH * kThinPW, kBatch = 3;
+        const size_t img = (size_t)n * A.Cout * pplane;
+#pragma unroll 1
+        for (int e0 = lane; e0 < kPix; e0 += 32 * kBatch) {
+            float dv[kBatch][kCos], yv[kBatch][kCos]; unsigned char av[kBatch][kCos]; bool in[kBatch];
 #pragma unroll
-            for (int it = 0; it < kIt; ++it) {
-                const int e = lane + 32 * it;
-                const int ly = e / kThinPW, lx = e - ly * kThinPW;
+            for (int i = 0; i < kBatch; ++i) {
+                const int e = min(e0 + 32 * i, kPix - 1), ly = e / kThinPW, lx = e - ly * kThinPW;
                 const int py = py0 + ly - 1, px = px0 + lx - 1;
-                dv[it] = 0.f; yv[it] = 0.f; av[it] = 0;
-                if (e < kThinPH * kThinPW && py >= 0 && py < A.OH && px >= 0 && px < A.OW) {
-                    const size_t gi = base + (size_t)py * A.OW + px;
-                    dv[it] = __ldg(A.dyp + gi); yv[it] = __ldg(A.yp + gi); av[it] = __ldg(A.arg + gi);
+                in[i] = py >= 0 && py < A.OH && px >= 0 && px < A.OW;
+                const size_t at = img + (size_t)min(max(py, 0), A.OH - 1) * A.OW + min(max(px, 0), A.OW - 1);
+#pragma unroll
+                for (int c = 0; c < kCos; ++c) {
+                    const size_t gi = at + (size_t)min(warp + c * kWarps, A.Cout - 1) * pplane;
+                    dv[i][c] = __ldg(A.dyp + gi); yv[i][c] = __ldg(A.yp + gi); av[i][c] = __ldg(A.arg + gi);
                 }
             }
 #pragma unroll
-            for (int it = 0; it < kIt; ++it) {
-                const int e = lane + 32 * it;
-                if (e < kThinPH * kThinPW) {
-                    sv[e * kThinVs + co] = dv[it] * (yv[it] > 0.f ? 1.f : A.slope);
-                    sa[e * kThinAs + co] = av[it];
+            for (int i = 0; i < kBatch; ++i)
+#pragma unroll
+                for (int c = 0; c < kCos; ++c) {
+                    const int e = e0 + 32 * i, co = warp + c * kWarps;
+                    if (e < kPix && co < A.Cout) {
+                        sv[e * kThinVs + co] = in[i] ? dv[i][c] * (yv[i][c] > 0.f ? 1.f : A.slope) : 0.f;
+                        sa[e * kThinAs + co] = in[i] ? av[i][c] : 0;
+                    }
                 }
+        }
+        // stage the input patch, the same way
+        constexpr int kRows = CIN * kThinXH, kRowIt = (kRows + kWarps - 1) / kWarps, kColIt = (kThinXW + 31) / 32;
+        float xv[kRowIt][kColIt];
+#pragma unroll
+        for (int i = 0; i < kRowIt; ++i) {
+            const int r = min(warp + i * kWarps, kRows - 1), ci = r / kThinXH, y = 2 * py0 - 1 + r - ci * kThinXH;
+            const float* src = A.x + ((size_t)n * CIN + ci) * plane + (size_t)min(max(y, 0), H - 1) * W;
+#pragma unroll
+            for (int j = 0; j < kColIt; ++j) {
+                const int xg = 2 * px0 - 1 + lane + 32 * j;
+                const float v = __ldg(src + min(max(xg, 0), W - 1));
+                xv[i][j] = y >= 0 && y < H && xg >= 0 && xg < W ? v : 0.f;
             }
         }
-        // stage the input patch
-        for (int r = warp; r < CIN * kThinXH; r += kStThreads / 32) {
-            const int ci = r / kThinXH, lr = r - ci * kThinXH, y = 2 * py0 - 1 + lr;
-            const bool row_ok = y >= 0 && y < H;
-            const float* src = A.x + ((size_t)n * CIN + ci) * plane + (size_t)(row_ok ? y : 0) * W;
-            for (int lc = lane; lc < kThinXW; lc += 32) {
-                const int xg = 2 * px0 - 1 + lc;
-                sx[(ci * kThinXH + lr) * kThinXP + lc] = (row_ok && xg >= 0 && xg < W) ? __ldg(src + xg) : 0.f;
-            }
-        }
+#pragma unroll
+        for (int i = 0; i < kRowIt; ++i)
+#pragma unroll
+            for (int j = 0; j < kColIt; ++j)
+                if (warp + i * kWarps < kRows && lane + 32 * j < kThinXW) sx[(warp + i * kWarps) * kThinXP + lane + 32 * j] = xv[i][j];
         __syncthreads();
 
         // filter gradient: lane = output channel, the warps take the tile's pooled pixels in turn
