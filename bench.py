@@ -41,13 +41,13 @@ KIND = {0: ("pack_filters", None), 1: ("fwd_group", 1), 2: ("loss_delta", None),
         9: ("unroll_windows", None), 10: ("fold_windows", None)}
 KERNEL = {("fwd_group", "fp32"): "fwd_group_kernel / conv_rows_kernel", ("bwd_group", "fp32"): "bwd_group_kernel / thin_bwd_kernel",
           ("filter_grad_rows", "fp32"): "filter_grad_rows_kernel", ("delta_conv_rows", "fp32"): "conv_rows_kernel (input delta)",
+          ("fwd_group", "split"): "conv_split_kernel / conv_rows_kernel", ("bwd_group", "split"): "thin_bwd_kernel",
+          ("filter_grad_rows", "split"): "fgrad_split_kernel", ("delta_conv_rows", "split"): "conv_split_kernel (input delta)",
           ("fwd_group", "bf16"): "conv_tc_rows_kernel / fwd_group_tc_kernel", ("bwd_group", "bf16"): "bwd_group_tc_kernel",
           ("filter_grad_rows", "bf16"): "filter_grad_tc_rows_kernel", ("delta_conv_rows", "bf16"): "conv_tc_rows_kernel (input delta)"}
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel, from the ncu captures summarised
 # under profiles/ (static: null for every kernel / workload without a capture of the current code)
-NCU_TRAFFIC = {("C3", "fp32", "fwd_group"): 128.4e6, ("C3", "fp32", "filter_grad_rows"): 245.8e6,
-               ("C3", "fp32", "delta_conv_rows"): 159.3e6, ("C3", "fp32", "bwd_group"): 950.4e6,
-               ("C3", "bf16", "fwd_group"): 84.7e6, ("C3", "bf16", "filter_grad_rows"): 153.2e6, ("C3", "bf16", "delta_conv_rows"): 201.5e6}
+NCU_TRAFFIC = {("C3", "bf16", "fwd_group"): 84.7e6, ("C3", "bf16", "filter_grad_rows"): 153.2e6, ("C3", "bf16", "delta_conv_rows"): 201.5e6}
 
 
 def measured_bf16_peak():
@@ -57,6 +57,19 @@ def measured_bf16_peak():
             return float(json.load(f)["bf16_tflops_sustained"]), "of measured (MEASURED_PEAKS.json, sustained cuBLAS bf16)"
     except (OSError, KeyError, ValueError):
         return 1400.0, "of fallback (1.4 PFLOP/s sustained)"
+
+
+def split_operands(wl, precision, stationary):
+    """Whether the fp32 plan runs its one-conv groups on the tensor cores (the rule of ftp_plan_opts.stationary)."""
+    if precision != "fp32" or stationary:
+        return False
+    h, w, macs = wl.H, wl.W, 0
+    for l in wl.layers:
+        if l.kind == "pool":
+            h, w = h // 2, w // 2
+        elif l.k in (1, 3) and l.cin >= 32:
+            macs += h * w * l.cin * l.cout * l.k * l.k
+    return macs >= 1.0e8
 
 
 def parse():
@@ -403,13 +416,17 @@ def measure(ctx, name, precision, extras=True, light=False, **plan_opts):
         peak, src, bound = *measured_bf16_peak(), "tensor"
     else:
         peak, src, bound = ctx["fma"]["tflops"], ctx["fma"]["source"], "alu"
+    split = split_operands(wl, precision, dict(dict(stationary=args.stationary), **plan_opts)["stationary"])
+    if split:                                   # three bf16 parts per value: six tensor-core products per fp32 product
+        tc_peak, tc_src = measured_bf16_peak()
+        peak, src, bound = tc_peak / 6, f"sixth {tc_src}: six bf16 products per fp32 product", "tensor"
     per_kernel = {k: {"ms_per_step": breakdown[k], "algorithmic_flops_per_step": f,
                       "achieved_tflops": f / (breakdown[k] / 1e3) / 1e12, "frac": f / (breakdown[k] / 1e3) / 1e12 / peak,
                       "launches_per_step": launches_kind[k]}
                   for k, f in flops_kind.items() if breakdown.get(k, 0.0) > 0}
     dom = max(per_kernel, key=lambda k: per_kernel[k]["ms_per_step"])
     d = per_kernel[dom]
-    roofline = {"bound": bound, "kernel": KERNEL.get((dom, precision), dom), "achieved": d["achieved_tflops"], "peak": peak,
+    roofline = {"bound": bound, "kernel": KERNEL.get((dom, "split" if split else precision), dom), "achieved": d["achieved_tflops"], "peak": peak,
                 "unit": "TFLOP/s", "frac": d["frac"], "traffic": NCU_TRAFFIC.get((wl.name, precision, dom)),
                 "traffic_unit": "bytes per launch (static, from the ncu captures under profiles/; null: no capture of the current kernel)",
                 "peak_source": src, "launches_per_step": d["launches_per_step"],

@@ -129,7 +129,11 @@ typedef struct {
                            and stream pixel tiles through it, and the layer's maps cross the group boundary in
                            global memory as at any group boundary (the paper's weight-dominated layers, Section 6).
                            Default (0): groups whose conv has at least 32 input channels; 1: every such group
-                           whatever its channel count; -1: never.
+                           whatever its channel count; -1: never.  With the default and at least 1e8 multiply-
+                           accumulates an image in those layers, their contractions run on the tensor cores: every fp32
+                           value as the sum of three bf16 parts, six products of parts per product, sums kept in fp32
+                           outside the tensor core (as accurate as the fp32 sums of the CUDA-core kernels); their maps
+                           then lie in the workspace as parts.  1 keeps them on the CUDA cores.
                            bf16 path: a conv layer with a 1x1 or 3x3 window on a map of at most 1008 columns (the first
                            layer: a 3x3 window and at most 7 input channels) becomes an executed group of its own (with
                            its pool).  Forward pass and input delta run as banded tensor-core convolutions (a band of
@@ -160,7 +164,7 @@ int ftp_plan_create_opts(const ftp_layer* layers, int n_layers,
 int ftp_plan_exec_groups(const ftp_plan* plan, int* n_groups, ftp_group* groups_out, int capacity);
 
 /* How executed group `group` (0-based index into ftp_plan_exec_groups) runs: *stationary = 1 if it is a one-conv
- * group run by the weight-stationary kernels of the fp32 path (see ftp_plan_opts.stationary), 2 if by the banded
+ * group run by the one-conv kernels of the fp32 path (see ftp_plan_opts.stationary), 2 if by the banded
  * tensor-core kernels of the bf16 path, 0 if as fused sub-tile stacks;
  * *partial_sets (may be NULL) = the partial gradient sets of the group that the cross-tile reduction sums
  * (Section 4.1).  FTP_ERR_ARG on a bad index or NULL. */
@@ -399,12 +403,12 @@ int ftp_fma_peak(float* out, size_t out_count, long long iters, double* flops, v
 long long ftp_plan_launch_count(const ftp_plan* plan);
 
 /*
- * Synchronises `stream` and reports whether a kernel of the bf16 tensor-core path gave up on one
- * of its bounded waits (for a filter stage to arrive or for the tensor core to finish) since the
+ * Synchronises `stream` and reports whether a tensor-core kernel (bf16 path, or fp32 path with
+ * split operands) gave up on one of its bounded waits (for a stage to arrive or for the tensor core to finish) since the
  * last ftp_forward / ftp_step* call on this plan and workspace: FTP_ERR_TIMEOUT if so -- the results
  * of that call are then invalid -- else FTP_OK.  Kernels never wait without a limit; after a
  * failed wait they skip the remaining waits, release their tensor memory and return.  Always
- * FTP_OK for the fp32 path, which has no device-side waits.
+ * FTP_OK for fp32 plans that run on the CUDA cores only, which have no device-side waits.
  */
 int ftp_plan_check(ftp_plan* plan, void* workspace, void* stream);
 
