@@ -206,7 +206,8 @@ __global__ void __launch_bounds__(T, 512 / T) conv_rows_kernel(const __grid_cons
     auto val = [&](int p, int j, int c) { return (c & 1) ? acc[p][j][c >> 1].y : acc[p][j][c >> 1].x; };
     const int rp = rp0 + rp_l;
     const int n = rp / A.rp_img, y = (rp - n * A.rp_img) * 2, x = x0 + cq_l * 4;
-    if (n >= A.N || x >= A.W) return;
+    const bool live = n < A.N && x < A.W;
+    if (!live && !A.pool) return;
     const int plane8 = (co0 >> 3) + cg;                      // 8-channel plane of this thread's output channels
     const size_t opart = (size_t)A.og.planes * A.og.tp;
     if (!A.pool) {
@@ -243,37 +244,58 @@ __global__ void __launch_bounds__(T, 512 / T) conv_rows_kernel(const __grid_cons
         }
     } else {
         const int OH = A.H >> 1, OW = A.W >> 1;
+        float best[2][8];
+        unsigned long long am[2] = {0ull, 0ull};
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if (x + 2 * h >= A.W) break;
-            float best[8];
-            unsigned long long am = 0ull;
+        for (int h = 0; h < 2; ++h)
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
                 float v00 = val(0, 2 * h, c), v01 = val(0, 2 * h + 1, c), v10 = val(1, 2 * h, c), v11 = val(1, 2 * h + 1, c);
                 v00 = v00 > 0.f ? v00 : A.slope * v00; v01 = v01 > 0.f ? v01 : A.slope * v01;
                 v10 = v10 > 0.f ? v10 : A.slope * v10; v11 = v11 > 0.f ? v11 : A.slope * v11;
-                best[c] = v00; unsigned m = 0;
-                if (v01 > best[c]) { best[c] = v01; m = 1; }
-                if (v10 > best[c]) { best[c] = v10; m = 2; }
-                if (v11 > best[c]) { best[c] = v11; m = 3; }
-                am |= (unsigned long long)m << (8 * c);
+                best[h][c] = v00; unsigned m = 0;
+                if (v01 > best[h][c]) { best[h][c] = v01; m = 1; }
+                if (v10 > best[h][c]) { best[h][c] = v10; m = 2; }
+                if (v11 > best[h][c]) { best[h][c] = v11; m = 3; }
+                am[h] |= (unsigned long long)m << (8 * c);
             }
-            const int py = y >> 1, px = (x >> 1) + h;
-            if (A.out || A.arg) {
+        // The lanes of a warp lie in 16 rows, so a store covers a piece of a sector per row: both pixels of the thread go into
+        // one store of the NCHW maps, and the entries of the split map change places between the two lanes of a row, which
+        // then write whole sectors
+        // (first layer, 16 images of 608 x 608, 3 -> 32 channels: 613 -> 63 us).
+        const int py = y >> 1, px = x >> 1;
+        if (live && (A.out || A.arg)) {
+            const bool both = x + 2 < A.W, wide = both && (OW & 1) == 0 && ((unsigned long long)A.out & 7) == 0;
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const int co = co0 + cg * 8 + c;
-                    if (co >= A.Cout) break;
-                    const size_t gi = (((size_t)n * A.Cout + co) * OH + py) * OW + px;
-                    if (A.out) A.out[gi] = best[c];
-                    if (A.arg) A.arg[gi] = (unsigned char)(am >> (8 * c));
+            for (int c = 0; c < 8; ++c) {
+                const int co = co0 + cg * 8 + c;
+                if (co >= A.Cout) break;
+                const size_t gi = (((size_t)n * A.Cout + co) * OH + py) * OW + px;
+                const unsigned m0 = (unsigned)(am[0] >> (8 * c)) & 255u, m1 = (unsigned)(am[1] >> (8 * c)) & 255u;
+                if (wide) {
+                    if (A.out) *reinterpret_cast<float2*>(A.out + gi) = make_float2(best[0][c], best[1][c]);
+                    if (A.arg) *reinterpret_cast<unsigned short*>(A.arg + gi) = (unsigned short)(m0 | m1 << 8);
+                } else {
+                    if (A.out) { A.out[gi] = best[0][c]; if (both) A.out[gi + 1] = best[1][c]; }
+                    if (A.arg) { A.arg[gi] = (unsigned char)m0; if (both) A.arg[gi + 1] = (unsigned char)m1; }
                 }
             }
-            if (plane8 < A.og.planes && (A.out_s || A.arg_s)) {
-                const size_t e = (size_t)plane8 * A.og.tp + kSplitLead + (size_t)(1 + n * (OH + 1) + py) * A.og.wp + px;
-                if (A.out_s) sp::store_split(A.out_s, opart, e, best);
-                if (A.arg_s) A.arg_s[e] = am;
+        }
+        if (A.out_s || A.arg_s) {
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const float r = __shfl_xor_sync(0xffffffffu, cq_l ? best[0][c] : best[1][c], 1);
+                if (cq_l) best[0][c] = r; else best[1][c] = r;
+            }
+            const unsigned long long r = __shfl_xor_sync(0xffffffffu, cq_l ? am[0] : am[1], 1);
+            if (cq_l) am[0] = r; else am[1] = r;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int pe = (x0 >> 1) + 2 * h + cq_l;
+                if (n >= A.N || 2 * pe >= A.W || plane8 >= A.og.planes) continue;
+                const size_t e = (size_t)plane8 * A.og.tp + kSplitLead + (size_t)(1 + n * (OH + 1) + py) * A.og.wp + pe;
+                if (A.out_s) sp::store_split(A.out_s, opart, e, best[h]);
+                if (A.arg_s) A.arg_s[e] = am[h];
             }
         }
     }
