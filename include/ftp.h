@@ -133,7 +133,9 @@ typedef struct {
                            accumulates an image in those layers, their contractions run on the tensor cores: every fp32
                            value as the sum of three bf16 parts, six products of parts per product, sums kept in fp32
                            outside the tensor core (as accurate as the fp32 sums of the CUDA-core kernels); their maps
-                           then lie in the workspace as parts.  1 keeps them on the CUDA cores.
+                           then lie in the workspace as parts.  Infinities and NaNs reach what they reach in a plain sum
+                           (the filter gradient may show a NaN for a window position that leads out of the map from an
+                           infinite value at its border).  1 keeps them on the CUDA cores.
                            bf16 path: a conv layer with a 1x1 or 3x3 window on a map of at most 1008 columns (the first
                            layer: a 3x3 window and at most 7 input channels) becomes an executed group of its own (with
                            its pool).  Forward pass and input delta run as banded tensor-core convolutions (a band of

@@ -3,7 +3,8 @@
 //
 // Operands.  Every fp32 value is kept as the sum of three bf16 values, a = a0 + a1 + a2: a0 = a rounded to 6 significant
 // bits, a1 = bf16(a - a0), a2 = a - a0 - a1, which together hold the 24 bits of an fp32 exactly (the differences are exact in
-// fp32; values below 2^-110, whose last part falls under the smallest bf16, lose bits there).  A product is formed as
+// fp32; values below 2^-110, whose last part falls under the smallest bf16, lose bits there, and values next to the largest
+// fp32 one bit, see split8).  A product is formed as
 // the six products a0 b0, a0 b1, a1 b0, a0 b2, a1 b1, a2 b0, each exact in fp32; what is left out (a1 b2, a2 b1, a2 b2) has
 // either sign and measures 2^-24 of |a b| in the 2-norm, the rounding of one fp32 multiply-add.
 //
@@ -56,6 +57,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
 constexpr int kMaxA = 3, kMaxB = 8;
 constexpr int kConvThreads = 384;             // 8 epilogue warps; producer, MMA issuers of the large and (two) of the small products
 constexpr int kEpiThreads = 256;
+constexpr float kSplitLargest = 1.2676506e30f; // 2^100: the sum of two such values times two slopes of 2^10 is far from infinity
 
 // ---------------------------------------------------------------------------------------------
 // Convolution.  A work item is a tile of nblk x 128 output entries x a slice of Ns <= 128 output channels.  The input
@@ -149,6 +151,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_split_kernel(const __gri
         const int q = warp & 3, half = warp >> 2, et = threadIdx.x;
         const size_t opart = (size_t)A.og.planes * A.og.tp;
         uint32_t gh = 0, gl = 0, k = 0;                       // chains and items of this half so far
+        const bool small_slopes = fabsf(A.slope) <= 1024.f && fabsf(A.prev_slope) <= 1024.f;
         for (int it = blockIdx.x; it < A.items; it += gridDim.x, ++k) {
             const Item I = item_of(it);
             const int co0 = I.slice * A.Ns;
@@ -158,7 +161,8 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_split_kernel(const __gri
             float acc[128];
 #pragma unroll
             for (int j = 0; j < 128; ++j) acc[j] = 0.f;
-            auto add = [&](uint32_t col) {
+            auto plain = [](float a, float b) { return a + b; };
+            auto add = [&](uint32_t col, auto sum) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int bl = half + 2 * (2 * i / UPB), c0 = (2 * i % UPB) * 16;      // two units at a time
@@ -166,23 +170,34 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_split_kernel(const __gri
                         float v[32];
                         tmem_ld32(tmem + col + ((uint32_t)(q * 32) << 16) + (uint32_t)(bl * A.Ns + c0), v);
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) acc[i * 32 + j] += v[j];
+                        for (int j = 0; j < 32; ++j) acc[i * 32 + j] = sum(acc[i * 32 + j], v[j]);
                     }
                 }
                 fence_before_sync();
                 __syncwarp();
             };
             bool ok = true;
+            uint32_t round = kRoundFirst;
+            auto item_round = [&](float) { return round; };
             if (half < I.nblk) {
                 for (int c = 0; c < kChains * A.nchunks; ++c, ++gh) {
                     if (!wait(&H->hdone[half], gh & 1u, 32)) { ok = false; break; }
                     fence_after_sync();
-                    add(0);
+                    add(0, plain);
                     if (lane == 0) mbar_arrive(smem_u32(&H->hfree[half]));
                 }
+                // Sums that are infinite or NaN, or so large that a value to be stored could be within 2^-7 of the largest: the small
+                // products are then added with care and first parts cut, not rounded.  (One answer for the warp; the comparison
+                // is false for a NaN.  Together 0.5 to 1 % of a step; 1.4 % with a look at every value, see split8.)
+                float top = max_abs(max_abs(bias[0], bias[1], bias[2]), bias[3], 0.f);
+#pragma unroll
+                for (int j = 0; j < 128; j += 2) top = max_abs(top, acc[j], acc[j + 1]);
+                const bool large = __any_sync(0xffffffffu, !(top < kSplitLargest && small_slopes));
+                round = large ? 0u : kRoundFirst;
                 if (ok && wait(&H->ldone[half], gl & 1u, 32)) {
                     fence_after_sync();
-                    add(256);
+                    if (large) add(256, add_small);
+                    else add(256, plain);
                     if (lane == 0) mbar_arrive(smem_u32(&H->lfree[half]));
                     ++gl;
                 } else ok = false;
@@ -240,8 +255,8 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_split_kernel(const __gri
                                 }
                             }
                             if (!A.prev_arg) {
-                                store_split(A.out_s, opart, (size_t)pl * A.og.tp + e, v);
-                                store_split(A.out_s, opart, (size_t)(pl + 1) * A.og.tp + e, v + 8);
+                                store_split(A.out_s, opart, (size_t)pl * A.og.tp + e, v, item_round);
+                                store_split(A.out_s, opart, (size_t)(pl + 1) * A.og.tp + e, v + 8, item_round);
                             }
                         }
                         if (A.prev_arg) {
@@ -260,7 +275,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_split_kernel(const __gri
                             for (int h = 0; h < 2; ++h) {
                                 const unsigned long long am = valid ? __ldg(A.prev_arg + (size_t)(pl + h) * A.g.tp + e) : 0ull;
                                 uint4 s[3];
-                                split8(v + h * 8, s[0], s[1], s[2]);
+                                split8(v + h * 8, s[0], s[1], s[2], item_round);
 #pragma unroll
                                 for (int k2 = 0; k2 < 2; ++k2) {
                                     const int src = 16 * k2 + (lane >> 1);
@@ -611,14 +626,15 @@ __global__ void __launch_bounds__(kFgThreads, 1) fgrad_split_kernel(const __grid
             for (int j = 0; j < 128; ++j) acc[j] = 0.f;
             float bacc = 0.f;
             const bool bias = with_bias && u == 0;
-            auto add = [&](uint32_t col) {
+            auto plain = [](float a, float b) { return a + b; };
+            auto add = [&](uint32_t col, auto sum) {
 #pragma unroll
                 for (int t = 0; t < 8; ++t)
                     if (t * 16 < cols) {
                         float v[16];
                         tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + col + (uint32_t)(t * 16), v);
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) acc[t * 16 + j] += v[j];
+                        for (int j = 0; j < 16; ++j) acc[t * 16 + j] = sum(acc[t * 16 + j], v[j]);
                     }
                 fence_before_sync();
                 __syncwarp();
@@ -626,16 +642,17 @@ __global__ void __launch_bounds__(kFgThreads, 1) fgrad_split_kernel(const __grid
             for (int i = 0; i < ns; ++i) {
                 if (!wait(&H->hdone[u], (uint32_t)i & 1u, 32)) break;
                 fence_after_sync();
-                add(hcol + (uint32_t)((i * steps + u) % slots * wide));
+                add(hcol + (uint32_t)((i * steps + u) % slots * wide), plain);
                 if (lane == 0) mbar_arrive(smem_u32(&H->hfree[u]));
                 if (bias) {
                     if (!wait(&H->hdone[3], (uint32_t)i & 1u, 32)) break;
                     fence_after_sync();
-                    uint32_t r;
-                    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r)
-                                 : "r"(tmem + ((uint32_t)(q * 32) << 16) + hcol + (uint32_t)((i * steps + nu) % slots * wide)) : "memory");
+                    const uint32_t at = tmem + ((uint32_t)(q * 32) << 16) + hcol + (uint32_t)((i * steps + nu) % slots * wide);
+                    uint32_t r, rs;
+                    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(at) : "memory");
+                    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(rs) : "r"(at + 16u) : "memory");
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    bacc += __uint_as_float(r);
+                    bacc = add_small(bacc + __uint_as_float(r), __uint_as_float(rs));
                     fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&H->hfree[3]));
@@ -643,7 +660,7 @@ __global__ void __launch_bounds__(kFgThreads, 1) fgrad_split_kernel(const __grid
                 if (i % kFgFlush == kFgFlush - 1 || i == ns - 1) {
                     if (!wait(&H->ldone[u], (uint32_t)(i / kFgFlush) & 1u, 32)) break;
                     fence_after_sync();
-                    add((uint32_t)(u * wide));
+                    add((uint32_t)(u * wide), add_small);       // (the large products of the same stages are in)
                     if (lane == 0) mbar_arrive(smem_u32(&H->lfree[u]));
                 }
             }
@@ -735,9 +752,9 @@ __global__ void __launch_bounds__(kFgThreads, 1) fgrad_split_kernel(const __grid
                                 for (int kx = 0; kx < (A.rows3 ? 3 : 1); ++kx)
                                     chain(tcol + (uint32_t)(kx * A.cin16), dz0, xu + (uint32_t)kx, idesc, false);
                             } else
-                                for (int part = 2; part >= 0; --part)                    // bias: sums of dz, a contraction with ones
-                                    for (int ks = 0; ks < nk; ++ks)
-                                        mma_bf16(tcol, desc64(a_hi, dz0 + (uint32_t)part * dz_part + 16u * (uint32_t)ks), ones_d, idb, part < 2 || ks > 0);
+                                for (int part = 2; part >= 0; --part)                    // bias: sums of dz, a contraction with ones; 16 columns for
+                                    for (int ks = 0; ks < nk; ++ks)                      // the first part, 16 for the others (a slot has 32 at least)
+                                        mma_bf16(tcol + (part ? 16u : 0u), desc64(a_hi, dz0 + (uint32_t)part * dz_part + 16u * (uint32_t)ks), ones_d, idb, part == 1 || ks > 0);
                             mma_commit(smem_u32(&H->hdone[k == nu ? 3 : k]));
                         }
                     } else {
@@ -839,7 +856,7 @@ __global__ void __launch_bounds__(256) pack_split_kernel(const __grid_constant__
 {
     previous_launches();
     __shared__ float s[kPackSmemFloats];
-    pack_tiles<3>(A, params, s, [](const float* v, uint4* p) { split8(v, p[0], p[1], p[2]); });
+    pack_tiles<3>(A, params, s, [](const float* v, uint4* p) { split8(v, p[0], p[1], p[2], round_first); });
 }
 
 }  // namespace sp

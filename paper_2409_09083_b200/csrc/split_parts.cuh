@@ -10,14 +10,24 @@
 namespace ftp {
 namespace sp {
 
-// three bf16 parts of eight values; the first one rounded to 6 significant bits (nearest, ties away from zero)
-__device__ __forceinline__ void split8(const float* v, uint4& p0, uint4& p1, uint4& p2)
+constexpr uint32_t kRoundFirst = 0x20000u;       // half of the last place of 6 significant bits
+
+// What turns a value into its first part: rounding to 6 significant bits, but for values within 2^-7 of the largest fp32, where that
+// would be an infinity, and for infinities and NaNs.  These are cut to 6 bits.
+__device__ __forceinline__ uint32_t round_first(float x) { return fabsf(x) < __int_as_float(0x7f7e0000) ? kRoundFirst : 0u; }
+
+// Three bf16 parts of eight values; the first one rounded to 6 significant bits (nearest, ties away from zero), or cut (the
+// three parts then hold 23 bits at least): `round(x)` says which, kRoundFirst or 0.  An infinity becomes (itself, NaN, NaN), a NaN
+// NaNs: see add_small.  (Not a branch every eight values to code for the rare ones: that made the unrolled output phases of
+// conv_split_kernel 6 % slower, and a comparison per value 1 %.)
+template <class Round>
+__device__ __forceinline__ void split8(const float* v, uint4& p0, uint4& p1, uint4& p2, Round round)
 {
     uint32_t* a = &p0.x; uint32_t* b = &p1.x; uint32_t* c = &p2.x;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const float x = v[2 * i], y = v[2 * i + 1];
-        const uint32_t bx = (__float_as_uint(x) + 0x20000u) & 0xfffc0000u, by = (__float_as_uint(y) + 0x20000u) & 0xfffc0000u;
+        const uint32_t bx = (__float_as_uint(x) + round(x)) & 0xfffc0000u, by = (__float_as_uint(y) + round(y)) & 0xfffc0000u;
         a[i] = __byte_perm(bx, by, 0x7632);
         const float rx = x - __uint_as_float(bx), ry = y - __uint_as_float(by);
         const __nv_bfloat162 h1 = __floats2bfloat162_rn(rx, ry);
@@ -27,11 +37,25 @@ __device__ __forceinline__ void split8(const float* v, uint4& p0, uint4& p1, uin
         c[i] = *reinterpret_cast<const uint32_t*>(&h2);
     }
 }
-__device__ __forceinline__ void store_split(uint4* base, size_t part_stride, size_t at, const float* v)
+template <class Round>
+__device__ __forceinline__ void store_split(uint4* base, size_t part_stride, size_t at, const float* v, Round round)
 {
     uint4 p0, p1, p2;
-    split8(v, p0, p1, p2);
+    split8(v, p0, p1, p2, round);
     base[at] = p0; base[at + part_stride] = p1; base[at + 2 * part_stride] = p2;
+}
+__device__ __forceinline__ void store_split(uint4* base, size_t part_stride, size_t at, const float* v) { store_split(base, part_stride, at, v, round_first); }
+
+// Adds the products of the lower parts (small) to a sum that holds those of the first parts (large).  Where an operand is infinite or
+// NaN, the products of the first parts alone have the sum that fp32 multiply-adds have; the others stay out.
+__device__ __forceinline__ float add_small(float large, float small) { return fabsf(large) < __int_as_float(0x7f800000) ? large + small : large; }
+
+// largest magnitude of three values, NaN if one of them is
+__device__ __forceinline__ float max_abs(float a, float b, float c)
+{
+    float d;
+    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
 }
 
 // pixel of an entry (n, y, x); false: a zero entry of the map (edge column, row between images, lead or tail)

@@ -103,3 +103,113 @@ def test_small_stacks_stay_on_the_multiply_add_kernels():
     assert small.workspace_bytes == plan(64, 64, 96, stationary=0).workspace_bytes
     assert plan(2, 88, 104).workspace_bytes != plan(2, 88, 104, stationary=1).workspace_bytes
     assert large.group_mode(1)[0] == 1
+
+
+# one layer on a batch of two, above the 1e8 rule: flat runs; tiles with a pool; a 1x1 layer; tiles of a wide map; the forward pass on
+# the row kernel
+SINGLE = {
+    "flat": W("i", (conv(64, 48, 3),), 2, 64, 66, 70, (2, 2), one(1)),
+    "pool": W("j", (conv(64, 48, 3), pool()), 2, 64, 66, 70, (2, 2), one(2)),
+    "one-by-one": W("k", (conv(256, 200, 1),), 2, 256, 50, 52, (2, 2), one(1)),
+    "wide": W("l", (conv(64, 48, 3),), 2, 64, 20, 320, (2, 2), one(1)),
+    "32-channels": W("m", (conv(32, 64, 3), pool()), 2, 32, 88, 90, (2, 2), one(2)),
+}
+# ... and with maps between the layers, written by an epilogue: without and with a pool, on the row kernel
+CHAINS = {
+    "chain": W("n", (conv(64, 64, 3), conv(64, 48, 1)), 2, 64, 50, 62, (2, 2), one(2)),
+    "chain-pool": W("o", (conv(64, 64, 3), pool(), conv(64, 48, 3)), 2, 64, 52, 64, (2, 2), one(3)),
+    "chain-32": W("p", (conv(32, 64, 3), conv(64, 64, 3)), 2, 32, 52, 64, (2, 2), one(2)),
+    "chain-32-pool": W("q", (conv(32, 64, 3), pool(), conv(64, 64, 3)), 2, 32, 84, 88, (2, 2), one(3)),
+}
+
+
+def draw_single(wl):
+    x, params, _ = synth.draw(wl, bias_std=0.1)
+    shape = (wl.N,) + tuple(synth.map_shapes(wl.layers, wl.C, wl.H, wl.W)[-1])
+    return x, params, np.random.default_rng(1).standard_normal(shape).astype(np.float32)
+
+
+def classes(a):
+    return np.where(np.isnan(a), 3, np.where(np.isposinf(a), 1, np.where(np.isneginf(a), 2, 0)))
+
+
+@pytest.mark.parametrize("where", ["x", "dy"])
+@pytest.mark.parametrize("name", sorted(SINGLE))
+def test_infinities_and_nans_reach_what_they_reach_in_a_plain_sum(name, where):
+    """An infinity stays one: in the last map and the input delta exactly the values of the untiled sums are infinite (with their
+    signs) or NaN, the others stay finite and accurate.  In the filter gradient too, but for the window positions that lead
+    out of the map from a pixel at its border: there a zero of the padding meets the infinity, and a NaN may stand for the
+    finite value (the multiply-add kernels do the same at the edges of their tiles)."""
+    wl = SINGLE[name]
+    x, params, dy = draw_single(wl)
+    if where == "x":
+        x[0, 5, 10, 12], x[1, 7, 9, 30], x[0, 9, 15, 40] = np.inf, -np.inf, np.nan
+        x[0, 11, 0, 0], x[1, 12, -1, -1], x[0, 13, 3, -1], x[0, 14, -1, 4] = np.inf, np.inf, np.inf, -np.inf
+    else:
+        dy[0, 5, 5, 6], dy[1, 7, 7, 9], dy[0, 9, 8, 20] = np.inf, -np.inf, np.nan
+        dy[0, 11, 0, 0], dy[1, 12, -1, -1] = np.inf, np.inf
+    ref, got = run_oracle(wl, x, params, dy=dy), run_gpu(wl, x, params, dy=dy)
+    for k in ("y", "dx", "dparams"):
+        g, r = got[k].astype(np.float64), ref[k]
+        cg, cr = classes(g), classes(r)
+        if k == "dparams":
+            cout, cin, kk = wl.layers[0].cout, wl.layers[0].cin, wl.layers[0].k ** 2
+            border = np.zeros((cout, cin, kk), bool)
+            if where == "x":
+                border[:, 11:15] = True
+            else:
+                border[11:13] = True
+            border = np.concatenate([border.ravel(), np.zeros(cout, bool)])
+            cg = np.where(border & (cg == 3) & (cr == 0), 0, cg)
+        assert np.array_equal(cg, cr), (k, int((cg != cr).sum()))
+        ok = np.isfinite(g) & np.isfinite(r)
+        assert np.linalg.norm(g[ok] - r[ok]) <= 2 * 6 * 2.0 ** -23 * np.linalg.norm(r[ok]), k
+
+
+@pytest.mark.parametrize("name", sorted(CHAINS))
+def test_infinities_and_nans_through_two_layers(name):
+    """The same through the maps and deltas that the epilogues write."""
+    wl = CHAINS[name]
+    x, params, dy = draw_single(wl)
+    x[0, 5, 10, 12], x[1, 7, 9, 30], x[0, 9, 15, 40], x[1, 3, 0, 0] = np.inf, -np.inf, np.nan, np.inf
+    dy[1, 5, 20, 16], dy[0, 9, 2, 3] = np.inf, np.nan
+    ref, got = run_oracle(wl, x, params, dy=dy), run_gpu(wl, x, params, dy=dy)
+    for k in ("y", "dx"):
+        assert np.array_equal(classes(got[k]), classes(ref[k])), k
+        ok = np.isfinite(ref[k])
+        assert ok.any() and not ok.all()
+    assert np.isnan(got["dparams"]).any()
+
+
+@pytest.mark.parametrize("pooled", [False, True])
+@pytest.mark.parametrize("cin", [32, 256])
+def test_the_largest_finite_values_between_layers(cin, pooled):
+    """A first layer that hands its input on (1x1, identity), so that its epilogue writes values next to the largest fp32."""
+    h, w = (200, 64) if cin == 32 else (50, 52)
+    layers = (conv(cin, 256, 1),) + ((pool(),) if pooled else ()) + (conv(256, 64, 1),)
+    wl = W("r", layers, 2, cin, h, w, (2, 2), one(len(layers)))
+    x, params, dy = draw_single(wl)
+    params[:256 * cin] = np.eye(256, cin, dtype=np.float32).ravel()
+    params[256 * cin:256 * cin + 256] = 0
+    params[256 * cin + 256:] *= np.float32(2.0 ** -20)
+    x[:, :, 3:9, 5:9] = np.float32(3.395e38) * np.random.default_rng(2).choice(np.float32([1, -1, 0.999]), x[:, :, 3:9, 5:9].shape)
+    ref, got = run_oracle(wl, x, params, dy=dy), run_gpu(wl, x, params, dy=dy)
+    for k in ("y", "dx"):
+        assert np.isfinite(got[k]).all(), k
+        scale = np.abs(ref[k]).max()
+        assert np.linalg.norm((got[k] - ref[k]) / scale) <= 2 * 7 * 2.0 ** -23 * np.linalg.norm(ref[k] / scale), k
+
+
+@pytest.mark.parametrize("name", sorted(SINGLE))
+def test_the_largest_finite_values(name):
+    """Inputs within 2^-7 of the largest fp32: their first part is cut instead of rounded up to infinity (bound: see the module's
+    docstring, one convolution, and 2^-23 for the bit that the three parts of a cut value may lack)."""
+    wl = SINGLE[name]
+    x, params, dy = draw_single(wl)
+    x[:, :, 3:9, 5:9] = np.float32(3.395e38) * np.random.default_rng(2).choice(np.float32([1, -1, 0.999]), x[:, :, 3:9, 5:9].shape)
+    params *= np.float32(2.0 ** -20)
+    ref, got = run_oracle(wl, x, params, dy=dy), run_gpu(wl, x, params, dy=dy)
+    for k in ("y", "dx"):
+        assert np.isfinite(got[k]).all(), k
+        scale = np.abs(ref[k]).max()
+        assert np.linalg.norm((got[k] - ref[k]) / scale) <= 7 * 2.0 ** -23 * np.linalg.norm(ref[k] / scale), k
