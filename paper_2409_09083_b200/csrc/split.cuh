@@ -178,7 +178,8 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_split_kernel(const __gri
             };
             bool ok = true;
             uint32_t round = kRoundFirst;
-            auto item_round = [&](float) { return round; };
+            auto delta_first = [&](float x) { return first_part(x, round); };
+            auto map_first = [&](float x) { return keep_sign(x, first_part(x, round)); };
             if (half < I.nblk) {
                 for (int c = 0; c < kChains * A.nchunks; ++c, ++gh) {
                     if (!wait(&H->hdone[half], gh & 1u, 32)) { ok = false; break; }
@@ -255,8 +256,8 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_split_kernel(const __gri
                                 }
                             }
                             if (!A.prev_arg) {
-                                store_split(A.out_s, opart, (size_t)pl * A.og.tp + e, v, item_round);
-                                store_split(A.out_s, opart, (size_t)(pl + 1) * A.og.tp + e, v + 8, item_round);
+                                store_split(A.out_s, opart, (size_t)pl * A.og.tp + e, v, map_first);
+                                store_split(A.out_s, opart, (size_t)(pl + 1) * A.og.tp + e, v + 8, map_first);
                             }
                         }
                         if (A.prev_arg) {
@@ -275,7 +276,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_split_kernel(const __gri
                             for (int h = 0; h < 2; ++h) {
                                 const unsigned long long am = valid ? __ldg(A.prev_arg + (size_t)(pl + h) * A.g.tp + e) : 0ull;
                                 uint4 s[3];
-                                split8(v + h * 8, s[0], s[1], s[2], item_round);
+                                split8(v + h * 8, s[0], s[1], s[2], delta_first);
 #pragma unroll
                                 for (int k2 = 0; k2 < 2; ++k2) {
                                     const int src = 16 * k2 + (lane >> 1);
@@ -856,7 +857,7 @@ __global__ void __launch_bounds__(256) pack_split_kernel(const __grid_constant__
 {
     previous_launches();
     __shared__ float s[kPackSmemFloats];
-    pack_tiles<3>(A, params, s, [](const float* v, uint4* p) { split8(v, p[0], p[1], p[2], round_first); });
+    pack_tiles<3>(A, params, s, [](const float* v, uint4* p) { split8(v, p[0], p[1], p[2], [](float x) { return first_part(x); }); });
 }
 
 }  // namespace sp

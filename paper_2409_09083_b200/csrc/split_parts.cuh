@@ -12,22 +12,27 @@ namespace sp {
 
 constexpr uint32_t kRoundFirst = 0x20000u;       // half of the last place of 6 significant bits
 
-// What turns a value into its first part: rounding to 6 significant bits, but for values within 2^-7 of the largest fp32, where that
-// would be an infinity, and for infinities and NaNs.  These are cut to 6 bits.
-__device__ __forceinline__ uint32_t round_first(float x) { return fabsf(x) < __int_as_float(0x7f7e0000) ? kRoundFirst : 0u; }
+// First part of a value, as the bits of an fp32: rounded to 6 significant bits (nearest, ties away from zero) or, with round = 0,
+// cut to 6 bits.
+__device__ __forceinline__ uint32_t first_part(float x, uint32_t round) { return (__float_as_uint(x) + round) & 0xfffc0000u; }
+// Of a value of any size: cut within 2^-7 of the largest fp32, where rounding would make an infinity, and beyond.
+__device__ __forceinline__ uint32_t first_part(float x) { return first_part(x, fabsf(x) < __int_as_float(0x7f7e0000) ? kRoundFirst : 0u); }
+// Of a value in a saved map, where the backward pass takes the sign of a value from its first part: positive for every positive
+// value (below 2^-132 the smallest bf16, 2^-133; the second part makes up for it).
+__device__ __forceinline__ uint32_t keep_sign(float x, uint32_t first) { return __float_as_int(x) > 0 ? max(first, 0x10000u) : first; }
 
-// Three bf16 parts of eight values; the first one rounded to 6 significant bits (nearest, ties away from zero), or cut (the
-// three parts then hold 23 bits at least): `round(x)` says which, kRoundFirst or 0.  An infinity becomes (itself, NaN, NaN), a NaN
-// NaNs: see add_small.  (Not a branch every eight values to code for the rare ones: that made the unrolled output phases of
+// Three bf16 parts of eight values: `first(x)`, the rest of x rounded to bf16, and the rest of that, which bf16 holds exactly (but for
+// a bit that may be lacking where the first part is cut).  An infinity becomes (itself, NaN, NaN), a NaN NaNs: see
+// add_small.  (Not a branch every eight values to code for the rare ones: that made the unrolled output phases of
 // conv_split_kernel 6 % slower, and a comparison per value 1 %.)
-template <class Round>
-__device__ __forceinline__ void split8(const float* v, uint4& p0, uint4& p1, uint4& p2, Round round)
+template <class First>
+__device__ __forceinline__ void split8(const float* v, uint4& p0, uint4& p1, uint4& p2, First first)
 {
     uint32_t* a = &p0.x; uint32_t* b = &p1.x; uint32_t* c = &p2.x;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const float x = v[2 * i], y = v[2 * i + 1];
-        const uint32_t bx = (__float_as_uint(x) + round(x)) & 0xfffc0000u, by = (__float_as_uint(y) + round(y)) & 0xfffc0000u;
+        const uint32_t bx = first(x), by = first(y);
         a[i] = __byte_perm(bx, by, 0x7632);
         const float rx = x - __uint_as_float(bx), ry = y - __uint_as_float(by);
         const __nv_bfloat162 h1 = __floats2bfloat162_rn(rx, ry);
@@ -37,14 +42,17 @@ __device__ __forceinline__ void split8(const float* v, uint4& p0, uint4& p1, uin
         c[i] = *reinterpret_cast<const uint32_t*>(&h2);
     }
 }
-template <class Round>
-__device__ __forceinline__ void store_split(uint4* base, size_t part_stride, size_t at, const float* v, Round round)
+template <class First>
+__device__ __forceinline__ void store_split(uint4* base, size_t part_stride, size_t at, const float* v, First first)
 {
     uint4 p0, p1, p2;
-    split8(v, p0, p1, p2, round);
+    split8(v, p0, p1, p2, first);
     base[at] = p0; base[at + part_stride] = p1; base[at + 2 * part_stride] = p2;
 }
-__device__ __forceinline__ void store_split(uint4* base, size_t part_stride, size_t at, const float* v) { store_split(base, part_stride, at, v, round_first); }
+__device__ __forceinline__ void store_split(uint4* base, size_t part_stride, size_t at, const float* v)
+{
+    store_split(base, part_stride, at, v, [](float x) { return keep_sign(x, first_part(x)); });
+}
 
 // Adds the products of the lower parts (small) to a sum that holds those of the first parts (large).  Where an operand is infinite or
 // NaN, the products of the first parts alone have the sum that fp32 multiply-adds have; the others stay out.

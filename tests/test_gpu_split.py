@@ -213,3 +213,19 @@ def test_the_largest_finite_values(name):
         assert np.isfinite(got[k]).all(), k
         scale = np.abs(ref[k]).max()
         assert np.linalg.norm((got[k] - ref[k]) / scale) <= 7 * 2.0 ** -23 * np.linalg.norm(ref[k] / scale), k
+
+
+@pytest.mark.parametrize("name", ["chain", "chain-pool", "chain-32", "chain-32-pool"])
+def test_the_smallest_positive_values_count_as_positive(name):
+    """Outputs of a first layer down to the smallest fp32 (its input is zero, its bias tiny, of either sign): the derivative of the
+    layer is decided by their sign."""
+    wl = synth.with_slope(CHAINS[name], 0.25)
+    x, params, dy = draw_single(wl)
+    x[:] = 0
+    l = wl.layers[0]
+    at, c = l.cout * l.cin * l.k * l.k, np.arange(l.cout)
+    params[at:at + l.cout] = np.where(c % 2, -1, 1) * np.float32(2.0) ** (-149 + c // 2).astype(np.float32)
+    assert (params[at:at + l.cout] != 0).all()
+    ref, got = run_oracle(wl, x, params, dy=dy), run_gpu(wl, x, params, dy=dy)
+    assert rel_err(got["dx"], ref["dx"]) <= FP32_TOL
+    assert rel_err(got["dparams"], ref["dparams"]) <= FP32_TOL
