@@ -497,14 +497,14 @@ __device__ __forceinline__ void filter_grad_mma(Pipe& p, uint32_t dz_run /*addre
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 2 : 1) fwd_group_tc_kernel(const __grid_constant__ TcGroupArgs A, int tile_bytes, int tmem_cols, int stages)
 {
-    next_launch();
-    previous_launches();
     using namespace tcd;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Header* H = reinterpret_cast<Header*>(smem_raw);
     unsigned char* tiles = smem_raw + (kTcHeader + stages * kTcStageBytes);
     Pipe pipe;
-    setup(H, pipe, smem_raw, A.error, (size_t)tile_bytes, tmem_cols, stages);
+    setup(H, pipe, smem_raw, A.error, (size_t)tile_bytes, tmem_cols, stages);      // tensor memory first: see launch.cuh
+    next_launch();
+    previous_launches();
     const bool tma_ok = (smem_u32(smem_raw) & 127u) == 0;       // tensor copies want 128-byte aligned destinations
     int* hdr = H->hdr;
     const int items = A.N * A.R * A.Q;
@@ -628,14 +628,14 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 2 : 1) fwd_group_tc_
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 2 : 1) bwd_group_tc_kernel(const __grid_constant__ TcGroupArgs A, int tile_bytes, int tmem_cols, int stages)
 {
-    next_launch();
-    previous_launches();
     using namespace tcd;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Header* H = reinterpret_cast<Header*>(smem_raw);
     unsigned char* tiles = smem_raw + (kTcHeader + stages * kTcStageBytes);
     Pipe pipe;
-    setup(H, pipe, smem_raw, A.error, (size_t)tile_bytes, tmem_cols, stages);
+    setup(H, pipe, smem_raw, A.error, (size_t)tile_bytes, tmem_cols, stages);      // tensor memory first: see launch.cuh
+    next_launch();
+    previous_launches();
     const bool tma_ok = (smem_u32(smem_raw) & 127u) == 0;       // tensor copies want 128-byte aligned destinations
     int* hdr = H->hdr;
 

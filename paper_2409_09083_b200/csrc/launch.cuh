@@ -3,11 +3,19 @@
 // slowest one, then through the launch, the set-up of the block (barriers, tensor memory, up to 200 KB of zeros) and the
 // first copies.
 //
-// The rules.  EVERY kernel calls previous_launches() before its first access to global memory: it returns when all launches
-// before it on the stream have completed and their writes are visible.  Since every kernel waits, a kernel's completion implies
-// that of all before it, so only the previous launch has to be waited for, and a buffer is never written before its
-// readers are through.  A launch behind an event or a copy, or with `overlap` off (per-launch timing), starts as any
-// launch does.
+// The rules.  Every kernel that launch() below starts calls previous_launches() before its first access to global memory: it
+// returns when all launches before it on the stream have completed and their writes are visible.  Since each of them waits, a
+// kernel's completion implies that of all before it, so only the previous launch has to be waited for, and a buffer is
+// never written before its readers are through.  A launch behind an event or a copy, with `overlap` off (per-launch
+// timing), or without launch() (sgd_kernel, fma_peak_kernel, wait_probe_kernel, noalloc.cu) starts as any launch does, when all before it have
+// ended.
+//
+// A kernel that takes tensor memory calls next_launch() only when its whole block is behind the allocation.  The next launch
+// may take all columns of an SM before it waits for this one, and tcgen05.alloc waits without a limit: a block of this
+// launch that had let it in without having its own columns would wait for columns that are given back only after it
+// has ended.  With the rule, whoever waits in an allocation waits for earlier launches alone, and these have what they need
+// (a launch starts only when all blocks of the one before have triggered or ended, so this holds along the stream,
+// helpers in between included; launches of other streams that share the SM depend on their own stream only).
 //
 // next_launch() lets the blocks of the next launch onto SMs that have room before this launch has ended.  Kernels whose blocks
 // fill the GPU once and end together gain from it when they are short; long ones lose, because the next kernel's blocks then
