@@ -59,19 +59,6 @@ def measured_bf16_peak():
         return 1400.0, "of fallback (1.4 PFLOP/s sustained)"
 
 
-def split_operands(wl, precision, stationary):
-    """Whether the fp32 plan runs its one-conv groups on the tensor cores (the rule of ftp_plan_opts.stationary)."""
-    if precision != "fp32" or stationary:
-        return False
-    h, w, macs = wl.H, wl.W, 0
-    for l in wl.layers:
-        if l.kind == "pool":
-            h, w = h // 2, w // 2
-        elif l.k in (1, 3) and l.cin >= 32:
-            macs += h * w * l.cin * l.cout * l.k * l.k
-    return macs >= 1.0e8
-
-
 def parse():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -416,7 +403,7 @@ def measure(ctx, name, precision, extras=True, light=False, **plan_opts):
         peak, src, bound = *measured_bf16_peak(), "tensor"
     else:
         peak, src, bound = ctx["fma"]["tflops"], ctx["fma"]["source"], "alu"
-    split = split_operands(wl, precision, dict(dict(stationary=args.stationary), **plan_opts)["stationary"])
+    split = any(plan.group_kernels(i, 1) == "split" for i in range(len(eg)))
     if split:                                   # three bf16 parts per value: six tensor-core products per fp32 product
         tc_peak, tc_src = measured_bf16_peak()
         peak, src, bound = tc_peak / 6, f"sixth {tc_src}: six bf16 products per fp32 product", "tensor"

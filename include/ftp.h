@@ -172,6 +172,17 @@ int ftp_plan_exec_groups(const ftp_plan* plan, int* n_groups, ftp_group* groups_
  * (Section 4.1).  FTP_ERR_ARG on a bad index or NULL. */
 int ftp_plan_group_mode(const ftp_plan* plan, int group, int* stationary, int* partial_sets);
 
+/* Which kernels run one pass (0 forward, 1 backward) of an EXECUTED group, and with that its arithmetic and order of sums.
+ * Activations are the same bits under every tile grid and grouping profile that leaves each layer on the same kernels; between
+ * two kinds of kernels results agree to rounding.  FTP_ERR_ARG on a bad index, pass or NULL. */
+enum {
+    FTP_KERNELS_FUSED  = 0,  /* fused sub-tile stacks (fp32: CUDA cores; bf16: tensor cores) */
+    FTP_KERNELS_ROWS   = 1,  /* fp32 one-conv groups: weight-stationary on the CUDA cores */
+    FTP_KERNELS_BANDED = 2,  /* bf16 one-conv groups: banded tensor-core kernels */
+    FTP_KERNELS_SPLIT  = 3   /* fp32 one-conv groups: tensor cores, three bf16 parts a value (see ftp_plan_opts.stationary) */
+};
+int ftp_plan_group_kernels(const ftp_plan* plan, int group, int pass, int* kernels);
+
 void ftp_plan_destroy(ftp_plan* plan);
 
 /*
@@ -205,7 +216,8 @@ int ftp_plan_sizes(const ftp_plan* plan, size_t* param_floats,
  * Sub-tiling chosen for an EXECUTED group (0-based index into the profile of
  * ftp_plan_exec_groups) and pass (0 forward, 1 backward):
  * number of sub-tile rows and columns over the whole map, dynamic shared
- * memory per block in bytes, and blocks launched.  Any out pointer may be NULL.
+ * memory per block in bytes, and blocks launched.  (Groups on the split kernels: the figures of the row kernels
+ * that run them with ftp_plan_opts.stationary = 1.)  Any out pointer may be NULL.
  */
 int ftp_plan_subtiles(const ftp_plan* plan, int pass, int group,
                       int* rows, int* cols, size_t* smem_bytes, int* blocks);
@@ -417,11 +429,11 @@ int ftp_plan_check(ftp_plan* plan, void* workspace, void* stream);
 /*
  * Diagnostic for the error path above (the paper has no counterpart): launches, on `stream`, one small
  * kernel whose only thread waits on a barrier that nothing arrives on, through the same bounded-wait
- * routine as the bf16 tile kernels but with a limit of about `limit_us` microseconds (1 .. 100000, counted
+ * routine as the tensor-core kernels but with a limit of about `limit_us` microseconds (1 .. 100000, counted
  * in SM clock cycles at a nominal 2 GHz).  The wait runs out, the kernel sets the workspace's error word
  * and returns; nothing faults and the context stays usable.  The next ftp_plan_check then reports
- * FTP_ERR_TIMEOUT; the next ftp_forward / ftp_step* clears the word again.  bf16 plans only
- * (FTP_ERR_PRECISION otherwise); FTP_ERR_ARG on a null or unaligned pointer or a limit out of range.
+ * FTP_ERR_TIMEOUT; the next ftp_forward / ftp_step* clears the word again.  Plans whose kernels have such waits only: bf16 plans and
+ * fp32 plans with split operands (FTP_ERR_PRECISION otherwise); FTP_ERR_ARG on a null or unaligned pointer or a limit out of range.
  */
 int ftp_plan_wait_probe(ftp_plan* plan, void* workspace, int limit_us, void* stream);
 

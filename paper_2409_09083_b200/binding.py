@@ -52,6 +52,8 @@ _lib.ftp_plan_exec_groups.argtypes = [_vp, ctypes.POINTER(_i), ctypes.POINTER(ft
 _lib.ftp_plan_exec_groups.restype = _i
 _lib.ftp_plan_group_mode.argtypes = [_vp, _i, ctypes.POINTER(_i), ctypes.POINTER(_i)]
 _lib.ftp_plan_group_mode.restype = _i
+_lib.ftp_plan_group_kernels.argtypes = [_vp, _i, _i, ctypes.POINTER(_i)]
+_lib.ftp_plan_group_kernels.restype = _i
 _lib.ftp_plan_destroy.argtypes = [_vp]
 _lib.ftp_plan_destroy.restype = None
 _lib.ftp_plan_region.argtypes = [_vp, _i, _i, _i, _i, _i, ctypes.POINTER(_i * 4)]
@@ -244,6 +246,13 @@ class Plan:
         _check(_lib.ftp_plan_group_mode(self._h, group, ctypes.byref(st), ctypes.byref(sets)))
         return st.value, sets.value
 
+    def group_kernels(self, group, pass_=0):
+        """Which kernels run a pass (0 forward, 1 backward) of executed group `group`: "fused", "rows" (fp32 one-conv groups on the
+        CUDA cores), "banded" (bf16 one-conv groups) or "split" (fp32 one-conv groups on the tensor cores)."""
+        k = _i()
+        _check(_lib.ftp_plan_group_kernels(self._h, group, pass_, ctypes.byref(k)))
+        return ("fused", "rows", "banded", "split")[k.value]
+
     def region(self, pass_, group, map_index, ty, tx):
         """(x1, y1, x2, y2), inclusive, of user tile (ty, tx) at map X_{map_index}."""
         out = (_i * 4)()
@@ -284,7 +293,7 @@ class Plan:
         return [(arr[i].kind, arr[i].group, arr[i].ms) for i in range(min(n.value, cap))]
 
     def check(self, workspace, stream=None):
-        """Synchronise and raise FtpError(FTP_ERR_TIMEOUT) if a device-side wait of the bf16 path ran out."""
+        """Synchronise and raise FtpError(FTP_ERR_TIMEOUT) if a bounded device-side wait ran out."""
         _check(_lib.ftp_plan_check(self._h, _workspace(self, workspace).ptr, _stream(stream)))
 
     def wait_probe(self, workspace, limit_us=2000, stream=None):

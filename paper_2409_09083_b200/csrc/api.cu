@@ -928,6 +928,15 @@ int ftp_plan_group_mode(const ftp_plan* plan, int group, int* stationary, int* p
     return FTP_OK;
 }
 
+int ftp_plan_group_kernels(const ftp_plan* plan, int group, int pass, int* kernels)
+{
+    if (!plan || !kernels || group < 0 || group >= (int)plan->groups.size() || pass < 0 || pass > 1) return FTP_ERR_ARG;
+    const GroupPlan& g = plan->groups[group];
+    *kernels = g.tfg.on ? FTP_KERNELS_BANDED : g.sp.on && (pass == 1 || !g.sp.rows_fwd) ? FTP_KERNELS_SPLIT
+             : g.st.on ? FTP_KERNELS_ROWS : FTP_KERNELS_FUSED;
+    return FTP_OK;
+}
+
 void ftp_plan_destroy(ftp_plan* plan)
 {
     if (!plan) return;
@@ -1239,7 +1248,7 @@ int ftp_plan_check(ftp_plan* plan, void* workspace, void* stream)
 int ftp_plan_wait_probe(ftp_plan* plan, void* workspace, int limit_us, void* stream)
 {
     if (!plan || !workspace || !aligned256(workspace) || limit_us <= 0 || limit_us > 100000) return FTP_ERR_ARG;
-    if (!is_tc(plan)) return FTP_ERR_PRECISION;
+    if (!is_tc(plan) && !plan->split) return FTP_ERR_PRECISION;
     ++plan->launches;
     tcd::wait_probe_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(err_ptr(workspace, plan), (long long)limit_us * 2000);
     return launched_ok() ? FTP_OK : FTP_ERR_CUDA;

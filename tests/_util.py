@@ -114,3 +114,20 @@ def draw_unambiguous(wl, bias_std=0.5, tau=2e-5, tries=200, store=None):
         if decision_margin(list(w.layers), ref) > tau:
             return w, x, params, target, ref
     raise RuntimeError("no seed with unambiguous decisions found")
+
+
+def kernels(plan):
+    """{layers of an executed group: (kernels of its forward pass, of its backward pass)}."""
+    return {g: (plan.group_kernels(i, 0), plan.group_kernels(i, 1)) for i, g in enumerate(plan.exec_groups())}
+
+
+def assert_split(plan, layers):
+    """Every conv layer with a 1x1 or 3x3 window and 32 input channels or more runs on the split kernels (with exactly 32 its
+    forward pass on the row kernel), no other layer does."""
+    for (a, b), k in kernels(plan).items():
+        convs = [l for l in layers[a - 1:b] if l.kind == "conv"]
+        if len(convs) == 1 and convs[0].k in (1, 3) and convs[0].cin >= 32:
+            assert k == ("rows" if convs[0].cin == 32 else "split", "split"), (a, b, k)
+        else:
+            assert "split" not in k, (a, b, k)
+    assert any("split" in k for k in kernels(plan).values())

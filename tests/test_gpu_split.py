@@ -17,7 +17,7 @@ import torch
 
 import paper_2409_09083_b200 as ftp
 from paper_2409_09083_b200 import synth
-from _util import FP32_TOL, rel_err, run_gpu, run_oracle
+from _util import FP32_TOL, assert_split, kernels, rel_err, run_gpu, run_oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -45,10 +45,6 @@ STACKS = {
 }
 
 
-def split_layers(plan):
-    return [g for i, g in enumerate(plan.exec_groups()) if plan.group_mode(i)[0] == 1]
-
-
 @pytest.mark.parametrize("name", sorted(STACKS))
 def test_split_stacks_match_oracle(name):
     """Dyadic data (the forward pass is exact in any order, so every decision agrees): activations bit for bit, gradients
@@ -62,7 +58,7 @@ def test_split_stacks_match_oracle(name):
     assert rel_err(got["dx"], ref["dx"]) <= FP32_TOL
     assert rel_err(got["dparams"], ref["dparams"]) <= FP32_TOL
     plan = got["plan"]
-    assert split_layers(plan)
+    assert_split(plan, wl.layers)
     ws = plan.new_workspace().fill_(0xff)
     xd, pd, td = (torch.from_numpy(a).cuda() for a in (x, params, target))
     grads = [torch.empty_like(pd) for _ in range(2)]
@@ -90,19 +86,32 @@ def test_split_kernels_keep_fp32_accuracy(name, convs):
     ref = run_oracle(wl, x, params, dy=dy)
     got = run_gpu(wl, x, params, dy=dy)
     fma = run_gpu(wl, x, params, dy=dy, stationary=1)
+    assert_split(got["plan"], wl.layers)
+    assert all("split" not in k for k in kernels(fma["plan"]).values())
     norm = lambda a, o: float(np.linalg.norm((a.astype(np.float64) - o).ravel()) / np.linalg.norm(o.ravel()))
     for k in ("y", "dx", "dparams"):
         assert norm(got[k], ref[k]) <= convs * 6 * 2.0 ** -23, k
         assert norm(got[k], ref[k]) <= 1.5 * norm(fma[k], ref[k]), k
 
 
-def test_small_stacks_stay_on_the_multiply_add_kernels():
-    """The rule looks at one image's multiply-accumulates, not at the batch: a batch and its halves take the same kernels."""
-    plan = lambda n, h, w, **kw: ftp.ftp_plan(tuple(synth.stack_yolo8()), n, 3, h, w, (2, 2), one(8), **kw)
-    small, large = plan(64, 64, 96), plan(1, 88, 104)
-    assert small.workspace_bytes == plan(64, 64, 96, stationary=0).workspace_bytes
-    assert plan(2, 88, 104).workspace_bytes != plan(2, 88, 104, stationary=1).workspace_bytes
-    assert large.group_mode(1)[0] == 1
+def test_wait_that_runs_out_is_reported():
+    """Split plans have bounded waits on the device: see the test of the same name on the bf16 path."""
+    from paper_2409_09083_b200 import binding
+    wl = STACKS["stack-8-ragged"]
+    x, params, _ = synth.draw(wl)
+    plan = ftp.ftp_plan(wl.layers, wl.N, wl.C, wl.H, wl.W, wl.grid, wl.groups)
+    ws = plan.new_workspace()
+    xd, pd = torch.from_numpy(x).cuda(), torch.from_numpy(params).cuda()
+    y = [torch.empty((wl.N,) + tuple(synth.map_shapes(wl.layers, wl.C, wl.H, wl.W)[-1]), device="cuda") for _ in range(2)]
+    ftp.ftp_forward(plan, xd, pd, y[0], ws)
+    plan.check(ws)
+    plan.wait_probe(ws, limit_us=2000)
+    with pytest.raises(binding.FtpError) as e:
+        plan.check(ws)
+    assert e.value.code == -7
+    ftp.ftp_forward(plan, xd, pd, y[1], ws)                  # clears the error word
+    plan.check(ws)
+    assert torch.equal(y[0], y[1])
 
 
 # one layer on a batch of two, above the 1e8 rule: flat runs; tiles with a pool; a 1x1 layer; tiles of a wide map; the forward pass on
@@ -149,6 +158,7 @@ def test_infinities_and_nans_reach_what_they_reach_in_a_plain_sum(name, where):
         dy[0, 5, 5, 6], dy[1, 7, 7, 9], dy[0, 9, 8, 20] = np.inf, -np.inf, np.nan
         dy[0, 11, 0, 0], dy[1, 12, -1, -1] = np.inf, np.inf
     ref, got = run_oracle(wl, x, params, dy=dy), run_gpu(wl, x, params, dy=dy)
+    assert_split(got["plan"], wl.layers)
     for k in ("y", "dx", "dparams"):
         g, r = got[k].astype(np.float64), ref[k]
         cg, cr = classes(g), classes(r)
@@ -174,6 +184,7 @@ def test_infinities_and_nans_through_two_layers(name):
     x[0, 5, 10, 12], x[1, 7, 9, 30], x[0, 9, 15, 40], x[1, 3, 0, 0] = np.inf, -np.inf, np.nan, np.inf
     dy[1, 5, 20, 16], dy[0, 9, 2, 3] = np.inf, np.nan
     ref, got = run_oracle(wl, x, params, dy=dy), run_gpu(wl, x, params, dy=dy)
+    assert_split(got["plan"], wl.layers)
     for k in ("y", "dx"):
         assert np.array_equal(classes(got[k]), classes(ref[k])), k
         ok = np.isfinite(ref[k])
@@ -194,6 +205,7 @@ def test_the_largest_finite_values_between_layers(cin, pooled):
     params[256 * cin + 256:] *= np.float32(2.0 ** -20)
     x[:, :, 3:9, 5:9] = np.float32(3.395e38) * np.random.default_rng(2).choice(np.float32([1, -1, 0.999]), x[:, :, 3:9, 5:9].shape)
     ref, got = run_oracle(wl, x, params, dy=dy), run_gpu(wl, x, params, dy=dy)
+    assert_split(got["plan"], wl.layers)
     for k in ("y", "dx"):
         assert np.isfinite(got[k]).all(), k
         scale = np.abs(ref[k]).max()
@@ -209,6 +221,7 @@ def test_the_largest_finite_values(name):
     x[:, :, 3:9, 5:9] = np.float32(3.395e38) * np.random.default_rng(2).choice(np.float32([1, -1, 0.999]), x[:, :, 3:9, 5:9].shape)
     params *= np.float32(2.0 ** -20)
     ref, got = run_oracle(wl, x, params, dy=dy), run_gpu(wl, x, params, dy=dy)
+    assert_split(got["plan"], wl.layers)
     for k in ("y", "dx"):
         assert np.isfinite(got[k]).all(), k
         scale = np.abs(ref[k]).max()
@@ -227,5 +240,6 @@ def test_the_smallest_positive_values_count_as_positive(name):
     params[at:at + l.cout] = np.where(c % 2, -1, 1) * np.float32(2.0) ** (-149 + c // 2).astype(np.float32)
     assert (params[at:at + l.cout] != 0).all()
     ref, got = run_oracle(wl, x, params, dy=dy), run_gpu(wl, x, params, dy=dy)
+    assert_split(got["plan"], wl.layers)
     assert rel_err(got["dx"], ref["dx"]) <= FP32_TOL
     assert rel_err(got["dparams"], ref["dparams"]) <= FP32_TOL

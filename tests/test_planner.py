@@ -11,6 +11,7 @@ import pytest
 import paper_2409_09083_b200 as ftp
 from oracle import spans
 from paper_2409_09083_b200 import binding, synth
+from _util import assert_split, kernels
 from test_spans_oracle import STACKS, read_golden
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -333,3 +334,20 @@ def test_small_launches_of_the_row_convolution_use_half_size_blocks():
     plan = ftp.ftp_plan(big.layers, big.N, big.C, big.H, big.W, big.grid, big.groups)
     st = plan.subtiles(0, plan.exec_groups().index((5, 5)))
     assert st["rows"] == (16 * 76 + 15) // 16
+
+
+def test_small_stacks_stay_on_the_multiply_add_kernels():
+    """The rule looks at one image's multiply-accumulates in the layers concerned (1e8 and more run split), not at the batch: a
+    batch and its parts take the same kernels.  On both sides of it, and with the options that switch the split kernels off."""
+    layers = tuple(synth.stack_yolo8())
+    plan = lambda n, h, w, **kw: ftp.ftp_plan(layers, n, 3, h, w, (2, 2), ((1, 8),), **kw)
+
+    def macs(h, w):
+        shapes = synth.map_shapes(layers, 3, h, w)
+        return sum(shapes[i][1] * shapes[i][2] * l.cin * l.cout * l.k ** 2 for i, l in enumerate(layers) if l.kind == "conv" and l.cin >= 32)
+    assert macs(64, 104) < 1e8 <= macs(64, 112)
+    for n in (1, 8, 64):
+        assert all("split" not in k for k in kernels(plan(n, 64, 104)).values())
+        assert_split(plan(n, 64, 112), layers)
+    for kw in (dict(stationary=1), dict(stationary=-1), dict(precision=1)):
+        assert all("split" not in k for k in kernels(plan(1, 64, 112, **kw)).values())
