@@ -57,7 +57,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
 constexpr int kMaxA = 3, kMaxB = 8;
 constexpr int kConvThreads = 384;             // 8 epilogue warps; producer, MMA issuers of the large and (two) of the small products
 constexpr int kEpiThreads = 256;
-constexpr float kSplitLargest = 1.2676506e30f; // 2^100: the sum of two such values times two slopes of 2^10 is far from infinity
 
 // ---------------------------------------------------------------------------------------------
 // Convolution.  A work item is a tile of nblk x 128 output entries x a slice of Ns <= 128 output channels.  The input
@@ -151,7 +150,6 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_split_kernel(const __gri
         const int q = warp & 3, half = warp >> 2, et = threadIdx.x;
         const size_t opart = (size_t)A.og.planes * A.og.tp;
         uint32_t gh = 0, gl = 0, k = 0;                       // chains and items of this half so far
-        const bool small_slopes = fabsf(A.slope) <= 1024.f && fabsf(A.prev_slope) <= 1024.f;
         for (int it = blockIdx.x; it < A.items; it += gridDim.x, ++k) {
             const Item I = item_of(it);
             const int co0 = I.slice * A.Ns;
@@ -177,9 +175,6 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_split_kernel(const __gri
                 __syncwarp();
             };
             bool ok = true;
-            uint32_t round = kRoundFirst;
-            auto delta_first = [&](float x) { return first_part(x, round); };
-            auto map_first = [&](float x) { return keep_sign(x, first_part(x, round)); };
             if (half < I.nblk) {
                 for (int c = 0; c < kChains * A.nchunks; ++c, ++gh) {
                     if (!wait(&H->hdone[half], gh & 1u, 32)) { ok = false; break; }
@@ -187,18 +182,9 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_split_kernel(const __gri
                     add(0, plain);
                     if (lane == 0) mbar_arrive(smem_u32(&H->hfree[half]));
                 }
-                // Sums that are infinite or NaN, or so large that a value to be stored could be within 2^-7 of the largest: the small
-                // products are then added with care and first parts cut, not rounded.  (One answer for the warp; the comparison
-                // is false for a NaN.  Together 0.5 to 1 % of a step; 1.4 % with a look at every value, see split8.)
-                float top = max_abs(max_abs(bias[0], bias[1], bias[2]), bias[3], 0.f);
-#pragma unroll
-                for (int j = 0; j < 128; j += 2) top = max_abs(top, acc[j], acc[j + 1]);
-                const bool large = __any_sync(0xffffffffu, !(top < kSplitLargest && small_slopes));
-                round = large ? 0u : kRoundFirst;
                 if (ok && wait(&H->ldone[half], gl & 1u, 32)) {
                     fence_after_sync();
-                    if (large) add(256, add_small);
-                    else add(256, plain);
+                    add(256, add_small);
                     if (lane == 0) mbar_arrive(smem_u32(&H->lfree[half]));
                     ++gl;
                 } else ok = false;
@@ -256,8 +242,8 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_split_kernel(const __gri
                                 }
                             }
                             if (!A.prev_arg) {
-                                store_split(A.out_s, opart, (size_t)pl * A.og.tp + e, v, map_first);
-                                store_split(A.out_s, opart, (size_t)(pl + 1) * A.og.tp + e, v + 8, map_first);
+                                store_split(A.out_s, opart, (size_t)pl * A.og.tp + e, v);
+                                store_split(A.out_s, opart, (size_t)(pl + 1) * A.og.tp + e, v + 8);
                             }
                         }
                         if (A.prev_arg) {
@@ -276,7 +262,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_split_kernel(const __gri
                             for (int h = 0; h < 2; ++h) {
                                 const unsigned long long am = valid ? __ldg(A.prev_arg + (size_t)(pl + h) * A.g.tp + e) : 0ull;
                                 uint4 s[3];
-                                split8(v + h * 8, s[0], s[1], s[2], delta_first);
+                                split8<false>(v + h * 8, s[0], s[1], s[2]);
 #pragma unroll
                                 for (int k2 = 0; k2 < 2; ++k2) {
                                     const int src = 16 * k2 + (lane >> 1);
@@ -857,7 +843,7 @@ __global__ void __launch_bounds__(256) pack_split_kernel(const __grid_constant__
 {
     previous_launches();
     __shared__ float s[kPackSmemFloats];
-    pack_tiles<3>(A, params, s, [](const float* v, uint4* p) { split8(v, p[0], p[1], p[2], [](float x) { return first_part(x); }); });
+    pack_tiles<3>(A, params, s, [](const float* v, uint4* p) { split8<false>(v, p[0], p[1], p[2]); });
 }
 
 }  // namespace sp

@@ -10,25 +10,32 @@
 namespace ftp {
 namespace sp {
 
-constexpr uint32_t kRoundFirst = 0x20000u;       // half of the last place of 6 significant bits
+// largest magnitude of three values, NaN if one of them is
+__device__ __forceinline__ float max_abs(float a, float b, float c)
+{
+    float d;
+    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
 
-// First part of a value, as the bits of an fp32: rounded to 6 significant bits (nearest, ties away from zero) or, with round = 0,
-// cut to 6 bits.
-__device__ __forceinline__ uint32_t first_part(float x, uint32_t round) { return (__float_as_uint(x) + round) & 0xfffc0000u; }
-// Of a value of any size: cut within 2^-7 of the largest fp32, where rounding would make an infinity, and beyond.
-__device__ __forceinline__ uint32_t first_part(float x) { return first_part(x, fabsf(x) < __int_as_float(0x7f7e0000) ? kRoundFirst : 0u); }
-// Of a value in a saved map, where the backward pass takes the sign of a value from its first part: positive for every positive
-// value (below 2^-132 the smallest bf16, 2^-133; the second part makes up for it).
-__device__ __forceinline__ uint32_t keep_sign(float x, uint32_t first) { return __float_as_int(x) > 0 ? max(first, 0x10000u) : first; }
-
-// Three bf16 parts of eight values: `first(x)`, the rest of x rounded to bf16, and the rest of that, which bf16 holds exactly (but for
-// a bit that may be lacking where the first part is cut).  An infinity becomes (itself, NaN, NaN), a NaN NaNs: see
-// add_small.  (Not a branch every eight values to code for the rare ones: that made the unrolled output phases of
-// conv_split_kernel 6 % slower, and a comparison per value 1 %.)
-template <class First>
-__device__ __forceinline__ void split8(const float* v, uint4& p0, uint4& p1, uint4& p2, First first)
+// Three bf16 parts of eight values: the value rounded to 6 significant bits (nearest, ties away from zero), the rest rounded to
+// bf16, and the rest of that, which bf16 holds exactly.  Where one of the eight is within 2^-7 of the largest fp32, so that its first
+// part would be an infinity, or is infinite or NaN, the first parts are cut to 6 bits instead (the three parts then hold
+// 23 bits at least).  An infinity becomes (itself, NaN, NaN), a NaN NaNs: see add_small.
+// (One comparison for the eight.  One per value: a step with 16 layers 0.8 % slower; a branch to code for the rare ones in the
+// midst of the unrolled output phases of conv_split_kernel: 5 %.)
+// kSign: a positive value has a positive first part, however small it is (below 2^-132 the smallest bf16, 2^-133; the second part
+// makes up for it): the backward pass takes the sign of a saved value from there.
+template <bool kSign>
+__device__ __forceinline__ void split8(const float* v, uint4& p0, uint4& p1, uint4& p2)
 {
     uint32_t* a = &p0.x; uint32_t* b = &p1.x; uint32_t* c = &p2.x;
+    const float top = max_abs(max_abs(max_abs(v[0], v[1], v[2]), v[3], v[4]), max_abs(v[5], v[6], v[7]), 0.f);
+    const uint32_t round = top < __int_as_float(0x7f7e0000) ? 0x20000u : 0u;
+    auto first = [&](float x) {
+        const uint32_t f = (__float_as_uint(x) + round) & 0xfffc0000u;
+        return kSign && __float_as_int(x) > 0 ? max(f, 0x10000u) : f;
+    };
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const float x = v[2 * i], y = v[2 * i + 1];
@@ -42,29 +49,16 @@ __device__ __forceinline__ void split8(const float* v, uint4& p0, uint4& p1, uin
         c[i] = *reinterpret_cast<const uint32_t*>(&h2);
     }
 }
-template <class First>
-__device__ __forceinline__ void store_split(uint4* base, size_t part_stride, size_t at, const float* v, First first)
-{
-    uint4 p0, p1, p2;
-    split8(v, p0, p1, p2, first);
-    base[at] = p0; base[at + part_stride] = p1; base[at + 2 * part_stride] = p2;
-}
 __device__ __forceinline__ void store_split(uint4* base, size_t part_stride, size_t at, const float* v)
 {
-    store_split(base, part_stride, at, v, [](float x) { return keep_sign(x, first_part(x)); });
+    uint4 p0, p1, p2;
+    split8<true>(v, p0, p1, p2);
+    base[at] = p0; base[at + part_stride] = p1; base[at + 2 * part_stride] = p2;
 }
 
 // Adds the products of the lower parts (small) to a sum that holds those of the first parts (large).  Where an operand is infinite or
 // NaN, the products of the first parts alone have the sum that fp32 multiply-adds have; the others stay out.
 __device__ __forceinline__ float add_small(float large, float small) { return fabsf(large) < __int_as_float(0x7f800000) ? large + small : large; }
-
-// largest magnitude of three values, NaN if one of them is
-__device__ __forceinline__ float max_abs(float a, float b, float c)
-{
-    float d;
-    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
 
 // pixel of an entry (n, y, x); false: a zero entry of the map (edge column, row between images, lead or tail)
 __device__ __forceinline__ bool pixel_of(const SplitGeom& g, int e, int& n, int& y, int& x)

@@ -126,7 +126,8 @@ def assert_split(plan, layers):
     forward pass on the row kernel), no other layer does."""
     for (a, b), k in kernels(plan).items():
         convs = [l for l in layers[a - 1:b] if l.kind == "conv"]
-        if len(convs) == 1 and convs[0].k in (1, 3) and convs[0].cin >= 32:
+        if any(l.k in (1, 3) and l.cin >= 32 for l in convs):
+            assert len(convs) == 1, (a, b, k)
             assert k == ("rows" if convs[0].cin == 32 else "split", "split"), (a, b, k)
         else:
             assert "split" not in k, (a, b, k)

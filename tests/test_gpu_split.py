@@ -243,3 +243,37 @@ def test_the_smallest_positive_values_count_as_positive(name):
     assert_split(got["plan"], wl.layers)
     assert rel_err(got["dx"], ref["dx"]) <= FP32_TOL
     assert rel_err(got["dparams"], ref["dparams"]) <= FP32_TOL
+
+
+def test_activations_do_not_depend_on_grid_profile_or_batch_split():
+    """Above the 1e8 rule, what the test of the same kind in test_gpu_parity.py shows below it: the same bits in the last map under
+    every tile grid and profile that leaves each layer on its kernels, gradients to 1e-5 (sums in another order), the same bits
+    from run to run; an image gives the same bits alone and in a batch.  Profiles that fuse layers run on other kernels: then
+    the maps agree within both sides' rounding."""
+    wl = STACKS["stack-8-ragged"].with_(groups=one(8))
+    convs = sum(l.kind == "conv" for l in wl.layers)
+    x, params, _ = synth.draw(wl, bias_std=0.1)
+    dy = np.random.default_rng(1).standard_normal((wl.N,) + tuple(synth.map_shapes(wl.layers, wl.C, wl.H, wl.W)[-1])).astype(np.float32)
+    base, again = run_gpu(wl, x, params, dy=dy), run_gpu(wl, x, params, dy=dy)
+    assert_split(base["plan"], wl.layers)
+    for k in ("y", "dx", "dparams"):
+        assert np.array_equal(base[k], again[k]), f"{k} differs from run to run"
+    variants = [dict(grid=(1, 1)), dict(grid=(4, 2), groups=((1, 4), (5, 8))), dict(grid=(2, 5), groups=synth.groups_per_layer(wl.layers)),
+                dict(grid=(11, 17), groups=synth.groups_per_maxpool(wl.layers)), dict(opts=dict(max_group_convs=1)),
+                dict(opts=dict(cost_model=1))]
+    for v in variants:
+        opts = v.get("opts", {})
+        got = run_gpu(wl.with_(**{k: v[k] for k in v if k != "opts"}), x, params, dy=dy, **opts)
+        assert_split(got["plan"], wl.layers)
+        assert np.array_equal(got["y"], base["y"]), v
+        assert rel_err(got["dx"], base["dx"]) <= 1e-5, v
+        assert rel_err(got["dparams"], base["dparams"]) <= 1e-5, v
+    for n in range(wl.N):
+        alone = run_gpu(wl.with_(N=1), x[n:n + 1], params, dy=dy[n:n + 1])
+        assert np.array_equal(alone["y"][0], base["y"][n])
+        assert np.array_equal(alone["dx"][0], base["dx"][n])
+    for opts in (dict(strict_groups=True), dict(cost_model=-1), dict(stationary=-1), dict(stationary=1)):
+        got = run_gpu(wl, x, params, dy=dy, **opts)
+        assert kernels(got["plan"]) != kernels(base["plan"])
+        d = np.linalg.norm((got["y"] - base["y"]).astype(np.float64)) / np.linalg.norm(base["y"].astype(np.float64))
+        assert d <= 2 * convs * 6 * 2.0 ** -23, opts
