@@ -515,15 +515,21 @@ bool split_conv_args(SplitConvArgs& a, const SplitConvPlan& c, const uint4* in, 
     return K == 3 || encode_split_map(a.tmap, in, g, false, 128, 0, c.kpc, 3);
 }
 
+// The input of a split group in split form, where it exists as an fp32 map only: the network input and what a fused stack wrote.
+void split_input(ftp_plan* p, const GroupPlan& g, int gi, const float* x, void* ws, cudaStream_t st)
+{
+    if (gi > 0 && p->groups[gi - 1].st.on) return;
+    const OpDesc& op = g.fwd_ops[0];
+    Timed t(p, st, 9, gi);
+    split_launch_planes(map_ptr(p, x, ws, g.first), split_ptr(ws, g.sp.in_off), in_geom(p, op), op.cin, t.ls());
+}
+
 bool split_forward(ftp_plan* p, const GroupPlan& g, int gi, const float* x, const float* params, void* ws, cudaStream_t st)
 {
     const OpDesc& op = g.fwd_ops[0];
     uint4* in = split_ptr(ws, g.sp.in_off);
-    if (gi == 0 || !p->groups[gi - 1].st.on) {      // a fused stack below wrote an fp32 map only
-        Timed t(p, st, 9, gi);
-        split_launch_planes(map_ptr(p, x, ws, g.first), in, in_geom(p, op), op.cin, t.ls());
-    }
     if (g.sp.rows_fwd) return stationary_forward(p, g, gi, x, params, ws, st);
+    split_input(p, g, gi, x, ws, st);
     SplitConvArgs a{};
     if (!split_conv_args(a, g.sp.f, in, in_geom(p, op), op.k, op.cout, op.cout16)) return false;
     a.w = split_ptr(ws, p->ws.sw_off) + g.sp.wf_off;
@@ -544,6 +550,7 @@ bool split_backward(ftp_plan* p, const GroupPlan& g, int gi, const float* x, con
 {
     const OpDesc& op = g.bwd_ops[0];
     uint4* dz = split_ptr(ws, p->ws.sdz_off[gi & 1]);
+    if (g.sp.rows_fwd) split_input(p, g, gi, x, ws, st);     // (the forward pass read the fp32 map: 305 -> 214 us, 32 -> 32, 1x1, 16 x 320 x 320)
     if (!split_at(p, gi + 1)) {
         SplitDeltaArgs d{};
         d.d = dout; d.y = map_ptr(p, x, ws, op.out_map); d.dz = dz; d.g = dz_geom(p, op); d.low = out_geom(p, op);

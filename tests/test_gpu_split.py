@@ -95,6 +95,25 @@ def test_split_kernels_keep_fp32_accuracy(name, convs):
         assert norm(got[k], ref[k]) <= 1.5 * norm(fma[k], ref[k]), k
 
 
+def test_forward_on_the_row_kernel_leaves_the_input_as_it_is():
+    """A first layer with 32 input channels: its forward pass reads the fp32 input, so the conversion to split form, which only the
+    filter gradient reads, is no part of ftp_forward (two packing launches and the convolution)."""
+    wl = SINGLE["32-channels"]
+    x, params, dy = draw_single(wl)
+    plan = ftp.ftp_plan(wl.layers, wl.N, wl.C, wl.H, wl.W, wl.grid, wl.groups)
+    assert_split(plan, wl.layers)
+    ws = plan.new_workspace().fill_(0xff)
+    xd, pd, dyd = (torch.from_numpy(a).cuda() for a in (x, params, dy))
+    ftp.ftp_forward(plan, xd, pd, None, ws)
+    assert plan.launch_count() == 3
+    grads = [torch.empty_like(pd) for _ in range(2)]
+    for g in grads:                                          # the backward pass can be repeated after one forward pass
+        ftp.ftp_backward(plan, xd, dyd, pd, None, g, ws)
+    plan.check(ws)
+    ref = run_oracle(wl, x, params, dy=dy)
+    assert torch.equal(*grads) and rel_err(grads[0].cpu().numpy(), ref["dparams"]) <= FP32_TOL
+
+
 def test_wait_that_runs_out_is_reported():
     """Split plans have bounded waits on the device: see the test of the same name on the bf16 path."""
     from paper_2409_09083_b200 import binding
