@@ -5,7 +5,8 @@
 
 A step is one pass of the whole hot path (forward, loss delta, backward with input gradient,
 cross-tile reduction of the partial gradient sets, SGD update) over one batch of synthetic input.
-Rank 0 prints ONE JSON line.  Without --workload the run measures the three benchmark workloads
+Rank 0 prints ONE JSON line, short enough for a log that keeps the end of the output; the whole record (rooflines of all kernel
+classes, breakdowns per group, executed groups) goes to standard error as one JSON line, or to --details FILE.  Without --workload the run measures the three benchmark workloads
 C3 (the largest; the headline of the line), C1 and C2 (under "workloads"), each with its roofline,
 end-to-end and CPU-oracle numbers, after measuring the fp32 FMA rate of the GPU with a register-only
 kernel of the library (the peak the fp32 roofline fractions are quoted against).  With --gpus N > 1
@@ -80,6 +81,7 @@ def parse():
                     help="one-conv groups on their own kernels (fp32: weight-stationary; bf16: banded tensor-core kernels): 0 planner default, "
                          "-1 never (fused stacks only)")
     ap.add_argument("--strict-groups", action="store_true", help="execute the requested grouping profile as it is (no cuts)")
+    ap.add_argument("--details", default=None, help="file for the whole record (default: one line on standard error)")
     ap.add_argument("--no-bf16", action="store_true", help="skip the second measurement on the bf16 tensor-core path")
     return ap.parse_args()
 
@@ -246,9 +248,42 @@ def run_ours(args):
                             sub[key] = {"unavailable": str(e)}
                 line["workloads"][name] = {k: sub[k] for k in sub if k not in ("metric", "unit", "n_gpus", "higher_is_better", "scaling",
                                                                             "vs_baseline", "data", "fp32_fma_peak")}
-        print(json.dumps(line))
+        if args.details:
+            with open(args.details, "w") as f:
+                json.dump(line, f)
+        else:
+            print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(brief(line)))
     if dist is not None:
         dist.destroy_process_group()
+
+
+def brief(line):
+    """The headline line: the keys a reader of the benchmark needs, figures to six digits."""
+    def rounded(v):
+        if isinstance(v, float):
+            return float(f"{v:.6g}")
+        if isinstance(v, dict):
+            return {k: rounded(x) for k, x in v.items()}
+        return [rounded(x) for x in v] if isinstance(v, list) else v
+    out = {k: line[k] for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                                "vs_baseline", "dtype", "data")}
+    cfg = line["config"]
+    out["config"] = {"workload": cfg["workload"].split(", tile grid")[0], "global_batch": cfg["global_batch"], "parallelism": cfg["parallelism"],
+                     "input_delta": True, "l2": "flushed"}
+    for k in ("clocks", "gpu_launches", "loss"):
+        out[k] = line[k]
+    if "e2e" in line:
+        out["e2e"] = {k: v for k, v in line["e2e"].items() if k != "pipeline"}
+    out["roofline"] = {k: line["roofline"][k] for k in ("bound", "kernel", "achieved", "peak", "unit", "frac", "step_frac_of_peak")}
+    if "cpu_baseline" in line:
+        out["cpu_baseline"] = {k: line["cpu_baseline"][k] for k in ("value", "cores", "kind")}
+    # per workload and path: images/s with the batch on the device, end to end from host batches
+    pair = lambda r: [r["value"], r["e2e"]["value"]] if r.get("e2e") else [r["value"]]                            # noqa: E731
+    both = lambda r: {"f32": pair(r), **({"bf16": pair(r["bf16_tensor_core_path"])} if "bf16_tensor_core_path" in r else {})}   # noqa: E731
+    if "bf16_tensor_core_path" in line or "workloads" in line:
+        out["images_per_s_device_e2e"] = dict({"headline": both(line)}, **{k: both(r) for k, r in line.get("workloads", {}).items()})
+    return rounded(out)
 
 
 def measure(ctx, name, precision, extras=True, light=False, **plan_opts):
