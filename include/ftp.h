@@ -135,7 +135,14 @@ typedef struct {
                            outside the tensor core (as accurate as the fp32 sums of the CUDA-core kernels); their maps
                            then lie in the workspace as parts.  Infinities and NaNs reach what they reach in a plain sum
                            (the filter gradient may show a NaN for a window position that leads out of the map from an
-                           infinite value at its border).  1 keeps them on the CUDA cores.
+                           infinite value at its border).  Limits: values below 2^-110 are held to 2^-134 and not to 24 bits (a
+                           layer whose operands measure 2^-115, 2^-120, 2^-125 has relative errors of 2e-6, 7e-5,
+                           2e-3); sums within 2^-5 of the largest fp32 may overflow.  The switch at 1e8 also means
+                           that activations are no longer bit-identical between profiles that give such a layer a
+                           group of its own and profiles that fuse it with others, only equal to rounding
+                           (ftp_plan_group_kernels says what runs; tile grids and batch sizes make no difference), and
+                           that an image and a slab of it, planned as an image, may run on different kernels.
+                           1 keeps them on the CUDA cores.
                            bf16 path: a conv layer with a 1x1 or 3x3 window on a map of at most 1008 columns (the first
                            layer: a 3x3 window and at most 7 input channels) becomes an executed group of its own (with
                            its pool).  Forward pass and input delta run as banded tensor-core convolutions (a band of

@@ -247,9 +247,6 @@ bool encode_split_map(unsigned char out[128], const uint4* base, const SplitGeom
     return true;
 }
 
-// Tensor-core cycles of one MMA with N accumulator columns and both operands in shared memory (M = 128, K = 16)
-inline double tc_mma_cycles(int n) { return std::max(32.0 + n / 4.0, n / 2.0); }
-
 // One launch of the banded convolution kernel: `in` planes (cin16 channels) -> `out` planes (cout16 channels).
 struct PrevLayer { const uint4* y; const unsigned long long* arg; float slope; };   // see TcConvRowsArgs::prev_y
 

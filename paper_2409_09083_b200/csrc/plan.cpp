@@ -640,7 +640,6 @@ void plan_stationary(const ftp_plan& p, GroupPlan& g, const PlanOpts& o)
 }
 
 // ---- split kernels (split.cuh) ----
-inline double split_mma_cycles(int n) { return std::max(32.0 + n / 4.0, n / 2.0); }   // both operands in shared memory
 
 // Launch shape of conv_split_kernel.  Items are 128-entry blocks of the flat batch where the halo of a flat run fits, else
 // (wide maps, and always with a pool) tiles of R rows x Cw columns; the candidate with the least rounds of items over the
@@ -673,8 +672,7 @@ SplitConvPlan plan_split_conv(const SplitGeom& g, int K, int cout16, bool pool)
         c.pool_bytes = pool ? nblk * 128 * 16 * 4 : 0;
         c.b_stage = K * K * kpc * Ns * 16;
         const int a_bytes = c.a_bytes;
-        c.a_stages = std::min(3, std::max(2, (K == 1 ? 3 : 2)));
-        for (; c.a_stages >= 2; --c.a_stages) {
+        for (c.a_stages = K == 1 ? 3 : 2; c.a_stages >= 2; --c.a_stages) {
             c.b_stages = std::min(K == 1 ? 8 : 5, (room - c.pool_bytes - c.a_stages * a_bytes) / c.b_stage);
             if (c.b_stages >= 3) break;
         }
@@ -683,7 +681,7 @@ SplitConvPlan plan_split_conv(const SplitGeom& g, int K, int cout16, bool pool)
         if (items > 0x7fffffffLL) return;
         c.items = (int)items; c.blocks = (int)std::min<long long>(items, kSmCount);
         c.smem = kSplitHeader + c.a_stages * a_bytes + c.b_stages * c.b_stage + c.pool_bytes;
-        const double mma = nblk * (K * K * 6.0 * (kpc / 2)) * split_mma_cycles(Ns);
+        const double mma = nblk * (K * K * 6.0 * (kpc / 2)) * tc_mma_cycles(Ns);
         const double load = (3.0 * kpc * c.nruns * c.run_len * 16 + 3.0 * c.b_stage) / 22.0;
         const double cost = (double)((items + kSmCount - 1) / kSmCount) * (nchunks * std::max(mma, load) + 300.0) + nchunks * 200.0;
         if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = c; best.on = 1; }
@@ -741,7 +739,7 @@ SplitFgPlan plan_split_fg(const SplitGeom& g, int K, int cin16, int cout16)
     const int roles = t.slices * t.nci * (t.rows3 ? 1 : K);
     double best = -1;
     const double set_cost = (double)K * K * cin16 * cout16 * 8.0 / 5e6 * 1900.0;        // cycles to write and read one set of the layer
-    const double stage_cost = (K == 1 ? t.units : t.rows3 ? 9 : 3) * (t.E / 16) * 6 * (t.rows3 ? 26.0 : split_mma_cycles(t.ncols));
+    const double stage_cost = (K == 1 ? t.units : t.rows3 ? 9 : 3) * (t.E / 16) * 6 * (t.rows3 ? 26.0 : tc_mma_cycles(t.ncols));
     for (int shares = 1; shares <= std::min(t.stages_total, std::max(1, 2 * kSmCount / roles)); ++shares) {
         const double rounds = (double)((roles * shares + kSmCount - 1) / kSmCount);
         const double cost = rounds * (((t.stages_total + shares - 1) / shares) * stage_cost + 6000.0) + shares * set_cost;
@@ -753,10 +751,13 @@ SplitFgPlan plan_split_fg(const SplitGeom& g, int K, int cin16, int cout16)
 
 // Whether the fp32 plan runs its one-conv groups on the split kernels: with the default options, and only where the layers
 // they take (1x1 or 3x3 window, at least 32 input channels) amount to kSplitMinMacs multiply-accumulates an image in a
-// forward pass.  Below that (the 8-layer stack on images of less than about 80 x 80 pixels) a step is mostly launches and
-// latencies, and the CUDA-core kernels, whose sums have the order of the fused stacks, keep the result bit-identical under
-// every grouping profile.  The rule does not look at the batch, so that the parts of a batch that is dealt out to several
-// replicas run as the whole does.
+// forward pass.  Below that (the 8-layer stack on images of less than about 83 x 83 pixels) a step of one image is mostly
+// launches and latencies, and the CUDA-core kernels, whose sums have the order of the fused stacks, keep the result
+// bit-identical under every grouping profile.  (It is no crossover of the times: right above it, at 64 x 112, a step is twice
+// as fast on the split kernels as on the row kernels, 249 against 502 us with one image, 779 against 1655 with 64.)  The rule
+// does not look at the batch, so that the parts of a batch that is dealt out to several replicas run as the whole does.
+// Parts of an image need not: the slabs of a row-sharded step are planned as images of their own, and may run on the
+// CUDA cores where the whole image would run split.  Such results agree to rounding.
 bool split_wanted(const ftp_plan& p, const PlanOpts& o)
 {
     if (p.precision != FTP_FP32 || o.stationary != 0) return false;
@@ -775,17 +776,17 @@ void plan_split(const ftp_plan& p, GroupPlan& g)
     if (!p.split || !g.st.on || g.st.thin) return;
     const OpDesc& op = g.fwd_ops[0];
     if (op.cin < kStatMinCin || op.in_W > 1008) return;
+    if ((long long)p.N * (op.in_H + 1) * (op.in_W + 1) > 0x3fffffffLL) return;      // entries and copy coordinates are 32-bit
     const SplitGeom in = split_geom(p.N, op.cin, op.in_H, op.in_W), out = split_geom(p.N, op.cout, op.in_H, op.in_W);
-    if ((long long)in.N * (in.H + 1) * in.wp > 0x3fffffffLL) return;
     g.sp.f = plan_split_conv(in, op.k, op.cout16, op.kind == kOpConvPool);
     g.sp.d = plan_split_conv(out, op.k, op.cin16, false);
     g.sp.g = plan_split_fg(in, op.k, op.cin16, op.cout16);
     g.sp.on = g.sp.f.on && g.sp.d.on && g.sp.g.shares > 0;
-    // Forward pass of the layers with at most 32 input channels: by the multiply-add kernel, whose sums they have always had.  Such a
-    // layer stands at the highest resolution, where the sign and pool decisions that fall on near-ties are most numerous and
-    // each moves a whole delta at the network input by up to its root mean square; bit for bit the same maps keep them
-    // where they were.  Its contraction is the shortest (288 terms), so it gains least: 16 x 304 x 304, 32 -> 64: 1.1 ms, on the
-    // split kernel 0.44 ms.
+    // Forward pass of the layers with at most 32 input channels: by the multiply-add kernel, bit for bit the maps of the plans that run
+    // on the CUDA cores.  Such a layer stands at the highest resolution, where the sign and pool decisions that fall on near-ties are
+    // most numerous, and each that is taken differently moves a whole delta at the network input.  This is agreement with those
+    // plans and not accuracy (the split kernels' maps are nearer to fp64, see tests/test_gpu_split.py), and it has its
+    // price: 16 x 304 x 304, 32 -> 64: 1.1 ms, on the split kernel 0.44 ms.
     g.sp.rows_fwd = g.sp.on && op.cin <= 32;
 }
 // 16-byte entries of one packed arrangement
@@ -796,7 +797,7 @@ double split_estimate_us(const ftp_plan& p, const GroupPlan& g, bool backward, b
 {
     const OpDesc& op = g.fwd_ops[0];
     const double px = (double)p.N * op.in_H * op.in_W, flops = 2.0 * px * op.cin16 * op.cout16 * op.k * op.k;
-    auto rate = [](int n) { return 150e6 * std::min(1.0, n / 2.0 / split_mma_cycles(n)); };
+    auto rate = [](int n) { return 150e6 * std::min(1.0, n / 2.0 / tc_mma_cycles(n)); };
     const double in_us = px * op.cin16 * 6.0 / 4e6, out_us = px * op.cout16 * 6.0 / 4e6;
     if (!backward) return flops / (g.sp.rows_fwd ? kStatTflops * 1e6 : rate(g.sp.f.Ns)) + in_us + out_us + 10.0;
     double t = flops / rate(g.sp.g.rows3 ? 40 : g.sp.g.ncols) * (128.0 / g.sp.g.Ms) + in_us + out_us + 12.0;
@@ -1306,8 +1307,9 @@ int build_plan(ftp_plan& p, const ftp_layer* layers, int n_layers, int N, int C,
             if (!(g.sp.on && &g != &p.groups.back() && (&g)[1].sp.on && !(&g)[1].sp.rows_fwd))
                 ws.map_off[op.out_map - 1] = take((size_t)N * s.C * s.H * s.W * 4);
             if (op.kind == kOpConvPool) {
-                const SplitGeom sg = split_geom(N, s.C, s.H, s.W);
-                ws.arg_off[op.out_map - 1] = take(g.sp.on ? (size_t)sg.planes * sg.tp * 8 : (size_t)N * s.C * s.H * s.W);
+                size_t words = 0;
+                if (g.sp.on) { const SplitGeom sg = split_geom(N, s.C, s.H, s.W); words = (size_t)sg.planes * sg.tp; }
+                ws.arg_off[op.out_map - 1] = take(g.sp.on ? words * 8 : (size_t)N * s.C * s.H * s.W);
             }
         }
     // Deltas at the inputs of the executed groups 1..: the backward pass of group gi reads the one at its output

@@ -162,6 +162,9 @@ constexpr int kTcMaxColChunks = 8;            // a band spans at most 126 column
 constexpr int kTcFgHeader = 1024;             // barriers, tensor-memory slot, a core matrix of ones
 constexpr int kTcFgSmemBudget = 200 * 1024;   // header + two stages
 
+// Tensor-core cycles of one MMA with N accumulator columns and both operands in shared memory (M = 128, K = 16)
+inline double tc_mma_cycles(int n) { return n < 128 ? 32.0 + n / 4.0 : n / 2.0; }
+
 // Split execution of a one-conv group of the fp32 path (split.cuh): the contractions on the tensor cores, every fp32
 // operand as the sum of three bf16 values.
 enum { kSplitFlat = 0, kSplitTile = 1, kSplitPool = 2 };
