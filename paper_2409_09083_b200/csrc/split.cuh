@@ -16,8 +16,8 @@
 // of the accumulator's 24 bits to the range of their sum, so that little is cut off; and a chain of them is 2 to 4 steps long
 // before the epilogue warps add it to their registers, rounded to nearest.  The five small products go to a second set of
 // accumulators (L): they measure 2^-7 of the sum and their signs have nothing to do with its sign, so their chains may last for
-// an item (64 stages of the filter gradient).  What is left is 2e-9 to 1e-8 a layer.  Against fp64 sums the maps are three
-// times closer than those of stationary.cuh and the gradients as close (table in tests/test_gpu_split.py).
+// an item (64 stages of the filter gradient).  What is left is 2e-9 to 1e-8 a layer.  Against fp64 sums maps, deltas and
+// gradients are 1.7 to 7 times closer than those of stationary.cuh (table in tests/test_gpu_split.py).
 //
 // Maps travel between the layers in split form (split_args.hpp): 6 bytes a value instead of 4, split once by the epilogue
 // that produces them, with the zero padding in memory so that any run of entries is a tile: one plain bulk copy per plane
