@@ -301,6 +301,25 @@ def test_activations_do_not_depend_on_grid_profile_or_batch_split():
         assert d <= 2 * convs * 6 * 2.0 ** -23, opts
 
 
+@pytest.mark.parametrize("name", sorted(STACKS))
+def test_results_do_not_depend_on_what_the_workspace_held(name):
+    """Tiles read around the maps they are about: zeros, NaNs or large values there leave the same bits in every result."""
+    wl = STACKS[name]
+    x, params, target = synth.draw(wl, bias_std=0.1)
+    plan = ftp.ftp_plan(wl.layers, wl.N, wl.C, wl.H, wl.W, wl.grid, wl.groups)
+    xd, pd, td = (torch.from_numpy(a).cuda() for a in (x, params, target))
+    results = []
+    for fill in (0x00, 0xff, 0x7e):                          # 0x7e7e7e7e is 8e37, its halves as bf16 too
+        ws = plan.new_workspace().fill_(fill)
+        y, grad, dx = torch.empty_like(td), torch.empty_like(pd), torch.empty_like(xd)
+        ftp.ftp_forward(plan, xd, pd, y, ws)
+        ftp.ftp_step_grad(plan, xd, pd, grad, ws, target=td, dx=dx)
+        plan.check(ws)
+        results.append((y, grad, dx))
+    for r in results[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(results[0], r))
+
+
 def norm_err(a, o):
     return float(np.linalg.norm((np.asarray(a, np.float64) - o).ravel()) / np.linalg.norm(np.asarray(o).ravel()))
 
