@@ -226,6 +226,26 @@ bool encode_rows_map(unsigned char out[128], const void* base, int N, int planes
     return true;
 }
 
+// Tensor map of bf16 planes of this GPU's memory for the bands of the filter gradient: {columns, rows, planes, images}, or with
+// the planes of a row next to one another {columns, planes, rows, images}; a pixel's 8 channels are two 8-byte elements.
+bool encode_band_map(unsigned char out[128], const void* base, int N, int planes, int H, int W, bool planes_inside, int box_w, int box_h, int box_planes)
+{
+    tensor_map_encode_fn enc = tensor_map_encoder();
+    if (!enc || box_h > 256 || box_w > 128 || box_planes > 256) return false;
+    const int r = planes_inside ? 2 : 1, q = planes_inside ? 1 : 2;              // dimension of the rows / of the planes
+    cuuint64_t dims[4], strides[3]; cuuint32_t box[4]; const cuuint32_t estr[4] = {1, 1, 1, 1};
+    dims[0] = 2 * (cuuint64_t)W; box[0] = 2 * (cuuint32_t)box_w;
+    dims[r] = (cuuint64_t)H; box[r] = (cuuint32_t)box_h; strides[r - 1] = (cuuint64_t)W * 16;
+    dims[q] = (cuuint64_t)planes; box[q] = (cuuint32_t)box_planes; strides[q - 1] = (cuuint64_t)H * W * 16;
+    dims[3] = (cuuint64_t)N; box[3] = 1; strides[2] = (cuuint64_t)planes * H * W * 16;
+    CUtensorMap m;
+    if (enc(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 4, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return false;
+    std::memcpy(out, &m, 128);
+    return true;
+}
+
 // Tensor map of a split map (three parts of bf16 planes, this GPU's memory) as flat planes {entries, planes, parts}, or as rows
 // {columns, rows, planes, parts}; an entry is two 8-byte elements, entries outside read as zeros.
 bool encode_split_map(unsigned char out[128], const uint4* base, const SplitGeom& g, bool rows, int box_x, int box_rows, int box_planes, int box_parts)
@@ -628,9 +648,9 @@ TcReduceLayer reduce_layer(const GroupPlan& g, const OpDesc& op, void* ws)
 {
     if (g.col_cin16)
         return TcReduceLayer{op.p_off, ws_ptr(ws, g.partial_off), (long long)g.param_floats, op.tgp_off, g.sets(), g.col_cin, op.cout, 1,
-                             g.col_cin16, op.cout16, 1};
+                             g.col_cin16, op.cout16, g.tfg.nci};
     return TcReduceLayer{op.p_off, ws_ptr(ws, g.partial_off), (long long)g.set_floats(), op.tgp_off, g.sets(), op.cin, op.cout, op.k,
-                         op.cin16, op.cout16, 1};
+                         op.cin16, op.cout16, g.tfg.on ? g.tfg.nci : 1};
 }
 
 // Sums the partial sets of executed groups [first, last]: whole gradients (grad_out) and / or the update.
@@ -710,19 +730,15 @@ bool tc_filter_grad(ftp_plan* p, const GroupPlan& g, int gi, const TcGroupArgs& 
     }
 
     TcFilterGradArgs f{};
-    for (int cc = 0; cc < t.ncc; ++cc)          // one dz map per column chunk: its columns only, zeros behind them
-        if (!encode_rows_map(f.tmap_dz[cc], dz + (size_t)cc * t.Cw, p->N, op.cout16 / 8, op.in_H, std::min(t.Cw, op.in_W - cc * t.Cw),
-                             op.in_W, t.R, t.Wp))
-            return false;
-    if (!encode_rows_map(f.tmap_x, xin, p->N, cin16 / 8, op.in_H, op.in_W, op.in_W, t.R + t.k - 1, t.Wp)) return false;
-    f.ncc = t.ncc; f.Cw = t.Cw;
+    if (!encode_band_map(f.tmap_dz, dz, p->N, op.cout16 / 8, op.in_H, op.in_W, false, t.Cw, t.R, t.dz_box) ||
+        !encode_band_map(f.tmap_x, xin, p->N, cin16 / 8, op.in_H, op.in_W, true, t.Cw + t.k - 1, t.R + t.k - 1, t.ncols / 8)) return false;
     f.partial = a.partial; f.set_floats = a.set_floats; f.tgp_off = op.tgp_off;
     f.error = a.error;
-    f.N = p->N; f.K = t.k; f.cout16 = op.cout16; f.cin16 = cin16;
-    f.Ms = t.Ms; f.slices = t.slices; f.ncols = t.ncols; f.nci = t.nci;
-    f.R = t.R; f.Wp = t.Wp; f.bands_img = t.bands_img; f.bands = t.bands; f.shares = t.shares;
-    f.dz_plane = t.dz_plane; f.x_plane = t.x_plane; f.stage_bytes = t.stage_bytes;
-    f.hurry = (double)((t.bands + t.shares - 1) / t.shares) * (t.k * t.k + 1) * ((t.R * t.Wp + 15) / 16) * tc_mma_cycles(t.ncols) < kHurryCycles;
+    f.K = t.k; f.H = op.in_H; f.W = op.in_W; f.cout16 = op.cout16; f.cin16 = cin16;
+    f.Ms = t.Ms; f.slices = t.slices; f.ncols = t.ncols; f.nci = t.nci; f.units = t.units;
+    f.R = t.R; f.Cw = t.Cw; f.ncc = t.ncc; f.bands_img = t.bands_img; f.bands = t.bands; f.shares = t.shares;
+    f.dz_box = t.dz_box; f.x_off = t.x_off; f.stage_bytes = t.stage_bytes;
+    f.hurry = t.cycles < kHurryCycles;
     { Timed tm(p, st, 7, gi);
       launch(filter_grad_tc_rows_kernel, t.blocks, kTcFgThreads, one_block_smem(t.smem_bytes), tm.ls(), f); }
     if (!launched_ok()) return false;

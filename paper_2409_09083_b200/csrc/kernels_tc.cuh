@@ -894,7 +894,7 @@ __global__ void halo_sum_planes_kernel(const __grid_constant__ HaloSumArgs A)
 // summed once per batch and the result updates F_l).
 // One layer's slice of the partial sets ([tap][cout16][cin16] filters, then the bias), or a whole group whose sets are arranged
 // like the parameters (cout = k = 1, cin = floats of a set, no bias).
-struct TcReduceLayer { long long p_off; const float* partial; long long set_floats, tgp_off; int sets, cin, cout, k, cin16, cout16, bias; };
+struct TcReduceLayer { long long p_off; const float* partial; long long set_floats, tgp_off; int sets, cin, cout, k, cin16, cout16, bias; };   // bias: its parts in a set (0: none)
 struct TcReduceArgs { int n; TcReduceLayer l[kMaxOps * 2]; };
 
 // 16 loads in flight a thread: with 4 (296 sets of the 896 parameters of an fp32 first layer) the sums were a chain of latencies,
@@ -923,8 +923,10 @@ __global__ void reduce_sgd_tc_kernel(const __grid_constant__ TcReduceArgs A, flo
         }
         const float* src = L.partial + L.tgp_off + e;
         float s = 0.f;
+        for (int part = 0; part < (e < nf ? 1 : L.bias); ++part, src += L.cout16) {
 #pragma unroll 16
-        for (int k = 0; k < L.sets; ++k) s += src[(size_t)k * L.set_floats];
+            for (int k = 0; k < L.sets; ++k) s += src[(size_t)k * L.set_floats];
+        }
         if (grad_out) grad_out[dst] = s;
         if (params) params[dst] = params[dst] - lr * s;
     }

@@ -891,10 +891,11 @@ TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, b
     return c;
 }
 
-// Launch shape of the weight-stationary filter gradient of a one-conv bf16 group (tc_stationary.cuh): slices of
-// Ms output x ncols input channels (all window positions of a slice fit the 512 tensor-memory columns), bands of
-// R rows chosen for the fewest K steps among those whose two stages fit in shared memory, and as many pixel
-// shares as fill the SMs once.
+// Launch shape of the weight-stationary filter gradient of a one-conv bf16 group (tc_stationary.cuh): slices of Ms output x
+// ncols input channels (all window positions of a slice fit the 512 tensor-memory columns), bands of R rows x Cw columns whose two
+// stages fit in shared memory, and pixel shares, at most one round of blocks where the slices leave SMs.  The shape with the
+// least expected time wins: bands of a share x the larger of their MMAs (shared memory delivers 128 bytes a cycle to
+// them) and their copies (22 bytes a cycle and SM from L2), plus writing and reading the partial sets.
 void plan_tc_filter_grad(const ftp_plan& p, GroupPlan& g, const PlanOpts& o)
 {
     g.tfg = TcFgPlan{};
@@ -905,44 +906,46 @@ void plan_tc_filter_grad(const ftp_plan& p, GroupPlan& g, const PlanOpts& o)
     const int col_cin16 = round_up(op.cin * 9, 16);
     const int H = op.in_H, W = op.in_W, K = unrolled ? 1 : op.k;
     const int cin16 = unrolled ? col_cin16 : op.cin16;
-    tc_col_chunks(W, &t.ncc, &t.Cw);
-    t.k = K; t.Wp = t.Cw + K - 1;
+    t.k = K;
     t.Ms = op.cout16 <= 64 ? 64 : 128;
     t.slices = (op.cout16 + t.Ms - 1) / t.Ms;
-    t.ncols = std::min(cin16, K == 1 ? 256 : 48);
-    if (K == 3 && cin16 > 32) {
-        // 48 or 32 input channels a block: the slowest block sets the time, i.e. rounds of blocks over the SMs x the pixels
-        // of a share x the cycles of an MMA that wide (32 + columns / 4: both operands come from shared memory).  32 wins
-        // where 48 leaves a ragged last slice as wide (64 = 48 + 16 against 32 + 32) or too few blocks for the SMs
-        // (512 -> 1024: 88 blocks against 128)
-        double best_cost = -1;
-        for (int nc : {48, 32}) {
-            const long long roles = (long long)t.slices * ((cin16 + nc - 1) / nc);
-            const long long shares = std::max<long long>(1, kSmCount / roles);
-            const double cost = (double)((roles * shares + kSmCount - 1) / kSmCount) / (double)shares * (32.0 + nc / 4.0);
-            if (best_cost < 0 || cost < best_cost) { best_cost = cost; t.ncols = nc; }
-        }
-    }
-    t.nci = (cin16 + t.ncols - 1) / t.ncols;
-    long long best = -1;
-    for (int R = 1; R <= std::min(H, 64); ++R) {
-        const size_t dzp = align_up(((size_t)R * t.Wp + 16) * 16, 128), xp = align_up(((size_t)(R + K - 1) * t.Wp + 32) * 16, 128);
-        const size_t stage = (size_t)(t.Ms / 8) * dzp + (size_t)(t.ncols / 8) * xp;
-        if (kTcFgHeader + 2 * stage > (size_t)kTcFgSmemBudget || R + K - 1 > 256) break;
-        const long long cost = (long long)((H + R - 1) / R) * ((R * t.Wp + 15) / 16 * 16 + 32);
-        if (best < 0 || cost <= best) {
-            best = cost; t.R = R; t.dz_plane = (int)dzp; t.x_plane = (int)xp; t.stage_bytes = (int)stage;
+    t.dz_box = std::min(t.Ms, op.cout16) / 8;
+    double best = -1;
+    for (int most : {256, 48, 32, 16}) {
+        if (K == 3 && most > 48) continue;
+        TcFgPlan c = t;
+        c.nci = (cin16 + most - 1) / most;
+        c.ncols = round_up((cin16 + c.nci - 1) / c.nci, 16);
+        if (c.ncols > most) continue;
+        const int wide = K * c.ncols, roles = c.slices * c.nci, max_g = (128 - (K - 1)) / 8, groups = (W + 7) / 8;
+        c.units = K == 3 || 3 * wide + 16 <= kTcTmemCols ? 3 : 1;
+        const double operands = (c.Ms + wide) * 32.0 / 128.0, mma = (K == 3 ? 3.0 : 1.0) * std::max(wide / 2.0, operands) + (c.Ms + 16) * 0.25 / c.nci;
+        const double set_cost = (double)(K * K * cin16 + 1) * op.cout16 * 8.0 / 5e6 * 1900.0;
+        for (int ncc = (groups + max_g - 1) / max_g, end = ncc + 4; ncc <= std::min(groups, end); ++ncc) {
+            c.Cw = (groups + ncc - 1) / ncc * 8;
+            c.ncc = (W + c.Cw - 1) / c.Cw;
+            for (c.R = 2; c.R <= std::min(round_up(H, 2), 64); c.R += 2) {
+                c.x_off = (int)align_up((size_t)(c.Ms / 8) * c.R * c.Cw * 16, 128);
+                const size_t xb = (size_t)(c.ncols / 8) * (c.R + K - 1) * (c.Cw + K - 1) * 16;
+                c.stage_bytes = (int)align_up((size_t)c.x_off + xb, 128);
+                c.smem_bytes = kTcFgHeader + 2 * c.stage_bytes;
+                if (c.smem_bytes > kTcFgSmemBudget) break;
+                c.bands_img = (H + c.R - 1) / c.R * c.ncc;
+                const long long bands = (long long)p.N * c.bands_img;
+                if (bands > 0x7fffffffLL) continue;
+                c.bands = (int)bands;
+                const double steps = (double)((H + 1) / 2) * groups / c.bands_img;            // K steps of an average band
+                const double band = std::max(steps * mma, ((double)c.dz_box * c.R * c.Cw * 16.0 + xb) / 22.0) + 300.0;
+                for (c.shares = (int)std::max<long long>(1, std::min<long long>(bands, kSmCount / roles)); c.shares >= 1; c.shares = c.shares * 3 / 4) {
+                    c.cycles = (double)((roles * c.shares + kSmCount - 1) / kSmCount) * ((bands + c.shares - 1) / c.shares * band + 6000.0);
+                    const double cost = c.cycles + c.shares * set_cost;
+                    if (best < 0 || cost < best) { best = cost; t = c; }
+                }
+            }
         }
     }
     if (best < 0) return;
-    t.smem_bytes = kTcFgHeader + 2 * t.stage_bytes;
-    t.bands_img = (H + t.R - 1) / t.R * t.ncc;
-    const long long bands = (long long)p.N * t.bands_img;
-    if (bands > 0x7fffffffLL) return;
-    t.bands = (int)bands;
-    const int roles = t.slices * t.nci;
-    t.shares = (int)std::max<long long>(1, std::min<long long>(bands, kSmCount / roles));
-    t.blocks = roles * t.shares;
+    t.blocks = t.slices * t.nci * t.shares;
     // the forward convolution, and the input delta as the convolution of dz (cout16 channels) with the rotated filters
     g.cf = plan_tc_conv(p.N, H, W, K, cin16, op.cout16, op.kind == kOpConvPool);
     g.cd = plan_tc_conv(p.N, H, W, K, op.cout16, cin16, false);
@@ -950,6 +953,7 @@ void plan_tc_filter_grad(const ftp_plan& p, GroupPlan& g, const PlanOpts& o)
     if (unrolled) { g.col_cin = op.cin * 9; g.col_cin16 = col_cin16; }
     t.on = 1;
     g.tfg = t;
+    g.param_floats += (size_t)(t.nci - 1) * op.cout16;          // the bias gradient comes in parts, one per slice of the input channels
     g.bwd.scratch_floats = 0;       // no per-sub-tile input deltas
 }
 

@@ -133,13 +133,15 @@ struct TcFgPlan {
     int on = 0;
     int k = 0, Ms = 0, slices = 0;          // output channels per block (64 or 128), number of slices
     int ncols = 0, nci = 0;                 // input channels per block (multiple of 16), number of slices
-    int R = 0, Wp = 0;                      // rows of a band, pitch of its tiles (Cw + k - 1)
-    int ncc = 1, Cw = 0;                    // column chunks of a row band (maps wider than 126 pixels) and their width
+    int units = 1;                          // accumulator units (see TcFilterGradArgs)
+    int R = 0;                              // rows of a band (even)
+    int ncc = 1, Cw = 0;                    // column chunks of a row band and their width (a multiple of 8)
     int bands_img = 0, bands = 0;           // bands per image and in the batch
     int shares = 0;                         // pixel shares = partial gradient sets of the group
     int blocks = 0;                         // slices * nci * shares
-    int dz_plane = 0, x_plane = 0;          // bytes between the planes of the two tiles
+    int dz_box = 0, x_off = 0;              // planes of a dz copy, bytes before the input tile
     int stage_bytes = 0, smem_bytes = 0;
+    double cycles = 0;                      // what the planner expects a block to take
 };
 // Banded tensor-core convolution of a one-conv bf16 group (conv_tc_rows_kernel): forward pass and input delta.
 struct TcConvPlan {
@@ -160,7 +162,7 @@ constexpr int kTcPoolStageBytes = 32 * 1024;  // least staging area of the fused
 constexpr int kTcConvSmemBudget = 224 * 1024; // banded convolution: header + stages + pool staging
 constexpr int kTcMaxColChunks = 8;            // a band spans at most 126 columns (a TMA box row of 128 pixels with the halo): wider maps are cut into chunks
 constexpr int kTcFgHeader = 1024;             // barriers, tensor-memory slot, a core matrix of ones
-constexpr int kTcFgSmemBudget = 200 * 1024;   // header + two stages
+constexpr int kTcFgSmemBudget = 224 * 1024;   // header + two stages
 
 // Tensor-core cycles of one MMA with N accumulator columns and both operands in shared memory (M = 128, K = 16)
 inline double tc_mma_cycles(int n) { return n < 128 ? 32.0 + n / 4.0 : n / 2.0; }

@@ -6,19 +6,25 @@
 // the block's partial set, because tensor memory cannot keep the accumulators of a wide layer across sub-tiles.
 // For layers with hundreds of channels that flush costs several times the MMAs.  Here the roles are turned
 // round: a block owns a slice of the FILTER GRADIENT (64 or 128 output channels x up to 48 input channels x all
-// window positions; K*K accumulators of `ncols` columns each, plus 16 columns for the bias gradient) and keeps
+// window positions; plus 16 columns for the bias gradient) and keeps
 // it in tensor memory while bands of rows of the whole batch stream past it, so the gradient leaves the SM
 // once.  The pixels are dealt out in `shares`; a share is one partial gradient set of Section 4.1, summed by
 // the same cross-tile reduction as the sets of the fused kernels.
 //
-// A band is R rows x Cw columns (Cw = W, or a column chunk of at most 126 columns of a wider map) of one image at
-// the conv's resolution.  The delta in front of the activation (dz, bf16 planes, written by the input-delta
-// kernel of the layer above or by delta_act_planes_kernel) and the layer's saved input map arrive by TMA tensor
-// copies into tiles of the same pitch Wp = Cw + K - 1: dz at columns 0 .. Cw-1 with zeros behind them (beyond
-// the edge of the chunk's tensor map), the input shifted by the padding.  With equal pitches one run of 16 consecutive tile entries
-// is a K step of both operands (MN-major, 8 pixels x 8 channels per core matrix), and window position (ky, kx)
-// only moves the start of the input operand by ky * Wp + kx entries.  Two stages: the copies of the next band
-// run behind the MMAs of the current one.
+// A band is R rows (even) x Cw columns (a multiple of 8, at most 128 tile entries with the halo) of one image at the conv's
+// resolution.  The delta in front of the activation (dz, bf16 planes, written by the input-delta kernel of the layer above or by
+// delta_act_planes_kernel) arrives by one TMA copy as [plane][row][Cw entries], the layer's saved input by another as
+// [row][plane][Cw + K - 1 entries] with its halo; what lies outside the map arrives as zeros.  Both operands are MN-major (8
+// pixels x 8 channels per core matrix).  A K step of 16 pixels is 8 pixels of a row and the 8 below them, so that only a width that
+// no multiple of 8 covers is padded (38 columns: 40 instead of the 48 of 16 pixels in a row).  Because the planes of a
+// row of the input lie between it and the next row, the 8-channel groups (window row ky, plane p) of ONE window column stand at one
+// stride: an MMA covers the three window rows of its column, K * ncols accumulator columns, and the window column moves the
+// start by an entry.  With one MMA per window position instead (48 columns each, both operands from shared memory) an MMA took
+// the 44 cycles in which shared memory delivers 5.5 KB, for 24 cycles of arithmetic, and dz was read nine times
+// for a K step; 144 columns take 72 cycles and dz is read three times.  Now the copies bound it: 93 KB a band at 20 bytes a cycle
+// and SM.  us before and after: 256 -> 512, 16 x 38 x 38: 97 -> 66 (826 TFLOP/s); 128 -> 256, 76 x 76: 81 -> 60; 64 -> 128,
+// 152 x 152: 91 -> 52; 32 -> 64, 304 x 304: 112 -> 76; 256 -> 512 on 8 x 13 x 13: 40 -> 26; 1x1 512 -> 256: 29 -> 21.
+// Two stages (copies of the next band behind the MMAs of this one).
 #pragma once
 
 #include <algorithm>
@@ -31,20 +37,19 @@ namespace ftp {
 // eight-byte elements (a pixel's 8 channels = two elements), so that a box row is one contiguous run of Wp pixels
 // instead of Wp separate 16-byte pieces; a box row holds at most 256 elements, i.e. Wp <= 128 pixels.
 struct TcFilterGradArgs {
-    // dz planes, one map per column chunk: the chunk's columns only (base moved to its first column, extent = its
-    // width), so that the box (Wp pixels x R rows) reads zeros behind the chunk's last column
-    alignas(64) unsigned char tmap_dz[kTcMaxColChunks][128];
-    alignas(64) unsigned char tmap_x[128];    // the layer's input planes, box = Wp pixels x (R + K - 1) rows
+    alignas(64) unsigned char tmap_dz[128];   // dz as {columns, rows, planes, images}: box = Cw columns x R rows x dz_box planes
+    alignas(64) unsigned char tmap_x[128];    // the layer's input as {columns, planes, rows, images}: box = (Cw + K - 1) x ncols / 8 x (R + K - 1)
     float* partial;                           // partial sets of the group
     long long set_floats, tgp_off;            // floats per set, offset of this layer inside a set
     int* error;
     int hurry;                                // a short launch: see kHurryCycles in launch.cuh
-    int N, K, cout16, cin16;
+    int K, H, W, cout16, cin16;
     int Ms, slices;                           // output channels per block (64 or 128) and number of such slices
     int ncols, nci;                           // input channels per block (multiple of 16) and number of such slices
-    int R, Wp, bands_img, bands, shares;      // rows per band, tile pitch, bands per image / in the batch, pixel shares
-    int ncc, Cw;                              // column chunks per row band and their width (Wp = Cw + K - 1)
-    int dz_plane, x_plane, stage_bytes;       // bytes between planes of the two tiles, bytes of one stage
+    int units;                                // accumulator units of K * ncols columns: 3x3: one per window column; 1x1: row pairs in turn
+    int R, Cw, ncc;                           // rows per band, columns of a band and column chunks per row band
+    int bands_img, bands, shares;             // bands per image / in the batch, pixel shares
+    int dz_box, x_off, stage_bytes;           // dz planes a copy brings, offset of the input tile in a stage, bytes of a stage
 };
 
 struct DeltaActPlanesArgs {
@@ -211,12 +216,10 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
     const int nroles = A.slices * A.nci;
     const int role = (int)blockIdx.x % nroles, share = (int)blockIdx.x / nroles;
     const int slice = role / A.nci, cs = role - slice * A.nci;
-    const int ci0 = cs * A.ncols, cols = min(A.ncols, A.cin16 - ci0);
-    const int mp = A.Ms / 8;                                            // dz planes of a full slice
-    const int nd = min(mp, A.cout16 / 8 - slice * mp), np = cols / 8;   // planes this block copies per band
-    const bool bias = cs == 0;
+    const int ci0 = cs * A.ncols, cols = min(A.ncols, A.cin16 - ci0), wide = K * A.ncols;
     const int b_lo = (int)((long long)share * A.bands / A.shares), b_hi = (int)((long long)(share + 1) * A.bands / A.shares);
     const int nb = b_hi - b_lo;
+    const int np = A.ncols / 8, Wx = A.Cw + K - 1;                       // planes and row pitch of the input tile
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&H->full[s]), 1); mbar_init(smem_u32(&H->empty[s]), kTcIssuers); }
@@ -225,8 +228,6 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
         fence_mbar_init();
     }
     if (warp == 0) { __syncwarp(); tmem_alloc(smem_u32(&H->tmem_base), (uint32_t)kTcTmemCols); }
-    // tails, planes that are never copied and everything else the tensor core may read: zeros from here on
-    tcd::zero_bytes(stages, 2 * (size_t)A.stage_bytes);
     for (int i = threadIdx.x; i < 64; i += blockDim.x) H->ones[i] = __float2bfloat16(1.0f);
     fence_async_smem();
     fence_before_sync();
@@ -246,54 +247,64 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
         if (threadIdx.x == 0) { H->failed = 1; atomicExch(A.error, 1); }
         __syncthreads();
     }
+    // image and origin of band b of the batch
+    auto band_of = [&](int b, int& n, int& y0, int& x0) {
+        n = b / A.bands_img;
+        const int bi = b - n * A.bands_img, rb = bi / A.ncc;
+        y0 = rb * A.R; x0 = (bi - rb * A.ncc) * A.Cw;
+    };
+    auto pairs_of = [&](int y0) { return (min(A.R, A.H - y0) + 1) >> 1; };       // row pairs with pixels
 
     if (warp == kTcIssuers && lane == 0) {
-        // producer: the two tiles of a band, one tensor copy per plane
+        // producer: the two tiles of a band, one tensor copy each
         int issued[2] = {0, 0};
         for (int i = 0; i < nb; ++i) {
             const int s = i & 1;
             if (!wait(&H->empty[s], ((uint32_t)(i >> 1) & 1u) ^ 1u)) break;
-            const int b = b_lo + i, n = b / A.bands_img, bi = b - n * A.bands_img;
-            const int cc = bi % A.ncc, y0 = (bi / A.ncc) * A.R, x0 = cc * A.Cw;
-            unsigned char* dzs = stages + (size_t)s * A.stage_bytes;
-            unsigned char* xs = dzs + (size_t)mp * A.dz_plane;
-            const uint32_t bar = smem_u32(&H->full[s]);
-            mbar_expect_tx(bar, (uint32_t)((nd * A.R + np * (A.R + K - 1)) * A.Wp) * 16u);
-            for (int pl = 0; pl < nd; ++pl)
-                tma_load_3d(smem_u32(dzs + (size_t)pl * A.dz_plane), A.tmap_dz[cc], 0, y0, n * (A.cout16 / 8) + slice * mp + pl, bar);
-            for (int pl = 0; pl < np; ++pl)
-                tma_load_3d(smem_u32(xs + (size_t)pl * A.x_plane), A.tmap_x, 2 * (x0 - K / 2), y0 - K / 2, n * (A.cin16 / 8) + ci0 / 8 + pl, bar);
+            int n, y0, x0;
+            band_of(b_lo + i, n, y0, x0);
+            const uint32_t dst = smem_u32(stages + (size_t)s * A.stage_bytes), bar = smem_u32(&H->full[s]);
+            mbar_expect_tx(bar, (uint32_t)(A.dz_box * A.R * A.Cw + np * (A.R + K - 1) * Wx) * 16u);
+            tma_load_4d(dst, A.tmap_dz, 2 * x0, y0, slice * (A.Ms / 8), n, bar);
+            tma_load_4d(dst + (uint32_t)A.x_off, A.tmap_x, 2 * (x0 - K / 2), ci0 / 8, y0 - K / 2, n, bar);
             ++issued[s];
         }
         if (H->failed)       // gave up somewhere: let the copies already under way land before the block leaves
             for (int s = 0; s < 2; ++s)
                 if (issued[s] > 0) mbar_wait(smem_u32(&H->full[s]), (uint32_t)(issued[s] - 1) & 1u, 200000000ll);
     } else if (warp < kTcIssuers && lane == 0) {
-        // MMA issue: every issuer takes every kTcIssuers-th accumulator (window positions, then the bias)
-        const uint32_t a_hi = desc_hi((uint32_t)A.dz_plane), x_hi = desc_hi((uint32_t)A.x_plane);
-        const uint32_t idesc = make_idesc(A.Ms, cols, true, true), idb = make_idesc(A.Ms, 16, true, true);
-        const uint64_t ones_d = make_desc(smem_u32(H->ones), 0, 0);
-        const int nunits = KK + (bias ? 1 : 0);
-        const int nk = (A.R * A.Wp + 15) >> 4;
+        // MMA issue: issuers 0 .. units - 1 an accumulator unit each, the last one the bias gradient (dz against ones).
+        // A block takes the bias of every nci-th row pair, so that the blocks of a share, one per slice of the input channels,
+        // have the same work; the reduction adds their parts.
+        const bool is_bias = warp == kTcIssuers - 1;
+        const uint32_t a_hi = desc_hi((uint32_t)(A.R * A.Cw) * 16u), x_hi = is_bias ? desc_hi(0) : desc_hi((uint32_t)Wx * 16u);
+        const uint32_t idesc = make_idesc(A.Ms, is_bias ? 16 : wide, true, true);
+        const uint32_t col = tmem + (uint32_t)((is_bias ? A.units : warp) * wide);
+        const uint32_t a_pair = 2u * (uint32_t)A.Cw, x_pair = is_bias ? 0u : 2u * (uint32_t)(np * Wx), x_step = is_bias ? 0u : 8u;
+        const int every = is_bias ? A.nci : K == 1 ? A.units : 1, first = is_bias ? cs : K == 1 ? warp : 0;
+        bool acc = false;
+        int turn = first;                                    // row pairs until this issuer's next one
         for (int i = 0; i < nb; ++i) {
             const int s = i & 1;
             if (!wait(&H->full[s], (uint32_t)(i >> 1) & 1u)) break;
             fence_after_sync();
-            const uint32_t dz_addr = smem_u32(stages + (size_t)s * A.stage_bytes);
-            const uint32_t dz_lo0 = desc_lo(dz_addr, 128), x_lo0 = desc_lo(dz_addr + (uint32_t)(mp * A.dz_plane), 128);
-            for (int u = warp; u < nunits; u += kTcIssuers) {
-                uint32_t a_lo = dz_lo0;
-                if (u < KK) {
-                    const int ky = u / K, kx = u - ky * K;
-                    uint32_t x_lo = x_lo0 + (uint32_t)(ky * A.Wp + kx);
-                    const uint32_t col = tmem + (uint32_t)(u * A.ncols);
-                    for (int ks = 0; ks < nk; ++ks) {
-                        mma_bf16(col, desc64(a_hi, a_lo), desc64(x_hi, x_lo), idesc, (i | ks) != 0);
-                        a_lo += 16; x_lo += 16;
+            if (is_bias || warp < A.units) {
+                int n, y0, x0;
+                band_of(b_lo + i, n, y0, x0);
+                const uint32_t dst = smem_u32(stages + (size_t)s * A.stage_bytes);
+                uint32_t ar = desc_lo(dst, (uint32_t)A.Cw * 16u);
+                uint32_t xr = is_bias ? desc_lo(smem_u32(H->ones), 0)
+                                      : desc_lo(dst + (uint32_t)A.x_off, (uint32_t)(np * Wx) * 16u) + (K == 3 ? (uint32_t)warp : 0u);
+                const int pairs = pairs_of(y0), groups = (min(A.Cw, A.W - x0) + 7) >> 3;
+                for (int r = 0; r < pairs; ++r, ar += a_pair, xr += x_pair) {
+                    if (turn > 0) { --turn; continue; }
+                    turn = every - 1;
+                    uint32_t a = ar, x = xr;
+#pragma unroll 4
+                    for (int g = 0; g < groups; ++g, a += 8u, x += x_step) {
+                        mma_bf16(col, desc64(a_hi, a), desc64(x_hi, x), idesc, acc);
+                        acc = true;
                     }
-                } else {
-                    const uint32_t col = tmem + (uint32_t)(KK * A.ncols);
-                    for (int ks = 0; ks < nk; ++ks) { mma_bf16(col, desc64(a_hi, a_lo), ones_d, idb, (i | ks) != 0); a_lo += 16; }
                 }
             }
             mma_commit(smem_u32(&H->empty[s]));
@@ -307,20 +318,34 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
 
     if (A.hurry) next_launch();
 
+    // what a block of few row pairs never touched: units and the bias beyond the number of its pairs
+    int pairs = 0;
+    for (int i = 0; i < nb && pairs <= max(A.units, cs); ++i) {
+        int n, y0, x0;
+        band_of(b_lo + i, n, y0, x0);
+        pairs += pairs_of(y0);
+    }
+    const int used = !have ? 0 : K == 3 ? 1 : min(A.units, pairs);
+
     // tensor memory -> this share's partial set; lane quarter q holds rows 32q.. (Ms = 128) or rows 16q.. in its
     // first 16 lanes (Ms = 64).  The slices of the blocks are disjoint: plain stores.
     const int q = warp & 3, half = warp >> 2;
     const int row = A.Ms == 128 ? q * 32 + lane : q * 16 + lane;
     const bool row_ok = (A.Ms == 128 || lane < 16) && slice * A.Ms + row < A.cout16;
     const int co = slice * A.Ms + row;
+    const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16);
     float* gset = A.partial + (size_t)share * A.set_floats + A.tgp_off;
-    for (int u = 0; u < KK; ++u)
+    for (int u = 0; u < KK; ++u) {
+        const int ky = u / K, kx = u - ky * K;
         for (int c0 = half * 16; c0 < cols; c0 += 32) {
             float v[16];
-            if (have) tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(u * A.ncols + c0), v);
-            else {
 #pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] = 0.f;
+            for (int j = 0; j < 16; ++j) v[j] = 0.f;
+            for (int w = 0; w < used; ++w) {
+                float t[16];
+                tmem_ld16(tq + (uint32_t)((kx + w) * wide + ky * A.ncols + c0), t);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] = w ? v[j] + t[j] : t[j];
             }
             if (row_ok) {
                 float* g = gset + ((size_t)u * A.cout16 + co) * A.cin16 + ci0 + c0;
@@ -329,11 +354,12 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
                     *reinterpret_cast<float4*>(g + 4 * j) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             }
         }
-    if (bias && half == 0) {
+    }
+    if (half == 0) {
         float v[16];
-        if (have) tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(KK * A.ncols), v);
-        else v[0] = 0.f;
-        if (row_ok) gset[(size_t)KK * A.cout16 * A.cin16 + co] = v[0];
+        v[0] = 0.f;
+        if (have && pairs > cs) tmem_ld16(tq + (uint32_t)(A.units * wide), v);
+        if (row_ok) gset[(size_t)KK * A.cout16 * A.cin16 + (size_t)cs * A.cout16 + co] = v[0];
     }
     fence_before_sync();
     __syncthreads();

@@ -529,3 +529,28 @@ def test_tma_and_thread_copies_of_the_tiles_give_the_same_bits():
     b = backward_bf16(wl, x, params, dy, tc_tma=-1)
     for u, v in zip(a[:3], b[:3]):
         assert np.array_equal(u, v)
+
+
+# (input channels, output channels, window, N, H, W) of the second of two conv layers: slices of 48 and 32 input channels and of the
+# output channels with a remainder, fewer row pairs than slices and units, odd heights, one row, one column, widths beside
+# a multiple of 8 and beside a column chunk, 1x1 windows with one and with three accumulator units
+FILTER_GRAD = [(16, 16, 3, 1, 1, 1), (32, 64, 3, 2, 13, 13), (64, 48, 3, 1, 5, 121), (80, 144, 3, 3, 7, 9), (128, 80, 3, 1, 2, 38),
+               (208, 128, 3, 2, 3, 8), (48, 130, 3, 1, 33, 250), (40, 24, 1, 1, 1, 7), (160, 64, 1, 2, 9, 129), (176, 144, 1, 1, 5, 17),
+               (320, 128, 1, 3, 3, 4)]
+
+
+@pytest.mark.parametrize("cin,cout,k,n,h,w", FILTER_GRAD)
+def test_filter_gradient_at_the_edges_of_its_slices_and_bands(cin, cout, k, n, h, w):
+    """Against the fp64 oracle on the same stored maps, without decisions (slope 1): delta and map enter as bf16 (2^-9 of a value
+    each), the sums are fp32, so an element of the gradient is within 2^-8 of its sum of magnitudes; 1e-2 of the largest element
+    is what the tests above use."""
+    layers = (conv(3, cin, 3, leaky=1.0), conv(cin, cout, k, leaky=1.0))
+    wl = W("fg", layers, n, 3, h, w, (1, 1), ((1, 1), (2, 2)), x_dist="normal")
+    x, params, target = synth.draw(wl, bias_std=0.3)
+    x, params = bf16_grid(x), bf16_grid(params)
+    dy = bf16_grid(np.random.default_rng(7).standard_normal(target.shape))
+    ref = run_oracle(wl, x, params, dy=dy, store="bf16")
+    _, _, dparams, plan = backward_bf16(wl, x, params, dy)
+    errors = per_layer_errors(list(layers), dparams, ref["dparams"])
+    print(plan.exec_groups(), errors)
+    assert len(errors) == 2 and all(max(e[1:]) <= 1e-2 for e in errors)
