@@ -660,7 +660,7 @@ int reduce_groups(ftp_plan* p, int first, int last, float* sgd_params, float lr,
     auto flush = [&]() {
         if (!ra.n) return;
         Timed t(p, st, 5, timed_group);
-        launch(reduce_sgd_tc_kernel, dim3(1184, ra.n), 128, 0, t.ls(), ra, sgd_params, lr, grad_out);
+        launch_reduce(ra, sgd_params, lr, grad_out, t.ls());
         ra.n = 0;
     };
     for (int gi = first; gi <= last; ++gi) {

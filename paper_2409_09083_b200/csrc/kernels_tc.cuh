@@ -894,42 +894,154 @@ __global__ void halo_sum_planes_kernel(const __grid_constant__ HaloSumArgs A)
 // summed once per batch and the result updates F_l).
 // One layer's slice of the partial sets ([tap][cout16][cin16] filters, then the bias), or a whole group whose sets are arranged
 // like the parameters (cout = k = 1, cin = floats of a set, no bias).
-struct TcReduceLayer { long long p_off; const float* partial; long long set_floats, tgp_off; int sets, cin, cout, k, cin16, cout16, bias; };   // bias: its parts in a set (0: none)
+struct TcReduceLayer {
+    long long p_off; const float* partial; long long set_floats, tgp_off;
+    int sets, cin, cout, k, cin16, cout16, bias;      // bias: its parts in a set (0: none)
+    int tile_begin, filter_tiles, quads;              // tiles of a launch: first tile of the layer, its tiles of filters, their size and form (see launch_reduce)
+};
 struct TcReduceArgs { int n; TcReduceLayer l[kMaxOps * 2]; };
+constexpr int kReduceThreads = 288;                   // a warp per window position
 
-// 16 loads in flight a thread: with 4 (296 sets of the 896 parameters of an fp32 first layer) the sums were a chain of latencies,
-// 52 us of an 8-layer step, now 27 us.  Measured and dropped: 3x3 tiles that leave through shared memory as contiguous runs of the
-// parameters, with the sets dealt out to warps or with several tiles a block (73-140 us on a 16-layer stack, this 75 us).
-__global__ void reduce_sgd_tc_kernel(const __grid_constant__ TcReduceArgs A, float* __restrict__ params, float lr,
-                                     float* __restrict__ grad_out)
+// Sums of the sets for 3x3 filters without padded input channels: Q x 128 consecutive filters (output channel, input channel) x 9
+// window positions.  A set has them as 9 runs, read 16 bytes a thread; parameters and gradient are one run of 9 floats a filter; the
+// sums change places in shared memory (a word of padding after the 36 of a thread: no bank conflicts).
+template <int Q>
+__device__ __forceinline__ void reduce_filter_tile(const TcReduceLayer& L, int t, float* s, float* __restrict__ params, float lr, float* __restrict__ grad_out)
+{
+    const int tap = threadIdx.x >> 5, lane = threadIdx.x & 31, f0 = t * Q * 128, left = L.cout * L.cin - f0;
+    const int run = min(Q * 128, left) * 9;
+    const long long dst = L.p_off + (long long)f0 * 9;
+    float p[4 * Q];
+#pragma unroll
+    for (int i = 0; i < 4 * Q; ++i) {
+        const int j = i * kReduceThreads + (int)threadIdx.x;
+        p[i] = (params && j < run) ? params[dst + j] : 0.f;
+    }
+    const float4* src = reinterpret_cast<const float4*>(L.partial + L.tgp_off + (long long)tap * L.cout16 * L.cin16 + f0) + lane;
+    const long long step = L.set_floats / 4;
+    float4 v[Q];
+    bool in[Q];                                       // (a set holds whole rows of filters: 16 bytes are inside)
+#pragma unroll
+    for (int q = 0; q < Q; ++q) { v[q] = make_float4(0.f, 0.f, 0.f, 0.f); in[q] = q * 128 + lane * 4 < left; }
+#pragma unroll 4
+    for (int k = 0; k < L.sets; ++k)
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+            if (in[q]) {
+                const float4 a = src[k * step + q * 32];
+                v[q].x += a.x; v[q].y += a.y; v[q].z += a.z; v[q].w += a.w;
+            }
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        float* d = s + (q * 32 + lane) * 37 + tap;
+        d[0] = v[q].x; d[9] = v[q].y; d[18] = v[q].z; d[27] = v[q].w;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4 * Q; ++i) {
+        const int j = i * kReduceThreads + (int)threadIdx.x;
+        if (j >= run) break;
+        const float sum = s[j + j / 36];
+        if (grad_out) grad_out[dst + j] = sum;
+        if (params) params[dst + j] = p[i] - lr * sum;
+    }
+}
+
+// The same for layers of many sets, 288 values a tile (32 filters of 3x3, or 288 of 1x1, which need no exchange): every fourth set
+// to one of four lanes, whose sums are added in a fixed order, so that the chain of loads is a quarter as long.
+__device__ __forceinline__ void reduce_split_tile(const TcReduceLayer& L, int t, float* s, float* __restrict__ params, float lr, float* __restrict__ grad_out)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, part = lane >> 3, l4 = (lane & 7) * 4, j = threadIdx.x;
+    const bool k3 = L.k == 3;
+    const int at = k3 ? t * 32 + l4 : t * kReduceThreads + warp * 32 + l4, count = L.cout * L.cin, left = count * L.k * L.k - t * kReduceThreads;
+    const long long dst = L.p_off + (long long)t * kReduceThreads + j;
+    const float p = (params && j < left) ? params[dst] : 0.f;
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    if (at < count) {
+        const float4* src = reinterpret_cast<const float4*>(L.partial + L.tgp_off + (k3 ? (long long)warp * L.cout16 * L.cin16 : 0ll) + at);
+        const long long step = L.set_floats / 4;
+#pragma unroll 10
+        for (int k = part; k < L.sets; k += 4) {
+            const float4 a = src[k * step];
+            v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        v[i] += __shfl_xor_sync(0xffffffffu, v[i], 8);
+        v[i] += __shfl_xor_sync(0xffffffffu, v[i], 16);
+        if (part == 0) s[k3 ? (l4 + i) * 9 + warp : warp * 32 + l4 + i] = v[i];
+    }
+    __syncthreads();
+    if (j >= left) return;
+    const float sum = s[j];
+    if (grad_out) grad_out[dst] = sum;
+    if (params) params[dst] = p - lr * sum;
+}
+
+// Bound: DRAM, the sets once, the parameters once each way.  One thread per value, with a scattered write at a stride of 36 bytes, was
+// bound by L2 sectors (a sector each for the read and the write of a parameter): 178 -> 113 us on the
+// 23-layer stack (sets and parameters: 442 MB), 88 -> 66 on the 16-layer one (259 MB), 24 -> 19 on the 8-layer one.  16 loads in flight a thread: with 4
+// (296 sets of the 896 parameters of an fp32 first layer) the sums were a chain of latencies, 52 us of an 8-layer step,
+// with 16 27 us.
+__global__ void __launch_bounds__(kReduceThreads) reduce_sgd_tc_kernel(const __grid_constant__ TcReduceArgs A, float* __restrict__ params, float lr,
+                                                                       float* __restrict__ grad_out)
 {
     previous_launches();
-    // Threads walk the set's own arrangement, so the reads of every set are coalesced (the sets are the
-    // bulk of the traffic); the one write per parameter goes to its place in the caller's arrangement.
-    const TcReduceLayer L = A.l[blockIdx.y];
-    const int KK = L.k * L.k;
-    const long long nf = (long long)KK * L.cout16 * L.cin16, total = nf + (L.bias ? L.cout16 : 0);
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
-        long long dst;
-        if (e < nf) {
-            const int ci = (int)(e % L.cin16); long long t = e / L.cin16;
-            const int co = (int)(t % L.cout16); const int tap = (int)(t / L.cout16);
-            if (ci >= L.cin || co >= L.cout) continue;
-            dst = L.p_off + ((long long)co * L.cin + ci) * KK + tap;
-        } else {
-            const int co = (int)(e - nf);
-            if (co >= L.cout) continue;
-            dst = L.p_off + (long long)L.cout * L.cin * KK + co;
-        }
-        const float* src = L.partial + L.tgp_off + e;
-        float s = 0.f;
-        for (int part = 0; part < (e < nf ? 1 : L.bias); ++part, src += L.cout16) {
-#pragma unroll 16
-            for (int k = 0; k < L.sets; ++k) s += src[(size_t)k * L.set_floats];
-        }
-        if (grad_out) grad_out[dst] = s;
-        if (params) params[dst] = params[dst] - lr * s;
+    __shared__ float s[2 * 32 * 37];
+    int l = 0;
+    while (l + 1 < A.n && (int)blockIdx.x >= A.l[l + 1].tile_begin) ++l;
+    const TcReduceLayer L = A.l[l];
+    const int t = (int)blockIdx.x - L.tile_begin;
+    if (t < L.filter_tiles) {
+        if (L.quads == 0) reduce_split_tile(L, t, s, params, lr, grad_out);
+        else if (L.quads == 2) reduce_filter_tile<2>(L, t, s, params, lr, grad_out);
+        else reduce_filter_tile<1>(L, t, s, params, lr, grad_out);
+        return;
     }
+    // 1x1 filters, sets arranged like the parameters, and biases: one thread per value, in the set's arrangement
+    const long long nf = (long long)L.k * L.k * L.cout16 * L.cin16, total = nf + (L.bias ? L.cout16 : 0);
+    const long long e = (L.filter_tiles ? nf : 0) + (long long)(t - L.filter_tiles) * kReduceThreads + threadIdx.x;
+    if (e >= total) return;
+    long long dst;
+    int parts = 1;
+    if (e < nf) {
+        const int ci = (int)(e % L.cin16), co = (int)(e / L.cin16 % L.cout16), tap = (int)(e / L.cin16 / L.cout16);
+        if (ci >= L.cin || co >= L.cout) return;
+        dst = L.p_off + ((long long)co * L.cin + ci) * L.k * L.k + tap;
+    } else {
+        const int co = (int)(e - nf);
+        if (co >= L.cout) return;
+        dst = L.p_off + (long long)L.cout * L.cin * L.k * L.k + co;
+        parts = L.bias;
+    }
+    const float* src = L.partial + L.tgp_off + e;
+    float sum = 0.f;
+    for (int part = 0; part < parts; ++part, src += L.cout16) {
+#pragma unroll 16
+        for (int k = 0; k < L.sets; ++k) sum += src[(size_t)k * L.set_floats];
+    }
+    if (grad_out) grad_out[dst] = sum;
+    if (params) params[dst] = params[dst] - lr * sum;
+}
+
+// Deals the layers of `a` out in tiles and launches the reduction.
+inline void launch_reduce(TcReduceArgs& a, float* params, float lr, float* grad_out, LaunchStream st)
+{
+    long long tiles = 0;
+    for (int i = 0; i < a.n; ++i) {
+        TcReduceLayer& L = a.l[i];
+        // filters in tiles where their sets are arranged without padding; those of more than 16 sets with the sets shared out
+        const bool plain = L.cin == L.cin16 && L.set_floats % 4 == 0 && (long long)L.cout * L.cin < (1ll << 27), many = L.sets > 16;
+        const bool filters = plain && (L.k == 3 || (L.k == 1 && many && L.bias));
+        const int count = filters ? L.cout * L.cin : 0, one = (count + 127) / 128;
+        L.tile_begin = (int)tiles;
+        L.quads = many ? 0 : one >= 2048 ? 2 : 1;     // (256 filters a tile only where 128 are several rounds of blocks)
+        L.filter_tiles = many ? (count * L.k * L.k + kReduceThreads - 1) / kReduceThreads : (one + L.quads - 1) / L.quads;
+        const long long rest = (filters ? 0 : (long long)L.k * L.k * L.cout16 * L.cin16) + (L.bias ? L.cout16 : 0);
+        tiles += L.filter_tiles + (rest + kReduceThreads - 1) / kReduceThreads;
+    }
+    launch(reduce_sgd_tc_kernel, dim3((unsigned)tiles), kReduceThreads, 0, st, a, params, lr, grad_out);
 }
 
 // fp32 NCHW view of a saved bf16 map (the network output handed back to the caller).
