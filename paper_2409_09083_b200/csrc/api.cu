@@ -697,6 +697,9 @@ int reduce_group_and_notify(ftp_plan* p, int gi, float* grad_out, void* ws, cuda
     return FTP_OK;
 }
 
+// dz planes of one-conv bf16 group gi (two areas in turn)
+inline uint4* dz_planes(const ftp_plan* p, void* ws, int gi) { return reinterpret_cast<uint4*>(ws_ptr(ws, p->ws.dz_off + (size_t)(gi & 1) * p->ws.dz_bytes)); }
+
 // Backward pass of a one-conv bf16 group: dz planes at the conv's resolution, the filter gradient by the
 // weight-stationary tensor-core kernel over bands of the whole batch (one partial set per pixel share), and the delta
 // at the group's input.
@@ -710,9 +713,9 @@ bool tc_filter_grad(ftp_plan* p, const GroupPlan& g, int gi, const TcGroupArgs& 
     // dz planes: the two areas take turns; when the group above is a one-conv group too, its input-delta kernel has
     // already written this group's dz (see below), otherwise delta_act_planes_kernel makes them from the stored delta
     const int G = (int)p->groups.size();
-    uint4* dz = reinterpret_cast<uint4*>(ws_ptr(ws, p->ws.dz_off + (size_t)(gi & 1) * p->ws.dz_bytes));
-    uint4* dz_below = reinterpret_cast<uint4*>(ws_ptr(ws, p->ws.dz_off + (size_t)((gi + 1) & 1) * p->ws.dz_bytes));
-    const bool dz_ready = gi + 1 < G && p->groups[gi + 1].tfg.on;
+    uint4 *dz = dz_planes(p, ws, gi), *dz_below = dz_planes(p, ws, gi + 1);
+    // (the last group's by loss_planes_kernel, when the step made the loss: no delta then)
+    const bool dz_ready = gi + 1 < G ? p->groups[gi + 1].tfg.on : a.dmap_out == nullptr;
     const bool feeds_below = gi > 0 && p->groups[gi - 1].tfg.on;
     DeltaActPlanesArgs d{};
     d.dmap = a.dmap_out; d.dmap_planes = a.dmap_planes;
@@ -1070,7 +1073,9 @@ static int step_impl(ftp_plan* plan, const float* x, const float* dy, const floa
     int rc = ensure_device(plan);
     if (rc != FTP_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    float* y32 = (is_tc(plan) && target) ? ws_ptr(workspace, plan->ws.y32_off) : nullptr;
+    const GroupPlan& top = plan->groups.back();
+    const bool planes = target && top.tfg.on;                 // loss from the saved planes to dz planes
+    float* y32 = (is_tc(plan) && target && !planes) ? ws_ptr(workspace, plan->ws.y32_off) : nullptr;
     rc = forward_impl(plan, x, params, y32, workspace, kPackForward | kPackDelta, st);
     if (rc != FTP_OK) return rc;
     const float* delta = dy;
@@ -1080,6 +1085,19 @@ static int step_impl(ftp_plan* plan, const float* x, const float* dy, const floa
         const size_t M = (size_t)plan->N * s.C * s.H * s.W;
         float* d = ws_ptr(workspace, plan->ws.dy_off);
         float* sums = ws_ptr(workspace, plan->ws.loss_off);
+        if (planes) {
+            const OpDesc& op = top.bwd_ops[0];
+            LossPlanesArgs a{};
+            a.y = reinterpret_cast<const uint4*>(map_ptr(plan, x, workspace, op.out_map));
+            a.pool = op.kind == kOpConvPool ? 1 : 0;
+            if (a.pool) a.arg = reinterpret_cast<const unsigned long long*>(static_cast<unsigned char*>(workspace) + plan->ws.arg_off[op.out_map - 1]);
+            a.target = target; a.block_sums = sums; a.slope = op.slope;
+            a.dz = dz_planes(plan, workspace, (int)plan->groups.size() - 1);
+            a.N = plan->N; a.C = s.C; a.C16 = op.cout16; a.H = s.H; a.W = s.W;
+            Timed t(plan, st, 2, -1);
+            launch(loss_planes_kernel, plan->loss_blocks, 256, 0, t.ls(), a);
+            d = nullptr;
+        } else
         { Timed t(plan, st, 2, -1);
           launch(mse_delta_kernel, plan->loss_blocks, 256, 0, t.ls(), y32 ? y32 : map_ptr(plan, x, workspace, (int)plan->layers.size() + 1),
                                                              target, d, M, sums); }

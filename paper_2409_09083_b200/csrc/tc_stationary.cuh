@@ -60,6 +60,23 @@ struct DeltaActPlanesArgs {
     float slope;
 };
 
+// Entry of dz for 8 channels of pixel (y, x) of an H x W output map, plane `plane` of the batch; arg: their arg-max bytes where a
+// pool follows (four entries at twice the resolution), else null.
+__device__ __forceinline__ void store_dz(uint4* dz, const float (&v)[8], const unsigned long long* arg, size_t plane, int y, int x, int H, int W)
+{
+    if (!arg) { dz[(plane * H + y) * W + x] = tcd::pack8(v); return; }
+    const unsigned long long am = *arg;
+    const int W2 = 2 * W;
+    uint4* o = dz + (plane * (2 * H) + 2 * y) * W2 + 2 * x;
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        float z[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) z[c] = (int)((am >> (c * 8)) & 3ull) == w ? v[c] : 0.f;
+        o[(w >> 1) * W2 + (w & 1)] = tcd::pack8(z);
+    }
+}
+
 // dz = delta * act'(y), routed through the arg-max of a fused pool (zeros at the three other positions of a
 // window): the same arithmetic and roundings as the fused backward kernel applies when it fills its dz tile.
 __global__ void delta_act_planes_kernel(const __grid_constant__ DeltaActPlanesArgs A)
@@ -85,18 +102,58 @@ __global__ void delta_act_planes_kernel(const __grid_constant__ DeltaActPlanesAr
         tcd::unpack8(__ldg(A.y + e), yv);
 #pragma unroll
         for (int c = 0; c < 8; ++c) v[c] *= yv[c] > 0.f ? 1.f : A.slope;
-        if (!A.pool) { A.dz[e] = tcd::pack8(v); continue; }
-        const unsigned long long am = A.arg[e];
-        const int W2 = 2 * A.out_W;
-        uint4* o = A.dz + (((size_t)n * planes + pl) * (2 * A.out_H) + 2 * y) * W2 + 2 * x;
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            float z[8];
-#pragma unroll
-            for (int c = 0; c < 8; ++c) z[c] = (int)((am >> (c * 8)) & 3ull) == w ? v[c] : 0.f;
-            o[(w >> 1) * W2 + (w & 1)] = tcd::pack8(z);
-        }
+        store_dz(A.dz, v, A.pool ? A.arg + e : nullptr, (size_t)n * planes + pl, y, x, A.out_H, A.out_W);
     }
+}
+
+// Mean-squared-error loss of a step whose last group is a one-conv group: from the saved output (planes) and the target straight to
+// that group's dz planes, and per-block partial sums of (y - t)^2.  The values are those of planes_to_nchw_kernel,
+// mse_delta_kernel and delta_act_planes_kernel one after another, which moved 24 bytes a value instead of 8.  Bound: DRAM.
+// us, with the kernels overlapping: 256 channels on 16 x 38 x 38, 51 -> 16; 64 images, 215 -> 70; 4 x 52 x 52, 23 -> 8.
+struct LossPlanesArgs {
+    const uint4* y; const unsigned long long* arg;   // saved output (planes) and, for a fused pool, its arg-max bytes
+    const float* target;                             // fp32 NCHW
+    uint4* dz;                                       // out: planes at the conv's resolution
+    float* block_sums;
+    int N, C, C16, H, W, pool;                       // output map
+    float slope;
+};
+
+__global__ void __launch_bounds__(256) loss_planes_kernel(const __grid_constant__ LossPlanesArgs A)
+{
+    next_launch();
+    previous_launches();
+    __shared__ float red[256];
+    const int planes = A.C16 / 8;
+    const size_t HW = (size_t)A.H * A.W, total = (size_t)A.N * planes * HW, M = (size_t)A.N * A.C * HW;
+    const float scale = 2.0f / (float)M;
+    float sum = 0.f;
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
+        const size_t px = e % HW, t = e / HW;
+        const int pl = (int)(t % planes), n = (int)(t / planes);
+        const float* tg = A.target + ((size_t)n * A.C + pl * 8) * HW + px;
+        float v[8], yv[8], tv[8];
+        const uint4 yq = __ldg(A.y + e);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) tv[c] = pl * 8 + c < A.C ? __ldg(tg + c * HW) : 0.f;
+        tcd::unpack8(yq, yv);
+        float part = 0.f;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const float diff = pl * 8 + c < A.C ? yv[c] - tv[c] : 0.f;
+            part += diff * diff;
+            v[c] = scale * diff * (yv[c] > 0.f ? 1.f : A.slope);
+        }
+        sum += part;
+        store_dz(A.dz, v, A.pool ? A.arg + e : nullptr, t, (int)(px / A.W), (int)(px % A.W), A.H, A.W);
+    }
+    red[threadIdx.x] = sum;
+    __syncthreads();
+    for (int k = 128; k >= 1; k >>= 1) {
+        if ((int)threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) A.block_sums[blockIdx.x] = red[0];
 }
 
 // First layer: the fp32 network input [N][C][H][W] -> window-unrolled bf16 planes [N][C16'/8][H][W][8] with channel
