@@ -272,7 +272,7 @@ struct PrevLayer { const uint4* y; const unsigned long long* arg; float slope; }
 
 bool launch_tc_conv(ftp_plan* p, const TcConvPlan& c, int kind, int gi, const void* in, const __nv_bfloat16* w, const float* bias,
                     void* out, unsigned char* arg, int K, int cin16, int cout16, int cout, int H, int W, bool pool, float slope,
-                    int* error, cudaStream_t st, const PrevLayer* prev = nullptr)
+                    int* error, cudaStream_t st, const PrevLayer* prev = nullptr, float* out_f = nullptr)
 {
     TcConvRowsArgs a{};
     if (!encode_rows_map(a.tmap_x, in, p->N, cin16 / 8, H, W, W, c.R + K - 1, c.Wp)) return false;
@@ -285,7 +285,8 @@ bool launch_tc_conv(ftp_plan* p, const TcConvPlan& c, int kind, int gi, const vo
     a.Ns = c.Ns; a.slices = c.slices; a.R = c.R; a.Wp = c.Wp; a.bands_img = c.bands_img; a.nblk = c.nblk; a.kpc = c.kpc;
     a.ncc = c.ncc; a.Cw = c.Cw; a.items = c.items; a.pool_planes = c.pool_planes; a.nbuf = c.nbuf;
     a.x_plane = c.x_plane; a.stage_bytes = c.stage_bytes; a.stages = c.stages;
-    a.hurry = (double)((c.items + c.blocks - 1) / c.blocks) * c.nblk * K * K * (cin16 / 16) * tc_mma_cycles(c.Ns) < kHurryCycles;
+    a.out_f = out_f; a.narrow = c.narrow; a.zero_off = c.zero_off;
+    a.hurry = (double)((c.items + c.blocks - 1) / c.blocks) * c.nblk * (c.narrow ? 5 : K * K * (cin16 / 16)) * tc_mma_cycles(c.Ns) < kHurryCycles;
     { Timed tm(p, st, kind, gi);
       launch(conv_tc_rows_kernel, c.blocks, kTcConvThreads, one_block_smem(c.smem_bytes), tm.ls(), a); }
     return launched_ok();
@@ -363,10 +364,8 @@ int pack_filters_tc(ftp_plan* p, const float* params, void* ws, int dirs, cudaSt
                 continue;
             }
             if (ba.n == kPackTilesLayers) flush_banded();
-            // (first layer on the window-unrolled input: a 1x1 conv with 9 cin input channels, same parameters)
-            const bool col = g.col_cin16 != 0;
             add_pack_tiles(ba, PackTilesLayer{op.p_off, reinterpret_cast<uint4*>(wf + op.twf_off), reinterpret_cast<uint4*>(wb + op.twb_off),
-                                              col ? g.col_cin : op.cin, op.cout, col ? 1 : op.k, col ? g.col_cin16 : op.cin16, op.cout16,
+                                              op.cin, op.cout, op.k, g.narrow ? 8 : op.cin16, op.cout16,
                                               g.cf.Ns, g.cf.kpc, g.cd.Ns, g.cd.kpc, 0});
         }
     flush();
@@ -387,15 +386,17 @@ int forward_tc(ftp_plan* p, const float* x, const float* params, float* y, void*
             const OpDesc& op = g.fwd_ops[0];
             const __nv_bfloat16* wf = reinterpret_cast<const __nv_bfloat16*>(ws_ptr(ws, p->ws.wf_off)) + op.twf_off;
             const void* in = a.map[0];
-            if (g.col_cin16) {                  // first layer: a 1x1 conv on the window-unrolled network input
+            if (g.narrow) {                     // first layer
                 uint4* col = reinterpret_cast<uint4*>(ws_ptr(ws, p->ws.col_off));
+                const size_t HW = (size_t)op.in_H * op.in_W;
                 { Timed t(p, st, 9, (int)gi);
-                  launch_unroll_windows(x, col, p->N, op.cin, op.in_H, op.in_W, t.ls()); }
+                  launch(input_entries_kernel, (int)std::min<size_t>((p->N * HW + 255) / 256, (size_t)kSmCount * 16), 256, 0, t.ls(),
+                         x, col, p->N, op.cin, HW); }
                 if (!launched_ok()) return FTP_ERR_CUDA;
                 in = col;
             }
             if (!launch_tc_conv(p, g.cf, 1, (int)gi, in, wf, params + op.p_off + (size_t)op.cout * op.cin * op.k * op.k,
-                                a.map_out[1], a.arg[0], g.tfg.k, g.col_cin16 ? g.col_cin16 : op.cin16, op.cout16, op.cout, op.in_H, op.in_W,
+                                a.map_out[1], a.arg[0], g.tfg.k, g.narrow ? 8 : op.cin16, op.cout16, op.cout, op.in_H, op.in_W,
                                 op.kind == kOpConvPool, op.slope, a.error, st))
                 return FTP_ERR_CUDA;
             continue;
@@ -642,15 +643,11 @@ int forward_impl(ftp_plan* p, const float* x, const float* params, float* y, voi
     return FTP_OK;
 }
 
-// A layer's entry for the cross-tile reduction: where its slice of the partial sets lies and how it is arranged (the
-// first layer on the window-unrolled input: as the 1x1 conv with 9 cin input channels that computed it).
+// A layer's entry for the cross-tile reduction: where its slice of the partial sets lies and how it is arranged.
 TcReduceLayer reduce_layer(const GroupPlan& g, const OpDesc& op, void* ws)
 {
-    if (g.col_cin16)
-        return TcReduceLayer{op.p_off, ws_ptr(ws, g.partial_off), (long long)g.param_floats, op.tgp_off, g.sets(), g.col_cin, op.cout, 1,
-                             g.col_cin16, op.cout16, g.tfg.nci};
     return TcReduceLayer{op.p_off, ws_ptr(ws, g.partial_off), (long long)g.set_floats(), op.tgp_off, g.sets(), op.cin, op.cout, op.k,
-                         op.cin16, op.cout16, g.tfg.on ? g.tfg.nci : 1};
+                         g.narrow ? g.tfg.ncols : op.cin16, op.cout16, g.tfg.on ? g.tfg.nci : 1};
 }
 
 // Sums the partial sets of executed groups [first, last]: whole gradients (grad_out) and / or the update.
@@ -707,9 +704,9 @@ bool tc_filter_grad(ftp_plan* p, const GroupPlan& g, int gi, const TcGroupArgs& 
 {
     const OpDesc& op = g.bwd_ops[0];
     const TcFgPlan& t = g.tfg;
-    // the layer's input as bf16 planes: the saved map, or (first layer) the window-unrolled network input of the forward pass
-    void* xin = g.col_cin16 ? static_cast<void*>(ws_ptr(ws, p->ws.col_off)) : const_cast<void*>(a.map[0]);
-    const int cin16 = g.col_cin16 ? g.col_cin16 : op.cin16;
+    // the layer's input as bf16 planes: the saved map, or (first layer) what the forward pass made of the network input
+    void* xin = g.narrow ? static_cast<void*>(ws_ptr(ws, p->ws.col_off)) : const_cast<void*>(a.map[0]);
+    const int cin16 = op.cin16;
     // dz planes: the two areas take turns; when the group above is a one-conv group too, its input-delta kernel has
     // already written this group's dz (see below), otherwise delta_act_planes_kernel makes them from the stored delta
     const int G = (int)p->groups.size();
@@ -734,10 +731,10 @@ bool tc_filter_grad(ftp_plan* p, const GroupPlan& g, int gi, const TcGroupArgs& 
 
     TcFilterGradArgs f{};
     if (!encode_band_map(f.tmap_dz, dz, p->N, op.cout16 / 8, op.in_H, op.in_W, false, t.Cw, t.R, t.dz_box) ||
-        !encode_band_map(f.tmap_x, xin, p->N, cin16 / 8, op.in_H, op.in_W, true, t.Cw + t.k - 1, t.R + t.k - 1, t.ncols / 8)) return false;
+        !encode_band_map(f.tmap_x, xin, p->N, g.narrow ? 1 : cin16 / 8, op.in_H, op.in_W, true, t.Cw + t.k - 1, t.R + t.k - 1, t.ncols / 8)) return false;
     f.partial = a.partial; f.set_floats = a.set_floats; f.tgp_off = op.tgp_off;
     f.error = a.error;
-    f.K = t.k; f.H = op.in_H; f.W = op.in_W; f.cout16 = op.cout16; f.cin16 = cin16;
+    f.K = t.k; f.H = op.in_H; f.W = op.in_W; f.cout16 = op.cout16; f.cin16 = g.narrow ? t.ncols : cin16; f.narrow = g.narrow;
     f.Ms = t.Ms; f.slices = t.slices; f.ncols = t.ncols; f.nci = t.nci; f.units = t.units;
     f.R = t.R; f.Cw = t.Cw; f.ncc = t.ncc; f.bands_img = t.bands_img; f.bands = t.bands; f.shares = t.shares;
     f.dz_box = t.dz_box; f.x_off = t.x_off; f.stage_bytes = t.stage_bytes;
@@ -749,7 +746,7 @@ bool tc_filter_grad(ftp_plan* p, const GroupPlan& g, int gi, const TcGroupArgs& 
     // input delta: the convolution of dz with the rotated filters (dz planes in, delta planes out)
     if (!need_dx) return true;
     const __nv_bfloat16* wb = reinterpret_cast<const __nv_bfloat16*>(ws_ptr(ws, p->ws.wb_off)) + op.twb_off;
-    if (!g.col_cin16) {
+    if (gi > 0) {
         if (!feeds_below)
             return launch_tc_conv(p, g.cd, 8, gi, dz, wb, nullptr, ws_ptr(ws, p->ws.dmap_off[gi]), nullptr, t.k, op.cout16, cin16, op.cin,
                                   op.in_H, op.in_W, false, 1.0f, a.error, st);
@@ -761,14 +758,9 @@ bool tc_filter_grad(ftp_plan* p, const GroupPlan& g, int gi, const TcGroupArgs& 
         return launch_tc_conv(p, g.cd, 8, gi, dz, wb, nullptr, dz_below, nullptr, t.k, op.cout16, cin16, op.cin,
                               op.in_H, op.in_W, false, 1.0f, a.error, st, &pv);
     }
-    // first layer: the delta of the window-unrolled input (in the dz area that is not in use, sized for it; the unrolled
-    // input stays as the forward pass left it), folded back into the caller's fp32 map
-    if (!launch_tc_conv(p, g.cd, 8, gi, dz, wb, nullptr, dz_below, nullptr, 1, op.cout16, cin16, g.col_cin, op.in_H, op.in_W, false, 1.0f,
-                        a.error, st))
-        return false;
-    { Timed tm(p, st, 10, gi);
-      launch_fold_windows(reinterpret_cast<const __nv_bfloat16*>(dz_below), dx, p->N, op.cin, op.in_H, op.in_W, tm.ls()); }
-    return launched_ok();
+    // first layer: straight into the caller's fp32 map
+    return launch_tc_conv(p, g.cd, 8, gi, dz, wb, nullptr, nullptr, nullptr, t.k, op.cout16, cin16, op.cin, op.in_H, op.in_W, false, 1.0f,
+                          a.error, st, nullptr, dx);
 }
 
 int backward_tc(ftp_plan* p, const float* x, const float* dy, const float* params, float* dx, float* grad_out,

@@ -35,7 +35,7 @@ __device__ __forceinline__ void pack_tile(const PackTilesLayer L, int t, int dir
         const bool fwd = i < total;
         const int j = fwd ? i : i - total, r = j & 31, o = (j >> 5) & 3, tap = j >> 7;   // row of the operand, octet of contraction channels
         const int row = (fwd ? co0 : ci0) + r, k0 = (fwd ? ci0 : co0) + o * 8;
-        if (row >= (fwd ? L.cout16 : L.cin16) || k0 >= (fwd ? L.cin16 : L.cout16)) continue;
+        if (row >= (fwd ? L.cout16 : max(L.cin16, 16)) || k0 >= (fwd ? L.cin16 : L.cout16)) continue;
         const int ns = fwd ? L.ns_f : L.ns_d, kpc = fwd ? L.kpc_f : L.kpc_d;
         const int nch = ((fwd ? L.cin16 : L.cout16) / 8 + kpc - 1) / kpc;
         float v[8];

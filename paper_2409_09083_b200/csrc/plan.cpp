@@ -506,14 +506,14 @@ double tc_stationary_estimate_us(const ftp_plan& p, const GroupPlan& g, bool bac
 {
     const OpDesc& op = g.fwd_ops[0];
     const double px = (double)p.N * op.in_H * op.in_W;
-    const int cin16 = g.col_cin16 ? g.col_cin16 : op.cin16, kk = g.col_cin16 ? 1 : op.k * op.k;
+    const int cin16 = g.narrow ? 8 : op.cin16, kk = op.k * op.k;
     const double flops = 2.0 * px * cin16 * op.cout16 * kk;
     auto rate = [](int ns) { return 800e6 * std::min(1.0, std::max(ns, 16) / 80.0); };           // flop per microsecond
     const double in_b = px * cin16 * 2.0, out_b = px * op.cout16 * 2.0 / (op.kind == kOpConvPool ? 4.0 : 1.0), dz_b = px * op.cout16 * 2.0;
-    if (!backward) return flops / rate(g.cf.Ns) + (in_b + out_b) / 5e6 + (g.col_cin16 ? in_b / 3e6 : 0.0) + 8.0;
+    if (!backward) return flops / rate(g.cf.Ns) + (in_b + out_b) / 5e6 + (g.narrow ? 1.5 * in_b / 5e6 : 0.0) + 8.0;
     double t = (2.0 * out_b + dz_b) / 5e6 + 4.0;                                               // dz planes
     t += flops / 600e6 + (in_b + dz_b) / 5e6 + 10.0;                                           // filter gradient
-    if (need_dx) t += flops / rate(g.cd.Ns) + (in_b + dz_b) / 5e6 + (g.col_cin16 ? in_b / 3e6 : 0.0) + 8.0;
+    if (need_dx) t += flops / rate(g.cd.Ns) + (in_b + dz_b) / 5e6 + 8.0;
     return t;
 }
 
@@ -813,8 +813,8 @@ bool tc_stationary_conv(const ftp_plan& p, int li /*0-based*/, const PlanOpts& o
 {
     const ftp_layer& l = p.layers[li];
     if (p.precision != FTP_BF16_FP32ACC || o.stationary < 0 || l.kind != FTP_CONV) return false;
-    // the first layer reads the fp32 network input: only as a 1x1 conv on its window-unrolled copy (3x3, at most 7 channels)
-    if (li == 0 && (l.k != 3 || l.cin * 9 > 64)) return false;
+    // the first layer reads the fp32 network input: only as 8-channel entries with a spare channel (3x3, at most 7 channels)
+    if (li == 0 && (l.k != 3 || l.cin > 7)) return false;
     return (l.k == 1 || l.k == 3) && p.maps[li].W <= kTcMaxColChunks * 126;
 }
 
@@ -855,6 +855,7 @@ TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, b
     c.nbuf = c.Ns <= 64 ? 2 : 1;
     const int max_blk = std::min(8, kTcTmemCols / c.nbuf / c.Ns);
     c.kpc = K == 1 ? std::min(cin16 / 8, 8) : kpc3;
+    c.narrow = cin16 == 8 ? 1 : 0;
     const int step = pool ? 2 : 1;
     const int r_max = std::min((max_blk * 128) / c.Wp, H) / step * step;
     if (r_max < step) return c;
@@ -867,10 +868,10 @@ TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, b
     }
     const size_t entries = std::max<size_t>((size_t)(c.R + K - 1) * c.Wp, (size_t)c.nblk * 128 + (size_t)(K - 1) * c.Wp + K);
     c.x_plane = (int)align_up(entries * 16, 128);
-    c.stage_bytes = c.kpc * c.x_plane + K * K * c.kpc * c.Ns * 16;
+    c.stage_bytes = c.kpc * c.x_plane + (K * K + c.narrow) * c.kpc * c.Ns * 16;         // (narrow: a tenth window position of zeros)
     // fused pool: the band as stored goes through a staging area, all channels of the slice at once where that leaves
     // three stages (two for short rings), else 16 channels or more at a time
-    const size_t room = (size_t)kTcConvSmemBudget - kTcFgHeader;
+    const size_t room = (size_t)kTcConvSmemBudget - kTcFgHeader - (c.narrow ? 2048 : 0);
     const size_t plane_pair = (size_t)c.nblk * 128 * 16 * 2, whole = (size_t)(c.Ns / 16) * plane_pair;
     size_t staging = pool ? kTcPoolStageBytes : 0;
     c.stages = (int)std::min<size_t>(4, (room - staging) / c.stage_bytes);
@@ -882,7 +883,8 @@ TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, b
         c.pool_stage_bytes = (int)staging;
     }
     if (c.stages < 2 || (pool && c.pool_planes < 2)) return c;
-    c.smem_bytes = kTcFgHeader + c.stages * c.stage_bytes + (int)staging;
+    c.zero_off = c.stages * c.stage_bytes + (int)staging;
+    c.smem_bytes = kTcFgHeader + c.zero_off + (c.narrow ? 2048 : 0);
     const long long items = (long long)N * c.bands_img * c.slices;
     if (items > 0x7fffffffLL) return c;
     c.items = (int)items;
@@ -902,10 +904,8 @@ void plan_tc_filter_grad(const ftp_plan& p, GroupPlan& g, const PlanOpts& o)
     if (g.n_ops != 1 || g.bwd_ops[0].kind == kOpPool || !tc_stationary_conv(p, g.first - 1, o)) return;
     const OpDesc& op = g.bwd_ops[0];
     TcFgPlan t;
-    const bool unrolled = g.first == 1;                         // first layer: 1x1 conv on the window-unrolled input
-    const int col_cin16 = round_up(op.cin * 9, 16);
-    const int H = op.in_H, W = op.in_W, K = unrolled ? 1 : op.k;
-    const int cin16 = unrolled ? col_cin16 : op.cin16;
+    const bool narrow = g.first == 1;                           // first layer: input entries of 8 channels
+    const int H = op.in_H, W = op.in_W, K = op.k;
     t.k = K;
     t.Ms = op.cout16 <= 64 ? 64 : 128;
     t.slices = (op.cout16 + t.Ms - 1) / t.Ms;
@@ -914,13 +914,14 @@ void plan_tc_filter_grad(const ftp_plan& p, GroupPlan& g, const PlanOpts& o)
     for (int most : {256, 48, 32, 16}) {
         if (K == 3 && most > 48) continue;
         TcFgPlan c = t;
-        c.nci = (cin16 + most - 1) / most;
-        c.ncols = round_up((cin16 + c.nci - 1) / c.nci, 16);
+        c.nci = (op.cin16 + most - 1) / most;
+        c.ncols = round_up((op.cin16 + c.nci - 1) / c.nci, 16);
         if (c.ncols > most) continue;
+        if (narrow && t.Ms == 64) c.ncols = 8;                   // (with 128 rows an MMA has multiples of 16 columns)
         const int wide = K * c.ncols, roles = c.slices * c.nci, max_g = (128 - (K - 1)) / 8, groups = (W + 7) / 8;
         c.units = K == 3 || 3 * wide + 16 <= kTcTmemCols ? 3 : 1;
-        const double operands = (c.Ms + wide) * 32.0 / 128.0, mma = (K == 3 ? 3.0 : 1.0) * std::max(wide / 2.0, operands) + (c.Ms + 16) * 0.25 / c.nci;
-        const double set_cost = (double)(K * K * cin16 + 1) * op.cout16 * 8.0 / 5e6 * 1900.0;
+        const double operands = (c.Ms + wide) * 32.0 / 128.0, mma = (K == 3 ? 3.0 : 1.0) * std::max(wide / 2.0, operands) + (narrow ? 0.0 : (c.Ms + 16) * 0.25 / c.nci);
+        const double set_cost = (double)(K * K * op.cin16 + 1) * op.cout16 * 8.0 / 5e6 * 1900.0;
         for (int ncc = (groups + max_g - 1) / max_g, end = ncc + 4; ncc <= std::min(groups, end); ++ncc) {
             c.Cw = (groups + ncc - 1) / ncc * 8;
             c.ncc = (W + c.Cw - 1) / c.Cw;
@@ -947,10 +948,11 @@ void plan_tc_filter_grad(const ftp_plan& p, GroupPlan& g, const PlanOpts& o)
     if (best < 0) return;
     t.blocks = t.slices * t.nci * t.shares;
     // the forward convolution, and the input delta as the convolution of dz (cout16 channels) with the rotated filters
-    g.cf = plan_tc_conv(p.N, H, W, K, cin16, op.cout16, op.kind == kOpConvPool);
-    g.cd = plan_tc_conv(p.N, H, W, K, op.cout16, cin16, false);
+    g.cf = narrow ? plan_tc_conv_kpc(p.N, H, W, K, 8, op.cout16, op.kind == kOpConvPool, 1)
+                  : plan_tc_conv(p.N, H, W, K, op.cin16, op.cout16, op.kind == kOpConvPool);
+    g.cd = plan_tc_conv(p.N, H, W, K, op.cout16, op.cin16, false);
     if (!g.cf.on || !g.cd.on) return;
-    if (unrolled) { g.col_cin = op.cin * 9; g.col_cin16 = col_cin16; }
+    g.narrow = narrow ? 1 : 0;
     t.on = 1;
     g.tfg = t;
     g.param_floats += (size_t)(t.nci - 1) * op.cout16;          // the bias gradient comes in parts, one per slice of the input channels
@@ -1355,10 +1357,9 @@ int build_plan(ftp_plan& p, const ftp_layer* layers, int n_layers, int N, int C,
         if (g.st.on && !g.st.thin && !g.sp.on)
             dz[0] = dz[1] = std::max(dz[0], (size_t)N * g.fwd_ops[0].cout * g.fwd_ops[0].in_H * g.fwd_ops[0].in_W * 4);
         if (g.tfg.on) dz[gi & 1] = std::max(dz[gi & 1], (size_t)N * g.fwd_ops[0].cout16 * g.fwd_ops[0].in_H * g.fwd_ops[0].in_W * 2);
-        if (gi == 0 && g.col_cin16) dz[1] = std::max(dz[1], (size_t)N * g.col_cin16 * H * W * 2);   // delta of the unrolled input
     }
     ws.scratch_off = take(scratch * 4);
-    if (!p.groups.empty() && p.groups[0].col_cin16) ws.col_off = take((size_t)N * p.groups[0].col_cin16 * H * W * 2);
+    if (!p.groups.empty() && p.groups[0].narrow) ws.col_off = take((size_t)N * H * W * 16);
     ws.dz_bytes = align_up(dz[0], 256);             // = offset of the second area
     ws.dz_off = take(ws.dz_bytes + align_up(dz[1], 256));
     ws.wf_off = take(p.wf_floats * (tcp ? 2 : 4));

@@ -46,6 +46,7 @@ struct TcFilterGradArgs {
     int K, H, W, cout16, cin16;
     int Ms, slices;                           // output channels per block (64 or 128) and number of such slices
     int ncols, nci;                           // input channels per block (multiple of 16) and number of such slices
+    int narrow;                               // first layer: x is input_entries_kernel's plane (ncols 8 or 16, the bias gradient its channel 7)
     int units;                                // accumulator units of K * ncols columns: 3x3: one per window column; 1x1: row pairs in turn
     int R, Cw, ncc;                           // rows per band, columns of a band and column chunks per row band
     int bands_img, bands, shares;             // bands per image / in the batch, pixel shares
@@ -156,98 +157,23 @@ __global__ void __launch_bounds__(256) loss_planes_kernel(const __grid_constant_
     if (threadIdx.x == 0) A.block_sums[blockIdx.x] = red[0];
 }
 
-// First layer: the fp32 network input [N][C][H][W] -> window-unrolled bf16 planes [N][C16'/8][H][W][8] with channel
-// ci * 9 + ky * 3 + kx of pixel (y, x) = input(ci, y + ky - 1, x + kx - 1) (zero outside the map and beyond 9 C).
-// One thread per pixel: it reads the 9 C values of its window once and writes its entry of every plane (the
-// channel -> (ci, ky, kx) arithmetic is resolved at compile time).
-template <int C>
-__global__ void unroll_windows_kernel(const float* __restrict__ x, uint4* __restrict__ col, int N, int H, int W)
+// First layer (at most 7 channels): the fp32 network input [N][C][H][W] -> one plane of 8-channel bf16 entries, channels
+// beyond C zero, the last one 1 (the filter gradient's sums of dz x that channel at the window's centre are the bias gradient; its
+// forward weights are zero).  16 bytes a pixel; the window-unrolled copy that stood here before (9 C channels, 64 bytes a
+// pixel with 3) was written once and read twice at four times the size: us for 16 x 608 x 608, 3 -> 32 channels,
+// copy / forward / filter gradient / input delta (and fold): 99 / 152 / 144 / 240 -> 34 / 152 / 142 / 166.
+__global__ void __launch_bounds__(256) input_entries_kernel(const float* __restrict__ x, uint4* __restrict__ out, int N, int C, size_t HW)
 {
     previous_launches();
-    constexpr int planes = (9 * C + 15) / 16 * 2;
-    const size_t HW = (size_t)H * W, total = (size_t)N * HW;
+    const size_t total = (size_t)N * HW;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const int px = (int)(e % W); size_t t = e / W;
-        const int py = (int)(t % H); const int n = (int)(t / H);
-        float v[planes * 8];
-        const float* ctr = x + (size_t)n * C * HW + (size_t)py * W + px;       // this pixel in channel 0
-        if (py > 0 && py < H - 1 && px > 0 && px < W - 1) {                    // the whole window lies inside the map
+        const size_t n = e / HW;
+        const float* src = x + n * C * HW + (e - n * HW);
+        float v[8];
 #pragma unroll
-            for (int j = 0; j < planes * 8; ++j) {
-                const int ci = j / 9, tap = j - ci * 9, ky = tap / 3, kx = tap - ky * 3;
-                v[j] = ci < C ? __ldg(ctr + (size_t)ci * HW + (ky - 1) * W + (kx - 1)) : 0.f;
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < planes * 8; ++j) {
-                const int ci = j / 9, tap = j - ci * 9, ky = tap / 3, kx = tap - ky * 3;
-                const int yy = py + ky - 1, xx = px + kx - 1;
-                v[j] = (ci < C && yy >= 0 && yy < H && xx >= 0 && xx < W) ? __ldg(ctr + (size_t)ci * HW + (ky - 1) * W + (kx - 1)) : 0.f;
-            }
-        }
-#pragma unroll
-        for (int pl = 0; pl < planes; ++pl) col[((size_t)n * planes + pl) * HW + (size_t)py * W + px] = tcd::pack8(v + 8 * pl);
-    }
-}
-
-// ... and back: the delta at the network input, fp32 NCHW, as the sum over the window positions of the delta planes of
-// the unrolled input: dx(ci, y, x) = sum over (ky, kx) of dcol(ci * 9 + ky * 3 + kx, y - ky + 1, x - kx + 1), in the
-// order of the window positions.  One thread per pixel and all its channels: of the neighbour at window position
-// (ky, kx) it needs channel ci * 9 + ky * 3 + kx for every ci.
-template <int C>
-__global__ void fold_windows_kernel(const __nv_bfloat16* __restrict__ dcol, float* __restrict__ dx, int N, int H, int W)
-{
-    previous_launches();
-    constexpr int planes = (9 * C + 15) / 16 * 2;
-    const size_t HW = (size_t)H * W, total = (size_t)N * HW;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const int px = (int)(e % W); size_t t = e / W;
-        const int py = (int)(t % H); const int n = (int)(t / H);
-        float s[C];
-#pragma unroll
-        for (int ci = 0; ci < C; ++ci) s[ci] = 0.f;
-#pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-            const int ky = tap / 3, kx = tap - ky * 3, yy = py - ky + 1, xx = px - kx + 1;
-            if (yy >= 0 && yy < H && xx >= 0 && xx < W) {
-                const __nv_bfloat16* src = dcol + ((size_t)n * planes * HW + (size_t)yy * W + xx) * 8;
-#pragma unroll
-                for (int ci = 0; ci < C; ++ci) {
-                    const int j = ci * 9 + tap;
-                    s[ci] += __bfloat162float(__ldg(src + (size_t)(j >> 3) * HW * 8 + (j & 7)));
-                }
-            }
-        }
-#pragma unroll
-        for (int ci = 0; ci < C; ++ci) dx[((size_t)n * C + ci) * HW + (size_t)py * W + px] = s[ci];
-    }
-}
-
-// the two kernels for the channel counts the route takes (9 C <= 64)
-inline void launch_unroll_windows(const float* x, uint4* col, int N, int C, int H, int W, LaunchStream st)
-{
-    const int blocks = (int)std::min<size_t>(((size_t)N * H * W + 255) / 256, (size_t)kSmCount * 16);
-    switch (C) {
-        case 1: launch(unroll_windows_kernel<1>, blocks, 256, 0, st, x, col, N, H, W); break;
-        case 2: launch(unroll_windows_kernel<2>, blocks, 256, 0, st, x, col, N, H, W); break;
-        case 3: launch(unroll_windows_kernel<3>, blocks, 256, 0, st, x, col, N, H, W); break;
-        case 4: launch(unroll_windows_kernel<4>, blocks, 256, 0, st, x, col, N, H, W); break;
-        case 5: launch(unroll_windows_kernel<5>, blocks, 256, 0, st, x, col, N, H, W); break;
-        case 6: launch(unroll_windows_kernel<6>, blocks, 256, 0, st, x, col, N, H, W); break;
-        default: launch(unroll_windows_kernel<7>, blocks, 256, 0, st, x, col, N, H, W); break;
-    }
-}
-inline void launch_fold_windows(const __nv_bfloat16* dcol, float* dx, int N, int C, int H, int W, LaunchStream st)
-{
-    const int blocks = (int)std::min<size_t>(((size_t)N * H * W + 255) / 256, (size_t)kSmCount * 16);
-    switch (C) {
-        case 1: launch(fold_windows_kernel<1>, blocks, 256, 0, st, dcol, dx, N, H, W); break;
-        case 2: launch(fold_windows_kernel<2>, blocks, 256, 0, st, dcol, dx, N, H, W); break;
-        case 3: launch(fold_windows_kernel<3>, blocks, 256, 0, st, dcol, dx, N, H, W); break;
-        case 4: launch(fold_windows_kernel<4>, blocks, 256, 0, st, dcol, dx, N, H, W); break;
-        case 5: launch(fold_windows_kernel<5>, blocks, 256, 0, st, dcol, dx, N, H, W); break;
-        case 6: launch(fold_windows_kernel<6>, blocks, 256, 0, st, dcol, dx, N, H, W); break;
-        default: launch(fold_windows_kernel<7>, blocks, 256, 0, st, dcol, dx, N, H, W); break;
+        for (int c = 0; c < 7; ++c) v[c] = c < C ? __ldg(src + c * HW) : 0.f;
+        v[7] = 1.f;
+        out[e] = tcd::pack8(v);
     }
 }
 
@@ -345,7 +271,7 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
             const int s = i & 1;
             if (!wait(&H->full[s], (uint32_t)(i >> 1) & 1u)) break;
             fence_after_sync();
-            if (is_bias || warp < A.units) {
+            if (is_bias ? !A.narrow : warp < A.units) {
                 int n, y0, x0;
                 band_of(b_lo + i, n, y0, x0);
                 const uint32_t dst = smem_u32(stages + (size_t)s * A.stage_bytes);
@@ -408,14 +334,15 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
                 float* g = gset + ((size_t)u * A.cout16 + co) * A.cin16 + ci0 + c0;
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    *reinterpret_cast<float4*>(g + 4 * j) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                    if (c0 + 4 * j < cols) *reinterpret_cast<float4*>(g + 4 * j) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             }
         }
     }
     if (half == 0) {
         float v[16];
         v[0] = 0.f;
-        if (have && pairs > cs) tmem_ld16(tq + (uint32_t)(A.units * wide), v);
+        if (A.narrow) { if (have) { tmem_ld16(tq + (uint32_t)(wide + A.ncols), v); v[0] = v[7]; } }
+        else if (have && pairs > cs) tmem_ld16(tq + (uint32_t)(A.units * wide), v);
         if (row_ok) gset[(size_t)KK * A.cout16 * A.cin16 + (size_t)cs * A.cout16 + co] = v[0];
     }
     fence_before_sync();
@@ -463,6 +390,8 @@ struct TcConvRowsArgs {
     // at twice the resolution if it ends with a pool): prev_y = that layer's saved output (= this conv's output shape),
     // prev_arg = its pool's arg-max bytes or null, prev_slope = its leaky slope.  prev_y null: plain delta planes.
     const uint4* prev_y; const unsigned long long* prev_arg; float prev_slope;
+    float* out_f;                             // fp32 NCHW output in the place of planes (delta at the network input), else null
+    int narrow, zero_off;                     // first layer's forward pass: in is one plane of 8 channels; offset of 2 KB of zeros behind the stages
     int nbuf;                                 // accumulator buffers (2: items of at most 256 columns alternate between the halves
                                               //   of the tensor memory, so the MMAs of one run while the other is read back)
 };
@@ -502,6 +431,7 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
     }
     if (warp == 0) { __syncwarp(); tmem_alloc(smem_u32(&H->tmem_base), (uint32_t)kTcTmemCols); }
     tcd::zero_bytes(stages, (size_t)A.stages * A.stage_bytes);       // what the copies never write is read as zeros
+    if (A.narrow) tcd::zero_bytes(stages + A.zero_off, 2048);
     fence_async_smem();
     fence_before_sync();
     __syncthreads();
@@ -589,7 +519,17 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                     for (int b = iw; b < I.nblk; b += kTcIssuers) {
                         const uint32_t tcol = tmem + buf * 256u + (uint32_t)(b * A.Ns);
                         const uint32_t a0 = desc_lo(xaddr + (uint32_t)b * 2048u, (uint32_t)A.x_plane);
-                        if (K == 3) {
+                        if (A.narrow) {
+                            // one plane: a K step is two window positions (the second LBO entries behind the first), the last one's
+                            // partner a block of zeros (an infinite pixel must not meet a zero weight)
+                            const uint32_t wp = (uint32_t)A.Wp, al = desc_lo(xaddr + (uint32_t)b * 2048u, 0), w2 = 2u * (uint32_t)A.Ns;
+                            const uint32_t last = al + 2 * wp + 2, zeros = desc_lo(smem_u32(stages + A.zero_off), 0);
+                            mma_bf16(tcol, desc64(a_hi, al | (1u << 16)), desc64(b_hi, b_lo0), idesc, false);
+                            mma_bf16(tcol, desc64(a_hi, (al + 2) | ((wp - 2) << 16)), desc64(b_hi, b_lo0 + w2), idesc, true);
+                            mma_bf16(tcol, desc64(a_hi, (al + wp + 1) | (1u << 16)), desc64(b_hi, b_lo0 + 2 * w2), idesc, true);
+                            mma_bf16(tcol, desc64(a_hi, (al + 2 * wp) | (1u << 16)), desc64(b_hi, b_lo0 + 3 * w2), idesc, true);
+                            mma_bf16(tcol, desc64(a_hi, last | ((zeros - last) << 16)), desc64(b_hi, b_lo0 + 4 * w2), idesc, true);
+                        } else if (K == 3) {
                             // nine MMAs per K step, one per window position, written out: the issuing thread runs a few dozen
                             // instructions per MMA if it has to loop, and then it, not the tensor core, sets the pace
                             // (measured: an MMA every 100 cycles with the loops, every 40-64 with straight-line code)
@@ -679,7 +619,13 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                     tmem_ld16(tbuf + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * A.Ns + c0), v);
 #pragma unroll
                     for (int j = 0; j < 16; ++j) { const float z = v[j] + H->bias[c0 + j]; v[j] = z > 0.f ? z : slope * z; }
-                    if (valid && !A.prev_y) {
+                    if (A.out_f) {
+                        if (!valid) continue;
+                        const int p = b * 128 + q * 32 + lane, r = p / A.Wp, c = p - r * A.Wp;
+                        float* dst = A.out_f + (((size_t)I.n * A.cout + I.co0 + c0) * A.H + I.y0 + r) * A.W + I.x0 + c;
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) if (I.co0 + c0 + j < A.cout) dst[j * gstep] = v[j];
+                    } else if (valid && !A.prev_y) {
                         A.out[g0] = tcd::pack8(v);
                         A.out[g0 + gstep] = tcd::pack8(v + 8);
                     } else if (valid) {
