@@ -285,7 +285,7 @@ bool launch_tc_conv(ftp_plan* p, const TcConvPlan& c, int kind, int gi, const vo
     a.Ns = c.Ns; a.slices = c.slices; a.R = c.R; a.Wp = c.Wp; a.bands_img = c.bands_img; a.nblk = c.nblk; a.kpc = c.kpc;
     a.ncc = c.ncc; a.Cw = c.Cw; a.items = c.items; a.pool_planes = c.pool_planes; a.nbuf = c.nbuf;
     a.x_plane = c.x_plane; a.stage_bytes = c.stage_bytes; a.stages = c.stages;
-    a.out_f = out_f; a.narrow = c.narrow; a.zero_off = c.zero_off;
+    a.out_f = out_f; a.row_blocks = c.row_blocks; a.blk_step = c.row_blocks ? c.Wp : 128; a.narrow = c.narrow; a.zero_off = c.zero_off;
     a.hurry = (double)((c.items + c.blocks - 1) / c.blocks) * c.nblk * (c.narrow ? 5 : K * K * (cin16 / 16)) * tc_mma_cycles(c.Ns) < kHurryCycles;
     { Timed tm(p, st, kind, gi);
       launch(conv_tc_rows_kernel, c.blocks, kTcConvThreads, one_block_smem(c.smem_bytes), tm.ls(), a); }

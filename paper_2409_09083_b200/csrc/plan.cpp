@@ -858,31 +858,40 @@ TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, b
     c.narrow = cin16 == 8 ? 1 : 0;
     const int step = pool ? 2 : 1;
     const int r_max = std::min((max_blk * 128) / c.Wp, H) / step * step;
-    if (r_max < step) return c;
+    // With a pool, accumulator blocks of one row each where that is the faster form: the epilogue then compares in registers (430
+    // cycles for 128 entries x 16 channels instead of 550 through the staging area), while rows of few columns
+    // leave most of a block's 128 entries empty.
+    const double mma = (c.narrow ? 5.0 : (double)K * K * cin16 / 16) * tc_mma_cycles(c.Ns), units = c.Ns / 16.0;
     double best = -1;
-    for (int R = step; R <= r_max; R += step) {
-        const int bands = (H + R - 1) / R * c.ncc, nblk = (R * c.Wp + 127) / 128;
-        const long long items = (long long)N * bands * c.slices;
-        const double cost = (double)((items + kSmCount - 1) / kSmCount) * (nblk + 0.5);      // rounds x (MMAs + fixed part) of a block
-        if (best < 0 || cost <= best) { best = cost; c.R = R; c.nblk = nblk; c.bands_img = bands; }
-    }
-    const size_t entries = std::max<size_t>((size_t)(c.R + K - 1) * c.Wp, (size_t)c.nblk * 128 + (size_t)(K - 1) * c.Wp + K);
+    for (int rows = 0; rows <= (pool ? 1 : 0); ++rows)
+        for (int R = step; R <= (rows ? std::min(max_blk, H) / step * step : r_max); R += step) {
+            const int bands = (H + R - 1) / R * c.ncc, nblk = rows ? R : (R * c.Wp + 127) / 128;
+            const long long items = (long long)N * bands * c.slices;
+            const double m = nblk * mma, epi = nblk * units * (rows ? 430.0 : 550.0);
+            const double block = !pool ? nblk + 0.5 : (c.nbuf == 2 ? std::max(m, epi) : m + epi) + 0.5 * mma;      // MMAs + fixed part
+            const double cost = (double)((items + kSmCount - 1) / kSmCount) * block;                                     // x rounds
+            if (best < 0 || cost <= best) { best = cost; c.R = R; c.nblk = nblk; c.bands_img = bands; c.row_blocks = rows; }
+        }
+    if (best < 0) return c;
+    const size_t last = c.row_blocks ? (size_t)(c.nblk - 1) * c.Wp + 128 : (size_t)c.nblk * 128;          // entries the blocks reach over
+    const size_t entries = std::max<size_t>((size_t)(c.R + K - 1) * c.Wp, last + (size_t)(K - 1) * c.Wp + K);
     c.x_plane = (int)align_up(entries * 16, 128);
     c.stage_bytes = c.kpc * c.x_plane + (K * K + c.narrow) * c.kpc * c.Ns * 16;         // (narrow: a tenth window position of zeros)
     // fused pool: the band as stored goes through a staging area, all channels of the slice at once where that leaves
     // three stages (two for short rings), else 16 channels or more at a time
     const size_t room = (size_t)kTcConvSmemBudget - kTcFgHeader - (c.narrow ? 2048 : 0);
     const size_t plane_pair = (size_t)c.nblk * 128 * 16 * 2, whole = (size_t)(c.Ns / 16) * plane_pair;
-    size_t staging = pool ? kTcPoolStageBytes : 0;
+    const bool staged = pool && !c.row_blocks;
+    size_t staging = staged ? kTcPoolStageBytes : 0;
     c.stages = (int)std::min<size_t>(4, (room - staging) / c.stage_bytes);
-    if (pool) {
+    if (staged) {
         const int keep = std::min(c.stages, 3);
         if (room >= (size_t)keep * c.stage_bytes + whole) { c.stages = std::min<int>(c.stages, (int)((room - whole) / c.stage_bytes)); staging = whole; }
         else staging = std::max<size_t>(staging, (room - (size_t)c.stages * c.stage_bytes) / plane_pair * plane_pair);
         c.pool_planes = (int)(staging / plane_pair) * 2;
         c.pool_stage_bytes = (int)staging;
     }
-    if (c.stages < 2 || (pool && c.pool_planes < 2)) return c;
+    if (c.stages < 2 || (staged && c.pool_planes < 2)) return c;
     c.zero_off = c.stages * c.stage_bytes + (int)staging;
     c.smem_bytes = kTcFgHeader + c.zero_off + (c.narrow ? 2048 : 0);
     const long long items = (long long)N * c.bands_img * c.slices;

@@ -391,6 +391,7 @@ struct TcConvRowsArgs {
     // prev_arg = its pool's arg-max bytes or null, prev_slope = its leaky slope.  prev_y null: plain delta planes.
     const uint4* prev_y; const unsigned long long* prev_arg; float prev_slope;
     float* out_f;                             // fp32 NCHW output in the place of planes (delta at the network input), else null
+    int row_blocks, blk_step;                 // pool: an accumulator block per row of the band (else blocks of 128 consecutive entries); entries between blocks
     int narrow, zero_off;                     // first layer's forward pass: in is one plane of 8 channels; offset of 2 KB of zeros behind the stages
     int nbuf;                                 // accumulator buffers (2: items of at most 256 columns alternate between the halves
                                               //   of the tensor memory, so the MMAs of one run while the other is read back)
@@ -400,6 +401,73 @@ constexpr int kTcConvMaxStages = 4;
 constexpr int kTcConvEpiWarps = 16;           // four per lane quarter of the tensor memory
 constexpr int kTcConvEpiThreads = kTcConvEpiWarps * 32;
 constexpr int kTcConvThreads = (kTcConvEpiWarps + kTcIssuers + 1) * 32;
+
+// bias and leaky ReLU of 8 accumulators, rounded: both sides of the activation are formed and rounded, the rounded sum's sign picks
+// (3 instructions a value instead of 5.5: pairs are added, multiplied, rounded and selected together; an epilogue warp is bound by
+// instruction issue).
+__device__ __forceinline__ uint4 act8(const float* v, const float* bias, float slope)
+{
+    const float2 s2 = make_float2(slope, slope);
+    uint32_t o[4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const float4 b = *reinterpret_cast<const float4*>(bias + 4 * h);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const float2 z = __fadd2_rn(make_float2(v[4 * h + 2 * j], v[4 * h + 2 * j + 1]), j ? make_float2(b.z, b.w) : make_float2(b.x, b.y));
+            const float2 n = __fmul2_rn(z, s2);
+            const __nv_bfloat162 zb = __float22bfloat162_rn(z), nb = __float22bfloat162_rn(n);
+            const uint32_t m = __hgt2_mask(zb, __nv_bfloat162(__ushort_as_bfloat16(0), __ushort_as_bfloat16(0)));
+            o[2 * h + j] = (*reinterpret_cast<const uint32_t*>(&zb) & m) | (*reinterpret_cast<const uint32_t*>(&nb) & ~m);
+        }
+    }
+    return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+// 8 deltas times the derivative of the layer below (1 where its stored output y is positive, else its slope), rounded
+__device__ __forceinline__ uint4 derive8(const uint4& d, const uint4& y, float slope)
+{
+    const uint32_t dw[4] = {d.x, d.y, d.z, d.w}, yw[4] = {y.x, y.y, y.z, y.w};
+    const float2 s2 = make_float2(slope, slope);
+    uint32_t o[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float2 n = __fmul2_rn(make_float2(__uint_as_float(dw[j] << 16), __uint_as_float(dw[j] & 0xffff0000u)), s2);
+        const __nv_bfloat162 nb = __float22bfloat162_rn(n);
+        const uint32_t m = __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&yw[j]), __nv_bfloat162(__ushort_as_bfloat16(0), __ushort_as_bfloat16(0)));
+        o[j] = (dw[j] & m) | (*reinterpret_cast<const uint32_t*>(&nb) & ~m);
+    }
+    return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+// Two neighbouring entries, the first at an even index of a 256-byte aligned area.
+__device__ __forceinline__ void store_pair(uint4* dst, const uint4& a, const uint4& b)
+{
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 :: "l"(dst), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w) : "memory");
+}
+
+// 2x2 maximum of 8 channels (bf16 pairs, compared as stored, two channels per instruction): the first maximum in window order,
+// i.e. a later member wins only if it is greater; returns the members' numbers, a byte per channel.
+__device__ __forceinline__ unsigned long long pool4(const uint4& m0, const uint4& m1, const uint4& m2, const uint4& m3, uint4& best)
+{
+    const uint32_t w[4][4] = {{m0.x, m1.x, m2.x, m3.x}, {m0.y, m1.y, m2.y, m3.y}, {m0.z, m1.z, m2.z, m3.z}, {m0.w, m1.w, m2.w, m3.w}};
+    uint32_t val[4], code[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        uint32_t m = w[j][0], a = 0u;
+#pragma unroll
+        for (int k = 1; k < 4; ++k) {
+            const uint32_t gt = __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&w[j][k]), *reinterpret_cast<const __nv_bfloat162*>(&m));
+            m = (w[j][k] & gt) | (m & ~gt);
+            a = (((uint32_t)k * 0x00010001u) & gt) | (a & ~gt);
+        }
+        val[j] = m; code[j] = a;
+    }
+    best = make_uint4(val[0], val[1], val[2], val[3]);
+    // channel 2j in the low half of code[j], channel 2j + 1 in the high half
+    return (unsigned long long)__byte_perm(code[0], code[1], 0x6420) | ((unsigned long long)__byte_perm(code[2], code[3], 0x6420) << 32);
+}
 
 __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const __grid_constant__ TcConvRowsArgs A)
 {
@@ -413,7 +481,7 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
         uint32_t tmem_base;
         volatile int failed;
         volatile int epi_stop[2];       // the epilogue warps' common view of `failed` (they meet at named barriers), items in turn
-        float bias[128];
+        __align__(16) float bias[128];
     };
     static_assert(sizeof(Hdr) <= kTcFgHeader, "header does not fit");
     Hdr* H = reinterpret_cast<Hdr*>(cv_smem);
@@ -461,7 +529,7 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
         I.y0 = (bi / A.ncc) * A.R; I.x0 = (bi % A.ncc) * A.Cw;
         I.rows = min(A.R, A.H - I.y0); I.cw = min(A.Cw, A.W - I.x0);
         I.co0 = I.slice * A.Ns; I.cols = min(A.Ns, A.cout16 - I.co0);
-        I.nblk = (I.rows * A.Wp + 127) >> 7;
+        I.nblk = A.row_blocks ? I.rows : (I.rows * A.Wp + 127) >> 7;
         return I;
     };
     const uint32_t w_tap = (uint32_t)A.kpc * (uint32_t)A.Ns * 16u;                      // filter bytes of one window position
@@ -518,11 +586,11 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                     // (the thread that issues is the bottleneck of a narrow MMA: descriptors advance by adds only)
                     for (int b = iw; b < I.nblk; b += kTcIssuers) {
                         const uint32_t tcol = tmem + buf * 256u + (uint32_t)(b * A.Ns);
-                        const uint32_t a0 = desc_lo(xaddr + (uint32_t)b * 2048u, (uint32_t)A.x_plane);
+                        const uint32_t a0 = desc_lo(xaddr + (uint32_t)(b * A.blk_step) * 16u, (uint32_t)A.x_plane);
                         if (A.narrow) {
                             // one plane: a K step is two window positions (the second LBO entries behind the first), the last one's
                             // partner a block of zeros (an infinite pixel must not meet a zero weight)
-                            const uint32_t wp = (uint32_t)A.Wp, al = desc_lo(xaddr + (uint32_t)b * 2048u, 0), w2 = 2u * (uint32_t)A.Ns;
+                            const uint32_t wp = (uint32_t)A.Wp, al = desc_lo(xaddr + (uint32_t)(b * A.blk_step) * 16u, 0), w2 = 2u * (uint32_t)A.Ns;
                             const uint32_t last = al + 2 * wp + 2, zeros = desc_lo(smem_u32(stages + A.zero_off), 0);
                             mma_bf16(tcol, desc64(a_hi, al | (1u << 16)), desc64(b_hi, b_lo0), idesc, false);
                             mma_bf16(tcol, desc64(a_hi, (al + 2) | ((wp - 2) << 16)), desc64(b_hi, b_lo0 + w2), idesc, true);
@@ -617,17 +685,15 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                     }
                     float v[16];
                     tmem_ld16(tbuf + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * A.Ns + c0), v);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) { const float z = v[j] + H->bias[c0 + j]; v[j] = z > 0.f ? z : slope * z; }
-                    if (A.out_f) {
+                    if (A.out_f) {                            // (a delta: neither bias nor activation)
                         if (!valid) continue;
                         const int p = b * 128 + q * 32 + lane, r = p / A.Wp, c = p - r * A.Wp;
                         float* dst = A.out_f + (((size_t)I.n * A.cout + I.co0 + c0) * A.H + I.y0 + r) * A.W + I.x0 + c;
 #pragma unroll
                         for (int j = 0; j < 16; ++j) if (I.co0 + c0 + j < A.cout) dst[j * gstep] = v[j];
                     } else if (valid && !A.prev_y) {
-                        A.out[g0] = tcd::pack8(v);
-                        A.out[g0 + gstep] = tcd::pack8(v + 8);
+                        A.out[g0] = act8(v, H->bias + c0, slope);
+                        A.out[g0 + gstep] = act8(v + 8, H->bias + c0 + 8, slope);
                     } else if (valid) {
                         // input delta straight into the dz planes of the layer below: rounded as a stored delta
                         // would be, times the derivative of that layer's activation, through its pool's arg-max
@@ -635,26 +701,49 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                         const int r = p / A.Wp, c = p - r * A.Wp;
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            float d[8], yv[8];
-                            tcd::unpack8(tcd::pack8(v + 8 * h), d);
-                            tcd::unpack8(yq[h], yv);
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) d[j] *= yv[j] > 0.f ? 1.f : A.prev_slope;
-                            const uint4 dq = tcd::pack8(d);
+                            const uint4 dq = derive8(tcd::pack8(v + 8 * h), yq[h], A.prev_slope);
                             if (!A.prev_arg) { A.out[g0 + h * gstep] = dq; continue; }
                             // the four members of every channel's pool window: the delta where the arg-max byte names the
                             // member, zero elsewhere (byte masks widened to the bf16 halves)
                             const uint32_t alo = (uint32_t)amq[h] & 0x03030303u, ahi = (uint32_t)(amq[h] >> 32) & 0x03030303u;
                             const int W2 = 2 * A.W;
                             uint4* o2 = A.out + (((size_t)I.n * oplanes + ((I.co0 + c0) >> 3) + h) * (2 * A.H) + 2 * (I.y0 + r)) * W2 + 2 * (I.x0 + c);
-#pragma unroll
-                            for (int w = 0; w < 4; ++w) {
-                                const uint32_t ml = __vcmpeq4(alo, (uint32_t)w * 0x01010101u), mh = __vcmpeq4(ahi, (uint32_t)w * 0x01010101u);
-                                o2[(w >> 1) * W2 + (w & 1)] = make_uint4(dq.x & __byte_perm(ml, 0u, 0x1100), dq.y & __byte_perm(ml, 0u, 0x3322),
-                                                                         dq.z & __byte_perm(mh, 0u, 0x1100), dq.w & __byte_perm(mh, 0u, 0x3322));
-                            }
+                            // (a 32-byte store covers a whole sector; as two of 16 bytes: us of the launch 178 -> 146, 64 -> 32 channels to
+                            // 16 x 608 x 608; 95 -> 75, 128 -> 64 channels to 304 x 304)
+                            auto member = [&](uint32_t w) {
+                                const uint32_t ml = __vcmpeq4(alo, w * 0x01010101u), mh = __vcmpeq4(ahi, w * 0x01010101u);
+                                return make_uint4(dq.x & __byte_perm(ml, 0u, 0x1100), dq.y & __byte_perm(ml, 0u, 0x3322),
+                                                  dq.z & __byte_perm(mh, 0u, 0x1100), dq.w & __byte_perm(mh, 0u, 0x3322));
+                            };
+                            store_pair(o2, member(0), member(1));
+                            store_pair(o2 + W2, member(2), member(3));
                         }
                     }
+                }
+            } else if (A.row_blocks) {
+                // The rows of a window are the same lanes of two blocks and its columns two neighbouring lanes: no staging area and
+                // no barriers.  The even lane takes the lower 8 channels of a unit, the odd lane the upper ones.
+                // us, staged and so: 3 -> 32, 16 x 608 x 608 164 -> 143; 32 -> 64, 304 x 304 127 -> 101.
+                const int OH = A.H >> 1, OW = A.W >> 1, nc = I.cols >> 4, odd = lane & 1, col = q * 32 + lane;
+                const bool valid = (col & ~1) < I.cw;
+                for (int u = part; u < (I.rows >> 1) * nc; u += kParts) {
+                    const int pr = u / nc, c0 = (u - pr * nc) << 4;
+                    const uint32_t at = tbuf + ((uint32_t)(q * 32) << 16) + (uint32_t)(2 * pr * A.Ns + c0);
+                    float v[2][16];
+                    tmem_ld16x2(at, at + (uint32_t)A.Ns, v[0], v[1]);
+                    uint4 own[2], got[2];
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const uint4 lo = act8(v[r], H->bias + c0, slope), hi = act8(v[r] + 8, H->bias + c0 + 8, slope);
+                        own[r] = odd ? hi : lo;
+                        const uint4 away = odd ? lo : hi;
+                        got[r] = make_uint4(__shfl_xor_sync(0xffffffffu, away.x, 1), __shfl_xor_sync(0xffffffffu, away.y, 1),
+                                            __shfl_xor_sync(0xffffffffu, away.z, 1), __shfl_xor_sync(0xffffffffu, away.w, 1));
+                    }
+                    uint4 best;
+                    const unsigned long long am = odd ? pool4(got[0], own[0], got[1], own[1], best) : pool4(own[0], got[0], own[1], got[1], best);
+                    const size_t gi = (((size_t)I.n * oplanes + ((I.co0 + c0) >> 3) + odd) * OH + (I.y0 >> 1) + pr) * OW + (I.x0 >> 1) + (col >> 1);
+                    if (valid) { A.out[gi] = best; A.arg[gi] = am; }
                 }
             } else {
                 const int OH = A.H / 2, OW = A.W / 2, prs = I.rows / 2, pcs = I.cw / 2;
@@ -668,40 +757,21 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                         {
                             float v[16];
                             tmem_ld16(tbuf + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * A.Ns + c0), v);
-#pragma unroll
-                            for (int j = 0; j < 16; ++j) { const float z = v[j] + H->bias[c0 + j]; v[j] = z > 0.f ? z : slope * z; }
-                            S[(size_t)((c0 >> 3) - pl0) * E + p] = tcd::pack8(v);
-                            S[(size_t)((c0 >> 3) - pl0 + 1) * E + p] = tcd::pack8(v + 8);
+                            S[(size_t)((c0 >> 3) - pl0) * E + p] = act8(v, H->bias + c0, slope);
+                            S[(size_t)((c0 >> 3) - pl0 + 1) * E + p] = act8(v + 8, H->bias + c0 + 8, slope);
                         }
                     }
                     asm volatile("bar.sync 1, %0;" :: "n"(kTcConvEpiThreads) : "memory");
-                    // one thread per pooled pixel and plane; the four window members are compared as stored, two
-                    // channels (a bf16 pair) per instruction: a later member wins only if it is greater
+                    // one thread per pooled pixel and plane
                     const int npix = prs * pcs, total = npl * npix;
                     for (int e = et; e < total; e += kTcConvEpiThreads) {
                         const int pl = e / npix, pix = e - pl * npix, pr = pix / pcs, pc = pix - pr * pcs;
                         const uint4* s4 = S + (size_t)pl * E + (size_t)(2 * pr) * A.Wp + 2 * pc;
                         const uint4 m0 = s4[0], m1 = s4[1], m2 = s4[A.Wp], m3 = s4[A.Wp + 1];
-                        const uint32_t* w0 = &m0.x; const uint32_t* w1 = &m1.x; const uint32_t* w2 = &m2.x; const uint32_t* w3 = &m3.x;
-                        uint32_t best[4], code[4];
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            uint32_t m = w0[j], a = 0u;
-                            const uint32_t cand[3] = {w1[j], w2[j], w3[j]};
-#pragma unroll
-                            for (int w = 0; w < 3; ++w) {
-                                const uint32_t gt = __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&cand[w]),
-                                                                *reinterpret_cast<const __nv_bfloat162*>(&m));
-                                m = (cand[w] & gt) | (m & ~gt);
-                                a = (((uint32_t)(w + 1) * 0x00010001u) & gt) | (a & ~gt);
-                            }
-                            best[j] = m; code[j] = a;
-                        }
-                        // arg-max bytes: channel 2j in the low half of code[j], channel 2j + 1 in the high half
-                        const unsigned long long am = (unsigned long long)__byte_perm(code[0], code[1], 0x6420) |
-                                                      ((unsigned long long)__byte_perm(code[2], code[3], 0x6420) << 32);
+                        uint4 best;
+                        const unsigned long long am = pool4(m0, m1, m2, m3, best);
                         const size_t gi = (((size_t)I.n * oplanes + (I.co0 >> 3) + pl0 + pl) * OH + (I.y0 >> 1) + pr) * OW + (I.x0 >> 1) + pc;
-                        A.out[gi] = make_uint4(best[0], best[1], best[2], best[3]);
+                        A.out[gi] = best;
                         A.arg[gi] = am;
                     }
                     asm volatile("bar.sync 1, %0;" :: "n"(kTcConvEpiThreads) : "memory");    // the staging area is free for the next planes
