@@ -285,8 +285,8 @@ bool launch_tc_conv(ftp_plan* p, const TcConvPlan& c, int kind, int gi, const vo
     a.Ns = c.Ns; a.slices = c.slices; a.R = c.R; a.Wp = c.Wp; a.bands_img = c.bands_img; a.nblk = c.nblk; a.kpc = c.kpc;
     a.ncc = c.ncc; a.Cw = c.Cw; a.items = c.items; a.pool_planes = c.pool_planes; a.nbuf = c.nbuf;
     a.x_plane = c.x_plane; a.stage_bytes = c.stage_bytes; a.stages = c.stages;
-    a.out_f = out_f; a.row_blocks = c.row_blocks; a.blk_step = c.row_blocks ? c.Wp : 128; a.narrow = c.narrow; a.zero_off = c.zero_off;
-    a.hurry = (double)((c.items + c.blocks - 1) / c.blocks) * c.nblk * (c.narrow ? 5 : K * K * (cin16 / 16)) * tc_mma_cycles(c.Ns) < kHurryCycles;
+    a.out_f = out_f; a.row_blocks = c.row_blocks; a.stack = c.stack; a.blk_step = c.row_blocks ? c.Wp : 128;
+    a.hurry = (double)((c.items + c.blocks - 1) / c.blocks) * c.nblk * K * K * (cin16 / 16) * tc_mma_cycles(c.Ns) < kHurryCycles;
     { Timed tm(p, st, kind, gi);
       launch(conv_tc_rows_kernel, c.blocks, kTcConvThreads, one_block_smem(c.smem_bytes), tm.ls(), a); }
     return launched_ok();
@@ -364,9 +364,16 @@ int pack_filters_tc(ftp_plan* p, const float* params, void* ws, int dirs, cudaSt
                 continue;
             }
             if (ba.n == kPackTilesLayers) flush_banded();
-            add_pack_tiles(ba, PackTilesLayer{op.p_off, reinterpret_cast<uint4*>(wf + op.twf_off), reinterpret_cast<uint4*>(wb + op.twb_off),
-                                              op.cin, op.cout, op.k, g.narrow ? 8 : op.cin16, op.cout16,
-                                              g.cf.Ns, g.cf.kpc, g.cd.Ns, g.cd.kpc, 0});
+            PackTilesLayer l{op.p_off, reinterpret_cast<uint4*>(wf + op.twf_off), reinterpret_cast<uint4*>(wb + op.twb_off), op.cin, op.cout,
+                             op.k, op.cin16, op.cout16, g.cf.Ns, g.cf.kpc, g.cd.Ns, g.cd.kpc, 0, g.cd.stack, 0};
+            if (g.narrow) {                     // first layer: a 1x1 conv with 9 cin input channels in the forward pass, same parameters
+                PackTilesLayer f = l;
+                f.cin = 9 * op.cin; f.k = 1; f.cin16 = g.col_cin16; f.only = kPackForward;
+                add_pack_tiles(ba, f);
+                l.only = kPackDelta;
+            }
+            if (ba.n == kPackTilesLayers) flush_banded();
+            add_pack_tiles(ba, l);
         }
     flush();
     flush_banded();
@@ -386,17 +393,16 @@ int forward_tc(ftp_plan* p, const float* x, const float* params, float* y, void*
             const OpDesc& op = g.fwd_ops[0];
             const __nv_bfloat16* wf = reinterpret_cast<const __nv_bfloat16*>(ws_ptr(ws, p->ws.wf_off)) + op.twf_off;
             const void* in = a.map[0];
-            if (g.narrow) {                     // first layer
+            if (g.narrow) {                     // first layer: a 1x1 conv on the window-unrolled network input
                 uint4* col = reinterpret_cast<uint4*>(ws_ptr(ws, p->ws.col_off));
-                const size_t HW = (size_t)op.in_H * op.in_W;
                 { Timed t(p, st, 9, (int)gi);
-                  launch(input_entries_kernel, (int)std::min<size_t>((p->N * HW + 255) / 256, (size_t)kSmCount * 16), 256, 0, t.ls(),
-                         x, col, p->N, op.cin, HW); }
+                  launch_unroll_windows(x, col, (pack & kPackDelta) ? reinterpret_cast<uint4*>(ws_ptr(ws, p->ws.ent_off)) : nullptr, p->N, op.cin,
+                                        op.in_H, op.in_W, t.ls()); }
                 if (!launched_ok()) return FTP_ERR_CUDA;
                 in = col;
             }
             if (!launch_tc_conv(p, g.cf, 1, (int)gi, in, wf, params + op.p_off + (size_t)op.cout * op.cin * op.k * op.k,
-                                a.map_out[1], a.arg[0], g.tfg.k, g.narrow ? 8 : op.cin16, op.cout16, op.cout, op.in_H, op.in_W,
+                                a.map_out[1], a.arg[0], g.narrow ? 1 : g.tfg.k, g.narrow ? g.col_cin16 : op.cin16, op.cout16, op.cout, op.in_H, op.in_W,
                                 op.kind == kOpConvPool, op.slope, a.error, st))
                 return FTP_ERR_CUDA;
             continue;
@@ -704,8 +710,8 @@ bool tc_filter_grad(ftp_plan* p, const GroupPlan& g, int gi, const TcGroupArgs& 
 {
     const OpDesc& op = g.bwd_ops[0];
     const TcFgPlan& t = g.tfg;
-    // the layer's input as bf16 planes: the saved map, or (first layer) what the forward pass made of the network input
-    void* xin = g.narrow ? static_cast<void*>(ws_ptr(ws, p->ws.col_off)) : const_cast<void*>(a.map[0]);
+    // the layer's input as bf16 planes: the saved map, or (first layer) the entries of the network input
+    void* xin = g.narrow ? static_cast<void*>(ws_ptr(ws, p->ws.ent_off)) : const_cast<void*>(a.map[0]);
     const int cin16 = op.cin16;
     // dz planes: the two areas take turns; when the group above is a one-conv group too, its input-delta kernel has
     // already written this group's dz (see below), otherwise delta_act_planes_kernel makes them from the stored delta
@@ -731,7 +737,8 @@ bool tc_filter_grad(ftp_plan* p, const GroupPlan& g, int gi, const TcGroupArgs& 
 
     TcFilterGradArgs f{};
     if (!encode_band_map(f.tmap_dz, dz, p->N, op.cout16 / 8, op.in_H, op.in_W, false, t.Cw, t.R, t.dz_box) ||
-        !encode_band_map(f.tmap_x, xin, p->N, g.narrow ? 1 : cin16 / 8, op.in_H, op.in_W, true, t.Cw + t.k - 1, t.R + t.k - 1, t.ncols / 8)) return false;
+        !encode_band_map(f.tmap_x, xin, p->N, g.narrow ? 1 : cin16 / 8, op.in_H, op.in_W, true, g.narrow ? t.Cw : t.Cw + t.k - 1,
+                         g.narrow ? 1 : t.R + t.k - 1, t.ncols / 8)) return false;
     f.partial = a.partial; f.set_floats = a.set_floats; f.tgp_off = op.tgp_off;
     f.error = a.error;
     f.K = t.k; f.H = op.in_H; f.W = op.in_W; f.cout16 = op.cout16; f.cin16 = g.narrow ? t.ncols : cin16; f.narrow = g.narrow;
@@ -1053,6 +1060,14 @@ int ftp_backward(ftp_plan* plan, const float* x, const float* dy, const float* p
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     rc = is_tc(plan) ? pack_filters_tc(plan, params, workspace, kPackDelta, st) : pack_filters(plan, params, workspace, kPackDelta, st);
     if (rc != FTP_OK) return rc;
+    const GroupPlan& g = plan->groups.front();
+    if (g.narrow) {                             // (a step's forward pass writes them along with its own copy)
+        const OpDesc& op = g.bwd_ops[0];
+        const size_t HW = (size_t)op.in_H * op.in_W;
+        Timed t(plan, st, 10, 0);
+        launch(input_entries_kernel, (int)std::min<size_t>((plan->N * HW + 255) / 256, (size_t)kSmCount * 16), 256, 0, t.ls(),
+               x, reinterpret_cast<uint4*>(ws_ptr(workspace, plan->ws.ent_off)), plan->N, op.cin, HW);
+    }
     return backward_impl(plan, x, dy, params, dx, dparams, nullptr, 0.f, workspace, st);
 }
 

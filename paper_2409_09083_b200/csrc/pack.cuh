@@ -35,7 +35,7 @@ __device__ __forceinline__ void pack_tile(const PackTilesLayer L, int t, int dir
         const bool fwd = i < total;
         const int j = fwd ? i : i - total, r = j & 31, o = (j >> 5) & 3, tap = j >> 7;   // row of the operand, octet of contraction channels
         const int row = (fwd ? co0 : ci0) + r, k0 = (fwd ? ci0 : co0) + o * 8;
-        if (row >= (fwd ? L.cout16 : max(L.cin16, 16)) || k0 >= (fwd ? L.cin16 : L.cout16)) continue;
+        if (row >= (fwd ? L.cout16 : L.cin16) || k0 >= (fwd ? L.cin16 : L.cout16)) continue;
         const int ns = fwd ? L.ns_f : L.ns_d, kpc = fwd ? L.kpc_f : L.kpc_d;
         const int nch = ((fwd ? L.cin16 : L.cout16) / 8 + kpc - 1) / kpc;
         float v[8];
@@ -45,7 +45,8 @@ __device__ __forceinline__ void pack_tile(const PackTilesLayer L, int t, int dir
         parts(v, p);
         const int sl = row / ns, rr = row - sl * ns, kp = k0 / 8, ch = kp / kpc, kj = kp - ch * kpc;
         const size_t stage = (size_t)KK * kpc * ns;
-        uint4* dst = (fwd ? L.wf : L.wd) + ((size_t)sl * nch + ch) * PARTS * stage + ((size_t)tap * kpc + kj) * ns + rr;
+        const size_t at = !fwd && L.stack_d ? (size_t)(tap % 3 * kpc + kj) * 3 + (2 - tap / 3) : (size_t)tap * kpc + kj;
+        uint4* dst = (fwd ? L.wf : L.wd) + ((size_t)sl * nch + ch) * PARTS * stage + at * ns + rr;
 #pragma unroll
         for (int q = 0; q < PARTS; ++q) dst[q * stage] = p[q];
     }
@@ -58,9 +59,10 @@ __device__ __forceinline__ void pack_tiles(const PackTilesArgs& A, const float* 
     int l = 0;
     while (l + 1 < A.n && (int)blockIdx.x >= A.l[l + 1].tile_begin) ++l;
     const PackTilesLayer L = A.l[l];                          // (a copy: through a reference every field is a memory load)
-    const int t = (int)blockIdx.x - L.tile_begin;
-    if (L.k == 3) pack_tile<9, PARTS>(L, t, A.dirs, params, s, parts);
-    else pack_tile<1, PARTS>(L, t, A.dirs, params, s, parts);
+    const int t = (int)blockIdx.x - L.tile_begin, dirs = L.only ? A.dirs & L.only : A.dirs;
+    if (!dirs) return;
+    if (L.k == 3) pack_tile<9, PARTS>(L, t, dirs, params, s, parts);
+    else pack_tile<1, PARTS>(L, t, dirs, params, s, parts);
 }
 
 constexpr int kPackSmemFloats = 32 * (32 * 9 + 1);

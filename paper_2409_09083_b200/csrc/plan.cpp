@@ -506,11 +506,11 @@ double tc_stationary_estimate_us(const ftp_plan& p, const GroupPlan& g, bool bac
 {
     const OpDesc& op = g.fwd_ops[0];
     const double px = (double)p.N * op.in_H * op.in_W;
-    const int cin16 = g.narrow ? 8 : op.cin16, kk = op.k * op.k;
+    const int cin16 = g.narrow ? g.col_cin16 : op.cin16, kk = g.narrow ? 1 : op.k * op.k;
     const double flops = 2.0 * px * cin16 * op.cout16 * kk;
     auto rate = [](int ns) { return 800e6 * std::min(1.0, std::max(ns, 16) / 80.0); };           // flop per microsecond
     const double in_b = px * cin16 * 2.0, out_b = px * op.cout16 * 2.0 / (op.kind == kOpConvPool ? 4.0 : 1.0), dz_b = px * op.cout16 * 2.0;
-    if (!backward) return flops / rate(g.cf.Ns) + (in_b + out_b) / 5e6 + (g.narrow ? 1.5 * in_b / 5e6 : 0.0) + 8.0;
+    if (!backward) return flops / rate(g.cf.Ns) + (in_b + out_b) / 5e6 + (g.narrow ? in_b / 3e6 : 0.0) + 8.0;
     double t = (2.0 * out_b + dz_b) / 5e6 + 4.0;                                               // dz planes
     t += flops / 600e6 + (in_b + dz_b) / 5e6 + 10.0;                                           // filter gradient
     if (need_dx) t += flops / rate(g.cd.Ns) + (in_b + dz_b) / 5e6 + 8.0;
@@ -813,7 +813,7 @@ bool tc_stationary_conv(const ftp_plan& p, int li /*0-based*/, const PlanOpts& o
 {
     const ftp_layer& l = p.layers[li];
     if (p.precision != FTP_BF16_FP32ACC || o.stationary < 0 || l.kind != FTP_CONV) return false;
-    // the first layer reads the fp32 network input: only as 8-channel entries with a spare channel (3x3, at most 7 channels)
+    // the first layer reads the fp32 network input: only as a window-unrolled copy and as 8-channel entries with a spare channel (3x3, at most 7 channels)
     if (li == 0 && (l.k != 3 || l.cin > 7)) return false;
     return (l.k == 1 || l.k == 3) && p.maps[li].W <= kTcMaxColChunks * 126;
 }
@@ -830,7 +830,7 @@ void tc_col_chunks(int W, int* ncc, int* Cw)
 // Launch shape of the banded convolution kernel for a conv with `cout16` output and `cin16` input channels (padded)
 // on N maps of H x W: bands as tall as the accumulators allow (512 columns = blocks of 128 entries x Ns channels),
 // among those the height with the fewest rounds of blocks over the SMs; as many stages as fit.
-TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, bool pool, int kpc3);
+TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, bool pool, int kpc3, bool stack = false);
 
 TcConvPlan plan_tc_conv(int N, int H, int W, int K, int cin16, int cout16, bool pool)
 {
@@ -843,7 +843,7 @@ TcConvPlan plan_tc_conv(int N, int H, int W, int K, int cin16, int cout16, bool 
     return plan_tc_conv_kpc(N, H, W, K, cin16, cout16, pool, 2);
 }
 
-TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, bool pool, int kpc3)
+TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, bool pool, int kpc3, bool stack)
 {
     TcConvPlan c;
     tc_col_chunks(W, &c.ncc, &c.Cw);
@@ -853,22 +853,23 @@ TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, b
     // slices of at most 64 channels: items of 256 columns in two alternating buffers (narrow MMAs leave the tensor
     // core idle while an item is read back); wider slices: one buffer of 512 columns (their filters are read per item)
     c.nbuf = c.Ns <= 64 ? 2 : 1;
-    const int max_blk = std::min(8, kTcTmemCols / c.nbuf / c.Ns);
+    const int max_blk = std::min(stack ? 16 : 8, kTcTmemCols / c.nbuf / c.Ns);
+    c.stack = stack ? 1 : 0;
     c.kpc = K == 1 ? std::min(cin16 / 8, 8) : kpc3;
-    c.narrow = cin16 == 8 ? 1 : 0;
     const int step = pool ? 2 : 1;
     const int r_max = std::min((max_blk * 128) / c.Wp, H) / step * step;
-    // With a pool, accumulator blocks of one row each where that is the faster form: the epilogue then compares in registers (430
-    // cycles for 128 entries x 16 channels instead of 550 through the staging area), while rows of few columns
+    // With a pool, accumulator blocks of one row each where that is the faster form: the epilogue then compares in registers (350
+    // cycles for 128 entries x 16 channels instead of 500 through the staging area), while rows of few columns
     // leave most of a block's 128 entries empty.
-    const double mma = (c.narrow ? 5.0 : (double)K * K * cin16 / 16) * tc_mma_cycles(c.Ns), units = c.Ns / 16.0;
+    const double mma = (double)K * K * cin16 / 16 * tc_mma_cycles(c.Ns), units = c.Ns / 16.0;
     double best = -1;
-    for (int rows = 0; rows <= (pool ? 1 : 0); ++rows)
+    for (int rows = stack ? 1 : 0; rows <= (pool || stack ? 1 : 0); ++rows)
         for (int R = step; R <= (rows ? std::min(max_blk, H) / step * step : r_max); R += step) {
             const int bands = (H + R - 1) / R * c.ncc, nblk = rows ? R : (R * c.Wp + 127) / 128;
             const long long items = (long long)N * bands * c.slices;
-            const double m = nblk * mma, epi = nblk * units * (rows ? 430.0 : 550.0);
-            const double block = !pool ? nblk + 0.5 : (c.nbuf == 2 ? std::max(m, epi) : m + epi) + 0.5 * mma;      // MMAs + fixed part
+            const double m = nblk * mma, epi = nblk * units * (rows ? 350.0 : 500.0);
+            const double block = stack ? R + 1.5 * ((R + 3) / 4) + 1.0             // (64 + 44 n cycles a K step and window column for n rows of an issuer)
+                               : !pool ? nblk + 0.5 : (c.nbuf == 2 ? std::max(m, epi) : m + epi) + 0.5 * mma + 1000.0;      // MMAs + fixed part
             const double cost = (double)((items + kSmCount - 1) / kSmCount) * block;                                     // x rounds
             if (best < 0 || cost <= best) { best = cost; c.R = R; c.nblk = nblk; c.bands_img = bands; c.row_blocks = rows; }
         }
@@ -876,10 +877,10 @@ TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, b
     const size_t last = c.row_blocks ? (size_t)(c.nblk - 1) * c.Wp + 128 : (size_t)c.nblk * 128;          // entries the blocks reach over
     const size_t entries = std::max<size_t>((size_t)(c.R + K - 1) * c.Wp, last + (size_t)(K - 1) * c.Wp + K);
     c.x_plane = (int)align_up(entries * 16, 128);
-    c.stage_bytes = c.kpc * c.x_plane + (K * K + c.narrow) * c.kpc * c.Ns * 16;         // (narrow: a tenth window position of zeros)
+    c.stage_bytes = c.kpc * c.x_plane + K * K * c.kpc * c.Ns * 16;
     // fused pool: the band as stored goes through a staging area, all channels of the slice at once where that leaves
     // three stages (two for short rings), else 16 channels or more at a time
-    const size_t room = (size_t)kTcConvSmemBudget - kTcFgHeader - (c.narrow ? 2048 : 0);
+    const size_t room = (size_t)kTcConvSmemBudget - kTcFgHeader;
     const size_t plane_pair = (size_t)c.nblk * 128 * 16 * 2, whole = (size_t)(c.Ns / 16) * plane_pair;
     const bool staged = pool && !c.row_blocks;
     size_t staging = staged ? kTcPoolStageBytes : 0;
@@ -892,8 +893,7 @@ TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, b
         c.pool_stage_bytes = (int)staging;
     }
     if (c.stages < 2 || (staged && c.pool_planes < 2)) return c;
-    c.zero_off = c.stages * c.stage_bytes + (int)staging;
-    c.smem_bytes = kTcFgHeader + c.zero_off + (c.narrow ? 2048 : 0);
+    c.smem_bytes = kTcFgHeader + c.stages * c.stage_bytes + (int)staging;
     const long long items = (long long)N * c.bands_img * c.slices;
     if (items > 0x7fffffffLL) return c;
     c.items = (int)items;
@@ -927,18 +927,21 @@ void plan_tc_filter_grad(const ftp_plan& p, GroupPlan& g, const PlanOpts& o)
         c.ncols = round_up((op.cin16 + c.nci - 1) / c.nci, 16);
         if (c.ncols > most) continue;
         if (narrow && t.Ms == 64) c.ncols = 8;                   // (with 128 rows an MMA has multiples of 16 columns)
-        const int wide = K * c.ncols, roles = c.slices * c.nci, max_g = (128 - (K - 1)) / 8, groups = (W + 7) / 8;
-        c.units = K == 3 || 3 * wide + 16 <= kTcTmemCols ? 3 : 1;
-        const double operands = (c.Ms + wide) * 32.0 / 128.0, mma = (K == 3 ? 3.0 : 1.0) * std::max(wide / 2.0, operands) + (narrow ? 0.0 : (c.Ms + 16) * 0.25 / c.nci);
+        const int wide = (narrow ? 9 : K) * c.ncols, roles = c.slices * c.nci, max_g = narrow ? 16 : (128 - (K - 1)) / 8, groups = (W + 7) / 8;
+        c.units = (K == 3 && !narrow) || 3 * wide + 16 <= kTcTmemCols ? 3 : 1;
+        const double operands = (c.Ms + wide) * 32.0 / 128.0, mma = (K == 3 && !narrow ? 3.0 : 1.0) * std::max(wide / 2.0, operands) + (narrow ? 0.0 : (c.Ms + 16) * 0.25 / c.nci);
         const double set_cost = (double)(K * K * op.cin16 + 1) * op.cout16 * 8.0 / 5e6 * 1900.0;
         for (int ncc = (groups + max_g - 1) / max_g, end = ncc + 4; ncc <= std::min(groups, end); ++ncc) {
             c.Cw = (groups + ncc - 1) / ncc * 8;
             c.ncc = (W + c.Cw - 1) / c.Cw;
             for (c.R = 2; c.R <= std::min(round_up(H, 2), 64); c.R += 2) {
-                c.x_off = (int)align_up((size_t)(c.Ms / 8) * c.R * c.Cw * 16, 128);
-                const size_t xb = (size_t)(c.ncols / 8) * (c.R + K - 1) * (c.Cw + K - 1) * 16;
+                // (rows of no channel read on into the input tile: a stage holds the planes that are copied, so that more of them
+                // are on their way: 32 channels at 608 x 608, 16 images, 126 -> 101 us)
+                const size_t dz_plane = (size_t)c.R * c.Cw * 16;
+                c.x_off = (int)align_up(c.dz_box * dz_plane, 128);
+                const size_t xb = (size_t)(c.ncols / 8) * (c.R + K - 1) * (narrow ? 3 * c.Cw : c.Cw + K - 1) * 16;
                 c.stage_bytes = (int)align_up((size_t)c.x_off + xb, 128);
-                c.smem_bytes = kTcFgHeader + 2 * c.stage_bytes;
+                c.smem_bytes = kTcFgHeader + c.stage_bytes + (int)std::max<size_t>(c.stage_bytes, c.Ms / 8 * dz_plane);
                 if (c.smem_bytes > kTcFgSmemBudget) break;
                 c.bands_img = (H + c.R - 1) / c.R * c.ncc;
                 const long long bands = (long long)p.N * c.bands_img;
@@ -957,11 +960,17 @@ void plan_tc_filter_grad(const ftp_plan& p, GroupPlan& g, const PlanOpts& o)
     if (best < 0) return;
     t.blocks = t.slices * t.nci * t.shares;
     // the forward convolution, and the input delta as the convolution of dz (cout16 channels) with the rotated filters
-    g.cf = narrow ? plan_tc_conv_kpc(p.N, H, W, K, 8, op.cout16, op.kind == kOpConvPool, 1)
-                  : plan_tc_conv(p.N, H, W, K, op.cin16, op.cout16, op.kind == kOpConvPool);
+    const int col_cin16 = round_up(9 * op.cin, 16);
+    g.cf = plan_tc_conv(p.N, H, W, narrow ? 1 : K, narrow ? col_cin16 : op.cin16, op.cout16, op.kind == kOpConvPool);
     g.cd = plan_tc_conv(p.N, H, W, K, op.cout16, op.cin16, false);
+    // delta at the network input (16 columns): with the window rows in one MMA where the rows are long enough.  A row, a block of 128
+    // entries whatever its length, costs 180 cycles a K step so; otherwise 128 entries cost 324, whole rows or not.
+    if (narrow && g.cd.on && g.cd.Wp >= 80) {
+        const TcConvPlan c = plan_tc_conv_kpc(p.N, H, W, K, op.cout16, op.cin16, false, 2, true);
+        if (c.on) g.cd = c;
+    }
     if (!g.cf.on || !g.cd.on) return;
-    g.narrow = narrow ? 1 : 0;
+    g.narrow = narrow ? 1 : 0; g.col_cin16 = narrow ? col_cin16 : 0;
     t.on = 1;
     g.tfg = t;
     g.param_floats += (size_t)(t.nci - 1) * op.cout16;          // the bias gradient comes in parts, one per slice of the input channels
@@ -1368,7 +1377,10 @@ int build_plan(ftp_plan& p, const ftp_layer* layers, int n_layers, int N, int C,
         if (g.tfg.on) dz[gi & 1] = std::max(dz[gi & 1], (size_t)N * g.fwd_ops[0].cout16 * g.fwd_ops[0].in_H * g.fwd_ops[0].in_W * 2);
     }
     ws.scratch_off = take(scratch * 4);
-    if (!p.groups.empty() && p.groups[0].narrow) ws.col_off = take((size_t)N * H * W * 16);
+    if (!p.groups.empty() && p.groups[0].narrow) {
+        ws.col_off = take((size_t)N * p.groups[0].col_cin16 * H * W * 2);
+        ws.ent_off = take((size_t)N * H * W * 16);
+    }
     ws.dz_bytes = align_up(dz[0], 256);             // = offset of the second area
     ws.dz_off = take(ws.dz_bytes + align_up(dz[1], 256));
     ws.wf_off = take(p.wf_floats * (tcp ? 2 : 4));

@@ -156,7 +156,7 @@ struct TcConvPlan {
     int blocks = 0;                         // persistent blocks: min(items, SMs)
     int pool_planes = 0;                    // fused pool: 8-channel planes the staging area holds
     int pool_stage_bytes = 0;               //             and its size
-    int narrow = 0, zero_off = 0, row_blocks = 0;   // see TcConvRowsArgs
+    int row_blocks = 0, stack = 0;          // see TcConvRowsArgs
     int nbuf = 1;                           // accumulator buffers (2 for slices of at most 64 channels)
 };
 constexpr int kTcPoolStageBytes = 32 * 1024;  // least staging area of the fused pool in the banded convolution (more where it fits)
@@ -203,9 +203,10 @@ struct GroupPlan {
     TcFgPlan tfg;
     TcConvPlan cf, cd;              // tfg.on: the forward convolution and the input-delta convolution (dz planes in, delta planes
                                     //   out: the conv with the channel counts exchanged and the filters rotated) as banded kernels
-    // First layer of the bf16 path (3x3, at most 7 channels): its one-conv kernels read the network input as one plane of
-    // 8-channel entries (input_entries_kernel)
-    int narrow = 0;
+    // First layer of the bf16 path (3x3, at most 7 channels).  Forward pass: a 1x1 conv with 9 cin input channels on a window-unrolled
+    // copy of the network input (channel ci * 9 + ky * 3 + kx of a pixel = the input of channel ci at window position (ky, kx));
+    // W[co][ci][ky][kx] is W'[co][ci * 9 + ky * 3 + kx].  Backward pass: the 3x3 conv, on entries of 8 channels.
+    int narrow = 0, col_cin16 = 0;      // 1 on this route; 9 cin padded to 16
     int sets() const { return tfg.on ? tfg.shares : sp.on ? sp.g.shares : bwd.blocks; }   // partial gradient sets the reduction sums
     int n_ops = 0;
     OpDesc fwd_ops[kMaxOps];
@@ -228,7 +229,7 @@ struct Workspace {                 // byte offsets, all 256-aligned
     std::vector<size_t> dmap_off;  // delta maps at group inputs of groups 1.. (index = group), and slot for dY
     size_t dy_off = 0;             // loss delta at the last map (ftp_step with target)
     size_t scratch_off = 0;
-    size_t col_off = 0;                // first layer of the bf16 path: the network input as one plane of 8-channel entries
+    size_t col_off = 0, ent_off = 0;   // first layer of the bf16 path: the window-unrolled network input, and its 8-channel entries
     size_t dz_off = 0, dz_bytes = 0;   // one-conv groups: two areas (taken in turn, the second dz_bytes behind the first) for the
                                        // delta in front of the activation at the conv's resolution
     size_t wf_off = 0, wb_off = 0; // packed filters

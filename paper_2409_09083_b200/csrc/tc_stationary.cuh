@@ -47,7 +47,8 @@ struct TcFilterGradArgs {
     int Ms, slices;                           // output channels per block (64 or 128) and number of such slices
     int ncols, nci;                           // input channels per block (multiple of 16) and number of such slices
     int narrow;                               // first layer: x is input_entries_kernel's plane (ncols 8 or 16, the bias gradient its channel 7)
-    int units;                                // accumulator units of K * ncols columns: 3x3: one per window column; 1x1: row pairs in turn
+    int units;                                // accumulator units: 3x3: K * ncols columns, one per window column; 1x1 and the first
+                                              //   layer (9 * ncols columns): row pairs in turn
     int R, Cw, ncc;                           // rows per band, columns of a band and column chunks per row band
     int bands_img, bands, shares;             // bands per image / in the batch, pixel shares
     int dz_box, x_off, stage_bytes;           // dz planes a copy brings, offset of the input tile in a stage, bytes of a stage
@@ -157,11 +158,68 @@ __global__ void __launch_bounds__(256) loss_planes_kernel(const __grid_constant_
     if (threadIdx.x == 0) A.block_sums[blockIdx.x] = red[0];
 }
 
-// First layer (at most 7 channels): the fp32 network input [N][C][H][W] -> one plane of 8-channel bf16 entries, channels
-// beyond C zero, the last one 1 (the filter gradient's sums of dz x that channel at the window's centre are the bias gradient; its
-// forward weights are zero).  16 bytes a pixel; the window-unrolled copy that stood here before (9 C channels, 64 bytes a
-// pixel with 3) was written once and read twice at four times the size: us for 16 x 608 x 608, 3 -> 32 channels,
-// copy / forward / filter gradient / input delta (and fold): 99 / 152 / 144 / 240 -> 34 / 152 / 142 / 166.
+// First layer: the fp32 network input [N][C][H][W] -> window-unrolled bf16 planes [N][C16'/8][H][W][8] with channel
+// ci * 9 + ky * 3 + kx of pixel (y, x) = input(ci, y + ky - 1, x + kx - 1) (zero outside the map and beyond 9 C).
+// One thread per pixel: it reads the 9 C values of its window once and writes its entry of every plane (the
+// channel -> (ci, ky, kx) arithmetic is resolved at compile time).  On that copy the forward pass is a 1x1 conv.  (On the entries
+// below it is a 3x3 conv without the copy, 99 us less for 16 x 608 x 608, but the sums of an MMA are then other ones, a few
+// rounded outputs in a million with them, and through the ties of the pools whole deltas at the network input.)
+// ent, if not null: the entries for the backward pass (see input_entries_kernel), written in the same pass.
+template <int C>
+__global__ void unroll_windows_kernel(const float* __restrict__ x, uint4* __restrict__ col, uint4* __restrict__ ent, int N, int H, int W)
+{
+    previous_launches();
+    constexpr int planes = (9 * C + 15) / 16 * 2;
+    const size_t HW = (size_t)H * W, total = (size_t)N * HW;
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
+        const int px = (int)(e % W); size_t t = e / W;
+        const int py = (int)(t % H); const int n = (int)(t / H);
+        float v[planes * 8];
+        const float* ctr = x + (size_t)n * C * HW + (size_t)py * W + px;       // this pixel in channel 0
+        if (py > 0 && py < H - 1 && px > 0 && px < W - 1) {                    // the whole window lies inside the map
+#pragma unroll
+            for (int j = 0; j < planes * 8; ++j) {
+                const int ci = j / 9, tap = j - ci * 9, ky = tap / 3, kx = tap - ky * 3;
+                v[j] = ci < C ? __ldg(ctr + (size_t)ci * HW + (ky - 1) * W + (kx - 1)) : 0.f;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < planes * 8; ++j) {
+                const int ci = j / 9, tap = j - ci * 9, ky = tap / 3, kx = tap - ky * 3;
+                const int yy = py + ky - 1, xx = px + kx - 1;
+                v[j] = (ci < C && yy >= 0 && yy < H && xx >= 0 && xx < W) ? __ldg(ctr + (size_t)ci * HW + (ky - 1) * W + (kx - 1)) : 0.f;
+            }
+        }
+#pragma unroll
+        for (int pl = 0; pl < planes; ++pl) col[((size_t)n * planes + pl) * HW + (size_t)py * W + px] = tcd::pack8(v + 8 * pl);
+        if (ent) {
+            float c[8];
+#pragma unroll
+            for (int ci = 0; ci < 7; ++ci) c[ci] = ci < C ? v[ci < C ? ci * 9 + 4 : 0] : 0.f;
+            c[7] = 1.f;
+            ent[e] = tcd::pack8(c);
+        }
+    }
+}
+
+// for the channel counts the route takes (9 C <= 64)
+inline void launch_unroll_windows(const float* x, uint4* col, uint4* ent, int N, int C, int H, int W, LaunchStream st)
+{
+    const int blocks = (int)std::min<size_t>(((size_t)N * H * W + 255) / 256, (size_t)kSmCount * 16);
+    switch (C) {
+        case 1: launch(unroll_windows_kernel<1>, blocks, 256, 0, st, x, col, ent, N, H, W); break;
+        case 2: launch(unroll_windows_kernel<2>, blocks, 256, 0, st, x, col, ent, N, H, W); break;
+        case 3: launch(unroll_windows_kernel<3>, blocks, 256, 0, st, x, col, ent, N, H, W); break;
+        case 4: launch(unroll_windows_kernel<4>, blocks, 256, 0, st, x, col, ent, N, H, W); break;
+        case 5: launch(unroll_windows_kernel<5>, blocks, 256, 0, st, x, col, ent, N, H, W); break;
+        case 6: launch(unroll_windows_kernel<6>, blocks, 256, 0, st, x, col, ent, N, H, W); break;
+        default: launch(unroll_windows_kernel<7>, blocks, 256, 0, st, x, col, ent, N, H, W); break;
+    }
+}
+
+// First layer's backward pass: the network input as one plane of 8-channel bf16 entries, channels beyond C zero, the last one 1 (the
+// filter gradient's sums of dz x that channel at the window's centre are the bias gradient).  16 bytes a pixel where the
+// unrolled copy, which the filter gradient read before, has 64 with 3 channels.  A step has it from the kernel above.
 __global__ void __launch_bounds__(256) input_entries_kernel(const float* __restrict__ x, uint4* __restrict__ out, int N, int C, size_t HW)
 {
     previous_launches();
@@ -199,10 +257,14 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
     const int nroles = A.slices * A.nci;
     const int role = (int)blockIdx.x % nroles, share = (int)blockIdx.x / nroles;
     const int slice = role / A.nci, cs = role - slice * A.nci;
-    const int ci0 = cs * A.ncols, cols = min(A.ncols, A.cin16 - ci0), wide = K * A.ncols;
+    const int ci0 = cs * A.ncols, cols = min(A.ncols, A.cin16 - ci0), wide = (A.narrow ? 9 : K) * A.ncols;
     const int b_lo = (int)((long long)share * A.bands / A.shares), b_hi = (int)((long long)(share + 1) * A.bands / A.shares);
     const int nb = b_hi - b_lo;
-    const int np = A.ncols / 8, Wx = A.Cw + K - 1;                       // planes and row pitch of the input tile
+    // input tile: planes, entries of a plane's row, entries from row to row.  First layer: each row three times, shifted by the window
+    // column, in the place of planes, so that all nine window positions of its few channels stand at one stride and share an
+    // MMA (three MMAs of 24 columns took 37 cycles each: 142 us a launch for 16 x 608 x 608, 3 -> 32, now 101, 473 MB).
+    const bool turns = K == 1 || A.narrow;
+    const int np = A.ncols / 8, Wx = A.narrow ? A.Cw : A.Cw + K - 1, pitch = (A.narrow ? 3 : 1) * np * Wx;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&H->full[s]), 1); mbar_init(smem_u32(&H->empty[s]), kTcIssuers); }
@@ -247,9 +309,14 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
             int n, y0, x0;
             band_of(b_lo + i, n, y0, x0);
             const uint32_t dst = smem_u32(stages + (size_t)s * A.stage_bytes), bar = smem_u32(&H->full[s]);
-            mbar_expect_tx(bar, (uint32_t)(A.dz_box * A.R * A.Cw + np * (A.R + K - 1) * Wx) * 16u);
+            mbar_expect_tx(bar, (uint32_t)(A.dz_box * A.R * A.Cw + (A.R + K - 1) * pitch) * 16u);
             tma_load_4d(dst, A.tmap_dz, 2 * x0, y0, slice * (A.Ms / 8), n, bar);
-            tma_load_4d(dst + (uint32_t)A.x_off, A.tmap_x, 2 * (x0 - K / 2), ci0 / 8, y0 - K / 2, n, bar);
+            if (A.narrow)
+                for (int r = 0; r < A.R + 2; ++r)
+                    for (int kx = 0; kx < 3; ++kx)
+                        tma_load_4d(dst + (uint32_t)(A.x_off + (r * 3 + kx) * np * Wx * 16), A.tmap_x, 2 * (x0 + kx - 1), 0, y0 + r - 1, n, bar);
+            else
+                tma_load_4d(dst + (uint32_t)A.x_off, A.tmap_x, 2 * (x0 - K / 2), ci0 / 8, y0 - K / 2, n, bar);
             ++issued[s];
         }
         if (H->failed)       // gave up somewhere: let the copies already under way land before the block leaves
@@ -263,8 +330,8 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
         const uint32_t a_hi = desc_hi((uint32_t)(A.R * A.Cw) * 16u), x_hi = is_bias ? desc_hi(0) : desc_hi((uint32_t)Wx * 16u);
         const uint32_t idesc = make_idesc(A.Ms, is_bias ? 16 : wide, true, true);
         const uint32_t col = tmem + (uint32_t)((is_bias ? A.units : warp) * wide);
-        const uint32_t a_pair = 2u * (uint32_t)A.Cw, x_pair = is_bias ? 0u : 2u * (uint32_t)(np * Wx), x_step = is_bias ? 0u : 8u;
-        const int every = is_bias ? A.nci : K == 1 ? A.units : 1, first = is_bias ? cs : K == 1 ? warp : 0;
+        const uint32_t a_pair = 2u * (uint32_t)A.Cw, x_pair = is_bias ? 0u : 2u * (uint32_t)pitch, x_step = is_bias ? 0u : 8u;
+        const int every = is_bias ? A.nci : turns ? A.units : 1, first = is_bias ? cs : turns ? warp : 0;
         bool acc = false;
         int turn = first;                                    // row pairs until this issuer's next one
         for (int i = 0; i < nb; ++i) {
@@ -277,7 +344,7 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
                 const uint32_t dst = smem_u32(stages + (size_t)s * A.stage_bytes);
                 uint32_t ar = desc_lo(dst, (uint32_t)A.Cw * 16u);
                 uint32_t xr = is_bias ? desc_lo(smem_u32(H->ones), 0)
-                                      : desc_lo(dst + (uint32_t)A.x_off, (uint32_t)(np * Wx) * 16u) + (K == 3 ? (uint32_t)warp : 0u);
+                                      : desc_lo(dst + (uint32_t)A.x_off, (uint32_t)pitch * 16u) + (turns ? 0u : (uint32_t)warp);
                 const int pairs = pairs_of(y0), groups = (min(A.Cw, A.W - x0) + 7) >> 3;
                 for (int r = 0; r < pairs; ++r, ar += a_pair, xr += x_pair) {
                     if (turn > 0) { --turn; continue; }
@@ -308,7 +375,7 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
         band_of(b_lo + i, n, y0, x0);
         pairs += pairs_of(y0);
     }
-    const int used = !have ? 0 : K == 3 ? 1 : min(A.units, pairs);
+    const int used = !have ? 0 : turns ? min(A.units, pairs) : 1;
 
     // tensor memory -> this share's partial set; lane quarter q holds rows 32q.. (Ms = 128) or rows 16q.. in its
     // first 16 lanes (Ms = 64).  The slices of the blocks are disjoint: plain stores.
@@ -326,7 +393,7 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
             for (int j = 0; j < 16; ++j) v[j] = 0.f;
             for (int w = 0; w < used; ++w) {
                 float t[16];
-                tmem_ld16(tq + (uint32_t)((kx + w) * wide + ky * A.ncols + c0), t);
+                tmem_ld16(tq + (uint32_t)((turns ? w : kx) * wide + (A.narrow ? u : ky) * A.ncols + c0), t);
 #pragma unroll
                 for (int j = 0; j < 16; ++j) v[j] = w ? v[j] + t[j] : t[j];
             }
@@ -341,7 +408,11 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
     if (half == 0) {
         float v[16];
         v[0] = 0.f;
-        if (A.narrow) { if (have) { tmem_ld16(tq + (uint32_t)(wide + A.ncols), v); v[0] = v[7]; } }
+        if (A.narrow) {
+            float sum = 0.f;
+            for (int w = 0; w < used; ++w) { tmem_ld16(tq + (uint32_t)(w * wide + 4 * A.ncols), v); sum += v[7]; }
+            v[0] = sum;
+        }
         else if (have && pairs > cs) tmem_ld16(tq + (uint32_t)(A.units * wide), v);
         if (row_ok) gset[(size_t)KK * A.cout16 * A.cin16 + (size_t)cs * A.cout16 + co] = v[0];
     }
@@ -391,8 +462,8 @@ struct TcConvRowsArgs {
     // prev_arg = its pool's arg-max bytes or null, prev_slope = its leaky slope.  prev_y null: plain delta planes.
     const uint4* prev_y; const unsigned long long* prev_arg; float prev_slope;
     float* out_f;                             // fp32 NCHW output in the place of planes (delta at the network input), else null
-    int row_blocks, blk_step;                 // pool: an accumulator block per row of the band (else blocks of 128 consecutive entries); entries between blocks
-    int narrow, zero_off;                     // first layer's forward pass: in is one plane of 8 channels; offset of 2 KB of zeros behind the stages
+    int row_blocks, blk_step;                 // an accumulator block per row of the band (else blocks of 128 consecutive entries); entries between blocks
+    int stack;                                // with it, 3x3 and slices of 16 channels: the window rows share an MMA (see the issuers)
     int nbuf;                                 // accumulator buffers (2: items of at most 256 columns alternate between the halves
                                               //   of the tensor memory, so the MMAs of one run while the other is read back)
 };
@@ -499,7 +570,6 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
     }
     if (warp == 0) { __syncwarp(); tmem_alloc(smem_u32(&H->tmem_base), (uint32_t)kTcTmemCols); }
     tcd::zero_bytes(stages, (size_t)A.stages * A.stage_bytes);       // what the copies never write is read as zeros
-    if (A.narrow) tcd::zero_bytes(stages + A.zero_off, 2048);
     fence_async_smem();
     fence_before_sync();
     __syncthreads();
@@ -583,21 +653,37 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                     const int nks = min(A.kpc, kplanes - c * A.kpc) >> 1;
                     const uint32_t xaddr = smem_u32(stages + (size_t)s * A.stage_bytes), waddr = xaddr + (uint32_t)(A.kpc * A.x_plane);
                     const uint32_t b_lo0 = desc_lo(waddr, (uint32_t)A.Ns * 16u);
+                    if (A.stack) {
+                        // An MMA reads 4 KB of A however narrow it is: with 16 columns it takes 36 cycles, with 48 44.  An input row
+                        // belongs to the three output rows around it, whose accumulators are neighbouring columns, so it meets
+                        // the filters of up to three window rows (packed bottom row first) in one MMA.  An issuer has four output rows
+                        // of its own; a row's accumulators start with the input row above it.
+                        const uint32_t wp = (uint32_t)A.Wp, kxw = (uint32_t)A.kpc * 48u;
+                        const int s0 = iw * 4, n = min(4, I.rows - s0);
+                        const uint32_t a0 = desc_lo(xaddr, (uint32_t)A.x_plane) + (uint32_t)s0 * wp, w0 = desc_lo(waddr, 768u);
+                        const uint32_t d0 = tmem + buf * 256u + (uint32_t)s0 * 16u;
+                        for (int kx = 0; kx < 3; ++kx)
+                            for (int ks = 0; ks < nks; ++ks) {
+                                const uint32_t w = w0 + (uint32_t)kx * kxw + (uint32_t)ks * 96u;
+                                const bool fresh = (c | kx | ks) == 0;
+                                uint32_t a = a0 + (uint32_t)kx + (uint32_t)ks * xstep;
+                                for (int r = 0; n > 0 && r < n + 2; ++r, a += wp) {          // input row s0 + r - 1: output rows r - 2 .. r of the issuer
+                                    const int lo = max(r - 2, 0), hi = min(r, n - 1);
+                                    const bool first = fresh && r < n;                       // output row r begins
+                                    const int joint = hi - lo + (first ? 0 : 1);
+                                    const uint32_t wl = w + (uint32_t)(lo + 2 - r) * 16u;
+                                    if (joint > 0) mma_bf16(d0 + (uint32_t)lo * 16u, desc64(a_hi, a), desc64(b_hi, wl), make_idesc(128, joint * 16, false, false), true);
+                                    if (first) mma_bf16(d0 + (uint32_t)r * 16u, desc64(a_hi, a), desc64(b_hi, w + 32u), make_idesc(128, 16, false, false), false);
+                                }
+                            }
+                        mma_commit(smem_u32(&H->empty[s]));
+                        continue;
+                    }
                     // (the thread that issues is the bottleneck of a narrow MMA: descriptors advance by adds only)
                     for (int b = iw; b < I.nblk; b += kTcIssuers) {
                         const uint32_t tcol = tmem + buf * 256u + (uint32_t)(b * A.Ns);
                         const uint32_t a0 = desc_lo(xaddr + (uint32_t)(b * A.blk_step) * 16u, (uint32_t)A.x_plane);
-                        if (A.narrow) {
-                            // one plane: a K step is two window positions (the second LBO entries behind the first), the last one's
-                            // partner a block of zeros (an infinite pixel must not meet a zero weight)
-                            const uint32_t wp = (uint32_t)A.Wp, al = desc_lo(xaddr + (uint32_t)(b * A.blk_step) * 16u, 0), w2 = 2u * (uint32_t)A.Ns;
-                            const uint32_t last = al + 2 * wp + 2, zeros = desc_lo(smem_u32(stages + A.zero_off), 0);
-                            mma_bf16(tcol, desc64(a_hi, al | (1u << 16)), desc64(b_hi, b_lo0), idesc, false);
-                            mma_bf16(tcol, desc64(a_hi, (al + 2) | ((wp - 2) << 16)), desc64(b_hi, b_lo0 + w2), idesc, true);
-                            mma_bf16(tcol, desc64(a_hi, (al + wp + 1) | (1u << 16)), desc64(b_hi, b_lo0 + 2 * w2), idesc, true);
-                            mma_bf16(tcol, desc64(a_hi, (al + 2 * wp) | (1u << 16)), desc64(b_hi, b_lo0 + 3 * w2), idesc, true);
-                            mma_bf16(tcol, desc64(a_hi, last | ((zeros - last) << 16)), desc64(b_hi, b_lo0 + 4 * w2), idesc, true);
-                        } else if (K == 3) {
+                        if (K == 3) {
                             // nine MMAs per K step, one per window position, written out: the issuing thread runs a few dozen
                             // instructions per MMA if it has to loop, and then it, not the tensor core, sets the pace
                             // (measured: an MMA every 100 cycles with the loops, every 40-64 with straight-line code)
@@ -664,16 +750,16 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                 const int nc = I.cols >> 4, nunits = I.nblk * nc;
                 const size_t gstep = (size_t)A.H * A.W;
                 // where unit u (accumulator block b, channels c0 .. c0 + 15) of this thread lies in the output planes
-                auto place = [&](int u, int& b, int& c0, size_t& g0) {
+                auto place = [&](int u, int& b, int& c0, size_t& g0, int& r, int& c) {
                     b = u / nc; c0 = (u - b * nc) << 4;
                     const int p = b * 128 + q * 32 + lane;
-                    const int r = p / A.Wp, c = p - r * A.Wp;
+                    r = A.row_blocks ? b : p / A.Wp; c = A.row_blocks ? q * 32 + lane : p - r * A.Wp;
                     g0 = (((size_t)I.n * oplanes + ((I.co0 + c0) >> 3)) * A.H + I.y0 + r) * A.W + I.x0 + c;
                     return r < I.rows && c < I.cw;
                 };
                 for (int u = part; u < nunits; u += kParts) {
-                    int b, c0; size_t g0;
-                    const bool valid = place(u, b, c0, g0);
+                    int b, c0, r, c; size_t g0;
+                    const bool valid = place(u, b, c0, g0, r, c);
                     // what the fused dz step reads of the layer below is requested before the accumulators, so that the
                     // latencies overlap (requested a whole unit ahead, even for the launches through a pool only, the
                     // kernel was measured slower)
@@ -687,7 +773,6 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                     tmem_ld16(tbuf + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * A.Ns + c0), v);
                     if (A.out_f) {                            // (a delta: neither bias nor activation)
                         if (!valid) continue;
-                        const int p = b * 128 + q * 32 + lane, r = p / A.Wp, c = p - r * A.Wp;
                         float* dst = A.out_f + (((size_t)I.n * A.cout + I.co0 + c0) * A.H + I.y0 + r) * A.W + I.x0 + c;
 #pragma unroll
                         for (int j = 0; j < 16; ++j) if (I.co0 + c0 + j < A.cout) dst[j * gstep] = v[j];
@@ -697,8 +782,6 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                     } else if (valid) {
                         // input delta straight into the dz planes of the layer below: rounded as a stored delta
                         // would be, times the derivative of that layer's activation, through its pool's arg-max
-                        const int p = b * 128 + q * 32 + lane;
-                        const int r = p / A.Wp, c = p - r * A.Wp;
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             const uint4 dq = derive8(tcd::pack8(v + 8 * h), yq[h], A.prev_slope);
@@ -741,7 +824,9 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                                             __shfl_xor_sync(0xffffffffu, away.z, 1), __shfl_xor_sync(0xffffffffu, away.w, 1));
                     }
                     uint4 best;
-                    const unsigned long long am = odd ? pool4(got[0], own[0], got[1], own[1], best) : pool4(own[0], got[0], own[1], got[1], best);
+                    // (operands picked before the comparison: two calls behind a branch would both run)
+                    auto pick = [&](const uint4& a, const uint4& b) { return make_uint4(odd ? b.x : a.x, odd ? b.y : a.y, odd ? b.z : a.z, odd ? b.w : a.w); };
+                    const unsigned long long am = pool4(pick(own[0], got[0]), pick(got[0], own[0]), pick(own[1], got[1]), pick(got[1], own[1]), best);
                     const size_t gi = (((size_t)I.n * oplanes + ((I.co0 + c0) >> 3) + odd) * OH + (I.y0 >> 1) + pr) * OW + (I.x0 >> 1) + (col >> 1);
                     if (valid) { A.out[gi] = best; A.arg[gi] = am; }
                 }

@@ -554,3 +554,41 @@ def test_filter_gradient_at_the_edges_of_its_slices_and_bands(cin, cout, k, n, h
     errors = per_layer_errors(list(layers), dparams, ref["dparams"])
     print(plan.exec_groups(), errors)
     assert len(errors) == 2 and all(max(e[1:]) <= 1e-2 for e in errors)
+
+
+# Stacks whose pools run on accumulator blocks of one row (rows of about 80 to 126 columns: 84, 126, 104 a chunk, an odd number of
+# row pairs, one row pair), whose input delta stacks the window rows (bands of 16 rows and of fewer, rows that the issuers share
+# unevenly) and whose first layer has 1, 3 and 7 channels, with 64 and with more rows an MMA; the loss below a pool and not.
+ROWS = {
+    "one-row-pair": W("o", (conv(3, 32, 3), pool(), conv(32, 64, 3)), 2, 3, 2, 252, (1, 1), ((1, 3),)),
+    "pools-of-narrow-layers": W("p", (conv(3, 32, 3), pool(), conv(32, 56, 3), pool()), 1, 3, 44, 336, (2, 2), ((1, 4),)),
+    "seven-channels": W("s", (conv(7, 80, 3), pool(), conv(80, 16, 1)), 3, 7, 38, 104, (1, 2), ((1, 3),)),
+    "one-channel-no-pool": W("c", (conv(1, 13, 3), conv(13, 32, 3), pool()), 2, 1, 22, 90, (1, 1), ((1, 3),)),
+    "narrow-map": W("n", (conv(3, 48, 3), pool(), conv(48, 32, 3), pool()), 2, 3, 20, 12, (1, 1), ((1, 4),)),
+}
+
+
+@pytest.mark.parametrize("name", sorted(ROWS))
+def test_first_layers_and_pools_in_rows_on_decision_safe_data(name):
+    """Forward pass bit for bit and gradients at BF16_TOL against the oracle on small integers (see the test of whole stacks above); a
+    step with a target then has the loss (1e-3 as above) and the gradient of the oracle's delta."""
+    wl = synth.with_slope(ROWS[name], 0.0)
+    x, params, target = synth.draw_integer_relu(wl)
+    dy = np.random.default_rng(3).standard_normal(target.shape).astype(np.float32)
+    y, dx, dparams, plan = backward_bf16(wl, x, params, dy)
+    assert all(plan.group_mode(i)[0] == 2 for i in range(len(plan.exec_groups())))
+    ref = run_oracle(wl, x, params, dy=dy, store="bf16")
+    assert np.array_equal(y.astype(np.float64), ref["y"])
+    assert np.abs(ref["dx"]).max() > 0
+    assert rel_err(dx, ref["dx"]) <= BF16_TOL
+    errs = per_layer_errors(list(wl.layers), dparams, ref["dparams"])
+    assert all(max(a, b) <= BF16_TOL for _, a, b in errs), errs
+
+    ref = run_oracle(wl, x, params, target=target, store="bf16")
+    ws = plan.new_workspace()
+    g, loss = torch.empty(params.size, device="cuda"), torch.zeros(1, device="cuda")
+    ftp.ftp_step_grad(plan, torch.from_numpy(x).cuda(), torch.from_numpy(params).cuda(), g, ws, target=torch.from_numpy(target).cuda(), loss_out=loss)
+    plan.check(ws)
+    assert loss.item() == pytest.approx(ref["loss"], rel=1e-3)
+    errs = per_layer_errors(list(wl.layers), g.cpu().numpy(), ref["dparams"])
+    assert all(max(a, b) <= BF16_TOL for _, a, b in errs), errs
