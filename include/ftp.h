@@ -149,8 +149,8 @@ typedef struct {
                            rows x a slice of output channels stays in tensor memory while the input channels stream
                            past; the delta is the convolution of dz with the rotated filters and writes every cell
                            once), the filter gradient by a weight-stationary kernel that keeps a slice of the gradient
-                           in tensor memory while the batch streams past; the first layer runs as a 1x1 conv on a
-                           window-unrolled bf16 copy of the network input, with the same parameters.
+                           in tensor memory while the batch streams past; the first layer's forward pass runs as a 1x1 conv on
+                           a window-unrolled bf16 copy of the network input, with the same parameters.
                            0 and 1: every such layer; -1: never (fused stacks only).  Conv layers with more than 512
                            input or output channels run this way only (the fused kernels keep all output channels of
                            an op in the 512 tensor-memory columns): a bf16 plan that would put such a layer into a

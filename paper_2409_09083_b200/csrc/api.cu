@@ -45,7 +45,10 @@ int ensure_device(ftp_plan* p)
         cudaFuncSetAttribute(bwd_group_tc_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemBudget) != cudaSuccess ||
         cudaFuncSetAttribute(bwd_group_tc_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemBudget) != cudaSuccess ||
         cudaFuncSetAttribute(filter_grad_tc_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcFgSmemBudget) != cudaSuccess ||
-        cudaFuncSetAttribute(conv_tc_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcConvSmemBudget) != cudaSuccess ||
+        cudaFuncSetAttribute(conv_tc_rows_kernel<kConvPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcConvSmemBudget) != cudaSuccess ||
+        cudaFuncSetAttribute(conv_tc_rows_kernel<kConvPool>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcConvSmemBudget) != cudaSuccess ||
+        cudaFuncSetAttribute(conv_tc_rows_kernel<kConvRowPool>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcConvSmemBudget) != cudaSuccess ||
+        cudaFuncSetAttribute(conv_tc_rows_kernel<kConvStack>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcConvSmemBudget) != cudaSuccess ||
         !st_prepare_device() || !split_prepare_device())
         return FTP_ERR_CUDA;
     if (!p->grad_stream) {
@@ -280,15 +283,19 @@ bool launch_tc_conv(ftp_plan* p, const TcConvPlan& c, int kind, int gi, const vo
     if (prev) { a.prev_y = prev->y; a.prev_arg = prev->arg; a.prev_slope = prev->slope; }
     a.bias = bias; a.out = static_cast<uint4*>(out); a.arg = reinterpret_cast<unsigned long long*>(arg);
     a.error = error;
-    a.N = p->N; a.K = K; a.cin16 = cin16; a.cout16 = cout16; a.cout = cout; a.H = H; a.W = W; a.pool = pool ? 1 : 0;
+    a.N = p->N; a.K = K; a.cin16 = cin16; a.cout16 = cout16; a.cout = cout; a.H = H; a.W = W;
     a.slope = slope;
     a.Ns = c.Ns; a.slices = c.slices; a.R = c.R; a.Wp = c.Wp; a.bands_img = c.bands_img; a.nblk = c.nblk; a.kpc = c.kpc;
     a.ncc = c.ncc; a.Cw = c.Cw; a.items = c.items; a.pool_planes = c.pool_planes; a.nbuf = c.nbuf;
     a.x_plane = c.x_plane; a.stage_bytes = c.stage_bytes; a.stages = c.stages;
-    a.out_f = out_f; a.row_blocks = c.row_blocks; a.stack = c.stack; a.blk_step = c.row_blocks ? c.Wp : 128;
+    a.out_f = out_f;
     a.hurry = (double)((c.items + c.blocks - 1) / c.blocks) * c.nblk * K * K * (cin16 / 16) * tc_mma_cycles(c.Ns) < kHurryCycles;
     { Timed tm(p, st, kind, gi);
-      launch(conv_tc_rows_kernel, c.blocks, kTcConvThreads, one_block_smem(c.smem_bytes), tm.ls(), a); }
+      const size_t smem = one_block_smem(c.smem_bytes);
+      if (c.stack) launch(conv_tc_rows_kernel<kConvStack>, c.blocks, kTcConvThreads, smem, tm.ls(), a);
+      else if (c.row_blocks) launch(conv_tc_rows_kernel<kConvRowPool>, c.blocks, kTcConvThreads, smem, tm.ls(), a);
+      else if (pool) launch(conv_tc_rows_kernel<kConvPool>, c.blocks, kTcConvThreads, smem, tm.ls(), a);
+      else launch(conv_tc_rows_kernel<kConvPlain>, c.blocks, kTcConvThreads, smem, tm.ls(), a); }
     return launched_ok();
 }
 

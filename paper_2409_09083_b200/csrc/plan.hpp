@@ -156,7 +156,7 @@ struct TcConvPlan {
     int blocks = 0;                         // persistent blocks: min(items, SMs)
     int pool_planes = 0;                    // fused pool: 8-channel planes the staging area holds
     int pool_stage_bytes = 0;               //             and its size
-    int row_blocks = 0, stack = 0;          // see TcConvRowsArgs
+    int row_blocks = 0, stack = 0;          // form of the kernel, see conv_tc_rows_kernel
     int nbuf = 1;                           // accumulator buffers (2 for slices of at most 64 channels)
 };
 constexpr int kTcPoolStageBytes = 32 * 1024;  // least staging area of the fused pool in the banded convolution (more where it fits)

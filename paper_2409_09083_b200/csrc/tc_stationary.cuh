@@ -1,6 +1,6 @@
 // bf16 path, executed groups of one conv layer (with its pool): the filter gradient by a weight-stationary
 // tensor-core kernel, the forward pass and the input delta by a banded tensor-core convolution (further down),
-// and their helpers (dz planes, window unroll / fold for the first layer).
+// and their helpers (dz planes, loss, window unroll and input entries for the first layer).
 //
 // Filter gradient.  In the fused tile-stack kernel every sub-tile adds its whole partial filter gradient (K*K*cout*cin fp32) to
 // the block's partial set, because tensor memory cannot keep the accumulators of a wide layer across sub-tiles.
@@ -448,7 +448,7 @@ struct TcConvRowsArgs {
     unsigned long long* arg;                  // pool: arg-max bytes in the same arrangement
     int* error;
     int hurry;                                // a short launch: see kHurryCycles in launch.cuh
-    int N, K, cin16, cout16, cout, H, W, pool;
+    int N, K, cin16, cout16, cout, H, W;
     float slope;
     int Ns, slices;                           // output channels per item, number of slices
     int R, Wp, bands_img, nblk;               // rows per band, tile pitch, bands per image, accumulator blocks of a full band
@@ -462,8 +462,8 @@ struct TcConvRowsArgs {
     // prev_arg = its pool's arg-max bytes or null, prev_slope = its leaky slope.  prev_y null: plain delta planes.
     const uint4* prev_y; const unsigned long long* prev_arg; float prev_slope;
     float* out_f;                             // fp32 NCHW output in the place of planes (delta at the network input), else null
-    int row_blocks, blk_step;                 // an accumulator block per row of the band (else blocks of 128 consecutive entries); entries between blocks
-    int stack;                                // with it, 3x3 and slices of 16 channels: the window rows share an MMA (see the issuers)
+    // forms of the kernel: accumulator blocks of 128 consecutive entries (plain, pool), or one per row of the band: with a pool, or, 3x3 with
+    // slices of 16 channels, with the window rows in one MMA (stack; see the issuers)
     int nbuf;                                 // accumulator buffers (2: items of at most 256 columns alternate between the halves
                                               //   of the tensor memory, so the MMAs of one run while the other is read back)
 };
@@ -540,6 +540,11 @@ __device__ __forceinline__ unsigned long long pool4(const uint4& m0, const uint4
     return (unsigned long long)__byte_perm(code[0], code[1], 0x6420) | ((unsigned long long)__byte_perm(code[2], code[3], 0x6420) << 32);
 }
 
+// One instance per form of the epilogue and the issue: a launch waits for its instructions too, and no instance spills (8 layers, 4
+// images: a step 283 us as one kernel with all forms, 276 so).
+enum { kConvPlain = 0, kConvPool = 1, kConvRowPool = 2, kConvStack = 3 };
+
+template <int FORM>
 __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const __grid_constant__ TcConvRowsArgs A)
 {
     using namespace tc;
@@ -599,7 +604,7 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
         I.y0 = (bi / A.ncc) * A.R; I.x0 = (bi % A.ncc) * A.Cw;
         I.rows = min(A.R, A.H - I.y0); I.cw = min(A.Cw, A.W - I.x0);
         I.co0 = I.slice * A.Ns; I.cols = min(A.Ns, A.cout16 - I.co0);
-        I.nblk = A.row_blocks ? I.rows : (I.rows * A.Wp + 127) >> 7;
+        I.nblk = FORM >= kConvRowPool ? I.rows : (I.rows * A.Wp + 127) >> 7;
         return I;
     };
     const uint32_t w_tap = (uint32_t)A.kpc * (uint32_t)A.Ns * 16u;                      // filter bytes of one window position
@@ -653,7 +658,7 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                     const int nks = min(A.kpc, kplanes - c * A.kpc) >> 1;
                     const uint32_t xaddr = smem_u32(stages + (size_t)s * A.stage_bytes), waddr = xaddr + (uint32_t)(A.kpc * A.x_plane);
                     const uint32_t b_lo0 = desc_lo(waddr, (uint32_t)A.Ns * 16u);
-                    if (A.stack) {
+                    if constexpr (FORM == kConvStack) {
                         // An MMA reads 4 KB of A however narrow it is: with 16 columns it takes 36 cycles, with 48 44.  An input row
                         // belongs to the three output rows around it, whose accumulators are neighbouring columns, so it meets
                         // the filters of up to three window rows (packed bottom row first) in one MMA.  An issuer has four output rows
@@ -676,13 +681,11 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                                     if (first) mma_bf16(d0 + (uint32_t)r * 16u, desc64(a_hi, a), desc64(b_hi, w + 32u), make_idesc(128, 16, false, false), false);
                                 }
                             }
-                        mma_commit(smem_u32(&H->empty[s]));
-                        continue;
-                    }
+                    } else {
                     // (the thread that issues is the bottleneck of a narrow MMA: descriptors advance by adds only)
                     for (int b = iw; b < I.nblk; b += kTcIssuers) {
                         const uint32_t tcol = tmem + buf * 256u + (uint32_t)(b * A.Ns);
-                        const uint32_t a0 = desc_lo(xaddr + (uint32_t)(b * A.blk_step) * 16u, (uint32_t)A.x_plane);
+                        const uint32_t a0 = desc_lo(xaddr + (uint32_t)(b * (FORM >= kConvRowPool ? A.Wp : 128)) * 16u, (uint32_t)A.x_plane);
                         if (K == 3) {
                             // nine MMAs per K step, one per window position, written out: the issuing thread runs a few dozen
                             // instructions per MMA if it has to loop, and then it, not the tensor core, sets the pace
@@ -708,6 +711,7 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                                 acc = true; a_lo += xstep; b_lo += wstep;
                             }
                         }
+                    }
                     }
                     mma_commit(smem_u32(&H->empty[s]));
                 }
@@ -746,14 +750,14 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
             wait(&H->done[buf], use & 1u, 128);                       // asleep between polls; (ran out: the item is written from
                                                                       // whatever is there; the error word is set)
             fence_after_sync();
-            if (!A.pool) {
+            if constexpr (FORM == kConvPlain || FORM == kConvStack) {
                 const int nc = I.cols >> 4, nunits = I.nblk * nc;
                 const size_t gstep = (size_t)A.H * A.W;
                 // where unit u (accumulator block b, channels c0 .. c0 + 15) of this thread lies in the output planes
                 auto place = [&](int u, int& b, int& c0, size_t& g0, int& r, int& c) {
                     b = u / nc; c0 = (u - b * nc) << 4;
                     const int p = b * 128 + q * 32 + lane;
-                    r = A.row_blocks ? b : p / A.Wp; c = A.row_blocks ? q * 32 + lane : p - r * A.Wp;
+                    r = FORM == kConvStack ? b : p / A.Wp; c = FORM == kConvStack ? q * 32 + lane : p - r * A.Wp;
                     g0 = (((size_t)I.n * oplanes + ((I.co0 + c0) >> 3)) * A.H + I.y0 + r) * A.W + I.x0 + c;
                     return r < I.rows && c < I.cw;
                 };
@@ -803,7 +807,7 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                         }
                     }
                 }
-            } else if (A.row_blocks) {
+            } else if constexpr (FORM == kConvRowPool) {
                 // The rows of a window are the same lanes of two blocks and its columns two neighbouring lanes: no staging area and
                 // no barriers.  The even lane takes the lower 8 channels of a unit, the odd lane the upper ones.
                 // us, staged and so: 3 -> 32, 16 x 608 x 608 164 -> 143; 32 -> 64, 304 x 304 127 -> 101.
