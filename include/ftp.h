@@ -150,7 +150,11 @@ typedef struct {
                            past; the delta is the convolution of dz with the rotated filters and writes every cell
                            once), the filter gradient by a weight-stationary kernel that keeps a slice of the gradient
                            in tensor memory while the batch streams past; the first layer's forward pass runs as a 1x1 conv on
-                           a window-unrolled bf16 copy of the network input, with the same parameters.
+                           a window-unrolled bf16 copy of the network input, with the same parameters.  Infinities and NaNs reach
+                           what they reach in a plain sum, with two exceptions, both NaN in the place of a finite value: a padding
+                           zero meets an infinite operand in the filter gradient (an infinite delta at the border of the map; in
+                           layers above the first, of a width that is no multiple of 8, an infinite value in the last column of the input) and
+                           in the first layer's forward pass and the input deltas (an infinite filter value, at the border of the map).
                            0 and 1: every such layer; -1: never (fused stacks only).  Conv layers with more than 512
                            input or output channels run this way only (the fused kernels keep all output channels of
                            an op in the 512 tensor-memory columns): a bf16 plan that would put such a layer into a

@@ -230,14 +230,15 @@ bool encode_rows_map(unsigned char out[128], const void* base, int N, int planes
 }
 
 // Tensor map of bf16 planes of this GPU's memory for the bands of the filter gradient: {columns, rows, planes, images}, or with
-// the planes of a row next to one another {columns, planes, rows, images}; a pixel's 8 channels are two 8-byte elements.
-bool encode_band_map(unsigned char out[128], const void* base, int N, int planes, int H, int W, bool planes_inside, int box_w, int box_h, int box_planes)
+// the planes of a row next to one another {columns, planes, rows, images}; a pixel's 8 channels are two 8-byte elements.  Columns from
+// `cols` on read as zeros.
+bool encode_band_map(unsigned char out[128], const void* base, int N, int planes, int H, int W, int cols, bool planes_inside, int box_w, int box_h, int box_planes)
 {
     tensor_map_encode_fn enc = tensor_map_encoder();
     if (!enc || box_h > 256 || box_w > 128 || box_planes > 256) return false;
     const int r = planes_inside ? 2 : 1, q = planes_inside ? 1 : 2;              // dimension of the rows / of the planes
     cuuint64_t dims[4], strides[3]; cuuint32_t box[4]; const cuuint32_t estr[4] = {1, 1, 1, 1};
-    dims[0] = 2 * (cuuint64_t)W; box[0] = 2 * (cuuint32_t)box_w;
+    dims[0] = 2 * (cuuint64_t)cols; box[0] = 2 * (cuuint32_t)box_w;
     dims[r] = (cuuint64_t)H; box[r] = (cuuint32_t)box_h; strides[r - 1] = (cuuint64_t)W * 16;
     dims[q] = (cuuint64_t)planes; box[q] = (cuuint32_t)box_planes; strides[q - 1] = (cuuint64_t)H * W * 16;
     dims[3] = (cuuint64_t)N; box[3] = 1; strides[2] = (cuuint64_t)planes * H * W * 16;
@@ -743,9 +744,11 @@ bool tc_filter_grad(ftp_plan* p, const GroupPlan& g, int gi, const TcGroupArgs& 
     }
 
     TcFilterGradArgs f{};
-    if (!encode_band_map(f.tmap_dz, dz, p->N, op.cout16 / 8, op.in_H, op.in_W, false, t.Cw, t.R, t.dz_box) ||
-        !encode_band_map(f.tmap_x, xin, p->N, g.narrow ? 1 : cin16 / 8, op.in_H, op.in_W, true, g.narrow ? t.Cw : t.Cw + t.k - 1,
-                         g.narrow ? 1 : t.R + t.k - 1, t.ncols / 8)) return false;
+    const int W = op.in_W;
+    if (!encode_band_map(f.tmap_dz, dz, p->N, op.cout16 / 8, op.in_H, W, W, false, t.Cw, t.R, t.dz_box) ||
+        !encode_band_map(f.tmap_x, xin, p->N, g.narrow ? 1 : cin16 / 8, op.in_H, W, W, true, g.narrow ? t.Cw : t.Cw + t.k - 1,
+                         g.narrow ? 1 : t.R + t.k - 1, t.ncols / 8) ||
+        (g.narrow && !encode_band_map(f.tmap_left, xin, p->N, 1, op.in_H, W, std::max(W - 1, 1), true, t.Cw, 1, t.ncols / 8))) return false;
     f.partial = a.partial; f.set_floats = a.set_floats; f.tgp_off = op.tgp_off;
     f.error = a.error;
     f.K = t.k; f.H = op.in_H; f.W = op.in_W; f.cout16 = op.cout16; f.cin16 = g.narrow ? t.ncols : cin16; f.narrow = g.narrow;

@@ -939,8 +939,8 @@ void plan_tc_filter_grad(const ftp_plan& p, GroupPlan& g, const PlanOpts& o)
                 // are on their way: 32 channels at 608 x 608, 16 images, 126 -> 101 us)
                 const size_t dz_plane = (size_t)c.R * c.Cw * 16;
                 c.x_off = (int)align_up(c.dz_box * dz_plane, 128);
-                const size_t xb = (size_t)(c.ncols / 8) * (c.R + K - 1) * (narrow ? 3 * c.Cw : c.Cw + K - 1) * 16;
-                c.stage_bytes = (int)align_up((size_t)c.x_off + xb, 128);
+                const size_t x_row = (size_t)(c.ncols / 8) * (narrow ? 3 * c.Cw : c.Cw + K - 1) * 16, xb = (c.R + K - 1) * x_row;
+                c.stage_bytes = (int)align_up((size_t)c.x_off + xb + (K == 3 && H % 2 ? x_row : 0), 128);      // (see odd_h in the kernel)
                 c.smem_bytes = kTcFgHeader + c.stage_bytes + (int)std::max<size_t>(c.stage_bytes, c.Ms / 8 * dz_plane);
                 if (c.smem_bytes > kTcFgSmemBudget) break;
                 c.bands_img = (H + c.R - 1) / c.R * c.ncc;

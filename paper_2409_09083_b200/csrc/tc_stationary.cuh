@@ -39,6 +39,7 @@ namespace ftp {
 struct TcFilterGradArgs {
     alignas(64) unsigned char tmap_dz[128];   // dz as {columns, rows, planes, images}: box = Cw columns x R rows x dz_box planes
     alignas(64) unsigned char tmap_x[128];    // the layer's input as {columns, planes, rows, images}: box = (Cw + K - 1) x ncols / 8 x (R + K - 1)
+    alignas(64) unsigned char tmap_left[128]; // first layer: the same without the map's last column, for the copies of window column 0
     float* partial;                           // partial sets of the group
     long long set_floats, tgp_off;            // floats per set, offset of this layer inside a set
     int* error;
@@ -265,6 +266,12 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
     // MMA (three MMAs of 24 columns took 37 cycles each: 142 us a launch for 16 x 608 x 608, 3 -> 32, now 101, 473 MB).
     const bool turns = K == 1 || A.narrow;
     const int np = A.ncols / 8, Wx = A.narrow ? A.Cw : A.Cw + K - 1, pitch = (A.narrow ? 3 : 1) * np * Wx;
+    // Pixels that only fill up a K step have zero dz, and a zero times an infinite input is NaN: they must not meet pixels of the map.
+    // Columns: the first layer's copies of window column 0 leave out the last column, which only the window columns 1 and 2 of
+    // a pixel read (elsewhere a row of the tile serves all window columns, and such a value at the end of a row shows).
+    // Rows: where the last row of an odd height stands alone, the second half of its K steps reads the input two rows on instead of one,
+    // below the map for all window rows; at the last row of a band that is one row behind the copied tile, zeros from here on.
+    const bool odd_h = K == 3 && (A.H & 1);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&H->full[s]), 1); mbar_init(smem_u32(&H->empty[s]), kTcIssuers); }
@@ -274,6 +281,8 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
     }
     if (warp == 0) { __syncwarp(); tmem_alloc(smem_u32(&H->tmem_base), (uint32_t)kTcTmemCols); }
     for (int i = threadIdx.x; i < 64; i += blockDim.x) H->ones[i] = __float2bfloat16(1.0f);
+    if (odd_h)
+        for (int s = 0; s < 2; ++s) tcd::zero_bytes(stages + (size_t)s * A.stage_bytes + A.x_off + (size_t)(A.R + K - 1) * pitch * 16, (size_t)pitch * 16);
     fence_async_smem();
     fence_before_sync();
     __syncthreads();
@@ -313,8 +322,9 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
             tma_load_4d(dst, A.tmap_dz, 2 * x0, y0, slice * (A.Ms / 8), n, bar);
             if (A.narrow)
                 for (int r = 0; r < A.R + 2; ++r)
-                    for (int kx = 0; kx < 3; ++kx)
-                        tma_load_4d(dst + (uint32_t)(A.x_off + (r * 3 + kx) * np * Wx * 16), A.tmap_x, 2 * (x0 + kx - 1), 0, y0 + r - 1, n, bar);
+                    for (int kx = 0; kx < 3; ++kx)      // (a map of one column: window column 0 has none, a box in front of the map)
+                        tma_load_4d(dst + (uint32_t)(A.x_off + (r * 3 + kx) * np * Wx * 16), kx ? A.tmap_x : A.tmap_left,
+                                    2 * (A.W == 1 && kx == 0 ? -A.Cw : x0 + kx - 1), 0, y0 + r - 1, n, bar);
             else
                 tma_load_4d(dst + (uint32_t)A.x_off, A.tmap_x, 2 * (x0 - K / 2), ci0 / 8, y0 - K / 2, n, bar);
             ++issued[s];
@@ -346,10 +356,11 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
                 uint32_t xr = is_bias ? desc_lo(smem_u32(H->ones), 0)
                                       : desc_lo(dst + (uint32_t)A.x_off, (uint32_t)pitch * 16u) + (turns ? 0u : (uint32_t)warp);
                 const int pairs = pairs_of(y0), groups = (min(A.Cw, A.W - x0) + 7) >> 3;
+                const int alone = odd_h && !is_bias && A.H - y0 < A.R ? pairs - 1 : -1;       // the pair of a last row without a second
                 for (int r = 0; r < pairs; ++r, ar += a_pair, xr += x_pair) {
                     if (turn > 0) { --turn; continue; }
                     turn = every - 1;
-                    uint32_t a = ar, x = xr;
+                    uint32_t a = ar, x = r == alone ? xr + ((uint32_t)pitch << 16) : xr;     // (desc_lo's stride: two rows)
 #pragma unroll 4
                     for (int g = 0; g < groups; ++g, a += 8u, x += x_step) {
                         mma_bf16(col, desc64(a_hi, a), desc64(x_hi, x), idesc, acc);

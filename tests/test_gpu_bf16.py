@@ -592,3 +592,55 @@ def test_first_layers_and_pools_in_rows_on_decision_safe_data(name):
     assert loss.item() == pytest.approx(ref["loss"], rel=1e-3)
     errs = per_layer_errors(list(wl.layers), g.cpu().numpy(), ref["dparams"])
     assert all(max(a, b) <= BF16_TOL for _, a, b in errs), errs
+
+
+def classes(a):
+    return np.where(np.isnan(a), 3, np.where(np.isposinf(a), 1, np.where(np.isneginf(a), 2, 0)))
+
+
+# (input channels, output channels, N, H, W) of a first layer: odd and even heights, one row, one column, widths beside a multiple of 8 and
+# beside a column chunk, 64 and 128 rows an MMA
+BORDERS = [(3, 16, 2, 5, 13), (1, 8, 1, 1, 1), (2, 16, 1, 7, 1), (7, 80, 2, 9, 3), (3, 32, 1, 2, 8), (3, 32, 2, 33, 121), (3, 24, 1, 4, 250),
+           (4, 130, 2, 13, 16)]
+
+
+@pytest.mark.filterwarnings("ignore:invalid value encountered")
+@pytest.mark.parametrize("cin,cout,n,h,w", BORDERS)
+def test_an_infinite_pixel_at_the_border_reaches_the_window_positions_that_read_it(cin, cout, n, h, w):
+    """First layer: the filter gradient is infinite or NaN where the untiled sums are, finite and accurate elsewhere."""
+    wl = W("inf", (conv(cin, cout, 3, leaky=0.5),), n, cin, h, w, (1, 1), ((1, 1),), x_dist="normal")
+    x, params, target = synth.draw(wl, bias_std=0.3)
+    x, params = bf16_grid(x), bf16_grid(params)
+    dy = bf16_grid(np.random.default_rng(7).standard_normal(target.shape))
+    x[0, 0, -1, -1], x[-1, -1, -1, w // 2], x[0, cin // 2, h // 2, -1], x[-1, 0, 0, 0] = np.inf, -np.inf, np.nan, np.inf
+    ref = run_oracle(wl, x, params, dy=dy, store="bf16")
+    y, dx, dparams, plan = backward_bf16(wl, x, params, dy)
+    assert plan.group_mode(0)[0] == 2
+    for k, g in (("y", y), ("dx", dx), ("dparams", dparams)):
+        assert np.array_equal(classes(g), classes(ref[k])), k
+        ok = np.isfinite(ref[k])
+        if ok.any():                                   # (sums of bf16 operands in fp32; y is stored in bf16)
+            assert rel_err(g[ok], ref[k][ok]) <= 1e-2, k
+
+
+@pytest.mark.filterwarnings("ignore:overflow encountered")
+@pytest.mark.parametrize("h", [3, 13, 33])
+def test_an_infinite_value_in_the_last_row_of_an_odd_height(h):
+    """A 3x3 layer above the first: the value that overflows stands in the last row of the first layer's output."""
+    wl = W("row", (conv(3, 32, 3, leaky=1.0), conv(32, 64, 3, leaky=1.0)), 1, 3, h, 16, (1, 1), ((1, 1), (2, 2)), x_dist="normal")
+    x, params, target = synth.draw(wl, bias_std=0.3)
+    params = bf16_grid(params)
+    params[:32 * 27] = 0
+    params[np.arange(32) * 27 + 4] = 2                       # every channel twice the first channel's pixel, and a bias
+    params[10 * 27 + 4] = 4
+    x = bf16_grid(x)
+    dy = bf16_grid(np.random.default_rng(7).standard_normal(target.shape))
+    grads = []
+    for v in (0.0, 1.5e38):                                  # 4 times it is infinite, twice it is not
+        x[0, 0, -1, 7] = v
+        y, _, dparams, plan = backward_bf16(wl, x, params, dy)
+        assert plan.exec_groups() == [(1, 1), (2, 2)] and plan.group_mode(1)[0] == 2
+        grads.append(dparams[32 * 28:32 * 28 + 64 * 32 * 9].reshape(64, 32, 3, 3))
+    a, b = grads
+    assert np.isinf(b[:, 10, 1:]).all()                      # two rows of window positions read it ...
+    assert np.array_equal(a[:, :, 0], b[:, :, 0])            # ... and the third does not
