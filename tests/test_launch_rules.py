@@ -66,3 +66,32 @@ def test_launches_that_may_overlap_wait_for_the_previous_ones(name):
     assert "previous_launches()" in text, name
     front = text[:text.index("previous_launches()")]
     assert not re.search(r"__ldg|tma_load|bulk_g2s|cp_async|atomic|A\.\w+\[", front), name
+
+
+def asm_statements():
+    """(file, instructions, outputs) of every asm statement: the instructions of its template, comments and declarations left out."""
+    for f, text in sources():
+        for m in re.finditer(r"\basm\s*(?:volatile)?\s*\(", text):
+            depth, i = 1, m.end()
+            while depth:
+                i += 1
+                depth += {"(": 1, ")": -1}.get(text[i], 0)
+            # (operands behind the first colon that stands outside the strings)
+            parts = re.split(r":(?=(?:[^\"]*\"[^\"]*\")*[^\"]*$)", text[m.end():i])
+            template = "".join(re.findall(r'"((?:[^"\\]|\\.)*)"', parts[0]))
+            code = [c.strip(" {}\t") for c in re.split(r";|\\n|\\t", template)]
+            yield f, [c for c in code if c and not c.startswith(".reg")], parts[1] if len(parts) > 1 else ""
+
+
+def test_outputs_written_before_the_last_input_is_read_have_registers_of_their_own():
+    """The compiler may give an output the register of an input unless the output is marked "=&r" (or "+r"): in a statement of several
+    instructions an output of any but the last one has to be, as a later instruction may still read the input."""
+    seen = 0
+    for f, code, outputs in asm_statements():
+        names = re.findall(r'"([=+]&?\w)"\s*\(', outputs)
+        last = max((i for i, c in enumerate(code) if "%" in c), default=0)
+        for i, c in enumerate(code[:last]):
+            written = {int(n) for n in re.findall(r"%(\d+)", c)} & set(range(len(names)))
+            seen += len(written)
+            assert all("&" in names[n] or "+" in names[n] for n in written), (f, c, [names[n] for n in written])
+    assert seen >= 16
