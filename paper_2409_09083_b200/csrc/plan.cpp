@@ -827,23 +827,37 @@ void tc_col_chunks(int W, int* ncc, int* Cw)
     if (*Cw > W) *Cw = W;
 }
 
-// Launch shape of the banded convolution kernel for a conv with `cout16` output and `cin16` input channels (padded)
-// on N maps of H x W: bands as tall as the accumulators allow (512 columns = blocks of 128 entries x Ns channels),
-// among those the height with the fewest rounds of blocks over the SMs; as many stages as fit.
-TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, bool pool, int kpc3, bool stack = false);
-
-TcConvPlan plan_tc_conv(int N, int H, int W, int K, int cin16, int cout16, bool pool)
+// Shared memory of a banded convolution with bands of c.R rows (c.row_blocks, c.nblk, c.kpc, c.Ns given): as many stages as fit, and with a
+// fused pool the staging area.  False if there is no room for two stages.
+bool fit_tc_conv(TcConvPlan& c, int K, bool pool)
 {
-    // input channels per chunk: 3x3: 16, or 32 with slices of at most 64 channels where two stages of that size fit
-    // (their filters are small, and every chunk costs the issuers a wait, a fence and a commit); 1x1: up to 64
-    if (K == 3 && std::min(cout16, 128) <= 64 && cin16 >= 32) {
-        const TcConvPlan c = plan_tc_conv_kpc(N, H, W, K, cin16, cout16, pool, 4);
-        if (c.on) return c;
+    const size_t last = c.row_blocks ? (size_t)(c.nblk - 1) * c.Wp + 128 : (size_t)c.nblk * 128;          // entries the blocks reach over
+    const size_t entries = std::max<size_t>((size_t)(c.R + K - 1) * c.Wp, last + (size_t)(K - 1) * c.Wp + K);
+    c.x_plane = (int)align_up(entries * 16, 128);
+    c.stage_bytes = c.kpc * c.x_plane + K * K * c.kpc * c.Ns * 16;
+    // fused pool: the band as stored goes through a staging area, all channels of the slice at once where that leaves
+    // three stages (two for short rings), else 16 channels or more at a time
+    const size_t room = (size_t)kTcConvSmemBudget - kTcFgHeader;
+    const size_t plane_pair = (size_t)c.nblk * 128 * 16 * 2, whole = (size_t)(c.Ns / 16) * plane_pair;
+    const bool staged = pool && !c.row_blocks;
+    size_t staging = staged ? kTcPoolStageBytes : 0;
+    c.pool_planes = c.pool_stage_bytes = 0;
+    c.stages = (int)std::min<size_t>(4, (room - staging) / c.stage_bytes);
+    if (staged) {
+        const int keep = std::min(c.stages, 3);
+        if (room >= (size_t)keep * c.stage_bytes + whole) { c.stages = std::min<int>(c.stages, (int)((room - whole) / c.stage_bytes)); staging = whole; }
+        else staging = std::max<size_t>(staging, (room - (size_t)c.stages * c.stage_bytes) / plane_pair * plane_pair);
+        c.pool_planes = (int)(staging / plane_pair) * 2;
+        c.pool_stage_bytes = (int)staging;
     }
-    return plan_tc_conv_kpc(N, H, W, K, cin16, cout16, pool, 2);
+    c.smem_bytes = kTcFgHeader + c.stages * c.stage_bytes + (int)staging;
+    return c.stages >= 2 && (!staged || c.pool_planes >= 2);
 }
 
-TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, bool pool, int kpc3, bool stack)
+// Launch shape of the banded convolution kernel for a conv with `cout16` output and `cin16` input channels (padded)
+// on N maps of H x W: bands as tall as the accumulators allow (512 columns = blocks of 128 entries x Ns channels),
+// among those that fit the height with the fewest rounds of blocks over the SMs; as many stages as fit.
+TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, bool pool, int kpc, bool stack = false)
 {
     TcConvPlan c;
     tc_col_chunks(W, &c.ncc, &c.Cw);
@@ -855,50 +869,44 @@ TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, b
     c.nbuf = c.Ns <= 64 ? 2 : 1;
     const int max_blk = std::min(stack ? 16 : 8, kTcTmemCols / c.nbuf / c.Ns);
     c.stack = stack ? 1 : 0;
-    c.kpc = K == 1 ? std::min(cin16 / 8, 8) : kpc3;
+    c.kpc = kpc;
     const int step = pool ? 2 : 1;
     const int r_max = std::min((max_blk * 128) / c.Wp, H) / step * step;
     // With a pool, accumulator blocks of one row each where that is the faster form: the epilogue then compares in registers (350
     // cycles for 128 entries x 16 channels instead of 500 through the staging area), while rows of few columns
     // leave most of a block's 128 entries empty.
     const double mma = (double)K * K * cin16 / 16 * tc_mma_cycles(c.Ns), units = c.Ns / 16.0;
-    double best = -1;
+    TcConvPlan best;
     for (int rows = stack ? 1 : 0; rows <= (pool || stack ? 1 : 0); ++rows)
         for (int R = step; R <= (rows ? std::min(max_blk, H) / step * step : r_max); R += step) {
-            const int bands = (H + R - 1) / R * c.ncc, nblk = rows ? R : (R * c.Wp + 127) / 128;
-            const long long items = (long long)N * bands * c.slices;
-            const double m = nblk * mma, epi = nblk * units * (rows ? 350.0 : 500.0);
+            c.R = R; c.row_blocks = rows;
+            c.bands_img = (H + R - 1) / R * c.ncc;
+            c.nblk = rows ? R : (R * c.Wp + 127) / 128;
+            const long long items = (long long)N * c.bands_img * c.slices;
+            const double m = c.nblk * mma, epi = c.nblk * units * (rows ? 350.0 : 500.0);
             const double block = stack ? R + 1.5 * ((R + 3) / 4) + 1.0             // (64 + 44 n cycles a K step and window column for n rows of an issuer)
-                               : !pool ? nblk + 0.5 : (c.nbuf == 2 ? std::max(m, epi) : m + epi) + 0.5 * mma + 1000.0;      // MMAs + fixed part
-            const double cost = (double)((items + kSmCount - 1) / kSmCount) * block;                                     // x rounds
-            if (best < 0 || cost <= best) { best = cost; c.R = R; c.nblk = nblk; c.bands_img = bands; c.row_blocks = rows; }
+                               : !pool ? c.nblk + 0.5 : (c.nbuf == 2 ? std::max(m, epi) : m + epi) + 0.5 * mma + 1000.0;      // MMAs + fixed part
+            c.cost = (double)((items + kSmCount - 1) / kSmCount) * block;                                                    // x rounds
+            if (items > 0x7fffffffLL || (best.on && c.cost > best.cost) || !fit_tc_conv(c, K, pool)) continue;
+            c.items = (int)items;
+            c.blocks = (int)std::min<long long>(items, kSmCount);
+            c.on = 1;
+            best = c;
         }
-    if (best < 0) return c;
-    const size_t last = c.row_blocks ? (size_t)(c.nblk - 1) * c.Wp + 128 : (size_t)c.nblk * 128;          // entries the blocks reach over
-    const size_t entries = std::max<size_t>((size_t)(c.R + K - 1) * c.Wp, last + (size_t)(K - 1) * c.Wp + K);
-    c.x_plane = (int)align_up(entries * 16, 128);
-    c.stage_bytes = c.kpc * c.x_plane + K * K * c.kpc * c.Ns * 16;
-    // fused pool: the band as stored goes through a staging area, all channels of the slice at once where that leaves
-    // three stages (two for short rings), else 16 channels or more at a time
-    const size_t room = (size_t)kTcConvSmemBudget - kTcFgHeader;
-    const size_t plane_pair = (size_t)c.nblk * 128 * 16 * 2, whole = (size_t)(c.Ns / 16) * plane_pair;
-    const bool staged = pool && !c.row_blocks;
-    size_t staging = staged ? kTcPoolStageBytes : 0;
-    c.stages = (int)std::min<size_t>(4, (room - staging) / c.stage_bytes);
-    if (staged) {
-        const int keep = std::min(c.stages, 3);
-        if (room >= (size_t)keep * c.stage_bytes + whole) { c.stages = std::min<int>(c.stages, (int)((room - whole) / c.stage_bytes)); staging = whole; }
-        else staging = std::max<size_t>(staging, (room - (size_t)c.stages * c.stage_bytes) / plane_pair * plane_pair);
-        c.pool_planes = (int)(staging / plane_pair) * 2;
-        c.pool_stage_bytes = (int)staging;
+    return best;
+}
+
+TcConvPlan plan_tc_conv(int N, int H, int W, int K, int cin16, int cout16, bool pool)
+{
+    // Input channels per chunk: 3x3: 16, or 32 with slices of at most 64 channels (their filters are small, and every chunk costs the
+    // issuers a wait, a fence and a commit); 1x1: up to 64.  Fewer where the bands that are taller for it are worth more.
+    const bool long_chunks = K == 1 || (std::min(cout16, 128) <= 64 && cin16 >= 32);
+    const int most = K == 1 ? std::min(cin16 / 8, 8) : long_chunks ? 4 : 2;
+    TcConvPlan c = plan_tc_conv_kpc(N, H, W, K, cin16, cout16, pool, most);
+    if (most > 2) {
+        const TcConvPlan d = plan_tc_conv_kpc(N, H, W, K, cin16, cout16, pool, (most / 2 + 1) / 2 * 2);
+        if (d.on && (!c.on || d.cost < c.cost || (d.cost == c.cost && d.R > c.R))) c = d;
     }
-    if (c.stages < 2 || (staged && c.pool_planes < 2)) return c;
-    c.smem_bytes = kTcFgHeader + c.stages * c.stage_bytes + (int)staging;
-    const long long items = (long long)N * c.bands_img * c.slices;
-    if (items > 0x7fffffffLL) return c;
-    c.items = (int)items;
-    c.blocks = (int)std::min<long long>(items, kSmCount);
-    c.on = 1;
     return c;
 }
 

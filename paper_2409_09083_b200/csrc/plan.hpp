@@ -158,6 +158,7 @@ struct TcConvPlan {
     int pool_stage_bytes = 0;               //             and its size
     int row_blocks = 0, stack = 0;          // form of the kernel, see conv_tc_rows_kernel
     int nbuf = 1;                           // accumulator buffers (2 for slices of at most 64 channels)
+    double cost = 0;                        // what the planner compares shapes by
 };
 constexpr int kTcPoolStageBytes = 32 * 1024;  // least staging area of the fused pool in the banded convolution (more where it fits)
 constexpr int kTcConvSmemBudget = 224 * 1024; // banded convolution: header + stages + pool staging

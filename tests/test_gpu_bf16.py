@@ -644,3 +644,27 @@ def test_an_infinite_value_in_the_last_row_of_an_odd_height(h):
     a, b = grads
     assert np.isinf(b[:, 10, 1:]).all()                      # two rows of window positions read it ...
     assert np.array_equal(a[:, :, 0], b[:, :, 0])            # ... and the third does not
+
+
+# Layers whose tallest bands do not leave room for two stages: lower ones, or fewer channels a chunk (1x1: 4 planes of 8, in a
+# first layer of 6 channels as 4 + 4 and of 5 as 4 + 2)
+LOW = {
+    "six-channels": W("x", (conv(6, 13, 3), pool(), conv(13, 16, 3)), 13, 6, 136, 72, (1, 1), ((1, 3),)),
+    "five-channels": W("v", (conv(5, 16, 3), pool()), 14, 5, 700, 28, (1, 1), ((1, 2),)),
+    "one-by-one-narrow": W("w", (conv(3, 64, 3), conv(64, 16, 1)), 4, 3, 124, 224, (1, 1), ((1, 2),)),
+    "one-by-one-from-many": W("m", (conv(3, 528, 3), conv(528, 16, 1)), 4, 3, 124, 224, (1, 1), ((1, 2),)),
+}
+
+
+@pytest.mark.parametrize("name", sorted(LOW))
+def test_layers_whose_tallest_bands_do_not_fit(name):
+    wl = synth.with_slope(LOW[name], 0.0)
+    x, params, target = synth.draw_integer_relu(wl)
+    dy = np.random.default_rng(3).standard_normal(target.shape).astype(np.float32)
+    y, dx, dparams, plan = backward_bf16(wl, x, params, dy)
+    assert all(plan.group_mode(i)[0] == 2 for i in range(len(plan.exec_groups())))
+    ref = run_oracle(wl, x, params, dy=dy, store="bf16")
+    assert np.array_equal(y.astype(np.float64), ref["y"])
+    assert rel_err(dx, ref["dx"]) <= BF16_TOL
+    errs = per_layer_errors(list(wl.layers), dparams, ref["dparams"])
+    assert all(max(a, b) <= BF16_TOL for _, a, b in errs), errs

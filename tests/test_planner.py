@@ -351,3 +351,31 @@ def test_small_stacks_stay_on_the_multiply_add_kernels():
         assert_split(plan(n, 64, 112), layers)
     for kw in (dict(stationary=1), dict(stationary=-1), dict(precision=1)):
         assert all("split" not in k for k in kernels(plan(1, 64, 112, **kw)).values())
+
+
+@pytest.mark.parametrize("cin", range(1, 8))
+def test_bf16_first_layers_keep_the_banded_route_at_every_size(cin):
+    """Bands whose stages do not fit give way to lower ones: a 3x3 first layer with at most 7 channels never falls to the fused stacks."""
+    for cout in (8, 16, 32, 64, 128):
+        for h, w in ((57, 83), (224, 224), (416, 416), (608, 608), (40, 1000)):
+            for n in (1, 4, 16):
+                for pooled in (False, True):
+                    layers = (synth.conv(cin, cout, 3),) + ((synth.pool(),) if pooled else ()) + (synth.conv(cout, 32, 3),)
+                    if pooled and (h % 2 or w % 2):
+                        continue
+                    plan = ftp.ftp_plan(layers, n, cin, h, w, (1, 1), ((1, len(layers)),), precision=1)
+                    got = [plan.group_kernels(i, 0) for i in range(len(plan.exec_groups()))]
+                    assert got == ["banded", "banded"], (cin, cout, h, w, n, pooled, got)
+
+
+@pytest.mark.parametrize("cin,cout", [(64, 16), (128, 32), (32, 640), (31, 563), (16, 520), (640, 24)])
+def test_bf16_1x1_layers_keep_the_banded_route_at_every_size(cin, cout):
+    """... nor does a 1x1 layer with few channels on one side, which with more than 512 on the other was refused."""
+    for n, h, w in ((4, 124, 224), (37, 124, 224), (5, 104, 250), (1, 13, 13), (2, 416, 416)):
+        for pooled in (False, True):
+            if pooled and h % 2:
+                continue
+            layers = (synth.conv(3, cin, 3), synth.conv(cin, cout, 1)) + ((synth.pool(),) if pooled else ())
+            plan = ftp.ftp_plan(layers, n, 3, h, w, (1, 1), ((1, len(layers)),), precision=1)
+            got = [plan.group_kernels(i, 0) for i in range(len(plan.exec_groups()))]
+            assert got == ["banded", "banded"], (cin, cout, n, h, w, pooled, got)
