@@ -1363,7 +1363,7 @@ int build_plan(ftp_plan& p, const ftp_layer* layers, int n_layers, int N, int C,
     {
         const MapShape& s = p.maps[n_layers];
         ws.dy_off = take((size_t)N * s.C * s.H * s.W * 4);
-        if (tcp) ws.y32_off = take((size_t)N * s.C * s.H * s.W * 4);
+        if (tcp && !p.groups.back().tfg.on) ws.y32_off = take((size_t)N * s.C * s.H * s.W * 4);      // (a one-conv group's loss reads the planes)
         size_t total = (size_t)N * s.C * s.H * s.W;
         p.loss_blocks = (int)std::min<size_t>(1024, (total + 1023) / 1024);
         ws.loss_off = take((size_t)p.loss_blocks * 4);

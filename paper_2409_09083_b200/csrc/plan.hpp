@@ -242,7 +242,7 @@ struct Workspace {                 // byte offsets, all 256-aligned
     size_t loss_val_off = 0;       // the loss value (ftp_step_host)
     size_t x_stage_off = 0, t_stage_off = 0;   // device copies of a host batch (ftp_step_host): two slots each, x_stage_bytes / t_stage_bytes apart
     size_t x_stage_bytes = 0, t_stage_bytes = 0;
-    size_t y32_off = 0;            // tensor-core path: fp32 NCHW copy of the last map for the loss (ftp_step with target)
+    size_t y32_off = 0;            // tensor-core path, last group fused: fp32 NCHW copy of the last map for the loss (ftp_step with target)
     size_t err_off = 0;            // device error word of the tensor-core kernels (a bounded wait ran out)
     size_t total = 0;
 };

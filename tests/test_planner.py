@@ -379,3 +379,14 @@ def test_bf16_1x1_layers_keep_the_banded_route_at_every_size(cin, cout):
             plan = ftp.ftp_plan(layers, n, 3, h, w, (1, 1), ((1, len(layers)),), precision=1)
             got = [plan.group_kernels(i, 0) for i in range(len(plan.exec_groups()))]
             assert got == ["banded", "banded"], (cin, cout, n, h, w, pooled, got)
+
+
+def test_bf16_workspace_holds_what_the_route_of_the_last_group_reads():
+    """Bytes an output value costs: the saved map 2, the loss delta 4, two staging slots of the target 8, dz 2; a copy of the map as fp32 for
+    the loss (4) only where the last group is a fused stack, here a 5x5 layer, which has no dz."""
+    def per_value(k, **opts):
+        a, b = (ftp.ftp_plan((synth.conv(3, 16, 3), synth.conv(16, c, k)), 8, 3, 208, 208, (1, 1), ((1, 2),), precision=1, **opts) for c in (64, 128))
+        assert a.group_kernels(len(a.exec_groups()) - 1, 0) == ("fused" if k == 5 else "banded")
+        return (b.workspace_bytes - a.workspace_bytes) / (8 * 64 * 208 * 208)
+    assert 16.0 <= per_value(1) < 16.5
+    assert 18.0 <= per_value(5) < 19.5                       # (the filters of the larger layer, in 148 partial sets, are in it)
