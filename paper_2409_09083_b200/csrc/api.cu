@@ -47,6 +47,7 @@ int ensure_device(ftp_plan* p)
         cudaFuncSetAttribute(filter_grad_tc_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcFgSmemBudget) != cudaSuccess ||
         cudaFuncSetAttribute(conv_tc_rows_kernel<kConvPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcConvSmemBudget) != cudaSuccess ||
         cudaFuncSetAttribute(conv_tc_rows_kernel<kConvPool>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcConvSmemBudget) != cudaSuccess ||
+        cudaFuncSetAttribute(conv_tc_rows_kernel<kConvInput>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcConvSmemBudget) != cudaSuccess ||
         cudaFuncSetAttribute(conv_tc_rows_kernel<kConvRowPool>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcConvSmemBudget) != cudaSuccess ||
         cudaFuncSetAttribute(conv_tc_rows_kernel<kConvStack>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcConvSmemBudget) != cudaSuccess ||
         !st_prepare_device() || !split_prepare_device())
@@ -295,6 +296,7 @@ bool launch_tc_conv(ftp_plan* p, const TcConvPlan& c, int kind, int gi, const vo
       const size_t smem = one_block_smem(c.smem_bytes);
       if (c.stack) launch(conv_tc_rows_kernel<kConvStack>, c.blocks, kTcConvThreads, smem, tm.ls(), a);
       else if (c.row_blocks) launch(conv_tc_rows_kernel<kConvRowPool>, c.blocks, kTcConvThreads, smem, tm.ls(), a);
+      else if (out_f) launch(conv_tc_rows_kernel<kConvInput>, c.blocks, kTcConvThreads, smem, tm.ls(), a);
       else if (pool) launch(conv_tc_rows_kernel<kConvPool>, c.blocks, kTcConvThreads, smem, tm.ls(), a);
       else launch(conv_tc_rows_kernel<kConvPlain>, c.blocks, kTcConvThreads, smem, tm.ls(), a); }
     return launched_ok();

@@ -552,8 +552,9 @@ __device__ __forceinline__ unsigned long long pool4(const uint4& m0, const uint4
 }
 
 // One instance per form of the epilogue and the issue: a launch waits for its instructions too, and no instance spills (8 layers, 4
-// images: a step 283 us as one kernel with all forms, 276 so).
-enum { kConvPlain = 0, kConvPool = 1, kConvRowPool = 2, kConvStack = 3 };
+// images: a step 283 us as one kernel with all forms, 276 so; the fp32 output inside the plain form: 64 -> 1024 forward on 7 x 84 x 116 416 us,
+// without 415).
+enum { kConvPlain, kConvPool, kConvInput, kConvRowPool, kConvStack };      // (input, stack: the delta at the network input, out_f)
 
 template <int FORM>
 __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const __grid_constant__ TcConvRowsArgs A)
@@ -761,7 +762,7 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
             wait(&H->done[buf], use & 1u, 128);                       // asleep between polls; (ran out: the item is written from
                                                                       // whatever is there; the error word is set)
             fence_after_sync();
-            if constexpr (FORM == kConvPlain || FORM == kConvStack) {
+            if constexpr (FORM == kConvPlain || FORM == kConvInput || FORM == kConvStack) {
                 const int nc = I.cols >> 4, nunits = I.nblk * nc;
                 const size_t gstep = (size_t)A.H * A.W;
                 // where unit u (accumulator block b, channels c0 .. c0 + 15) of this thread lies in the output planes
@@ -780,13 +781,13 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                     // kernel was measured slower)
                     uint4 yq[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
                     unsigned long long amq[2] = {0ull, 0ull};
-                    if (A.prev_y && valid) {
+                    if (FORM == kConvPlain && A.prev_y && valid) {
                         yq[0] = __ldg(A.prev_y + g0); yq[1] = __ldg(A.prev_y + g0 + gstep);
                         if (A.prev_arg) { amq[0] = __ldg(A.prev_arg + g0); amq[1] = __ldg(A.prev_arg + g0 + gstep); }
                     }
                     float v[16];
                     tmem_ld16(tbuf + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * A.Ns + c0), v);
-                    if (A.out_f) {                            // (a delta: neither bias nor activation)
+                    if constexpr (FORM != kConvPlain) {       // (a delta: neither bias nor activation)
                         if (!valid) continue;
                         float* dst = A.out_f + (((size_t)I.n * A.cout + I.co0 + c0) * A.H + I.y0 + r) * A.W + I.x0 + c;
 #pragma unroll
