@@ -39,7 +39,7 @@ FP32_NOMINAL_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12
 # executed group's multiply-accumulates the launch performs (None: a memory-bound helper)
 KIND = {0: ("pack_filters", None), 1: ("fwd_group", 1), 2: ("loss_delta", None), 3: ("bwd_group", 2), 4: ("halo_sum", None),
         5: ("reduce_sgd", None), 6: ("delta_act", None), 7: ("filter_grad_rows", 1), 8: ("delta_conv_rows", 1),
-        9: ("unroll_windows", None), 10: ("input_entries", None)}
+        9: ("unroll_windows", None)}
 KERNEL = {("fwd_group", "fp32"): "fwd_group_kernel / conv_rows_kernel", ("bwd_group", "fp32"): "bwd_group_kernel / thin_bwd_kernel",
           ("filter_grad_rows", "fp32"): "filter_grad_rows_kernel", ("delta_conv_rows", "fp32"): "conv_rows_kernel (input delta)",
           ("fwd_group", "split"): "conv_split_kernel / conv_rows_kernel", ("bwd_group", "split"): "thin_bwd_kernel",

@@ -342,12 +342,18 @@ void fill_common_tc(const ftp_plan* p, const GroupPlan& g, bool backward, const 
     }
 }
 
-int pack_filters_tc(ftp_plan* p, const float* params, void* ws, int dirs, cudaStream_t st)
+// entries_x: the network input, where the first layer's entries for the backward pass are wanted along with the filters, else null
+int pack_filters_tc(ftp_plan* p, const float* params, void* ws, int dirs, cudaStream_t st, const float* entries_x = nullptr)
 {
     __nv_bfloat16* wf = reinterpret_cast<__nv_bfloat16*>(ws_ptr(ws, p->ws.wf_off));
     __nv_bfloat16* wb = reinterpret_cast<__nv_bfloat16*>(ws_ptr(ws, p->ws.wb_off));
     TcPackArgs pa{};
     PackTilesArgs ba{};
+    InputEntries e{};
+    if (entries_x && p->groups.front().narrow) {
+        const OpDesc& op = p->groups.front().fwd_ops[0];
+        e = InputEntries{entries_x, reinterpret_cast<uint4*>(ws_ptr(ws, p->ws.ent_off)), p->N, op.cin, (size_t)op.in_H * op.in_W};
+    }
     pa.dirs = ba.dirs = dirs;
     int* clear = (dirs & kPackForward) ? err_ptr(ws, p) : nullptr;       // by the first launch
     auto flush = [&]() {
@@ -361,8 +367,9 @@ int pack_filters_tc(ftp_plan* p, const float* params, void* ws, int dirs, cudaSt
         if (!ba.n) return;
         ba.error = clear; clear = nullptr;
         Timed t(p, st, 0, -1);
-        launch(pack_banded_kernel, ba.tiles, 256, 0, t.ls(), ba, params);
-        ba.n = ba.tiles = 0;
+        if (e.x) launch(pack_banded_entries_kernel, ba.tiles + (int)std::min<size_t>((e.N * e.HW + 255) / 256, (size_t)kSmCount * 16), 256, 0, t.ls(), ba, params, e);
+        else launch(pack_banded_kernel, ba.tiles, 256, 0, t.ls(), ba, params);
+        ba.n = ba.tiles = 0; e.x = nullptr;
     };
     for (const GroupPlan& g : p->groups)
         for (int i = 0; i < g.n_ops; ++i) {
@@ -1070,16 +1077,8 @@ int ftp_backward(ftp_plan* plan, const float* x, const float* dy, const float* p
     int rc = ensure_device(plan);
     if (rc != FTP_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    rc = is_tc(plan) ? pack_filters_tc(plan, params, workspace, kPackDelta, st) : pack_filters(plan, params, workspace, kPackDelta, st);
+    rc = is_tc(plan) ? pack_filters_tc(plan, params, workspace, kPackDelta, st, x) : pack_filters(plan, params, workspace, kPackDelta, st);
     if (rc != FTP_OK) return rc;
-    const GroupPlan& g = plan->groups.front();
-    if (g.narrow) {                             // (a step's forward pass writes them along with its own copy)
-        const OpDesc& op = g.bwd_ops[0];
-        const size_t HW = (size_t)op.in_H * op.in_W;
-        Timed t(plan, st, 10, 0);
-        launch(input_entries_kernel, (int)std::min<size_t>((plan->N * HW + 255) / 256, (size_t)kSmCount * 16), 256, 0, t.ls(),
-               x, reinterpret_cast<uint4*>(ws_ptr(workspace, plan->ws.ent_off)), plan->N, op.cin, HW);
-    }
     return backward_impl(plan, x, dy, params, dx, dparams, nullptr, 0.f, workspace, st);
 }
 

@@ -1094,11 +1094,42 @@ __global__ void pack_filters_tc_kernel(const __grid_constant__ TcPackArgs A, con
     }
 }
 
+// First layer's backward pass on the banded kernels: the network input as one plane of 8-channel bf16 entries, channels beyond C zero, the
+// last one 1 (the filter gradient's sums of dz x that channel at the window's centre are the bias gradient).  16 bytes a pixel
+// where the unrolled copy of the forward pass has 64 with 3 channels.
+struct InputEntries { const float* x; uint4* out; int N, C; size_t HW; };      // x null: none wanted
+
+__device__ __forceinline__ void input_entries(const InputEntries& E, size_t block, size_t blocks)
+{
+    const size_t total = (size_t)E.N * E.HW;
+    for (size_t e = block * blockDim.x + threadIdx.x; e < total; e += blocks * blockDim.x) {
+        const size_t n = e / E.HW;
+        const float* src = E.x + n * E.C * E.HW + (e - n * E.HW);
+        float v[8];
+#pragma unroll
+        for (int c = 0; c < 7; ++c) v[c] = c < E.C ? __ldg(src + c * E.HW) : 0.f;
+        v[7] = 1.f;
+        E.out[e] = tcd::pack8(v);
+    }
+}
+
 // ... and of the banded kernels (pack.cuh)
 __global__ void __launch_bounds__(256) pack_banded_kernel(const __grid_constant__ PackTilesArgs A, const float* __restrict__ params)
 {
     previous_launches();
     __shared__ float s[kPackSmemFloats];
+    pack_tiles<1>(A, params, s, [](const float* v, uint4* p) { p[0] = tcd::pack8(v); });
+}
+
+// The same for ftp_backward; the blocks behind the tiles write the entries, which do not depend on the filters (a step's forward pass has
+// them from unroll_windows_kernel).  As a launch of their own they cost 1 to 1.5 us of a call's 35 on small maps; inside the
+// kernel above its longer code cost every forward pass 1 us.
+__global__ void __launch_bounds__(256) pack_banded_entries_kernel(const __grid_constant__ PackTilesArgs A, const float* __restrict__ params,
+                                                                  const __grid_constant__ InputEntries E)
+{
+    previous_launches();
+    __shared__ float s[kPackSmemFloats];
+    if ((int)blockIdx.x >= A.tiles) { input_entries(E, blockIdx.x - A.tiles, gridDim.x - A.tiles); return; }
     pack_tiles<1>(A, params, s, [](const float* v, uint4* p) { p[0] = tcd::pack8(v); });
 }
 

@@ -47,7 +47,7 @@ struct TcFilterGradArgs {
     int K, H, W, cout16, cin16;
     int Ms, slices;                           // output channels per block (64 or 128) and number of such slices
     int ncols, nci;                           // input channels per block (multiple of 16) and number of such slices
-    int narrow;                               // first layer: x is input_entries_kernel's plane (ncols 8 or 16, the bias gradient its channel 7)
+    int narrow;                               // first layer: x is the plane of InputEntries (ncols 8 or 16, the bias gradient its channel 7)
     int units;                                // accumulator units: 3x3: K * ncols columns, one per window column; 1x1 and the first
                                               //   layer (9 * ncols columns): row pairs in turn
     int R, Cw, ncc;                           // rows per band, columns of a band and column chunks per row band
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(256) loss_planes_kernel(const __grid_constant_
 // channel -> (ci, ky, kx) arithmetic is resolved at compile time).  On that copy the forward pass is a 1x1 conv.  (On the entries
 // below it is a 3x3 conv without the copy, 99 us less for 16 x 608 x 608, but the sums of an MMA are then other ones, a few
 // rounded outputs in a million with them, and through the ties of the pools whole deltas at the network input.)
-// ent, if not null: the entries for the backward pass (see input_entries_kernel), written in the same pass.
+// ent, if not null: the entries for the backward pass (see InputEntries), written in the same pass.
 template <int C>
 __global__ void unroll_windows_kernel(const float* __restrict__ x, uint4* __restrict__ col, uint4* __restrict__ ent, int N, int H, int W)
 {
@@ -215,24 +215,6 @@ inline void launch_unroll_windows(const float* x, uint4* col, uint4* ent, int N,
         case 5: launch(unroll_windows_kernel<5>, blocks, 256, 0, st, x, col, ent, N, H, W); break;
         case 6: launch(unroll_windows_kernel<6>, blocks, 256, 0, st, x, col, ent, N, H, W); break;
         default: launch(unroll_windows_kernel<7>, blocks, 256, 0, st, x, col, ent, N, H, W); break;
-    }
-}
-
-// First layer's backward pass: the network input as one plane of 8-channel bf16 entries, channels beyond C zero, the last one 1 (the
-// filter gradient's sums of dz x that channel at the window's centre are the bias gradient).  16 bytes a pixel where the
-// unrolled copy, which the filter gradient read before, has 64 with 3 channels.  A step has it from the kernel above.
-__global__ void __launch_bounds__(256) input_entries_kernel(const float* __restrict__ x, uint4* __restrict__ out, int N, int C, size_t HW)
-{
-    previous_launches();
-    const size_t total = (size_t)N * HW;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const size_t n = e / HW;
-        const float* src = x + n * C * HW + (e - n * HW);
-        float v[8];
-#pragma unroll
-        for (int c = 0; c < 7; ++c) v[c] = c < C ? __ldg(src + c * HW) : 0.f;
-        v[7] = 1.f;
-        out[e] = tcd::pack8(v);
     }
 }
 
