@@ -1017,9 +1017,26 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_sgd_tc_kernel(const __g
     }
     const float* src = L.partial + L.tgp_off + e;
     float sum = 0.f;
-    for (int part = 0; part < parts; ++part, src += L.cout16) {
+    if (parts == 1) {
 #pragma unroll 16
         for (int k = 0; k < L.sets; ++k) sum += src[(size_t)k * L.set_floats];
+    } else {
+        // The parts of a bias have few sets each: 8 loads in flight through all of them.  (Part by part every load waited for the one
+        // before: 16 parts of 9 sets, 512 -> 32 channels on 304 x 104, the reduction 50 us, so 19; 16 layers, 2 x 336 x 464,
+        // forward pass, loss and backward pass 506 -> 477.)
+        long long at = 0;
+        int k = 0;
+        for (int left = parts * L.sets; left > 0; left -= 8) {
+            float v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                v[j] = j < left ? src[at] : 0.f;
+                at += L.set_floats;
+                if (++k == L.sets) { k = 0; at += L.cout16 - L.sets * L.set_floats; }
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) sum += v[j];
+        }
     }
     if (grad_out) grad_out[dst] = sum;
     if (params) params[dst] = params[dst] - lr * sum;
