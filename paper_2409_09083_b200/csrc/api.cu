@@ -290,7 +290,7 @@ bool launch_tc_conv(ftp_plan* p, const TcConvPlan& c, int kind, int gi, const vo
     a.Ns = c.Ns; a.slices = c.slices; a.R = c.R; a.Wp = c.Wp; a.bands_img = c.bands_img; a.nblk = c.nblk; a.kpc = c.kpc;
     a.ncc = c.ncc; a.Cw = c.Cw; a.items = c.items; a.pool_planes = c.pool_planes; a.nbuf = c.nbuf;
     a.x_plane = c.x_plane; a.stage_bytes = c.stage_bytes; a.stages = c.stages;
-    a.out_f = out_f;
+    a.out_f = out_f; a.share = c.share;
     a.hurry = (double)((c.items + c.blocks - 1) / c.blocks) * c.nblk * K * K * (cin16 / 16) * tc_mma_cycles(c.Ns) < kHurryCycles;
     { Timed tm(p, st, kind, gi);
       const size_t smem = one_block_smem(c.smem_bytes);

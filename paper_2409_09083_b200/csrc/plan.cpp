@@ -884,7 +884,12 @@ TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, b
             c.nblk = rows ? R : (R * c.Wp + 127) / 128;
             const long long items = (long long)N * c.bands_img * c.slices;
             const double m = c.nblk * mma, epi = c.nblk * units * (rows ? 350.0 : 500.0);
-            const double block = stack ? R + 1.5 * ((R + 3) / 4) + 1.0             // (64 + 44 n cycles a K step and window column for n rows of an issuer)
+            // stack: an issuer has n rows and issues n + 2 MMAs a K step and window column, one every 220 cycles almost whatever the others
+            // do (slopes over 128 to 512 channels, cycles a K step: 3 rows 2180, 6 rows 2670, 11 and 12 rows 3190 and 3350, 13 rows 3700,
+            // 16 rows 3890)
+            const int n = (R + kTcIssuers - 1) / kTcIssuers;
+            c.share = stack ? n : 0;
+            const double block = stack ? cin16 / 16 * 3.0 * ((n + 2) * 220.0 + 2.0 * R) + 2000.0
                                : !pool ? c.nblk + 0.5 : (c.nbuf == 2 ? std::max(m, epi) : m + epi) + 0.5 * mma + 1000.0;      // MMAs + fixed part
             c.cost = (double)((items + kSmCount - 1) / kSmCount) * block;                                                    // x rounds
             if (items > 0x7fffffffLL || (best.on && c.cost > best.cost) || !fit_tc_conv(c, K, pool)) continue;
@@ -972,7 +977,7 @@ void plan_tc_filter_grad(const ftp_plan& p, GroupPlan& g, const PlanOpts& o)
     g.cf = plan_tc_conv(p.N, H, W, narrow ? 1 : K, narrow ? col_cin16 : op.cin16, op.cout16, op.kind == kOpConvPool);
     g.cd = plan_tc_conv(p.N, H, W, K, op.cout16, op.cin16, false);
     // delta at the network input (16 columns): with the window rows in one MMA where the rows are long enough.  A row, a block of 128
-    // entries whatever its length, costs 180 cycles a K step so; otherwise 128 entries cost 324, whole rows or not.
+    // entries whatever its length, costs 245 cycles a K step so (16 rows on four issuers); otherwise 128 entries cost 324, whole rows or not.
     if (narrow && g.cd.on && g.cd.Wp >= 80) {
         const TcConvPlan c = plan_tc_conv_kpc(p.N, H, W, K, op.cout16, op.cin16, false, 2, true);
         if (c.on) g.cd = c;

@@ -157,6 +157,7 @@ struct TcConvPlan {
     int pool_planes = 0;                    // fused pool: 8-channel planes the staging area holds
     int pool_stage_bytes = 0;               //             and its size
     int row_blocks = 0, stack = 0;          // form of the kernel, see conv_tc_rows_kernel
+    int share = 0;                          // stack: output rows of an issuer
     int nbuf = 1;                           // accumulator buffers (2 for slices of at most 64 channels)
     double cost = 0;                        // what the planner compares shapes by
 };

@@ -445,6 +445,7 @@ struct TcConvRowsArgs {
     float slope;
     int Ns, slices;                           // output channels per item, number of slices
     int R, Wp, bands_img, nblk;               // rows per band, tile pitch, bands per image, accumulator blocks of a full band
+    int share;                                // stack: output rows of an issuer
     int ncc, Cw;                              // column chunks per row band and their width (even with the pool; Wp = Cw + K - 1)
     int kpc;                                  // 8-channel planes per chunk (3x3: 2, or 4 with narrow slices; 1x1: up to 8)
     int x_plane, stage_bytes, stages;
@@ -655,10 +656,10 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                     if constexpr (FORM == kConvStack) {
                         // An MMA reads 4 KB of A however narrow it is: with 16 columns it takes 36 cycles, with 48 44.  An input row
                         // belongs to the three output rows around it, whose accumulators are neighbouring columns, so it meets
-                        // the filters of up to three window rows (packed bottom row first) in one MMA.  An issuer has four output rows
-                        // of its own; a row's accumulators start with the input row above it.
+                        // the filters of up to three window rows (packed bottom row first) in one MMA.  An issuer has up to four output
+                        // rows of its own (A.share); a row's accumulators start with the input row above it.
                         const uint32_t wp = (uint32_t)A.Wp, kxw = (uint32_t)A.kpc * 48u;
-                        const int s0 = iw * 4, n = min(4, I.rows - s0);
+                        const int s0 = iw * A.share, n = min(4, min(A.share, I.rows - s0));      // (a bound that the compiler sees: the rows unroll)
                         const uint32_t a0 = desc_lo(xaddr, (uint32_t)A.x_plane) + (uint32_t)s0 * wp, w0 = desc_lo(waddr, 768u);
                         const uint32_t d0 = tmem + buf * 256u + (uint32_t)s0 * 16u;
                         for (int kx = 0; kx < 3; ++kx)
