@@ -467,8 +467,8 @@ constexpr int kTcConvEpiWarps = 16;           // four per lane quarter of the te
 constexpr int kTcConvEpiThreads = kTcConvEpiWarps * 32;
 constexpr int kTcConvThreads = (kTcConvEpiWarps + kTcIssuers + 1) * 32;
 
-// bias and leaky ReLU of 8 accumulators, rounded: both sides of the activation are formed and rounded, the rounded sum's sign picks
-// (3 instructions a value instead of 5.5: pairs are added, multiplied, rounded and selected together; an epilogue warp is bound by
+// bias and leaky ReLU of 8 accumulators, rounded: both sides of the activation are formed and rounded, the sign of the sum picks, which a
+// sum that rounds to zero keeps: with a slope above 1 a positive one must not become slope times itself (3 instructions a value instead of 5.5: pairs are added, multiplied, rounded and selected together; an epilogue warp is bound by
 // instruction issue).
 __device__ __forceinline__ uint4 act8(const float* v, const float* bias, float slope)
 {
@@ -482,8 +482,10 @@ __device__ __forceinline__ uint4 act8(const float* v, const float* bias, float s
             const float2 z = __fadd2_rn(make_float2(v[4 * h + 2 * j], v[4 * h + 2 * j + 1]), j ? make_float2(b.z, b.w) : make_float2(b.x, b.y));
             const float2 n = __fmul2_rn(z, s2);
             const __nv_bfloat162 zb = __float22bfloat162_rn(z), nb = __float22bfloat162_rn(n);
-            const uint32_t m = __hgt2_mask(zb, __nv_bfloat162(__ushort_as_bfloat16(0), __ushort_as_bfloat16(0)));
-            o[2 * h + j] = (*reinterpret_cast<const uint32_t*>(&zb) & m) | (*reinterpret_cast<const uint32_t*>(&nb) & ~m);
+            const uint32_t zw = *reinterpret_cast<const uint32_t*>(&zb);
+            uint32_t m;
+            asm("prmt.b32 %0, %1, 0, 0xBB99;" : "=r"(m) : "r"(zw));      // the halves' signs, spread over their bits
+            o[2 * h + j] = (*reinterpret_cast<const uint32_t*>(&nb) & m) | (zw & ~m);
         }
     }
     return make_uint4(o[0], o[1], o[2], o[3]);

@@ -668,3 +668,19 @@ def test_layers_whose_tallest_bands_do_not_fit(name):
     assert rel_err(dx, ref["dx"]) <= BF16_TOL
     errs = per_layer_errors(list(wl.layers), dparams, ref["dparams"])
     assert all(max(a, b) <= BF16_TOL for _, a, b in errs), errs
+
+
+@pytest.mark.parametrize("slope", [0.0, 0.1, 4.0])
+@pytest.mark.parametrize("pooled", [False, True])
+def test_sums_that_round_to_zero_keep_their_side_of_the_activation(slope, pooled):
+    """Biases below half of the smallest bf16 value (2^-134) on a zero input: a positive sum is stored as it rounds, 0, not as `slope` times
+    itself; a negative one as slope times itself rounds."""
+    layers = (conv(3, 16, 3, leaky=slope), conv(16, 16, 1, leaky=slope)) + ((pool(),) if pooled else ())
+    wl = W("tiny", layers, 1, 3, 8, 24, (1, 1), ((1, 1), (2, len(layers))))
+    params = np.zeros(16 * 28 + 16 * 17, np.float32)
+    z = np.array([1, -1, 0.9, -0.9, 0.3, -0.3, 1.1, -1.1] * 2, np.float64) * 2.0 ** -134
+    params[-16:] = z
+    y, plan = forward_bf16(wl, np.zeros((1, 3, 8, 24), np.float32), params)
+    assert plan.group_mode(1)[0] == 2
+    want = np.where(z > 0, z, slope * z).astype(np.float32)
+    assert np.array_equal(y, np.broadcast_to(bf16_grid(want)[None, :, None, None], y.shape))
