@@ -194,6 +194,16 @@ enum {
 };
 int ftp_plan_group_kernels(const ftp_plan* plan, int group, int pass, int* kernels);
 
+/* Shape of one launch (0 forward convolution, 1 input delta, 2 filter gradient) of an EXECUTED group on FTP_KERNELS_BANDED: the rows and
+ * columns of a band and, for the convolutions, how its pixels are dealt out to accumulator blocks.  Any out pointer may be NULL.
+ * FTP_ERR_ARG on a bad index or launch and for groups on other kernels. */
+enum {
+    FTP_BANDS_ENTRIES = 0,   /* 128 consecutive pixels of the band */
+    FTP_BANDS_ROWS    = 1,   /* a row each: the 2x2 maximum is then taken in registers */
+    FTP_BANDS_STACKED = 2    /* a row each, an input row multiplied with the filters of three window rows at once (delta at the network input) */
+};
+int ftp_plan_bands(const ftp_plan* plan, int group, int launch, int* form, int* rows, int* columns);
+
 void ftp_plan_destroy(ftp_plan* plan);
 
 /*

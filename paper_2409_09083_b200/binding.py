@@ -54,6 +54,8 @@ _lib.ftp_plan_group_mode.argtypes = [_vp, _i, ctypes.POINTER(_i), ctypes.POINTER
 _lib.ftp_plan_group_mode.restype = _i
 _lib.ftp_plan_group_kernels.argtypes = [_vp, _i, _i, ctypes.POINTER(_i)]
 _lib.ftp_plan_group_kernels.restype = _i
+_lib.ftp_plan_bands.argtypes = [_vp, _i, _i, ctypes.POINTER(_i), ctypes.POINTER(_i), ctypes.POINTER(_i)]
+_lib.ftp_plan_bands.restype = _i
 _lib.ftp_plan_destroy.argtypes = [_vp]
 _lib.ftp_plan_destroy.restype = None
 _lib.ftp_plan_region.argtypes = [_vp, _i, _i, _i, _i, _i, ctypes.POINTER(_i * 4)]
@@ -252,6 +254,13 @@ class Plan:
         k = _i()
         _check(_lib.ftp_plan_group_kernels(self._h, group, pass_, ctypes.byref(k)))
         return ("fused", "rows", "banded", "split")[k.value]
+
+    def bands(self, group, launch=0):
+        """(form, rows, columns) of the bands of one launch (0 forward, 1 input delta, 2 filter gradient) of executed group `group` on
+        the banded kernels; form "entries", "rows" or "stacked"."""
+        f, r, c = _i(), _i(), _i()
+        _check(_lib.ftp_plan_bands(self._h, group, launch, ctypes.byref(f), ctypes.byref(r), ctypes.byref(c)))
+        return ("entries", "rows", "stacked")[f.value], r.value, c.value
 
     def region(self, pass_, group, map_index, ty, tx):
         """(x1, y1, x2, y2), inclusive, of user tile (ty, tx) at map X_{map_index}."""

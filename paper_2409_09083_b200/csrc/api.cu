@@ -978,6 +978,18 @@ int ftp_plan_group_kernels(const ftp_plan* plan, int group, int pass, int* kerne
     return FTP_OK;
 }
 
+int ftp_plan_bands(const ftp_plan* plan, int group, int launch, int* form, int* rows, int* columns)
+{
+    if (!plan || group < 0 || group >= (int)plan->groups.size() || launch < 0 || launch > 2) return FTP_ERR_ARG;
+    const GroupPlan& g = plan->groups[group];
+    if (!g.tfg.on) return FTP_ERR_ARG;
+    const TcConvPlan& c = launch ? g.cd : g.cf;
+    if (form) *form = launch == 2 ? FTP_BANDS_ENTRIES : c.stack ? FTP_BANDS_STACKED : c.row_blocks ? FTP_BANDS_ROWS : FTP_BANDS_ENTRIES;
+    if (rows) *rows = launch == 2 ? g.tfg.R : c.R;
+    if (columns) *columns = launch == 2 ? g.tfg.Cw : c.Cw;
+    return FTP_OK;
+}
+
 void ftp_plan_destroy(ftp_plan* plan)
 {
     if (!plan) return;

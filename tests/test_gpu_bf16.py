@@ -556,9 +556,9 @@ def test_filter_gradient_at_the_edges_of_its_slices_and_bands(cin, cout, k, n, h
     assert len(errors) == 2 and all(max(e[1:]) <= 1e-2 for e in errors)
 
 
-# Stacks whose pools run on accumulator blocks of one row (rows of about 80 to 126 columns: 84, 126, 104 a chunk, an odd number of
-# row pairs, one row pair), whose input delta stacks the window rows (bands of 16 rows and of fewer, rows that the issuers share
-# unevenly) and whose first layer has 1, 3 and 7 channels, with 64 and with more rows an MMA; the loss below a pool and not.
+# Stacks whose pools run on accumulator blocks of one row (rows of about 80 to 126 columns: 84, 126, 104 a chunk, one row pair a band), whose input
+# delta stacks the window rows (one row a band) and whose first layer has 1, 3 and 7 channels, with 64 and with more rows an MMA; the
+# loss below a pool and not.  Bands of several rows and pairs: BANDS below.
 ROWS = {
     "one-row-pair": W("o", (conv(3, 32, 3), pool(), conv(32, 64, 3)), 2, 3, 2, 252, (1, 1), ((1, 3),)),
     "pools-of-narrow-layers": W("p", (conv(3, 32, 3), pool(), conv(32, 56, 3), pool()), 1, 3, 44, 336, (2, 2), ((1, 4),)),
@@ -684,3 +684,99 @@ def test_sums_that_round_to_zero_keep_their_side_of_the_activation(slope, pooled
     assert plan.group_mode(1)[0] == 2
     want = np.where(z > 0, z, slope * z).astype(np.float32)
     assert np.array_equal(y, np.broadcast_to(bf16_grid(want)[None, :, None, None], y.shape))
+
+
+# One first layer: (output channels, pooled, N, H, W, rows of a band of the forward pass and of the input delta).  Row pools of two to four
+# pairs with a short last band; stacked deltas of 13 rows (four issuers with 4, 4, 4 and 1; last band 5), 10 (3, 3, 3, 1; last band 6), 9 (3, 3, 3;
+# last band 4), 7 (2, 2, 2, 1), 5 (2, 2, 1) and 4 (one each; last band 1)
+BANDS = [(32, True, 6, 50, 76, 4, None), (32, True, 3, 200, 90, 6, 5), (16, True, 6, 146, 84, 8, 7), (32, False, 3, 200, 312, None, 13),
+         (32, False, 2, 336, 464, None, 10), (24, False, 1, 1210, 90, None, 9), (32, False, 2, 160, 224, None, 5), (48, False, 4, 61, 224, None, 4)]
+
+
+@pytest.mark.parametrize("cout,pooled,n,h,w,rows,delta_rows", BANDS)
+def test_bands_of_several_rows(cout, pooled, n, h, w, rows, delta_rows):
+    """Integers in the forward pass: bit for bit.  A delta on the bf16 grid and slope 0: dz is exact, so the input delta is a sum of 9 cout exact
+    products in fp32, within 9 x 48 x 2^-23 (5e-5) of the sum of magnitudes, taken as 1e-4 of the largest; the filter
+    gradient sums up to 3e5 products of random signs, 1e-3."""
+    layers = (conv(3, cout, 3),) + ((pool(),) if pooled else ())
+    wl = synth.with_slope(W("bands", layers, n, 3, h, w, (1, 1), ((1, len(layers)),)), 0.0)
+    x, params, target = synth.draw_integer_relu(wl)
+    dy = bf16_grid(np.random.default_rng(3).standard_normal(target.shape))
+    y, dx, dparams, plan = backward_bf16(wl, x, params, dy)
+    if rows:
+        assert plan.bands(0, 0)[:2] == ("rows", rows)
+    if delta_rows:
+        assert plan.bands(0, 1)[:2] == ("stacked", delta_rows)
+    ref = run_oracle(wl, x, params, dy=dy, store="bf16")
+    assert np.array_equal(y.astype(np.float64), ref["y"])
+    assert rel_err(dx, ref["dx"]) <= 1e-4
+    errs = per_layer_errors(list(wl.layers), dparams, ref["dparams"])
+    assert all(max(a, b) <= 1e-3 for _, a, b in errs), errs
+
+
+# (input channels, output channels, window, N, H, W, more than 16 sets?) of a second layer: sets shared out to lanes with a last tile that is half
+# full (3x3: 16 x 13 filters; 1x1) or holds one row; one thread a value with several parts of a bias beside padded input channels; the
+# parts of a bias beyond a batch of 8 loads and not a multiple of it
+SETS = [(16, 13, 3, 8, 24, 24, True), (48, 13, 1, 8, 24, 24, True), (16, 2, 3, 8, 24, 24, True), (56, 24, 3, 8, 24, 24, True), (104, 130, 3, 3, 20, 20, False),
+        (528, 16, 3, 2, 12, 20, False), (560, 40, 1, 4, 12, 20, False)]
+
+
+@pytest.mark.parametrize("cin,cout,k,n,h,w,many", SETS)
+def test_reduction_of_the_sets_at_the_edges_of_its_tiles(cin, cout, k, n, h, w, many):
+    layers = (conv(3, cin, 3, leaky=1.0), conv(cin, cout, k, leaky=1.0))
+    plan = ftp.ftp_plan(layers, n, 3, h, w, (1, 1), ((1, 1), (2, 2)), precision=BF16)
+    assert (plan.group_mode(1)[1] > 16) == many, plan.group_mode(1)
+    test_filter_gradient_at_the_edges_of_its_slices_and_bands(cin, cout, k, n, h, w)
+
+
+NONFINITE = {
+    "chain": W("a", (conv(3, 32, 3), conv(32, 64, 3), conv(64, 16, 1)), 2, 3, 22, 90, (1, 1), ((1, 3),), x_dist="normal"),
+    "pools": W("b", (conv(3, 32, 3), pool(), conv(32, 80, 3), pool()), 2, 3, 44, 168, (1, 1), ((1, 4),), x_dist="normal"),
+    "staged-pools": W("c", (conv(3, 16, 3), pool(), conv(16, 140, 3), pool(), conv(140, 16, 1)), 2, 3, 48, 40, (1, 1), ((1, 5),), x_dist="normal"),
+}
+
+
+@pytest.mark.filterwarnings("ignore:invalid value encountered")
+@pytest.mark.parametrize("name", sorted(NONFINITE))
+def test_infinities_and_nans_through_the_banded_epilogues(name):
+    """Activation, pool, un-pooled delta and derivative: the last map and the input delta are infinite (with their signs) or NaN exactly where the
+    untiled sums are."""
+    wl = NONFINITE[name]
+    x, params, target = synth.draw(wl, bias_std=0.1)
+    x, params = bf16_grid(x), bf16_grid(params)
+    dy = bf16_grid(np.random.default_rng(1).standard_normal(target.shape))
+    x[0, 1, 9, 12], x[1, 2, 5, 30], x[0, 0, 19, 35] = np.inf, -np.inf, np.nan
+    dy[1, 5, 3, 4], dy[1, 2, -1, -1] = np.inf, np.nan
+    ref = run_oracle(wl, x, params, dy=dy, store="bf16")
+    y, dx, _, plan = backward_bf16(wl, x, params, dy)
+    assert all(plan.group_mode(i)[0] == 2 for i in range(len(plan.exec_groups())))
+    for k, g in (("y", y), ("dx", dx)):
+        assert np.array_equal(classes(g), classes(ref[k])), (k, int((classes(g) != classes(ref[k])).sum()))
+        assert np.isfinite(ref[k]).any() and not np.isfinite(ref[k]).all()
+
+
+@pytest.mark.parametrize("name", sorted(NONFINITE))
+@pytest.mark.parametrize("finite", [True, False])
+def test_a_step_has_the_delta_of_its_loss(name, finite):
+    """The loss pass of a step makes dz from the saved planes; forward pass, ftp_loss_mse and ftp_backward go through the fp32 map and delta: the same
+    bits, infinities and NaNs among them."""
+    wl = NONFINITE[name]
+    x, params, target = synth.draw(wl, bias_std=0.1)
+    if not finite:
+        target[0, 3, 2, 5], target[1, 0, -1, -1], x[0, 1, 9, 12] = np.inf, np.nan, -np.inf
+    plan = ftp.ftp_plan(wl.layers, wl.N, wl.C, wl.H, wl.W, wl.grid, wl.groups, precision=BF16)
+    ws = plan.new_workspace()
+    xd, pd, td = (torch.from_numpy(a).cuda() for a in (x, params, target))
+    a, b = (dict(g=torch.empty_like(pd), dx=torch.empty_like(xd), loss=torch.zeros(1, device="cuda")) for _ in range(2))
+    ftp.ftp_step_grad(plan, xd, pd, a["g"], ws, target=td, loss_out=a["loss"], dx=a["dx"])
+    y, dy = torch.empty_like(td), torch.empty_like(td)
+    ftp.ftp_forward(plan, xd, pd, y, ws)
+    ftp.ftp_loss_mse(plan, y, td, dy, b["loss"], ws)
+    ftp.ftp_backward(plan, xd, dy, pd, b["dx"], b["g"], ws)
+    plan.check(ws)
+    for k in ("g", "dx"):
+        assert np.array_equal(a[k].cpu().numpy(), b[k].cpu().numpy(), equal_nan=True), k
+    if finite:
+        assert a["loss"].item() == pytest.approx(b["loss"].item(), rel=1e-5)      # (two orders of fp32 sums)
+    else:
+        assert np.isnan(a["loss"].item()) and np.isnan(b["loss"].item())

@@ -390,3 +390,17 @@ def test_bf16_workspace_holds_what_the_route_of_the_last_group_reads():
         return (b.workspace_bytes - a.workspace_bytes) / (8 * 64 * 208 * 208)
     assert 16.0 <= per_value(1) < 16.5
     assert 18.0 <= per_value(5) < 19.5                       # (the filters of the larger layer, in 148 partial sets, are in it)
+
+
+def test_bands_of_a_banded_group():
+    """Forms and rows that the planner reports; only groups on the banded kernels have bands."""
+    plan = ftp.ftp_plan((synth.conv(3, 32, 3), synth.pool(), synth.conv(32, 32, 3)), 3, 3, 200, 312, (1, 1), ((1, 3),), precision=1)
+    for gi, forms in enumerate((("rows", "stacked", "entries"), ("entries",) * 3)):
+        for launch in range(3):
+            form, rows, cols = plan.bands(gi, launch)
+            h, w = ((200, 312), (100, 156))[gi]
+            assert form == forms[launch] and 1 <= rows <= h + 1 and 1 <= cols <= min(128, w + 7)
+    for gi, launch in ((-1, 0), (2, 0), (0, -1), (0, 3)):
+        assert _code(lambda: plan.bands(gi, launch)) == -1
+    fused = ftp.ftp_plan((synth.conv(3, 16, 5),), 1, 3, 32, 32, (1, 1), ((1, 1),), precision=1)
+    assert _code(lambda: fused.bands(0, 0)) == -1
