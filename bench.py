@@ -48,7 +48,7 @@ KERNEL = {("fwd_group", "fp32"): "fwd_group_kernel / conv_rows_kernel", ("bwd_gr
           ("filter_grad_rows", "bf16"): "filter_grad_tc_rows_kernel", ("delta_conv_rows", "bf16"): "conv_tc_rows_kernel (input delta)"}
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel, from the ncu captures summarised
 # under profiles/ (static: null for every kernel / workload without a capture of the current code)
-NCU_TRAFFIC = {("C3", "bf16", "fwd_group"): 84.7e6, ("C3", "bf16", "filter_grad_rows"): 153.2e6, ("C3", "bf16", "delta_conv_rows"): 201.5e6}
+NCU_TRAFFIC = {("C3", "bf16", "fwd_group"): 84.8e6, ("C3", "bf16", "filter_grad_rows"): 130.0e6, ("C3", "bf16", "delta_conv_rows"): 180.1e6}
 
 
 def measured_bf16_peak():

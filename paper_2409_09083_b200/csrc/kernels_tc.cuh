@@ -1042,7 +1042,9 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_sgd_tc_kernel(const __g
     if (params) params[dst] = params[dst] - lr * sum;
 }
 
-// Deals the layers of `a` out in tiles and launches the reduction.
+// Deals the layers of `a` out in tiles and launches the reduction.  Where the lines lie, us a step: sets shared out to lanes from more than
+// 16 of them (more than 8: 16 layers on 2 x 336 x 464 477 -> 482; more than 32: the same); 256 filters a tile from 2048 tiles of
+// 128 on (never: 23 layers with 8 images 1352 -> 1365; from 256 tiles: the same).
 inline void launch_reduce(TcReduceArgs& a, float* params, float lr, float* grad_out, LaunchStream st)
 {
     long long tiles = 0;

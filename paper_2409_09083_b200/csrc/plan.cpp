@@ -889,6 +889,8 @@ TcConvPlan plan_tc_conv_kpc(int N, int H, int W, int K, int cin16, int cout16, b
             // 16 rows 3890)
             const int n = (R + kTcIssuers - 1) / kTcIssuers;
             c.share = stack ? n : 0;
+            // The others have a fixed part for their first copies, MMAs and the hand-over.  (Without it bands get too low, a step of 8 layers with 4
+            // images 268 -> 283 us, 16 layers with 16 images 2234 -> 2457; twice as large it changes nothing.)
             const double block = stack ? cin16 / 16 * 3.0 * ((n + 2) * 220.0 + 2.0 * R) + 2000.0
                                : !pool ? c.nblk + 0.5 : (c.nbuf == 2 ? std::max(m, epi) : m + epi) + 0.5 * mma + 1000.0;      // MMAs + fixed part
             c.cost = (double)((items + kSmCount - 1) / kSmCount) * block;                                                    // x rounds
@@ -919,7 +921,10 @@ TcConvPlan plan_tc_conv(int N, int H, int W, int K, int cin16, int cout16, bool 
 // ncols input channels (all window positions of a slice fit the 512 tensor-memory columns), bands of R rows x Cw columns whose two
 // stages fit in shared memory, and pixel shares, at most one round of blocks where the slices leave SMs.  The shape with the
 // least expected time wins: bands of a share x the larger of their MMAs (shared memory delivers 128 bytes a cycle to
-// them) and their copies (22 bytes a cycle and SM from L2), plus writing and reading the partial sets.
+// them) and their copies (22 bytes a cycle and SM from L2, a little above the 20 that the widest layers reach), a hand-over of 300 cycles a
+// band and 6000 cycles a block for its start, its last band and the set that it writes, plus writing and reading the partial sets.
+// us a step of 8 layers with 4 images | 16 with 16 | 16, 2 x 336 x 464 | 23 with 8: so 268 | 2234 | 477 | 1352; without the 300 and 6000
+// 268 | 2295 | 503 | 1390; with 900 and 15000 271 | 2224 | 484 | 1367; with 16 bytes a cycle 277 | 2241 | 480 | 1358.
 void plan_tc_filter_grad(const ftp_plan& p, GroupPlan& g, const PlanOpts& o)
 {
     g.tfg = TcFgPlan{};
@@ -976,8 +981,9 @@ void plan_tc_filter_grad(const ftp_plan& p, GroupPlan& g, const PlanOpts& o)
     const int col_cin16 = round_up(9 * op.cin, 16);
     g.cf = plan_tc_conv(p.N, H, W, narrow ? 1 : K, narrow ? col_cin16 : op.cin16, op.cout16, op.kind == kOpConvPool);
     g.cd = plan_tc_conv(p.N, H, W, K, op.cout16, op.cin16, false);
-    // delta at the network input (16 columns): with the window rows in one MMA where the rows are long enough.  A row, a block of 128
-    // entries whatever its length, costs 245 cycles a K step so (16 rows on four issuers); otherwise 128 entries cost 324, whole rows or not.
+    // Delta at the network input (16 columns): with the window rows in one MMA where the rows are long enough, as a row is then a block
+    // of 128 entries whatever its length.  us of the launch, entries | stacked, 16 images of 96 rows: 70 columns, 32 channels 12.8 | 14.8;
+    // 78 columns 14.8 | 14.9; 86 columns, 64 channels 19.0 | 16.9; 104 columns 21.0 | 16.9.
     if (narrow && g.cd.on && g.cd.Wp >= 80) {
         const TcConvPlan c = plan_tc_conv_kpc(p.N, H, W, K, op.cout16, op.cin16, false, 2, true);
         if (c.on) g.cd = c;

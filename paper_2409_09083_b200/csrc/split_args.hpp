@@ -83,7 +83,7 @@ void split_launch_delta(const SplitDeltaArgs& a, LaunchStream ls);
 
 // Packing launches (pack.cuh): 32 x 32 channel tiles [tile_begin, next layer's tile_begin) of a layer.
 struct PackTilesLayer { long long p_off; uint4* wf; uint4* wd; int cin, cout, k, cin16, cout16, ns_f, kpc_f, ns_d, kpc_d, tile_begin;
-                        int stack_d;      // the rotated arrangement by window column, its rows from the last to the first (see TcConvRowsArgs::stack)
+                        int stack_d;      // the rotated arrangement by window column, its rows from the last to the first (the stacked form of conv_tc_rows_kernel)
                         int only; };      // 1 / 2: the forward arrangement / the rotated one only
 constexpr int kPackTilesLayers = 32;
 struct PackTilesArgs {

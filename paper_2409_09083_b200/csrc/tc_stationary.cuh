@@ -21,8 +21,9 @@
 // stride: an MMA covers the three window rows of its column, K * ncols accumulator columns, and the window column moves the
 // start by an entry.  With one MMA per window position instead (48 columns each, both operands from shared memory) an MMA took
 // the 44 cycles in which shared memory delivers 5.5 KB, for 24 cycles of arithmetic, and dz was read nine times
-// for a K step; 144 columns take 72 cycles and dz is read three times.  Now the copies bound it: 93 KB a band at 20 bytes a cycle
-// and SM.  us before and after: 256 -> 512, 16 x 38 x 38: 97 -> 66 (826 TFLOP/s); 128 -> 256, 76 x 76: 81 -> 60; 64 -> 128,
+// for a K step; 144 columns take 72 cycles and dz is read three times.  Now it waits for copies: no unit is near its limit (4 images of
+// 38 x 38, 256 -> 512: tensor core 33 %, L2 26 %, shared memory 39 %), but of the two stages one is read while the other's 93 KB
+// arrive, at about 20 bytes a cycle and SM.  us before and after: 256 -> 512, 16 x 38 x 38: 97 -> 66 (826 TFLOP/s); 128 -> 256, 76 x 76: 81 -> 60; 64 -> 128,
 // 152 x 152: 91 -> 52; 32 -> 64, 304 x 304: 112 -> 76; 256 -> 512 on 8 x 13 x 13: 40 -> 26; 1x1 512 -> 256: 29 -> 21.
 // Two stages (copies of the next band behind the MMAs of this one).
 #pragma once
@@ -245,7 +246,7 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
     const int nb = b_hi - b_lo;
     // input tile: planes, entries of a plane's row, entries from row to row.  First layer: each row three times, shifted by the window
     // column, in the place of planes, so that all nine window positions of its few channels stand at one stride and share an
-    // MMA (three MMAs of 24 columns took 37 cycles each: 142 us a launch for 16 x 608 x 608, 3 -> 32, now 101, 473 MB).
+    // MMA (on the unrolled copy with K = 1 144 us a launch for 16 x 608 x 608, 3 -> 32; with three MMAs of 24 columns 142; now 101, 479 MB).
     const bool turns = K == 1 || A.narrow;
     const int np = A.ncols / 8, Wx = A.narrow ? A.Cw : A.Cw + K - 1, pitch = (A.narrow ? 3 : 1) * np * Wx;
     // Pixels that only fill up a K step have zero dz, and a zero times an infinite input is NaN: they must not meet pixels of the map.
@@ -426,11 +427,11 @@ __global__ void __launch_bounds__(kTcFgThreads, 1) filter_grad_tc_rows_kernel(co
 // streams all filters of the layer once per 128 pixels, the filters read per pixel shrink by the number of
 // accumulator blocks and the pixels per block no longer depend on the grid.
 //
-// Persistent blocks (one per SM) walk over the items; the warps have fixed roles: warps 0-7 read the accumulators
-// back (bias, leaky ReLU, bf16 planes; with a fused 2x2 pool through a small staging area, 16 channels or more at
-// a time, first maximum in window order, with the arg-max bytes the backward pass routes deltas by), lane 0 of
-// warps 8-11 issues the MMAs (each for its own accumulator blocks), lane 0 of warp 12 issues the copies and runs
-// ahead into the next item while the accumulators of the current one are read back.
+// Persistent blocks (one per SM) walk over the items; the warps have fixed roles: warps 0-15 read the accumulators
+// back (bias, leaky ReLU, bf16 planes; with a fused 2x2 pool the first maximum in window order, with the arg-max bytes the
+// backward pass routes deltas by: from accumulator blocks of one row in registers, from blocks of 128 entries through a staging
+// area, 16 channels or more at a time), lane 0 of warps 16-19 issues the MMAs (each for its own accumulator blocks), lane 0 of
+// warp 20 issues the copies and runs ahead into the next item while the accumulators of the current one are read back.
 // ---------------------------------------------------------------------------------------------
 struct TcConvRowsArgs {
     alignas(64) unsigned char tmap_x[128];    // input planes (rows of 2 W eight-byte elements): box = Wp pixels x (R + K - 1) rows
@@ -717,8 +718,7 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
             mma_commit(smem_u32(&H->drain));
         }
     } else {
-        // epilogue warps: lane quarter q = warp % 4 of every accumulator block; the two warps of a quarter take
-        // alternate blocks
+        // epilogue warps: lane quarter q = warp % 4 of every accumulator block
         const int q = warp & 3, part = warp >> 2;                  // the warps of a quarter share its (block, 16 columns) units
         constexpr int kParts = kTcConvEpiWarps / 4;
         const int oplanes = A.cout16 / 8;
@@ -792,8 +792,8 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
                             const uint32_t alo = (uint32_t)amq[h] & 0x03030303u, ahi = (uint32_t)(amq[h] >> 32) & 0x03030303u;
                             const int W2 = 2 * A.W;
                             uint4* o2 = A.out + (((size_t)I.n * oplanes + ((I.co0 + c0) >> 3) + h) * (2 * A.H) + 2 * (I.y0 + r)) * W2 + 2 * (I.x0 + c);
-                            // (a 32-byte store covers a whole sector; as two of 16 bytes: us of the launch 178 -> 146, 64 -> 32 channels to
-                            // 16 x 608 x 608; 95 -> 75, 128 -> 64 channels to 304 x 304)
+                            // (a 32-byte store covers a whole sector; as two of 16 bytes: us of the launch 177 -> 150, 64 -> 32 channels to
+                            // 16 x 608 x 608; 96 -> 76, 128 -> 64 channels to 304 x 304)
                             auto member = [&](uint32_t w) {
                                 const uint32_t ml = __vcmpeq4(alo, w * 0x01010101u), mh = __vcmpeq4(ahi, w * 0x01010101u);
                                 return make_uint4(dq.x & __byte_perm(ml, 0u, 0x1100), dq.y & __byte_perm(ml, 0u, 0x3322),
@@ -807,7 +807,8 @@ __global__ void __launch_bounds__(kTcConvThreads, 1) conv_tc_rows_kernel(const _
             } else if constexpr (FORM == kConvRowPool) {
                 // The rows of a window are the same lanes of two blocks and its columns two neighbouring lanes: no staging area and
                 // no barriers.  The even lane takes the lower 8 channels of a unit, the odd lane the upper ones.
-                // us, staged and so: 3 -> 32, 16 x 608 x 608 164 -> 143; 32 -> 64, 304 x 304 127 -> 101.
+                // us, staged and so (with the cheaper activation and an instance of its own): 3 -> 32, 16 x 608 x 608 152 -> 130; 32 -> 64,
+                // 304 x 304 123 -> 95.
                 const int OH = A.H >> 1, OW = A.W >> 1, nc = I.cols >> 4, odd = lane & 1, col = q * 32 + lane;
                 const bool valid = (col & ~1) < I.cw;
                 for (int u = part; u < (I.rows >> 1) * nc; u += kParts) {
